@@ -82,9 +82,10 @@ typedef int32_t pc_status;
                                   Sec. II.B), so the reached set decides every
                                   configuration first and the FP32 recursion
                                   then runs, for exactly first_hit - 1 steps,
-                                  on the percolating ones only.  In pc_inspect
-                                  and pc_inspect_occupancy both solvers apply
-                                  it; on the streamed path the call waits for
+                                  on the percolating ones only.  The wavefront
+                                  solver always decides first; the forced
+                                  solvers do with this flag, and with
+                                  PC_MODE_STREAM the call waits for
                                   the verdicts before it starts the FP32
                                   solves (it synchronises cuda_stream even with
                                   PC_OUT_DEVICE).  pc_batch_run's streamed
@@ -140,11 +141,17 @@ pc_status pc_occupancy_fixed(int32_t W, int32_t L, int64_t n_metallic, uint64_t 
  * Errors: PC_ERR_ARG, PC_ERR_OOM, PC_ERR_CUDA, PC_ERR_INTERNAL, and
  * PC_ERR_TIMEOUT if a bounded device wait of the streamed solver expires
  * (host outputs only: with PC_OUT_DEVICE the call returns before the device
- * work ends, except with PC_VERDICT_FIRST on the streamed path).
- * Solvers: the resident one where a configuration's state fits one CTA's
- * shared memory, else the streamed one; with PC_BITS_ONLY the streamed path
- * runs 32 steps per visit of a slab where one thread-block cluster holds the
- * cross-section (pc_bits_blocked_shape).
+ * work ends, except with PC_VERDICT_FIRST and PC_MODE_STREAM).
+ * Solvers: without a PC_MODE flag the wavefront solver, which updates each
+ * reached site once, at the step at which mass first arrives there (the
+ * probability at the first hit is a sum over shortest walks, so nothing else
+ * of the vector enters it; its terms and their additions are the full
+ * recursion's, only the last sum over the end layer has a fixed order of its
+ * own).  PC_MODE_RESIDENT and PC_MODE_STREAM run the full recursion over the
+ * causal window: the resident one keeps a configuration's state in one CTA's
+ * shared memory (PC_ERR_OOM where it does not fit), the streamed one in HBM;
+ * with PC_BITS_ONLY the streamed path runs 32 steps per visit of a slab where
+ * one thread-block cluster holds the cross-section (pc_bits_blocked_shape).
  */
 pc_status pc_inspect(int32_t W, int32_t L, double p, uint64_t seed,
                      int64_t config_begin, int64_t n_configs,

@@ -1,0 +1,891 @@
+// wave.cu -- wavefront solver: every reached site is updated once, at the
+// step at which mass first arrives there (Sec. II.B, Eqs. (2)-(4)).
+//
+// Why once is enough.  The outputs are the first step with non-zero detector
+// probability, whether there is one, the step at which the reached set stops
+// growing, and the detector probability at the first hit.  That probability is
+// a sum over the walks that reach the detector in exactly first_hit moves; none
+// is shorter, so after k moves each of them stands on a site at distance k
+// from the start layer.  Of the vector nu_k only the entries of the sites whose
+// distance is k ("level" k, the sites that enter the reached set at step k)
+// ever reach the detector, and for such a site the sum over its 14 contacts is
+// the sum over its contacts of level k - 1: contacts at distance k and k + 1
+// hold nothing at step k - 1.  The terms and their additions are those of the
+// full recursion with zeros in the other places, so that the sums are equal
+// to it to the bit.  Once every entry of a level has underflowed to 0 all
+// later ones are 0, as in the full FP32 recursion.
+//
+// wave_kernel<.., false>: levels of every configuration (verdict, first_hit,
+//   m_stop), and the list of the percolating ones.
+// wave_kernel<.., true>: the levels of the listed configurations again, with
+//   nu, until the end layer is reached or nu has vanished.
+//
+// A "group" (one warp, or one CTA) takes configurations from a counter.  It
+// keeps
+//   U      bits: metallic and not yet reached, word [w][pos] = tubes 32w ..
+//          32w + 31 at plane position pos (layout in lattice.cu: contacts lie
+//          at fixed offsets from the position, and positions outside the
+//          hexagon are zero).  Word rows [wb, wb + NR) live in shared memory
+//          (a ring), the others in device scratch, where the few sites whose
+//          contacts lie outside the window are handled with global atomics.
+//   queues the sites of the current and of the next level, packed t << pb |
+//          pos.  Sites beyond the queue's capacity are kept as bits of an
+//          overflow map in device scratch, so that no level is too large.
+// A level: each site of the current one tests its 14 contacts in U and claims
+// the set ones (atomicAnd), the winner appends the site to the next level.
+// One barrier per level.  Occupancy is drawn a few layers ahead of the
+// frontier from the same Philox stream as every other path.
+//
+// What bounds it: a level is a chain of dependent shared-memory accesses and
+// integer instructions of one or a few warps (a warp issues one every 4.8
+// cycles), and there are first_hit - 1 of them; HBM traffic is nil.  Against
+// the full recursion, which updates every site of the window at every step
+// (us per call): W = 8, L = 64, p = 0.185, 10^4 configurations 7,230 -> 698;
+// W = 46, L = 400, p = 0.165, 32 configurations 273,000 -> 3,840; W = 64,
+// L = 4096, p = 0.17, one configuration 1,248,000 -> 41,700.
+#include <algorithm>
+#include <cstddef>
+#include <vector>
+
+#include "common.cuh"
+#include "kernels.cuh"
+#include "wave.cuh"
+
+namespace pc {
+
+namespace {
+
+constexpr int kPosBits = 18;  // plane position of a frontier entry; its hexagon row above
+constexpr uint32_t kPosMask = (1u << kPosBits) - 1u;
+constexpr int kDrawLayers = 8;  // layers drawn at a time (divides 32)
+
+// Contact directions (order of common.cuh, then the end contacts): offset
+// along the row, row offset index (0: r-2, 1: r-1, 2: r+1, 3: r+2, 4: own
+// row), tube offset: fixed (end contacts), +1 from sublattice 2 (up), -1 from
+// sublattice 0 (down).
+__host__ __device__ constexpr int c_dq(int d) { return d < 12 ? dir_dq(d) : 0; }
+__host__ __device__ constexpr int c_row(int d) {
+  return d >= 12 ? 4 : dir_dr(d) == -2 ? 0 : dir_dr(d) == -1 ? 1 : dir_dr(d) == 0 ? 4 : dir_dr(d) == 1 ? 2 : 3;
+}
+__host__ __device__ constexpr int c_drow(int d) { return d < 12 ? dir_dr(d) : 0; }
+__host__ __device__ constexpr int c_end(int d) { return d == 12 ? -1 : d == 13 ? 1 : 0; }
+__host__ __device__ constexpr int c_up(int d) { return d >= 6 && d < 9; }
+__host__ __device__ constexpr int c_dn(int d) { return d >= 9 && d < 12; }
+
+// Direction d for the claims: c_ent is added to a frontier entry (hexagon row
+// and offset along the row; the row offset comes on top); c_cls = byte of the
+// row offset in a row's table | tube offset + 1 at sublattice s in bits
+// 8 + 2s.
+__host__ __device__ constexpr uint32_t c_ent(int d) { return (uint32_t)(c_drow(d) * (1 << kPosBits) + c_dq(d)); }
+__host__ __device__ constexpr uint32_t c_cls(int d) {
+  return (uint32_t)(4 * c_row(d)) | (uint32_t)(1 + c_end(d) - c_dn(d)) << 8 | (uint32_t)(1 + c_end(d)) << 10 |
+         (uint32_t)(1 + c_end(d) + c_up(d)) << 12;
+}
+
+// What the claims of a level report (rare: tested by one comparison a site)
+enum : unsigned { F_NEED = 1u, F_HIT = 2u, F_OUT = 4u };
+
+// Scalars of a group, rotated over three levels: a level reads the previous
+// one's, writes its own and clears the next one's.
+struct GroupShared {
+  unsigned cf[3][2];      // sites of the level, flags
+  int olo[3], ohi[3];     // word rows of the level's overflow bits (ohi < 0: none)
+  int span[2];            // tubes of a level (level_span)
+  unsigned nz[2];
+  long long item;
+  uint2 dir[16];          // c_ent, c_cls of the 14 directions
+};
+constexpr int kSharedHead = 224;
+static_assert(sizeof(GroupShared) <= kSharedHead && offsetof(GroupShared, dir) % 8 == 0, "group scalars");
+
+template <bool kWarp>
+__device__ __forceinline__ void group_sync() {
+  if (kWarp) __syncwarp();
+  else __syncthreads();
+}
+
+// ld.shared at a 32-bit shared address plus an immediate
+template <int OFF>
+__device__ __forceinline__ uint32_t lds_u(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
+  return v;
+}
+
+// Shared-memory atomics at 32-bit shared addresses.
+__device__ __forceinline__ uint32_t atoms_and(uint32_t a, uint32_t v) {
+  uint32_t r;
+  asm volatile("atom.shared.and.b32 %0, [%1], %2;" : "=r"(r) : "r"(a), "r"(v) : "memory");
+  return r;
+}
+__device__ __forceinline__ uint32_t atoms_add(uint32_t a, uint32_t v) {
+  uint32_t r;
+  asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(r) : "r"(a), "r"(v) : "memory");
+  return r;
+}
+// the same under a condition, as predicated instructions (no branches)
+__device__ __forceinline__ uint32_t lds_if(bool c, uint32_t a) {
+  uint32_t v = 0u;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.shared.u32 %0, [%2];\n\t}" : "+r"(v) : "r"((uint32_t)c), "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t atoms_and_if(uint32_t c, uint32_t a, uint32_t m) {
+  uint32_t v = 0u;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p atom.shared.and.b32 %0, [%2], %3;\n\t}"
+               : "+r"(v) : "r"(c), "r"(a), "r"(m) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts_u2_if(bool c, uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.v2.u32 [%1], {%2, %3};\n\t}"
+               :: "r"((uint32_t)c), "r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void reds_min(uint32_t a, int v) {
+  asm volatile("red.shared.min.s32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void reds_max(uint32_t a, int v) {
+  asm volatile("red.shared.max.s32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void reds_or(uint32_t a, uint32_t v) {
+  asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint2 lds_u2(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts_u2(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" :: "r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ uint32_t smem_at(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+template <bool kWarp, bool kPart, bool kMass>
+__device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, char* scratch) {
+  const int tid = kWarp ? (threadIdx.x & 31) : threadIdx.x;
+  const int size = kWarp ? 32 : blockDim.x;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  GroupShared* gs = reinterpret_cast<GroupShared*>(sm);
+  int* roff = reinterpret_cast<int*>(sm + kSharedHead);  // [row][8]: offsets to rows r-2, r-1, r+1, r+2, then 0
+  const uint32_t gs_s = smem_at(gs), roff_s = smem_at(roff);
+  int cur_q = -1;
+#pragma unroll
+  for (int d = 0; d < 14; ++d)
+    if (tid == d) gs->dir[d] = make_uint2(c_ent(d), c_cls(d));
+  if (tid == 14 || tid == 15) gs->dir[tid] = make_uint2(0u, 16u | 0x1500u);
+  const uint32_t dir_s = gs_s + (uint32_t)offsetof(GroupShared, dir);
+  // this lane's contact when sixteen lanes share a site (lanes 14 and 15 idle)
+  const bool has16 = (lane & 15) < 14;
+  const uint32_t e16 = has16 ? c_ent(lane & 15) : 0u, y16 = has16 ? c_cls(lane & 15) : 16u | 0x1500u;
+
+  for (;;) {
+    long long item;
+    {
+      unsigned long long v = 0;
+      if (tid == 0) v = atomicAdd(a.work, 1ull);
+      if (kWarp) {
+        item = (long long)__shfl_sync(0xffffffffu, v, 0);
+      } else {
+        if (tid == 0) gs->item = (long long)v;
+        __syncthreads();
+        item = gs->item;
+      }
+    }
+    if (kMass) {
+      if (item >= (long long)*a.list_n) break;
+      item = (long long)a.list[item];
+    } else if (item >= a.n_items) {
+      break;
+    }
+    int qi = 0;
+    if (a.nq > 1) {
+      int hi = a.nq - 1;
+      while (qi < hi) {
+        const int mid = (qi + hi + 1) >> 1;
+        if (a.qs[mid].item0 <= item) qi = mid; else hi = mid - 1;
+      }
+    }
+    const WaveQuery& Q = a.nq > 1 ? a.qs[qi] : a.q0;
+    const int L = Q.L, A = Q.A, P = Q.P, NR = Q.NR, cap = Q.cap, sb = Q.s_begin, nr_mask = Q.nr_mask;
+    const int32_t* ppos = Q.ppos;
+    const int16_t* strip_row = Q.strip_row;
+    uint32_t* win = reinterpret_cast<uint32_t*>(sm + Q.o_win);
+    uint2* queue = reinterpret_cast<uint2*>(sm + Q.o_queue);
+    const uint32_t win_s = smem_at(win), queue_s = smem_at(queue);
+    uint32_t* back = reinterpret_cast<uint32_t*>(scratch + Q.a_back);
+    uint32_t* over = reinterpret_cast<uint32_t*>(scratch + Q.a_over);  // two maps of TW rows
+    const size_t over_n = (size_t)Q.TW * P;
+    uint32_t* occ = reinterpret_cast<uint32_t*>(scratch + Q.a_occ);
+    float* nu = reinterpret_cast<float*>(scratch + Q.a_nu);            // two rings of planes
+    const int ring_mask = Q.ring_mask;
+    const size_t nu_n = (size_t)(ring_mask < 0 ? L : ring_mask + 1) * P;
+    const long long rel = item - Q.item0;
+    if (qi != cur_q) {
+      cur_q = qi;
+      for (int k = tid; k < 8 * (2 * Q.W + 1); k += size) roff[k] = (k & 7) < 4 ? Q.row_off[(k >> 3) * 4 + (k & 7)] : 0;
+    }
+    if (tid == 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        gs->cf[k][0] = 0u; gs->cf[k][1] = 0u; gs->olo[k] = 0x7fffffff; gs->ohi[k] = -1;
+      }
+    }
+    group_sync<kWarp>();
+
+    int G = 0;   // layers drawn
+    int wb = 0;  // lowest word row of the window; row w has slot w & nr_mask
+    auto resident = [&](int w) { return !kPart || (unsigned)(w - wb) < (unsigned)NR; };
+    auto word_ptr = [&](int w, int pos) -> uint32_t* {  // any row
+      return resident(w) ? win + (w & nr_mask) * P + pos : back + (size_t)w * P + pos;
+    };
+    auto plane = [&](int t) -> size_t { return (size_t)(t & ring_mask) * P; };
+    auto row_of = [&](int pos) -> int { return strip_row[(int)__umulhi((unsigned)pos, 0x55555556u) - sb]; };
+    // Slide the window by one row: the row that leaves is written back if it
+    // was drawn, the row that enters (the same slot) read if it was.
+    // Group-uniform.
+    auto slide = [&](int dir) {
+      const int out = dir > 0 ? wb : wb + NR - 1, in = dir > 0 ? wb + NR : wb - 1;
+      uint32_t* row = win + (out & nr_mask) * P;
+      const bool w_out = 32 * out < G, r_in = 32 * in < G;
+      for (int k = tid; k < P; k += size) {
+        if (w_out) back[(size_t)out * P + k] = row[k];
+        if (r_in) row[k] = back[(size_t)in * P + k];
+      }
+      wb += dir;
+      group_sync<kWarp>();
+    };
+    // Draw the next layers (within one word row).  Group-uniform.
+    auto draw = [&]() {
+      const int Gn = min(G + kDrawLayers, L), w = G >> 5;
+      if (kPart && NR > 0) {
+        while (w >= wb + NR) slide(1);
+        while (w < wb) slide(-1);
+      }
+      uint32_t* row = !kPart || NR > 0 ? win + (w & nr_mask) * P : back + (size_t)w * P;
+      const uint32_t row_s = win_s + 4u * (uint32_t)((!kPart || NR > 0 ? w & nr_mask : 0) * P);
+      uint32_t* row_g = back + (size_t)w * P;
+      if ((G & 31) == 0) {  // first layers of the row
+        for (int k = tid; k < P; k += size) {
+          row[k] = 0u;
+          over[(size_t)w * P + k] = 0u;
+          over[over_n + (size_t)w * P + k] = 0u;
+        }
+        group_sync<kWarp>();
+      }
+      const uint32_t i0 = (uint32_t)G * (uint32_t)A, i1 = (uint32_t)Gn * (uint32_t)A;
+      const uint32_t divM = Q.divM;
+      const int divS = 31 + Q.divS;
+      auto set_site = [&](int t, int pos) {
+        if (!kPart || NR > 0) reds_or(row_s + 4u * (uint32_t)pos, 1u << (t & 31));
+        else atomicOr(row_g + pos, 1u << (t & 31));
+      };
+      if (Q.occ_bits) {
+        const uint32_t* cb = Q.occ_bits + (size_t)rel * Q.words_per_cfg;
+        for (uint32_t wi = (i0 >> 5) + tid; wi <= (i1 - 1) >> 5; wi += size) {
+          uint32_t bits = cb[wi];
+          while (bits) {
+            const uint32_t i = (wi << 5) + __ffs(bits) - 1;
+            bits &= bits - 1;
+            if (i < i0 || i >= i1) continue;
+            const int t = (int)(((uint64_t)i * divM) >> divS), c = (int)(i - (uint32_t)t * A);
+            set_site(t, __ldg(ppos + c));
+          }
+        }
+      } else {
+        OccStream os = Q.occ;
+        os.cfg = Q.cfg0 + (uint32_t)rel;
+        const uint32_t b_end = (i1 - 1) >> 2;
+        uint32_t bi = (i0 >> 2) + tid;
+        int t = (int)(((uint64_t)(bi << 2) * divM) >> divS), c = (int)((bi << 2) - (uint32_t)t * A);
+        const int dt = (int)(((uint64_t)(4 * size) * divM) >> divS), dc = 4 * size - dt * A;  // one round further
+        for (; bi <= b_end; bi += size) {
+          // the four positions are fetched while the block is drawn
+          int tj[4], pj[4];
+          {
+            int t1 = t, c1 = c;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              tj[j] = t1;
+              pj[j] = __ldg(ppos + c1);
+              if (++c1 == A) { c1 = 0; ++t1; }
+            }
+          }
+          const uint32_t bits = os.block_bits(bi);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (((bits >> j) & 1u) && tj[j] >= G && tj[j] < Gn) set_site(tj[j], pj[j]);
+          t += dt;
+          c += dc;
+          if (c >= A) { c -= A; ++t; }
+        }
+      }
+      group_sync<kWarp>();
+      if (kMass) {  // the degrees need the occupancy itself
+        const int nl = Gn - G;
+        const uint32_t mask = (nl == 32 ? 0xffffffffu : (1u << nl) - 1u) << (G & 31);
+        for (int k = tid; k < P; k += size) {
+          uint32_t* o = occ + (size_t)w * P + k;
+          *o = ((G & 31) ? *o : 0u) | (row[k] & mask);
+        }
+        group_sync<kWarp>();
+      }
+      G = Gn;
+    };
+
+    draw();
+    // level 0: the metallic sites of t = 0
+    unsigned total = 0;
+    {
+      uint32_t* row = !kPart || NR > 0 ? win : back;
+      for (int k0 = tid & ~31; k0 < P; k0 += size) {
+        const int pos = k0 + lane;
+        bool c = false;
+        if (pos < P) {
+          const uint32_t w = row[pos];
+          c = w & 1u;
+          if (c) row[pos] = w & ~1u;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, c);
+        if (bal) {
+          unsigned base = 0;
+          if (kWarp) {
+            base = total;
+            total += __popc(bal);
+          } else {
+            if (lane == 0) base = atoms_add(gs_s + (uint32_t)offsetof(GroupShared, cf), (unsigned)__popc(bal));
+            base = __shfl_sync(0xffffffffu, base, 0);
+          }
+          base += __popc(bal & lt);
+          if (c) {
+            if (base < (unsigned)cap) queue[base] = make_uint2((uint32_t)pos | (uint32_t)row_of(pos) << kPosBits, 0u);
+            else { atomicOr(over + pos, 1u); gs->olo[0] = 0; gs->ohi[0] = 0; }
+          }
+        }
+      }
+      group_sync<kWarp>();
+      if (!kWarp) total = gs->cf[0][0];
+    }
+    const unsigned n0 = total;
+
+    // nu of a new site: (1/degree) x the sum over the contacts of the previous
+    // level, whose values lie in src (at level 0: (1/degree) x 1/n0)
+    auto site_value = [&](int t, int pos, int hrow, const float* src) -> float {
+      const int sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
+      const int4 o4 = reinterpret_cast<const int4*>(roff)[2 * hrow];
+      const int ro[5] = {o4.x, o4.y, o4.z, o4.w, 0};
+      float v[14];
+      int deg = t == L - 1;  // the detector edge
+      uint32_t ow[14];
+#pragma unroll
+      for (int d = 0; d < 14; ++d) {
+        const int tt = t + c_end(d) + (c_up(d) & (sg == 2)) - (c_dn(d) & (sg == 0));
+        const int np = pos + c_dq(d) + ro[c_row(d)];
+        ow[d] = (unsigned)tt < (unsigned)L ? occ[(size_t)(tt >> 5) * P + np] >> (tt & 31) : 0u;
+      }
+#pragma unroll
+      for (int d = 0; d < 14; ++d) {
+        v[d] = 0.f;
+        if (ow[d] & 1u) {
+          ++deg;
+          if (src) {
+            const int tt = t + c_end(d) + (c_up(d) & (sg == 2)) - (c_dn(d) & (sg == 0));
+            const int np = pos + c_dq(d) + ro[c_row(d)];
+            if (!((*word_ptr(tt >> 5, np) >> (tt & 31)) & 1u)) v[d] = src[plane(tt) + np];
+          }
+        }
+      }
+      const float inv = deg ? __frcp_rn((float)deg) : 0.f;
+      if (!src) return inv * __frcp_rn((float)n0);
+      // the addition trees of the full recursion (strip_sums in tiling.cuh)
+      const float e = v[6] + v[9], h = v[12] + v[13], g = v[5] + v[2];
+      const float pa = v[7] + v[0], pbs = v[8] + v[1], pcs = v[4] + v[11], pd = v[3] + v[10];
+      float r;
+      if (sg == 0) r = (((pa + pbs) + pcs) + (pd + e)) + (h + g);
+      else if (sg == 1) r = ((pcs + pd) + (pa + pbs)) + ((e + h) + g);
+      else r = (((pcs + pd) + pa) + (pbs + e)) + (h + g);
+      return inv * r;
+    };
+    // nu of the sites of level m (queue qn, overflow rows [lo, hi]); true if any is not 0
+    auto level_values = [&](int m, unsigned n, const uint2* qn, int lo, int hi) -> bool {
+      const float* src = m ? nu + (size_t)((m - 1) & 1) * nu_n : nullptr;
+      float* dst = nu + (size_t)(m & 1) * nu_n;
+      if (tid == 0) gs->nz[m & 1] = 0u;
+      group_sync<kWarp>();
+      bool nz = false;
+      const unsigned stored = min(n, (unsigned)cap);
+      for (unsigned i = tid; i < stored; i += size) {
+        const uint2 e = qn[i];
+        const int t = (int)e.y, pos = (int)(e.x & kPosMask);
+        const float x = site_value(t, pos, (int)(e.x >> kPosBits), src);
+        dst[plane(t) + pos] = x;
+        nz |= x != 0.f;
+      }
+        for (int w = lo; w <= hi; ++w)
+          for (int pos = tid; pos < P; pos += size) {
+            uint32_t word = over[(size_t)(m & 1) * over_n + (size_t)w * P + pos];
+            while (word) {
+              const int t = 32 * w + __ffs(word) - 1;
+              word &= word - 1;
+              const float x = site_value(t, pos, row_of(pos), src);
+              dst[plane(t) + pos] = x;
+              nz |= x != 0.f;
+            }
+          }
+      if (nz) gs->nz[m & 1] = 1u;
+      group_sync<kWarp>();
+      return gs->nz[m & 1] != 0u;
+    };
+    // detector mass: nu over the reached sites of t = L - 1, by the group's
+    // first warp in a fixed order (the same for every group size)
+    auto detector_mass = [&](int m) -> float {
+      const float* dst = nu + (size_t)(m & 1) * nu_n;
+      float part_sum = 0.f;
+      if (tid < 32)
+        for (int c = tid; c < A; c += 32) {
+          const int pos = __ldg(ppos + c), w = (L - 1) >> 5;
+          const uint32_t bit = (occ[(size_t)w * P + pos] & ~*word_ptr(w, pos)) >> ((L - 1) & 31);
+          if (bit & 1u) part_sum += dst[plane(L - 1) + pos];
+        }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) part_sum += __shfl_xor_sync(0xffffffffu, part_sum, o);
+      return part_sum;  // valid in the first warp
+    };
+
+    int verdict = 0, fh = -1, mstop = 0;
+    float mass = 0.f;
+    bool hard = false;
+    if (n0 > 0 && L == 1) {
+      verdict = 1; fh = 1; mstop = 1;
+      if (kMass) {
+        level_values(0, total, queue, 0, gs->ohi[0]);
+        mass = detector_mass(0);
+      }
+    } else if (n0 > 0) {
+      if (kMass) level_values(0, total, queue, 0, gs->ohi[0]);
+      int cu_ = 0;  // rotating index of the current level
+      for (int m = 1;; ++m) {
+        const int nx = cu_ == 2 ? 0 : cu_ + 1, nn = nx == 2 ? 0 : nx + 1;
+        const uint32_t qc_s = queue_s + 8u * (uint32_t)(((m - 1) & 1) * cap), qn_s = queue_s + 8u * (uint32_t)((m & 1) * cap);
+        uint32_t* on = over + (size_t)(m & 1) * over_n;
+        const uint32_t cf_s = gs_s + (uint32_t)offsetof(GroupShared, cf) + 8u * (uint32_t)nx;
+        float* zero = nu + (size_t)((m - 1) & 1) * nu_n;
+        // tubes [t_lo, t_lo + t_span) call for nothing; t_need: contacts in
+        // layers not drawn yet
+        const int t_need = G < L ? G - 1 : 0x7fffffff;
+        const int t_lo = kPart ? 32 * wb : 0;
+        const unsigned t_span = (unsigned)(min(min(t_need, L - 1), kPart ? 32 * (wb + NR) : 0x7fffffff) - t_lo);
+        unsigned count = 0, f = 0;
+        // the site (ent, tt) enters level m as entry idx
+        auto put = [&](bool won, unsigned idx, uint32_t ent, int tt) {
+          sts_u2_if(won && idx < (unsigned)cap, qn_s + 8u * idx, ent, (uint32_t)tt);
+          if (won && (idx >= (unsigned)cap || (unsigned)(tt - t_lo) >= t_span)) {
+            if (idx >= (unsigned)cap) {
+              const int w = tt >> 5;
+              atomicOr(on + (size_t)w * P + (ent & kPosMask), 1u << (tt & 31));
+              reds_min(gs_s + (uint32_t)offsetof(GroupShared, olo) + 4u * (uint32_t)nx, w);
+              reds_max(gs_s + (uint32_t)offsetof(GroupShared, ohi) + 4u * (uint32_t)nx, w);
+            }
+            f |= (tt >= t_need ? F_NEED : 0u) | (tt == L - 1 ? F_HIT : 0u) | (resident(tt >> 5) ? 0u : F_OUT);
+          }
+          if (kMass && won) zero[plane(tt) + (ent & kPosMask)] = 0.f;  // level m holds nothing at step m - 1
+        };
+        // n entries of the next level for this warp
+        auto reserve = [&](unsigned n) -> unsigned {
+          unsigned base = 0;
+          if (kWarp) {
+            base = count;
+            count += n;
+          } else {
+            if (lane == 0) base = atoms_add(cf_s, n);
+            base = __shfl_sync(0xffffffffu, base, 0);
+          }
+          return base;
+        };
+        // where the word of (entry, tube) lies in the window
+        auto at_of = [&](uint32_t ent, int tt) -> uint32_t {
+          return win_s + 4u * (uint32_t)(((tt >> 5) & nr_mask) * P + (int)(ent & kPosMask));
+        };
+        auto back_of = [&](uint32_t ent, int tt) -> uint32_t* { return back + (size_t)(tt >> 5) * P + (ent & kPosMask); };
+        // Few sites: sixteen lanes to a site, one contact each, U pairs of
+        // sites at a time, so that the chain of a level is short.
+        auto expand16 = [&](unsigned first, unsigned step, unsigned stored) {
+          constexpr int U = kWarp ? 4 : 2;
+          uint32_t en[U], at[U], got[U];
+          int tt[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const unsigned i = first + (unsigned)u * step + (unsigned)(lane >> 4);
+            const bool act = i < stored && has16;
+            const uint2 e = lds_u2(qc_s + 8u * (act ? i : 0u));
+            const int pos = (int)(e.x & kPosMask), sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
+            en[u] = e.x + e16 + lds_u<0>(roff_s + ((e.x >> (kPosBits - 5)) & ~31u) + (y16 & 255u));
+            tt[u] = (int)e.y + (int)((y16 >> (8 + 2 * sg)) & 3u) - 1;
+            at[u] = at_of(en[u], tt[u]);
+            bool ok = act && tt[u] >= 0;
+            got[u] = 0u;
+            if (kPart && ok && !resident(tt[u] >> 5)) {
+              got[u] = *back_of(en[u], tt[u]);
+              ok = false;
+            }
+            const uint32_t wd = lds_if(ok, at[u]);
+            if (!kPart || ok) got[u] = wd;
+            got[u] &= 1u << (tt[u] & 31);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const uint32_t bit = got[u];
+            if (kPart && !resident(tt[u] >> 5)) {
+              if (bit) got[u] = atomicAnd(back_of(en[u], tt[u]), ~bit) & bit;
+            } else {
+              got[u] = atoms_and_if(bit, at[u], ~bit) & bit;
+            }
+          }
+          unsigned bal[U], n = 0;
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            bal[u] = __ballot_sync(0xffffffffu, got[u] != 0u);
+            n += (unsigned)__popc(bal[u]);
+          }
+          if (n == 0) return;
+          unsigned base = reserve(n);
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            put(got[u] != 0u, base + (unsigned)__popc(bal[u] & lt), en[u], tt[u]);
+            base += (unsigned)__popc(bal[u]);
+          }
+        };
+        // Many sites: a lane per site.
+        auto expand1 = [&](bool act, uint32_t ent, int t) {
+          const int pos = (int)(ent & kPosMask);
+          const int sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
+          const uint32_t ro_s = roff_s + 32u * (ent >> kPosBits);
+          const int w = t >> 5, b = t & 31;
+          const bool s2 = sg == 2, sz = sg == 0;
+          // c: bit d = contact d is metallic and not reached yet.  Each word
+          // is shifted so that the contact's bit comes first and a funnel
+          // shift takes it in.
+          uint32_t c = 0u;
+          bool in = act;
+          if (kPart) in = act && resident(w) && (b != 31 || resident(w + 1)) && (b != 0 || t == 0 || resident(w - 1));
+          if (in) {
+            uint4 o;  // offsets to rows r-2, r-1, r+1, r+2
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(o.x), "=r"(o.y), "=r"(o.z), "=r"(o.w) : "r"(ro_s));
+            const uint32_t base = at_of(ent, t);
+            const uint32_t nb = b == 31 ? at_of(ent, t + 1) : base, pbs = b == 0 && t ? at_of(ent, t - 1) : base;
+            const uint32_t ub = s2 ? nb : base, db = sz ? pbs : base;
+            const uint32_t o2 = 4u * o.x, o1 = 4u * o.y, p1 = 4u * o.z, p2 = 4u * o.w;
+            const uint32_t w13 = lds_u<0>(nb), w12 = lds_u<0>(pbs), w11 = lds_u<0>(db + p1), w10 = lds_u<4>(db + o1),
+                           w9 = lds_u<-4>(db), w8 = lds_u<0>(ub + o1), w7 = lds_u<-4>(ub + p1), w6 = lds_u<4>(ub),
+                           w5 = lds_u<-4>(base + p2), w4 = lds_u<-8>(base + p1), w3 = lds_u<-4>(base + o1),
+                           w2 = lds_u<4>(base + o2), w1 = lds_u<8>(base + o1), w0 = lds_u<4>(base + p1);
+            const int xs = 31 - b, xn = 31 - ((b + 1) & 31), xp = 31 - ((b - 1) & 31);
+            const int xu = s2 ? xn : xs, xd = sz ? xp : xs;
+            auto take = [&](uint32_t v, int sh) { c = __funnelshift_l(v << sh, c, 1); };
+            take(w13, xn); take(w12, xp); take(w11, xd); take(w10, xd); take(w9, xd); take(w8, xu); take(w7, xu);
+            take(w6, xu); take(w5, xs); take(w4, xs); take(w3, xs); take(w2, xs); take(w1, xs); take(w0, xs);
+          } else if (act) {  // a row outside the window
+            const int4 o = *reinterpret_cast<const int4*>(roff + 8 * (ent >> kPosBits));
+            const int ro[5] = {o.x, o.y, o.z, o.w, 0};
+            uint32_t v[14];
+#pragma unroll
+            for (int d = 0; d < 14; ++d) {
+              const int tt = t + c_end(d) + (c_up(d) & s2) - (c_dn(d) & sz);
+              v[d] = tt < 0 ? 0u : *word_ptr(tt >> 5, pos + c_dq(d) + ro[c_row(d)]) >> (tt & 31);
+            }
+#pragma unroll
+            for (int d = 0; d < 14; ++d) c |= (v[d] & 1u) << d;
+          }
+          if (t == 0) c &= sz ? ~((1u << 12) | (7u << 9)) : ~(1u << 12);
+          while (__any_sync(0xffffffffu, c != 0u)) {
+            constexpr int K = 3;  // candidates of a lane at a time: their atomics overlap
+            uint32_t en[K], got[K];
+            int tt[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+              const uint2 y = lds_u2(dir_s + 8u * (uint32_t)((__ffs(c) - 1) & 15));
+              en[k] = ent + y.x + lds_u<0>(ro_s + (y.y & 255u));
+              tt[k] = t + (int)((y.y >> (8 + 2 * sg)) & 3u) - 1;
+              const uint32_t bit = c ? 1u << (tt[k] & 31) : 0u;
+              c &= c - 1u;
+              if (kPart && !resident(tt[k] >> 5)) {
+                got[k] = bit ? atomicAnd(back_of(en[k], tt[k]), ~bit) & bit : 0u;
+              } else {
+                got[k] = atoms_and_if(bit, at_of(en[k], tt[k]), ~bit) & bit;
+              }
+            }
+            unsigned bal[K], n = 0;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+              bal[k] = __ballot_sync(0xffffffffu, got[k] != 0u);
+              n += (unsigned)__popc(bal[k]);
+            }
+            if (n == 0) continue;
+            unsigned base = reserve(n);
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+              put(got[k] != 0u, base + (unsigned)__popc(bal[k] & lt), en[k], tt[k]);
+              base += (unsigned)__popc(bal[k]);
+            }
+          }
+        };
+        const unsigned stored = min(total, (unsigned)cap);
+        if (stored <= (kWarp ? 16u : (unsigned)size >> 2)) {
+          const unsigned nw2 = (unsigned)(size >> 5) * 2u;  // sites of all warps in one round
+          constexpr unsigned U = kWarp ? 4u : 2u;
+          for (unsigned i = (unsigned)(tid >> 5) * 2u; i < stored; i += U * nw2) expand16(i, nw2, stored);
+        } else {
+          for (unsigned i0 = (unsigned)(tid & ~31); i0 < stored; i0 += (unsigned)size) {
+            const unsigned i = i0 + (unsigned)lane;
+            const uint2 e = lds_u2(qc_s + 8u * (i < stored ? i : i0));
+            expand1(i < stored, e.x, (int)e.y);
+          }
+        }
+        if (total > (unsigned)cap) {  // sites of this level beyond the queue
+          uint32_t* oc = over + (size_t)((m - 1) & 1) * over_n;
+          const int lo = gs->olo[cu_], hi = gs->ohi[cu_];
+          for (int w = lo; w <= hi; ++w)
+            for (int p0 = tid & ~31; p0 < P; p0 += size) {
+              const int pos = p0 + lane;
+              uint32_t word = pos < P ? oc[(size_t)w * P + pos] : 0u;
+              if (word) oc[(size_t)w * P + pos] = 0u;
+              uint32_t ent = 0u;
+              if (word) ent = (uint32_t)pos | (uint32_t)row_of(pos) << kPosBits;
+              while (__any_sync(0xffffffffu, word != 0u)) {
+                const bool act = word != 0u;
+                const int b = act ? __ffs(word) - 1 : 0;
+                word &= word - 1u;
+                expand1(act, ent, 32 * w + b);
+              }
+            }
+        }
+        __syncwarp();
+        if (kWarp) {
+          total = count;
+          f = __any_sync(0xffffffffu, f != 0u) ? __reduce_or_sync(0xffffffffu, f) : 0u;
+          if (lane == 0) { gs->olo[nn] = 0x7fffffff; gs->ohi[nn] = -1; }
+          __syncwarp();
+        } else {
+          if (f) reds_or(cf_s + 4u, f);
+          if (tid == 0) { gs->cf[nn][0] = 0u; gs->cf[nn][1] = 0u; gs->olo[nn] = 0x7fffffff; gs->ohi[nn] = -1; }
+          __syncthreads();
+          total = gs->cf[nx][0];
+          f = gs->cf[nx][1];
+        }
+        cu_ = nx;
+        if (total == 0) { mstop = m; break; }
+        if (f & F_NEED) draw();  // the new sites have contacts in the next layers
+        if (kMass || (kPart && NR > 0 && (f & F_OUT))) {
+          int lo = 0, hi = 0;  // tubes of the new level
+          if (!kMass || ring_mask >= 0) {
+            if (tid == 0) { gs->span[0] = gs->olo[nx] < 0x7fffffff ? 32 * gs->olo[nx] : 0x7fffffff; gs->span[1] = 32 * gs->ohi[nx] + 31; }
+            group_sync<kWarp>();
+            lo = 0x7fffffff; hi = -1;
+            for (unsigned i = tid; i < min(total, (unsigned)cap); i += size) {
+              const int t = (int)lds_u2(qn_s + 8u * i).y;
+              lo = min(lo, t);
+              hi = max(hi, t);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0) { atomicMin(&gs->span[0], lo); atomicMax(&gs->span[1], hi); }
+            group_sync<kWarp>();
+            lo = gs->span[0];
+            hi = gs->span[1];
+            group_sync<kWarp>();
+          }
+          if (kMass) {
+            // the rings hold the levels m - 1 and m only while their tubes
+            // (a level lies within one tube of the previous one's) and the
+            // tubes around them are fewer than the rings' planes
+            if (ring_mask >= 0 && hi - lo + 5 > ring_mask + 1) { hard = true; break; }
+            const bool live = level_values(m, total, queue + (m & 1) * cap, gs->olo[nx], gs->ohi[nx]);
+            if (f & F_HIT) { mass = detector_mass(m); break; }
+            if (!live) break;  // nu has underflowed everywhere: the mass is 0
+          }
+          if (kPart && NR > 0 && (f & F_OUT)) {  // keep the window on the frontier
+            if ((lo >> 5) < wb && (hi >> 5) < wb + NR - 1) slide(-1);
+            else if ((hi >> 5) >= wb + NR && (lo >> 5) > wb) slide(1);
+          }
+        }
+        if (!kMass && (f & F_HIT)) {
+          verdict = 1; fh = m + 1; mstop = m + 1;
+          break;
+        }
+      }
+    }
+    if (tid == 0) {
+      if (kMass) {
+        if (hard) a.hard[atomicAdd(a.hard_n, 1ull)] = (unsigned long long)item;
+        else Q.out.mass[rel] = mass;
+      } else {
+        Q.out.verdict[rel] = (uint8_t)verdict;
+        if (Q.out.first_hit) Q.out.first_hit[rel] = fh;
+        if (Q.out.mass) Q.out.mass[rel] = 0.f;
+        if (Q.out.m_stop) Q.out.m_stop[rel] = mstop;
+        if (verdict) {
+          if (Q.out.n_perc) atomicAdd(Q.out.n_perc, 1ull);
+          if (a.want_mass && Q.out.mass) a.list[atomicAdd(a.list_n, 1ull)] = (unsigned long long)item;
+        }
+      }
+    }
+    group_sync<kWarp>();
+  }
+}
+
+// A warp group's registers are bounded so that 24 warps fit an SM.
+template <bool kWarp, bool kPart, bool kMass>
+__global__ void __launch_bounds__(kWarp ? 128 : 512, kWarp ? 6 : 1) wave_kernel(const __grid_constant__ WaveArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (kWarp) {
+    const int w = threadIdx.x >> 5;
+    wave_body<true, kPart, kMass>(a, smem_raw + (size_t)w * a.group_smem,
+                                  a.scratch + ((long long)blockIdx.x * (blockDim.x >> 5) + w) * a.scratch_stride);
+  } else {
+    wave_body<false, kPart, kMass>(a, smem_raw, a.scratch + (long long)blockIdx.x * a.scratch_stride);
+  }
+}
+
+const void* wave_fn(bool warp, bool part, bool mass) {
+  static const void* const f[8] = {
+      (const void*)wave_kernel<false, false, false>, (const void*)wave_kernel<false, false, true>,
+      (const void*)wave_kernel<false, true, false>,  (const void*)wave_kernel<false, true, true>,
+      (const void*)wave_kernel<true, false, false>,  (const void*)wave_kernel<true, false, true>,
+      (const void*)wave_kernel<true, true, false>,   (const void*)wave_kernel<true, true, true>};
+  return f[(warp ? 4 : 0) + (part ? 2 : 0) + (mass ? 1 : 0)];
+}
+
+int ceil_log2(long long x) {
+  int b = 0;
+  while ((1ll << b) < x) ++b;
+  return b;
+}
+
+inline size_t up(size_t x, size_t m) { return (x + m - 1) / m * m; }
+
+void fill_lattice(WaveQuery& w, const Lattice& lat) {
+  w.W = lat.W; w.L = lat.L; w.A = lat.A; w.P = lat.P; w.TW = lat.TW;
+  w.s_begin = lat.s_begin; w.n_strips = lat.n_strips;
+  w.divS = ceil_log2(lat.A);
+  w.divM = (uint32_t)((1ull << (31 + w.divS)) / (unsigned long long)lat.A + 1ull);
+  w.strip_row = lat.strip_row; w.row_off = lat.row_off; w.ppos = lat.ppos;
+}
+
+}  // namespace
+
+bool wave_takes(const Lattice& lat) { return lat.P <= (1 << kPosBits); }
+
+pc_status run_wave(const StreamQuery& job, cudaStream_t st) {
+  if (job.n_cfg <= 0) return PC_OK;
+  const Lattice& lat = job.lat;
+  WaveArgs a = {};
+  WaveQuery& w = a.q0;
+  fill_lattice(w, lat);
+  w.occ = job.occ; w.occ_bits = job.occ_bits; w.words_per_cfg = job.words_per_cfg; w.cfg0 = job.cfg0;
+  w.out = job.out; w.item0 = 0;
+  a.nq = 1; a.qs = nullptr; a.n_items = job.n_cfg;
+  a.want_mass = (!job.bits_only && job.out.mass) ? 1 : 0;
+
+  int dev = 0, nsm = 0, optin = 0, per_sm_smem = 0;
+  PC_CUDA(cudaGetDevice(&dev));
+  PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  PC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  PC_CUDA(cudaDeviceGetAttribute(&per_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+  const bool warp = lat.A <= 640;
+  const int threads = warp ? 128 : lat.A <= 2000 ? 128 : lat.A <= 5000 ? 256 : 512;
+  const size_t row_b = sizeof(uint32_t) * (size_t)lat.P;
+  const size_t head = kSharedHead + 32 * (size_t)(2 * lat.W + 1);
+  // shared memory per group: every word row if they fit the target, else a
+  // power of two of them
+  const size_t most = (size_t)optin - 64;
+  const size_t target = warp ? 12 * 1024 : lat.A <= 5000 ? 72 * 1024 : most;
+  w.cap = (int)std::min<long long>(lat.A, warp ? 512 : 1200);
+  const size_t fixed = head + 2 * sizeof(uint2) * (size_t)w.cap + 32;
+  auto fits = [&](int rows, size_t lim) { return fixed + (size_t)rows * row_b <= lim; };
+  if (fits(lat.TW, target)) {
+    w.NR = lat.TW; w.nr_mask = -1;
+  } else {
+    w.NR = 0;
+    for (int r = 1; r < lat.TW && (fits(r, target) || (r <= 2 && fits(r, most))); r *= 2) w.NR = r;
+    w.nr_mask = w.NR - 1;
+  }
+  w.o_win = (int)head;
+  w.o_queue = (int)up(w.o_win + w.NR * row_b, 16);
+  const size_t group_smem = up(w.o_queue + 2 * sizeof(uint2) * (size_t)w.cap, 16);
+  a.group_smem = (int)group_smem;
+  const int groups_per_cta = warp ? threads / 32 : 1;
+  const size_t smem = group_smem * groups_per_cta;
+
+  // device scratch of a group
+  const size_t map_b = up(row_b * lat.TW, 256);
+  size_t off = 0;
+  w.a_over = (long long)off; off += 2 * row_b * lat.TW; off = up(off, 256);
+  w.a_back = (long long)off; if (w.NR < lat.TW) off += map_b;
+  w.a_occ = 0; w.a_nu = 0;
+  const int ring = lat.L <= 128 ? -1 : 127;
+  w.ring_mask = ring;
+  size_t stride_b = off, stride_m = off;
+  if (a.want_mass) {
+    w.a_occ = (long long)stride_m; stride_m += map_b;
+    w.a_nu = (long long)stride_m; stride_m += up(2 * row_b * (size_t)(ring < 0 ? lat.L : ring + 1), 256);
+  }
+  const void* fb = wave_fn(warp, w.NR < lat.TW, false);
+  const void* fm = wave_fn(warp, w.NR < lat.TW, true);
+  auto grid_of = [&](const void* f, long long items, size_t stride, size_t budget, long long* g) -> pc_status {
+    // the same limit on every call: calls from several threads never lower it
+    PC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+    int per_sm = 0;
+    PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem));
+    if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
+    long long n = (long long)per_sm * nsm;
+    n = std::min<long long>(n, (items + groups_per_cta - 1) / groups_per_cta);
+    n = std::min<long long>(n, std::max<long long>(1, (long long)(budget / (stride * groups_per_cta))));
+    *g = std::max<long long>(n, 1);
+    return PC_OK;
+  };
+  pc_status rc;
+  long long gb = 0, gm = 0, gh = 0;
+  const size_t budget = 24ull << 30;
+  if ((rc = grid_of(fb, job.n_cfg, std::max<size_t>(stride_b, 256), budget, &gb))) return rc;
+  if (a.want_mass && (rc = grid_of(fm, job.n_cfg, stride_m, budget, &gm))) return rc;
+  size_t stride_h = 0;
+  WaveQuery wh = w;
+  if (a.want_mass && ring >= 0) {
+    wh.ring_mask = -1;
+    stride_h = (size_t)wh.a_nu + up(2 * row_b * (size_t)lat.L, 256);
+    if ((rc = grid_of(fm, job.n_cfg, stride_h, stride_m * (size_t)gm * groups_per_cta, &gh))) return rc;
+  }
+  const size_t pool = std::max(std::max(stride_b * gb, stride_m * gm), stride_h * gh) * groups_per_cta;
+  const size_t list_b = a.want_mass ? up(8 * (size_t)job.n_cfg, 256) : 0;
+  char* mem = nullptr;
+  PC_CUDA(cudaMallocAsync((void**)&mem, 256 + list_b * (ring >= 0 ? 2 : 1) + pool + 256, st));
+  unsigned long long* ctr = (unsigned long long*)mem;
+  a.list = (unsigned long long*)(mem + 256);
+  a.hard = (unsigned long long*)(mem + 256 + list_b);
+  a.list_n = ctr + 1;
+  a.hard_n = ctr + 2;
+  char* scratch = mem + 256 + list_b * (ring >= 0 ? 2 : 1);
+  a.scratch = scratch;
+  cudaError_t e = cudaMemsetAsync(mem, 0, 256, st);
+  auto launch = [&](const void* f, long long g) {
+    void* args[] = {&a};
+    if (e == cudaSuccess) e = cudaLaunchKernel(f, dim3((unsigned)g), dim3(threads), args, smem, st);
+  };
+  a.work = ctr; a.scratch_stride = (long long)stride_b;
+  launch(fb, gb);
+  if (a.want_mass) {
+    a.work = ctr + 3; a.scratch_stride = (long long)stride_m;
+    launch(fm, gm);
+    if (ring >= 0) {  // frontiers that outgrew the rings: a plane for every layer
+      a.q0 = wh;
+      a.work = ctr + 4; a.scratch_stride = (long long)stride_h;
+      a.list = a.hard; a.list_n = a.hard_n;
+      launch(fm, gh);
+    }
+  }
+  rc = e == cudaSuccess ? PC_OK : cuda_fail(e, "wavefront solver");
+  cudaFreeAsync(mem, st);
+  return rc;
+}
+
+}  // namespace pc
