@@ -191,43 +191,29 @@ typedef struct pc_query {
 typedef struct pc_result {
   int64_t n_percolating;
   double Pi;
-  int32_t solver;           /* 0 = shared-memory resident, 1 = streamed,
-                               2 = verdict-only with temporal blocking */
-  int32_t threads;          /* CTA size the resident solver ran with */
+  int32_t solver;           /* size class of the lattice: 0 = its state fits one
+                               CTA's shared memory, 2 = synchronous PC_BITS_ONLY
+                               batches: one thread-block cluster holds its
+                               cross-section (pc_bits_blocked_shape), 1 = else */
+  int32_t threads;          /* class 0: threads that worked on a configuration */
 } pc_result;
 
 /*
  * Inspect many queries of mixed lattice sizes in one GPU submission (the
- * batching of a finite-size-scaling sweep, Sec. III): the queries whose
- * configuration state fits one CTA's shared memory run the resident solver
- * in at most three persistent launches, one per shared-memory class (up to
- * a quarter, a half, or all of an SM's shared memory), each taking the
- * configurations of its queries from one list ordered by decreasing lattice
- * size; every other query shares one pool of streamed-solver slots that
- * refill as configurations finish, largest lattices first.  The whole batch
- * is one CUDA graph, built on the first call and replayed when the same
- * batch (same queries and output pointers) is submitted again.  The
- * resident CTA size of each (W, L, p bin of width 0.025) is picked by timing
- * candidates on first use (autotuner; choices kept in memory and in the JSON
- * file named by the environment variable PC_TUNE_FILE, if set); a launch
- * runs with the size tuned for its heaviest query (sites x configurations),
- * reported in pc_result.threads.
+ * batching of a finite-size-scaling sweep, Sec. III) on the wavefront solver:
+ * one persistent launch for the levels, and one for the masses, of each group
+ * size that the batch's lattices take (a warp, or a CTA of 128 to 512
+ * threads), each taking the configurations of its queries from one list
+ * ordered by decreasing lattice size.
  * out: [n_queries] host summaries, or NULL.  Unless flags has PC_ASYNC the
  * call synchronises cuda_stream and fills out; with PC_ASYNC (requires
  * PC_OUT_DEVICE and out == NULL) it returns after enqueueing.  PC_BITS_ONLY
  * and PC_VERDICT_FIRST apply to every query of the batch; any other flag bit
- * is PC_ERR_ARG.  With PC_BITS_ONLY and without PC_ASYNC, a streamed query
- * whose cross-section one thread-block cluster holds (pc_bits_blocked_shape)
- * runs on the verdict-only solver with temporal blocking, on cuda_stream
- * after the batch's graph (solver 2 in out).
+ * is PC_ERR_ARG.
  * Results equal those of pc_inspect on each query.
- * Threads: calls from several host threads are safe.  A cached batch is
- * reference counted, so evicting it (or pc_shutdown) never frees one that a
- * running call uses.  Replays of the same batch are serialised: each waits,
- * on its own stream, for the previous replay (of any stream, PC_ASYNC
- * included) to finish, because they share counters and the output buffers
- * named in the queries.  A PC_ASYNC batch's outputs are therefore rewritten
- * by the next submission of the same batch once that one runs.
+ * Threads: calls from several host threads are safe; nothing is shared
+ * between calls.  Batches on several streams that name the same output
+ * buffers rewrite them without waiting for one another.
  * Errors: PC_ERR_ARG, PC_ERR_OOM, PC_ERR_CUDA, PC_ERR_INTERNAL.
  */
 #define PC_ASYNC 0x2
@@ -398,7 +384,7 @@ pc_status pc_bits_blocked_shape(int32_t W, int32_t* cluster_size, int32_t* colum
 pc_status pc_lazy_mass(const int32_t* first_hit, const float* mass, int64_t n_configs,
                        double hold, float* mass_lazy, int32_t flags, void* cuda_stream);
 
-/* Release cached lattice tables, batch graphs and scratch of every device,
+/* Release cached lattice tables of every device,
  * and forget the static array's cached device addresses (pc_inspect_static).
  * Call it after cudaDeviceReset, before any further call of the library. */
 pc_status pc_shutdown(void);

@@ -225,7 +225,7 @@ def pc_inspect(W: int, L: int, p: float, seed: int, config_begin: int, n_configs
     bits_only: propagate the exact reached set alone (verdicts, first_hit,
     m_stop; mass is 0).
     verdict_first: the same outputs, bit for bit, with the FP32 recursion run
-    only on the configurations that percolate (resident solver).
+    only on the configurations that percolate (the default solver always does).
 
     device=False: numpy outputs plus ``n_percolating`` and ``Pi`` (the call
     synchronises).  device=True: torch CUDA tensors written asynchronously on
@@ -345,10 +345,9 @@ def pc_batch_run(specs, *, device: bool = False, async_: bool = False, stream=No
                  outs: list | None = None, queries=None, bits_only: bool = False,
                  verdict_first: bool = False):
     """Inspect a batch of queries [(W, L, p, seed, config_begin, n_configs)] in
-    one submission (one cached CUDA graph).  Returns (outs, results): per-query
-    outputs (numpy, or torch CUDA tensors with ``device``) and the host
-    summaries (None with ``async_``).  Passing the same ``outs`` (and
-    ``queries``) again replays the cached graph."""
+    one submission.  Returns (outs, results): per-query outputs (numpy, or
+    torch CUDA tensors with ``device``) and the host summaries (None with
+    ``async_``).  ``outs`` (and ``queries``) may be passed again."""
     if queries is None:
         queries, outs = batch_queries(specs, device=device, outs=outs)
     flags = ((PC_OUT_DEVICE if device else 0) | (PC_ASYNC if async_ else 0) | (PC_BITS_ONLY if bits_only else 0)

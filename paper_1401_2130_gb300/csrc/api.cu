@@ -145,14 +145,14 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
     if ((flags & PC_MODE_RESIDENT) && !resident) {
       set_error("PC_MODE_RESIDENT: lattice state exceeds shared memory"); rc = PC_ERR_OOM; break;
     }
-    if (!(flags & (PC_MODE_RESIDENT | PC_MODE_STREAM)) && wave_takes(lat)) {
+    if (!(flags & (PC_MODE_RESIDENT | PC_MODE_STREAM))) {
       StreamQuery j;
       j.lat = lat; j.occ = os; j.occ_bits = occ_bits; j.words_per_cfg = wpc;
       j.n_cfg = n; j.cfg0 = (uint32_t)cfg0;
       j.out.verdict = s.verdict; j.out.first_hit = s.first_hit; j.out.mass = s.mass;
       j.out.m_stop = s.m_stop; j.out.n_perc = s.n_perc;
       j.bits_only = (flags & PC_BITS_ONLY) ? 1 : 0;
-      rc = run_wave(j, st);
+      rc = run_wave(&j, 1, st);
     } else if (resident) {
       ResidentArgs a;
       a.lat = lat; a.occ = os; a.occ_bits = occ_bits; a.words_per_cfg = wpc;
@@ -286,7 +286,6 @@ pc_status pc_inspect_occupancy(int32_t W, int32_t L, const uint32_t* occ_bits, i
 }
 
 pc_status pc_shutdown(void) {
-  release_batches();
   release_lattices();
   release_static();
   return PC_OK;

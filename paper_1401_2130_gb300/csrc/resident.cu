@@ -467,37 +467,6 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(ResidentArgs P
   }
 }
 
-// Many queries in one persistent launch: their configurations form one
-// list of items (query q owns [item0[q], item0[q + 1])), taken in order from
-// one counter.  The host orders the queries by decreasing lattice size, so
-// the longest configurations start first and the short ones fill the tails;
-// a CTA reloads the lattice tables only when its next item belongs to
-// another query.
-__global__ void __launch_bounds__(kMaxThreads, 1) resident_multi_kernel(ResidentBatch B) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ long long s_item;
-  QueryState qs;
-  int cur = -1;
-  const long long n_items = B.item0[B.nq];
-  for (;;) {
-    if (threadIdx.x == 0) s_item = (long long)atomicAdd(B.work, 1ull);
-    __syncthreads();
-    const long long item = s_item;
-    if (item >= n_items) break;
-    int lo = 0, hi = B.nq - 1;  // last q with item0[q] <= item
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (B.item0[mid] <= item) lo = mid; else hi = mid - 1;
-    }
-    const ResidentArgs& Pa = B.qs[lo];
-    if (lo != cur) {
-      setup_query(Pa, smem_raw, qs);
-      cur = lo;
-    }
-    solve_config(Pa, qs, item - B.item0[lo]);
-  }
-}
-
 // Kernel, dynamic shared memory and grid of a resident launch.
 static pc_status resident_config(const ResidentArgs& args, int threads, void** func, size_t* smem,
                                  long long* grid) {
@@ -523,55 +492,6 @@ static pc_status resident_config(const ResidentArgs& args, int threads, void** f
   if (g > args.n_cfg) g = args.n_cfg;
   *grid = g;
   *func = (void*)resident_kernel;
-  return PC_OK;
-}
-
-pc_status resident_add_node(const ResidentArgs& args, int threads, cudaGraph_t g,
-                            const cudaGraphNode_t* deps, size_t ndeps, cudaGraphNode_t* out) {
-  void* func = nullptr;
-  size_t smem = 0;
-  long long grid = 0;
-  pc_status rc = resident_config(args, threads, &func, &smem, &grid);
-  if (rc) return rc;
-  ResidentArgs a = args;
-  void* params[] = {&a};
-  cudaKernelNodeParams kp = {};
-  kp.func = func;
-  kp.gridDim = dim3((unsigned)(grid < 1 ? 1 : grid));
-  kp.blockDim = dim3(threads);
-  kp.sharedMemBytes = (unsigned)smem;
-  kp.kernelParams = params;
-  PC_CUDA(cudaGraphAddKernelNode(out, g, deps, ndeps, &kp));
-  return PC_OK;
-}
-
-pc_status resident_multi_add_node(const ResidentBatch& b, long long n_items, size_t smem, int threads,
-                                  cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps,
-                                  cudaGraphNode_t* out) {
-  if (threads > kMaxThreads || threads < 32 || threads % 32) {
-    set_error("resident solver: CTA size must be a multiple of 32 in [32, 640]");
-    return PC_ERR_ARG;
-  }
-  PC_CUDA(cudaFuncSetAttribute(resident_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int dev = 0, nsm = 0, per_sm = 0;
-  PC_CUDA(cudaGetDevice(&dev));
-  PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_multi_kernel, threads, smem));
-  if (per_sm < 1) {
-    set_error("resident solver: lattice does not fit one CTA");
-    return PC_ERR_OOM;
-  }
-  long long grid = (long long)per_sm * nsm;
-  if (grid > n_items) grid = n_items;
-  ResidentBatch a = b;
-  void* params[] = {&a};
-  cudaKernelNodeParams kp = {};
-  kp.func = (void*)resident_multi_kernel;
-  kp.gridDim = dim3((unsigned)(grid < 1 ? 1 : grid));
-  kp.blockDim = dim3(threads);
-  kp.sharedMemBytes = (unsigned)smem;
-  kp.kernelParams = params;
-  PC_CUDA(cudaGraphAddKernelNode(out, g, deps, ndeps, &kp));
   return PC_OK;
 }
 

@@ -113,11 +113,6 @@ __device__ __forceinline__ uint32_t lds_u(uint32_t a) {
 }
 
 // Shared-memory atomics at 32-bit shared addresses.
-__device__ __forceinline__ uint32_t atoms_and(uint32_t a, uint32_t v) {
-  uint32_t r;
-  asm volatile("atom.shared.and.b32 %0, [%1], %2;" : "=r"(r) : "r"(a), "r"(v) : "memory");
-  return r;
-}
 __device__ __forceinline__ uint32_t atoms_add(uint32_t a, uint32_t v) {
   uint32_t r;
   asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(r) : "r"(a), "r"(v) : "memory");
@@ -152,9 +147,6 @@ __device__ __forceinline__ uint2 lds_u2(uint32_t a) {
   uint2 v;
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
   return v;
-}
-__device__ __forceinline__ void sts_u2(uint32_t a, uint32_t x, uint32_t y) {
-  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" :: "r"(a), "r"(x), "r"(y) : "memory");
 }
 __device__ __forceinline__ uint32_t smem_at(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -199,11 +191,15 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       break;
     }
     int qi = 0;
-    if (a.nq > 1) {
-      int hi = a.nq - 1;
-      while (qi < hi) {
-        const int mid = (qi + hi + 1) >> 1;
-        if (a.qs[mid].item0 <= item) qi = mid; else hi = mid - 1;
+    if (a.nq > 1) {  // items come in order: mostly the previous one's query
+      if (cur_q >= 0 && item >= a.qs[cur_q].item0 && item < a.qs[cur_q].item0 + a.qs[cur_q].n_cfg) {
+        qi = cur_q;
+      } else {
+        int hi = a.nq - 1;
+        while (qi < hi) {
+          const int mid = (qi + hi + 1) >> 1;
+          if (a.qs[mid].item0 <= item) qi = mid; else hi = mid - 1;
+        }
       }
     }
     const WaveQuery& Q = a.nq > 1 ? a.qs[qi] : a.q0;
@@ -725,7 +721,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         if (Q.out.m_stop) Q.out.m_stop[rel] = mstop;
         if (verdict) {
           if (Q.out.n_perc) atomicAdd(Q.out.n_perc, 1ull);
-          if (a.want_mass && Q.out.mass) a.list[atomicAdd(a.list_n, 1ull)] = (unsigned long long)item;
+          if (Q.want_mass) a.list[atomicAdd(a.list_n, 1ull)] = (unsigned long long)item;
         }
       }
     }
@@ -773,117 +769,219 @@ void fill_lattice(WaveQuery& w, const Lattice& lat) {
 
 }  // namespace
 
-bool wave_takes(const Lattice& lat) { return lat.P <= (1 << kPosBits); }
+namespace {
 
-pc_status run_wave(const StreamQuery& job, cudaStream_t st) {
-  if (job.n_cfg <= 0) return PC_OK;
-  const Lattice& lat = job.lat;
-  WaveArgs a = {};
-  WaveQuery& w = a.q0;
-  fill_lattice(w, lat);
-  w.occ = job.occ; w.occ_bits = job.occ_bits; w.words_per_cfg = job.words_per_cfg; w.cfg0 = job.cfg0;
-  w.out = job.out; w.item0 = 0;
-  a.nq = 1; a.qs = nullptr; a.n_items = job.n_cfg;
-  a.want_mass = (!job.bits_only && job.out.mass) ? 1 : 0;
+// The query table goes through kernel parameters: asynchronous, and no
+// pageable host copy.
+constexpr int kUpload = 16;
+struct UploadChunk {
+  int n;
+  WaveQuery q[kUpload];
+};
+static_assert(sizeof(UploadChunk) <= 4000, "kernel parameters");
+__global__ void wave_upload_kernel(WaveQuery* dst, const __grid_constant__ UploadChunk c) {
+  if ((int)threadIdx.x < c.n) dst[threadIdx.x] = c.q[threadIdx.x];
+}
 
-  int dev = 0, nsm = 0, optin = 0, per_sm_smem = 0;
-  PC_CUDA(cudaGetDevice(&dev));
-  PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  PC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  PC_CUDA(cudaDeviceGetAttribute(&per_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-  const bool warp = lat.A <= 640;
-  const int threads = warp ? 128 : lat.A <= 2000 ? 128 : lat.A <= 5000 ? 256 : 512;
-  const size_t row_b = sizeof(uint32_t) * (size_t)lat.P;
-  const size_t head = kSharedHead + 32 * (size_t)(2 * lat.W + 1);
-  // shared memory per group: every word row if they fit the target, else a
-  // power of two of them
-  const size_t most = (size_t)optin - 64;
-  const size_t target = warp ? 12 * 1024 : lat.A <= 5000 ? 72 * 1024 : most;
-  w.cap = (int)std::min<long long>(lat.A, warp ? 512 : 1200);
+// One launch: the queries that run with the same group size.
+struct WaveClass {
+  int threads = 0;           // 32: a group is a warp (four to a CTA), else the CTA
+  std::vector<WaveQuery> q;
+  long long items = 0, mass_items = 0;
+  bool part = false, ring = false;
+  size_t group_smem = 0;
+  size_t stride_b = 256, stride_m = 256, stride_h = 256;
+  long long grid_b = 0, grid_m = 0, grid_h = 0;
+  size_t scratch = 0, list_b = 0, table_b = 0;
+};
+
+// Threads of a group.  With more configurations than groups fit the device,
+// few (more configurations in flight; a level's fixed cost is paid by every
+// warp); else more (a level is a chain of instructions: more warps, fewer
+// sites each).
+int group_threads(int A, long long n, int nsm) {
+  if (A <= 640) return n <= 8ll * nsm ? 128 : 32;
+  if (A <= 2000) return n <= 2ll * nsm ? 256 : 128;
+  if (A <= 5000) return n <= nsm ? 512 : 256;
+  return 512;
+}
+
+// Shared memory and scratch of query w in a class.
+void place(WaveQuery& w, WaveClass& c, size_t most) {
+  const size_t row_b = sizeof(uint32_t) * (size_t)w.P;
+  const size_t head = kSharedHead + 32 * (size_t)(2 * w.W + 1);
+  // every word row in shared memory if they fit the target, else a power of
+  // two of them
+  const size_t target = c.threads == 32 ? 12 * 1024 : c.threads <= 256 ? 72 * 1024 : most;
+  w.cap = (int)std::min<long long>(w.A, c.threads == 32 ? 512 : 1200);
   const size_t fixed = head + 2 * sizeof(uint2) * (size_t)w.cap + 32;
   auto fits = [&](int rows, size_t lim) { return fixed + (size_t)rows * row_b <= lim; };
-  if (fits(lat.TW, target)) {
-    w.NR = lat.TW; w.nr_mask = -1;
+  if (fits(w.TW, target)) {
+    w.NR = w.TW; w.nr_mask = -1;
   } else {
     w.NR = 0;
-    for (int r = 1; r < lat.TW && (fits(r, target) || (r <= 2 && fits(r, most))); r *= 2) w.NR = r;
+    for (int r = 1; r < w.TW && (fits(r, target) || (r <= 2 && fits(r, most))); r *= 2) w.NR = r;
     w.nr_mask = w.NR - 1;
   }
   w.o_win = (int)head;
   w.o_queue = (int)up(w.o_win + w.NR * row_b, 16);
-  const size_t group_smem = up(w.o_queue + 2 * sizeof(uint2) * (size_t)w.cap, 16);
-  a.group_smem = (int)group_smem;
-  const int groups_per_cta = warp ? threads / 32 : 1;
-  const size_t smem = group_smem * groups_per_cta;
+  c.group_smem = std::max(c.group_smem, up(w.o_queue + 2 * sizeof(uint2) * (size_t)w.cap, 16));
+  c.part = c.part || w.NR < w.TW;
+  const size_t map_b = up(row_b * w.TW, 256);
+  size_t off = up(2 * row_b * w.TW, 256);
+  w.a_over = 0;
+  w.a_back = (long long)off;
+  if (w.NR < w.TW) off += map_b;
+  c.stride_b = std::max(c.stride_b, off);
+  w.ring_mask = w.L <= 128 ? -1 : 127;
+  if (w.want_mass) {
+    w.a_occ = (long long)off; off += map_b;
+    w.a_nu = (long long)off;
+    const size_t ring = w.ring_mask < 0 ? (size_t)w.L : 128;
+    c.stride_m = std::max(c.stride_m, off + up(2 * row_b * ring, 256));
+    c.stride_h = std::max(c.stride_h, off + up(2 * row_b * (size_t)w.L, 256));
+    c.ring = c.ring || w.ring_mask >= 0;
+  }
+}
 
-  // device scratch of a group
-  const size_t map_b = up(row_b * lat.TW, 256);
-  size_t off = 0;
-  w.a_over = (long long)off; off += 2 * row_b * lat.TW; off = up(off, 256);
-  w.a_back = (long long)off; if (w.NR < lat.TW) off += map_b;
-  w.a_occ = 0; w.a_nu = 0;
-  const int ring = lat.L <= 128 ? -1 : 127;
-  w.ring_mask = ring;
-  size_t stride_b = off, stride_m = off;
-  if (a.want_mass) {
-    w.a_occ = (long long)stride_m; stride_m += map_b;
-    w.a_nu = (long long)stride_m; stride_m += up(2 * row_b * (size_t)(ring < 0 ? lat.L : ring + 1), 256);
+}  // namespace
+
+int wave_threads(int A, long long n_all) {
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return group_threads(A, n_all, nsm);
+}
+
+pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st) {
+  int dev = 0, nsm = 0, optin = 0;
+  PC_CUDA(cudaGetDevice(&dev));
+  PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  PC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  // classes; within one, larger lattices first (their configurations run longest)
+  std::vector<int> order;
+  for (int i = 0; i < nq; ++i)
+    if (qs[i].n_cfg > 0) order.push_back(i);
+  if (order.empty()) return PC_OK;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return qs[x].lat.N > qs[y].lat.N; });
+  long long n_all = 0;
+  for (int i : order) n_all += qs[i].n_cfg;
+  std::vector<WaveClass> cls;
+  for (int i : order) {
+    const StreamQuery& s = qs[i];
+    const int threads = group_threads(s.lat.A, n_all, nsm);
+    auto c = std::find_if(cls.begin(), cls.end(), [&](const WaveClass& x) { return x.threads == threads; });
+    if (c == cls.end()) {
+      cls.emplace_back();
+      c = cls.end() - 1;
+      c->threads = threads;
+    }
+    WaveQuery w = {};
+    fill_lattice(w, s.lat);
+    w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
+    w.out = s.out;
+    w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
+    w.item0 = c->items; w.n_cfg = s.n_cfg;
+    place(w, *c, (size_t)optin - 64);
+    c->items += s.n_cfg;
+    if (w.want_mass) c->mass_items += s.n_cfg;
+    c->q.push_back(w);
   }
-  const void* fb = wave_fn(warp, w.NR < lat.TW, false);
-  const void* fm = wave_fn(warp, w.NR < lat.TW, true);
-  auto grid_of = [&](const void* f, long long items, size_t stride, size_t budget, long long* g) -> pc_status {
-    // the same limit on every call: calls from several threads never lower it
-    PC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    int per_sm = 0;
-    PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem));
-    if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
-    long long n = (long long)per_sm * nsm;
-    n = std::min<long long>(n, (items + groups_per_cta - 1) / groups_per_cta);
-    n = std::min<long long>(n, std::max<long long>(1, (long long)(budget / (stride * groups_per_cta))));
-    *g = std::max<long long>(n, 1);
-    return PC_OK;
-  };
-  pc_status rc;
-  long long gb = 0, gm = 0, gh = 0;
-  const size_t budget = 24ull << 30;
-  if ((rc = grid_of(fb, job.n_cfg, std::max<size_t>(stride_b, 256), budget, &gb))) return rc;
-  if (a.want_mass && (rc = grid_of(fm, job.n_cfg, stride_m, budget, &gm))) return rc;
-  size_t stride_h = 0;
-  WaveQuery wh = w;
-  if (a.want_mass && ring >= 0) {
-    wh.ring_mask = -1;
-    stride_h = (size_t)wh.a_nu + up(2 * row_b * (size_t)lat.L, 256);
-    if ((rc = grid_of(fm, job.n_cfg, stride_h, stride_m * (size_t)gm * groups_per_cta, &gh))) return rc;
-  }
-  const size_t pool = std::max(std::max(stride_b * gb, stride_m * gm), stride_h * gh) * groups_per_cta;
-  const size_t list_b = a.want_mass ? up(8 * (size_t)job.n_cfg, 256) : 0;
+  // grids and device memory: fewer groups where the scratch of all of them
+  // cannot be had
   char* mem = nullptr;
-  PC_CUDA(cudaMallocAsync((void**)&mem, 256 + list_b * (ring >= 0 ? 2 : 1) + pool + 256, st));
-  unsigned long long* ctr = (unsigned long long*)mem;
-  a.list = (unsigned long long*)(mem + 256);
-  a.hard = (unsigned long long*)(mem + 256 + list_b);
-  a.list_n = ctr + 1;
-  a.hard_n = ctr + 2;
-  char* scratch = mem + 256 + list_b * (ring >= 0 ? 2 : 1);
-  a.scratch = scratch;
-  cudaError_t e = cudaMemsetAsync(mem, 0, 256, st);
-  auto launch = [&](const void* f, long long g) {
-    void* args[] = {&a};
-    if (e == cudaSuccess) e = cudaLaunchKernel(f, dim3((unsigned)g), dim3(threads), args, smem, st);
-  };
-  a.work = ctr; a.scratch_stride = (long long)stride_b;
-  launch(fb, gb);
-  if (a.want_mass) {
-    a.work = ctr + 3; a.scratch_stride = (long long)stride_m;
-    launch(fm, gm);
-    if (ring >= 0) {  // frontiers that outgrew the rings: a plane for every layer
-      a.q0 = wh;
-      a.work = ctr + 4; a.scratch_stride = (long long)stride_h;
-      a.list = a.hard; a.list_n = a.hard_n;
-      launch(fm, gh);
+  for (size_t total = 24ull << 30;; total /= 8) {
+    const size_t budget = total / cls.size();
+    size_t bytes = 256 * cls.size();
+    for (WaveClass& c : cls) {
+      const size_t per_cta = c.threads == 32 ? 4 : 1;
+      const int block = c.threads * (int)per_cta;
+      const size_t smem = c.group_smem * per_cta;
+      auto grid_of = [&](bool mass, long long items, size_t stride, size_t most, long long* g) -> pc_status {
+        const void* f = wave_fn(c.threads == 32, c.part, mass);
+        // the same limit on every call: calls from several threads never lower it
+        PC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+        int per_sm = 0;
+        PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, block, smem));
+        if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
+        long long n = std::min<long long>((long long)per_sm * nsm, (items + (long long)per_cta - 1) / (long long)per_cta);
+        n = std::min<long long>(n, (long long)(most / (stride * per_cta)));
+        *g = std::max<long long>(n, 1);
+        return PC_OK;
+      };
+      pc_status rc = grid_of(false, c.items, c.stride_b, budget, &c.grid_b);
+      if (rc) return rc;
+      c.scratch = c.stride_b * (size_t)c.grid_b * per_cta;
+      if (c.mass_items) {
+        if ((rc = grid_of(true, c.mass_items, c.stride_m, budget, &c.grid_m))) return rc;
+        c.scratch = std::max(c.scratch, c.stride_m * (size_t)c.grid_m * per_cta);
+        c.list_b = up(8 * (size_t)c.mass_items, 256);
+        if (c.ring) {
+          if ((rc = grid_of(true, c.mass_items, c.stride_h, c.scratch, &c.grid_h))) return rc;
+          c.scratch = std::max(c.scratch, c.stride_h * (size_t)c.grid_h * per_cta);
+        }
+      }
+      c.table_b = c.q.size() > 1 ? up(sizeof(WaveQuery) * c.q.size(), 256) : 0;
+      bytes += c.table_b * (c.ring ? 2 : 1) + c.list_b * (c.ring ? 2 : 1) + c.scratch;
+    }
+    cudaError_t e = cudaMallocAsync((void**)&mem, bytes, st);
+    if (e == cudaSuccess) break;
+    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "wavefront solver: scratch");
+    cudaGetLastError();
+    if (total < (1ull << 20)) {
+      set_error("wavefront solver: no memory for one configuration's state");
+      return PC_ERR_OOM;
     }
   }
-  rc = e == cudaSuccess ? PC_OK : cuda_fail(e, "wavefront solver");
+  cudaError_t e = cudaMemsetAsync(mem, 0, 256 * cls.size(), st);
+  char* at = mem + 256 * cls.size();
+  for (size_t k = 0; k < cls.size(); ++k) {
+    WaveClass& c = cls[k];
+    const int per_cta = c.threads == 32 ? 4 : 1;  // groups to a CTA
+    unsigned long long* ctr = (unsigned long long*)(mem + 256 * k);
+    WaveArgs a = {};
+    a.q0 = c.q[0];
+    a.nq = (int)c.q.size();
+    a.n_items = c.items;
+    a.group_smem = (int)c.group_smem;
+    auto upload = [&](char* to) {
+      for (size_t b = 0; b < c.q.size() && e == cudaSuccess; b += kUpload) {
+        UploadChunk u = {};
+        u.n = (int)std::min<size_t>(kUpload, c.q.size() - b);
+        for (int i = 0; i < u.n; ++i) u.q[i] = c.q[b + i];
+        wave_upload_kernel<<<1, kUpload, 0, st>>>((WaveQuery*)to + b, u);
+        e = cudaGetLastError();
+      }
+    };
+    if (c.table_b) { a.qs = (const WaveQuery*)at; upload(at); at += c.table_b; }
+    a.list = (unsigned long long*)at; at += c.list_b;
+    a.list_n = ctr + 1;
+    a.hard_n = ctr + 2;
+    if (c.ring) { a.hard = (unsigned long long*)at; at += c.list_b; }
+    auto launch = [&](bool mass, long long grid, unsigned long long* work, size_t stride) {
+      a.work = work;
+      a.scratch_stride = (long long)stride;
+      void* args[] = {&a};
+      if (e == cudaSuccess)
+        e = cudaLaunchKernel(wave_fn(c.threads == 32, c.part, mass), dim3((unsigned)grid), dim3(c.threads * per_cta),
+                             args, c.group_smem * per_cta, st);
+    };
+    char* table_h = at;
+    if (c.ring) at += c.table_b;
+    a.scratch = at; at += c.scratch;
+    launch(false, c.grid_b, ctr, c.stride_b);
+    if (c.mass_items) {
+      launch(true, c.grid_m, ctr + 3, c.stride_m);
+      if (c.ring) {  // frontiers that outgrew the mass rings: a plane for every layer
+        for (WaveQuery& w : c.q) w.ring_mask = -1;
+        a.q0 = c.q[0];
+        if (c.table_b) { a.qs = (const WaveQuery*)table_h; upload(table_h); }
+        a.list = a.hard; a.list_n = a.hard_n;
+        launch(true, c.grid_h, ctr + 4, c.stride_h);
+      }
+    }
+  }
+  pc_status rc = e == cudaSuccess ? PC_OK : cuda_fail(e, "wavefront solver");
   cudaFreeAsync(mem, st);
   return rc;
 }

@@ -20,7 +20,8 @@ struct WaveQuery {
   int64_t words_per_cfg;
   uint32_t cfg0;
   Outputs out;
-  long long item0;           // first work item of the query
+  int want_mass;
+  long long item0, n_cfg;    // the query's work items
   int NR;                    // word rows of the unvisited map held in shared memory
   int nr_mask;               // row w has slot w & nr_mask
   int cap;                   // frontier entries held in shared memory (two levels)
@@ -34,7 +35,6 @@ struct WaveArgs {
   WaveQuery q0;              // the query, if nq == 1
   const WaveQuery* qs;       // [nq] by increasing item0
   int nq;
-  int want_mass;
   long long n_items;
   unsigned long long* work;     // next work item (or entry of list)
   unsigned long long* list;     // percolating items whose mass is wanted
@@ -46,10 +46,10 @@ struct WaveArgs {
   long long scratch_stride;
 };
 
-// Whether the wavefront solver takes the lattice: a plane position has to fit
-// a frontier entry (every W <= 255 does).
-bool wave_takes(const Lattice& lat);
-// Inspects one query (stream-ordered, no host synchronisation).
-pc_status run_wave(const StreamQuery& q, cudaStream_t st);
+// Inspects the queries (stream-ordered, no host synchronisation).
+pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st);
+// Threads that work on one configuration of an A-column lattice when n_all
+// configurations are inspected together on the current device.
+int wave_threads(int A, long long n_all);
 
 }  // namespace pc
