@@ -223,27 +223,25 @@ pc_status pc_batch_run(const pc_query* queries, int64_t n_queries, pc_result* ou
 /*
  * Serving: a continuous-batching request loop on one device (the current
  * device at pc_server_create).  Queries are admitted in arrival order as soon
- * as their HBM footprint -- output buffers, plus the streamed solver's state
- * for max(1, min(slots free, max_slots_per_query)) configurations when the
- * lattice exceeds shared memory -- fits the server's device arena of
- * hbm_budget_bytes.  Admitted queries run concurrently on the device:
- * resident-size queries as persistent kernels on side streams, the others in
- * the streamed solver's slots, which refill on the device while the query
- * has configurations left.  New arrivals are admitted between chunks of
- * ticks_per_poll device ticks.  Lattice state and occupancy counters stay on
- * the device.  Each query's results equal pc_inspect's on the same query.
+ * as their HBM footprint -- output buffers, plus the state of max(1, min(slots
+ * free, max_slots_per_query)) configurations when the lattice exceeds shared
+ * memory -- fits the server's device arena of hbm_budget_bytes.  Each admitted
+ * query is one run of the wavefront solver on a side stream, in its own
+ * memory: as many configurations in work at once as it has slots, the next
+ * ones taken on the device; queries run beside each other, and new ones are
+ * admitted when one ends.  (A query without slots uses at most 64 MB of
+ * stream-ordered scratch besides.)  Each query's results equal pc_inspect's on
+ * the same query.
  */
 typedef struct pc_server pc_server;
 
 typedef struct pc_server_opts {
   uint64_t hbm_budget_bytes;   /* device arena (default 8 GiB) */
-  int32_t max_slots;           /* streamed-solver slots, 1..4096 (default 256) */
+  int32_t max_slots;           /* configurations in HBM slots at once, 1..4096 (default 256) */
   int32_t max_slots_per_query; /* cap per query (default 64) */
-  int32_t ticks_per_poll;      /* device ticks between admissions (default 8) */
+  int32_t ticks_per_poll;      /* >= 1; kept for callers that set it, without effect (default 8) */
   int64_t max_pending;         /* queue bound; submit returns PC_ERR_BUSY beyond */
-  int32_t max_W;               /* widest lattice solved in HBM slots, 0..255 (0 = 255):
-                                  sizes the sweep's shared-memory staging; a
-                                  narrower bound lets more planes be in flight */
+  int32_t max_W;               /* widest lattice accepted in HBM slots, 0..255 (0 = 255) */
 } pc_server_opts;
 
 typedef struct pc_server_stats {

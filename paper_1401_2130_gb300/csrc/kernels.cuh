@@ -81,23 +81,6 @@ pc_status run_blocked(const StreamJob& job, cudaStream_t st, bool* handled);
 // Whether run_blocked takes PC_BITS_ONLY jobs of this lattice on this device.
 bool blocked_takes(const Lattice& lat);
 
-// Server engine (stream.cu): streamed-solver slots bound to queries by the host.
-struct ServerEngine;
-pc_status server_engine_create(int max_slots, int max_queries, int ticks_per_chunk, int max_W,
-                               cudaStream_t st, ServerEngine** out);
-void server_engine_destroy(ServerEngine* E);
-int server_engine_slots(const ServerEngine* E);
-pc_status server_engine_set_query(ServerEngine* E, int qi, const StreamQuery& q, cudaStream_t st);
-pc_status server_engine_bind(ServerEngine* E, const int* slots, const int* queries, char* const* bases,
-                             int n, cudaStream_t st);
-pc_status server_engine_run_chunk(ServerEngine* E, cudaStream_t st);
-// Enqueue a status read into host buffer buf (0 or 1): slot phases and
-// per-query completion counts; the buffers are valid once the stream passes.
-pc_status server_engine_status(ServerEngine* E, cudaStream_t st, int buf, const int** phases,
-                               const unsigned long long** qdone);
-const int* server_engine_phase_buffer(const ServerEngine* E, int buf);
-const unsigned long long* server_engine_qdone_buffer(const ServerEngine* E, int buf);
-
 // Standalone occupancy draw, occupancy.cu.
 pc_status launch_occupancy(const Lattice& lat, const OccStream& os, uint32_t cfg0,
                            int64_t n_cfg, uint32_t* occ_bits, cudaStream_t st);

@@ -116,10 +116,6 @@ struct Ctx {
   int nring;                    // ring slots (3 .. kMaxRing)
   int fp;                       // some query runs the FP32 recursion (else: the bits-only kernel)
   int use_cond;                 // set the WHILE condition at the end of a tick
-  int server;                   // 1: slots are bound to a query by the host
-  char** slot_base;             // [K] state of each slot (server mode)
-  unsigned long long* qnext;    // [nq] next configuration of a query (server mode)
-  unsigned long long* qdone;    // [nq] finished configurations (server mode)
 };
 
 
@@ -158,7 +154,7 @@ __host__ __device__ inline size_t slot_bytes_of(int A, int L, int P) {
 
 __device__ inline SlotView view_of(const Ctx& x, int slot, const Lattice& lat) {
   const size_t S = (size_t)lat.S;
-  char* b = x.server ? x.slot_base[slot] : x.pool + (size_t)slot * x.slot_bytes;
+  char* b = x.pool + (size_t)slot * x.slot_bytes;
   SlotView v;
   const size_t nu_b = a256(sizeof(float) * (size_t)(lat.L + 4) * lat.P);
   const size_t w_b = a256(sizeof(uint32_t) * (size_t)lat.TWP * S);
@@ -169,10 +165,6 @@ __device__ inline SlotView view_of(const Ctx& x, int slot, const Lattice& lat) {
   v.R0 = (uint32_t*)b; b += w_b;
   v.R1 = (uint32_t*)b;
   return v;
-}
-
-__device__ inline uint32_t bit_at(const uint32_t* w, int S, int col, int tt) {
-  return (w[((tt >> 5) + 1) * S + col] >> (tt & 31)) & 1u;
 }
 
 // query of a global work item (queries are few; linear scan)
@@ -671,7 +663,7 @@ __global__ void __launch_bounds__(kCols, kFP ? 2 : 4) sweep_kernel(Ctx x) {
     } else {  // U_DRAW: one word row of occupancy, 32 tubes per word
       const int tw = p.lo[U_DRAW] + rchunk;
       if (a < A) {
-        const long long rel = x.server ? c.item : config_of(Q, c.item - Q.item0);
+        const long long rel = config_of(Q, c.item - Q.item0);
         uint32_t word = 0;
         if (Q.occ_bits) {
           const uint32_t* cb = Q.occ_bits + (size_t)rel * Q.words_per_cfg;
@@ -808,25 +800,14 @@ __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
     }
     if (tid == 0) {
       if (finish) {
-        const long long rel = x.server ? c.item : config_of(Q, c.item - Q.item0);
+        const long long rel = config_of(Q, c.item - Q.item0);
         Q.out.verdict[rel] = (uint8_t)verdict;
         if (Q.out.first_hit) Q.out.first_hit[rel] = fh;
         if (Q.out.mass) Q.out.mass[rel] = mass;
         if (Q.out.m_stop) Q.out.m_stop[rel] = mstop;
         if (verdict && Q.out.n_perc) atomicAdd(Q.out.n_perc, 1ull);
         atomicAdd(x.n_done, 1ull);
-        if (x.server) {
-          // the slot stays with its query while it has configurations left
-          atomicAdd(&x.qdone[c.q], 1ull);
-          const unsigned long long nxt = atomicAdd(&x.qnext[c.q], 1ull);
-          const int q = c.q;
-          c.item = (long long)nxt; c.m = 0; c.G = 0; c.F = 0; c.flags = 0u;
-          for (int k = 0; k < U_KINDS; ++k) c.units[k] = 0;
-          if ((long long)nxt < x.qs[q].n_cfg) { c.phase = PH_DRAW0; fill_plan(c, x.qs[q]); }
-          else c.phase = PH_EMPTY;
-        } else {
-          assign(x, c, atomicAdd(x.work, 1ull));
-        }
+        assign(x, c, atomicAdd(x.work, 1ull));
       } else {
         fill_plan(c, Q);
       }
@@ -918,7 +899,7 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   q += 256;
   x.pool = q;
   x.slot_bytes = slot;
-  x.use_cond = 0; x.server = 0; x.slot_base = nullptr; x.qnext = nullptr; x.qdone = nullptr;
+  x.use_cond = 0;
   x.fp = 0;
   for (int i = 0; i < nq; ++i) x.fp |= qs[i].bits_only ? 0 : 1;
   {
@@ -991,203 +972,6 @@ void stream_plan_release(StreamPlan* P, cudaStream_t st) {
   if (!P) return;
   if (P->mem) cudaFreeAsync(P->mem, st);
   delete P;
-}
-
-// ---------------------------------------------------------------------------
-// Server engine: the same ticks, with slots bound to queries by the host
-// (continuous batching).  The host uploads query entries, binds free slots to
-// admitted queries, runs chunks of ticks and reads back slot phases and
-// per-query completion counts between chunks.
-// ---------------------------------------------------------------------------
-namespace {
-
-constexpr int kBindChunk = 64;
-struct BindList {
-  int n;
-  int slot[kBindChunk];
-  int query[kBindChunk];
-  char* base[kBindChunk];
-};
-
-__global__ void __launch_bounds__(1024) server_bind_kernel(Ctx x, BindList b) {
-  if ((int)threadIdx.x < b.n) {
-    const int s = b.slot[threadIdx.x], q = b.query[threadIdx.x];
-    x.slot_base[s] = b.base[threadIdx.x];
-    Ctl c;
-    const unsigned long long nxt = atomicAdd(&x.qnext[q], 1ull);
-    c.item = (long long)nxt; c.q = q; c.m = 0; c.G = 0; c.F = 0; c.flags = 0u;
-    for (int k = 0; k < U_KINDS; ++k) c.units[k] = 0;
-    if ((long long)nxt < x.qs[q].n_cfg) { c.phase = PH_DRAW0; fill_plan(c, x.qs[q]); }
-    else c.phase = PH_EMPTY;
-    x.ctl[s] = c;
-  }
-  __threadfence();
-  __syncthreads();
-  plan_prefix(x);
-}
-
-__global__ void server_reset_kernel(Ctx x) {
-  for (int s = threadIdx.x; s < x.K; s += blockDim.x) {
-    Ctl c;
-    c.item = 0; c.q = 0; c.phase = PH_EMPTY; c.m = 0; c.G = 0; c.F = 0; c.flags = 0u;
-    for (int k = 0; k < U_KINDS; ++k) c.units[k] = 0;
-    x.ctl[s] = c;
-    x.pre[s] = 0;
-  }
-  if (threadIdx.x == 0) { x.pre[x.K] = 0; *x.arrive = 0u; *x.next_unit = 0u; *x.ticks = 0u; *x.n_done = 0ull; }
-}
-
-__global__ void server_status_kernel(Ctx x, int* phases) {
-  for (int s = threadIdx.x; s < x.K; s += blockDim.x) phases[s] = x.ctl[s].phase;
-}
-
-}  // namespace
-
-struct ServerEngine {
-  Ctx x;
-  char* mem = nullptr;
-  int* d_phase = nullptr;
-  int* h_phase[2] = {};                 // pinned [K], one per status buffer
-  unsigned long long* h_qdone[2] = {};  // pinned [nq]
-  cudaGraphExec_t chunk = nullptr;
-  int max_queries = 0;
-};
-
-pc_status server_engine_create(int max_slots, int max_queries, int ticks_per_chunk, int max_W,
-                               cudaStream_t st, ServerEngine** out) {
-  *out = nullptr;
-  ServerEngine* E = new ServerEngine();
-  Ctx& x = E->x;
-  const int K = std::max(1, std::min(max_slots, kMaxSlots));
-  const int nq = std::max(1, max_queries);
-  const size_t bytes = a256(sizeof(QDev) * nq) + a256(sizeof(Ctl) * K) + a256(sizeof(int) * (K + 1)) +
-                       a256(sizeof(char*) * K) + 2 * a256(sizeof(unsigned long long) * nq) +
-                       a256(sizeof(int) * K) + 256;
-  cudaError_t e = cudaMalloc((void**)&E->mem, bytes);
-  if (e != cudaSuccess) { delete E; return cuda_fail(e, "server engine alloc"); }
-  char* q = E->mem;
-  x = Ctx{};
-  x.qs = (const QDev*)q; q += a256(sizeof(QDev) * nq);
-  x.nq = nq; x.n_items = 0; x.K = K;
-  x.ctl = (Ctl*)q; q += a256(sizeof(Ctl) * K);
-  x.pre = (int*)q; q += a256(sizeof(int) * (K + 1));
-  x.slot_base = (char**)q; q += a256(sizeof(char*) * K);
-  x.qnext = (unsigned long long*)q; q += a256(sizeof(unsigned long long) * nq);
-  x.qdone = (unsigned long long*)q; q += a256(sizeof(unsigned long long) * nq);
-  E->d_phase = (int*)q; q += a256(sizeof(int) * K);
-  x.work = (unsigned long long*)q;
-  x.n_done = x.work + 1;
-  x.ticks = (unsigned int*)(x.work + 2);
-  x.arrive = x.ticks + 1;
-  x.error = (int*)(x.ticks + 2);
-  x.next_unit = x.ticks + 3;
-  x.pool = nullptr; x.slot_bytes = 0; x.max_ticks = 0xffffffffu;
-  x.use_cond = 0; x.server = 1; x.fp = 1;  // served queries may run the FP32 recursion
-  x.seg_cap = max_pair_segment(max_W, kCols) + 16;  // any lattice the server accepts
-  x.nring = ring_depth(x.seg_cap);
-  E->max_queries = nq;
-  pc_status rc = PC_OK;
-  do {
-    if ((e = cudaMemsetAsync(E->mem, 0, bytes, st)) != cudaSuccess) { rc = cuda_fail(e, "server memset"); break; }
-    server_reset_kernel<<<1, 1024, 0, st>>>(x);
-    if ((e = cudaGetLastError()) != cudaSuccess) { rc = cuda_fail(e, "server reset"); break; }
-    for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
-      e = cudaMallocHost((void**)&E->h_phase[b], sizeof(int) * K);
-      if (e == cudaSuccess) e = cudaMallocHost((void**)&E->h_qdone[b], sizeof(unsigned long long) * nq);
-    }
-    if (e != cudaSuccess) { rc = cuda_fail(e, "pinned"); break; }
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if ((e = cudaFuncSetAttribute(sweep_fn(x), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  sweep_smem_bytes(x.seg_cap, x.nring, x.K))) != cudaSuccess) {
-      rc = cuda_fail(e, "sweep smem"); break;
-    }
-    cudaGraph_t g;
-    if ((e = cudaGraphCreate(&g, 0)) != cudaSuccess) { rc = cuda_fail(e, "graph"); break; }
-    void* args[] = {&x};
-    cudaGraphNode_t prev = nullptr;
-    for (int t = 0; t < std::max(1, ticks_per_chunk) && rc == PC_OK; ++t) {
-      cudaKernelNodeParams sp = {};
-      sp.func = const_cast<void*>(sweep_fn(x)); sp.gridDim = dim3(sweep_grid(x)); sp.blockDim = dim3(kCols);
-      sp.kernelParams = args;
-      sp.sharedMemBytes = (unsigned)sweep_smem_bytes(x.seg_cap, x.nring, x.K);
-      cudaGraphNode_t ns, nc;
-      if ((e = cudaGraphAddKernelNode(&ns, g, prev ? &prev : nullptr, prev ? 1 : 0, &sp)) != cudaSuccess) { rc = cuda_fail(e, "node"); break; }
-      cudaKernelNodeParams cp = {};
-      cp.func = (void*)control_kernel; cp.gridDim = dim3(K); cp.blockDim = dim3(kCols);
-      cp.kernelParams = args;
-      if ((e = cudaGraphAddKernelNode(&nc, g, &ns, 1, &cp)) != cudaSuccess) { rc = cuda_fail(e, "node"); break; }
-      prev = nc;
-    }
-    if (rc == PC_OK && (e = cudaGraphInstantiate(&E->chunk, g, 0)) != cudaSuccess) rc = cuda_fail(e, "instantiate");
-    cudaGraphDestroy(g);
-    if (rc == PC_OK && (e = cudaStreamSynchronize(st)) != cudaSuccess) rc = cuda_fail(e, "server init sync");
-  } while (0);
-  if (rc) { server_engine_destroy(E); return rc; }
-  *out = E;
-  return PC_OK;
-}
-
-void server_engine_destroy(ServerEngine* E) {
-  if (!E) return;
-  if (E->chunk) cudaGraphExecDestroy(E->chunk);
-  for (int b = 0; b < 2; ++b) {
-    if (E->h_phase[b]) cudaFreeHost(E->h_phase[b]);
-    if (E->h_qdone[b]) cudaFreeHost(E->h_qdone[b]);
-  }
-  if (E->mem) cudaFree(E->mem);
-  delete E;
-}
-
-int server_engine_slots(const ServerEngine* E) { return E->x.K; }
-
-pc_status server_engine_set_query(ServerEngine* E, int qi, const StreamQuery& sq, cudaStream_t st) {
-  if (qi < 0 || qi >= E->max_queries) { set_error("server: query index out of range"); return PC_ERR_ARG; }
-  QChunk ch;
-  ch.base = qi; ch.n = 1;
-  QDev& d = ch.q[0];
-  d.lat = stream_view(sq.lat); d.occ = sq.occ; d.occ_bits = sq.occ_bits; d.words_per_cfg = sq.words_per_cfg;
-  d.n_cfg = sq.n_cfg; d.cfg0 = sq.cfg0; d.out = sq.out; d.item0 = 0; d.bits_only = sq.bits_only; d.sel = nullptr;
-  upload_queries_kernel<<<1, kQChunk, 0, st>>>((QDev*)E->x.qs, ch);
-  PC_CUDA(cudaGetLastError());
-  PC_CUDA(cudaMemsetAsync(E->x.qnext + qi, 0, sizeof(unsigned long long), st));
-  PC_CUDA(cudaMemsetAsync(E->x.qdone + qi, 0, sizeof(unsigned long long), st));
-  return PC_OK;
-}
-
-pc_status server_engine_bind(ServerEngine* E, const int* slots, const int* queries, char* const* bases,
-                             int n, cudaStream_t st) {
-  for (int b = 0; b < n; b += kBindChunk) {
-    BindList bl;
-    bl.n = std::min(kBindChunk, n - b);
-    for (int i = 0; i < bl.n; ++i) { bl.slot[i] = slots[b + i]; bl.query[i] = queries[b + i]; bl.base[i] = bases[b + i]; }
-    server_bind_kernel<<<1, 1024, 0, st>>>(E->x, bl);
-    PC_CUDA(cudaGetLastError());
-  }
-  return PC_OK;
-}
-
-pc_status server_engine_run_chunk(ServerEngine* E, cudaStream_t st) {
-  PC_CUDA(cudaGraphLaunch(E->chunk, st));
-  return PC_OK;
-}
-
-// Enqueue the copy of slot phases and per-query completion counts to pinned
-// host memory; valid after st reaches this point.
-const int* server_engine_phase_buffer(const ServerEngine* E, int buf) { return E->h_phase[buf]; }
-const unsigned long long* server_engine_qdone_buffer(const ServerEngine* E, int buf) { return E->h_qdone[buf]; }
-
-pc_status server_engine_status(ServerEngine* E, cudaStream_t st, int buf, const int** phases,
-                               const unsigned long long** qdone) {
-  server_status_kernel<<<1, 1024, 0, st>>>(E->x, E->d_phase);
-  PC_CUDA(cudaGetLastError());
-  PC_CUDA(cudaMemcpyAsync(E->h_phase[buf], E->d_phase, sizeof(int) * E->x.K, cudaMemcpyDeviceToHost, st));
-  PC_CUDA(cudaMemcpyAsync(E->h_qdone[buf], E->x.qdone, sizeof(unsigned long long) * E->max_queries,
-                          cudaMemcpyDeviceToHost, st));
-  *phases = E->h_phase[buf];
-  *qdone = E->h_qdone[buf];
-  return PC_OK;
 }
 
 // Single-query convenience used by pc_inspect: build, run, release (stream

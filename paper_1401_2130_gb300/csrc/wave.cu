@@ -16,9 +16,9 @@
 // later ones are 0, as in the full FP32 recursion.
 //
 // wave_kernel<.., false>: levels of every configuration (verdict, first_hit,
-//   m_stop), and the list of the percolating ones.
-// wave_kernel<.., true>: the levels of the listed configurations again, with
-//   nu, until the end layer is reached or nu has vanished.
+//   m_stop; mass 0).
+// wave_kernel<.., true>: the levels of the percolating ones again, with nu,
+//   until the end layer is reached or nu has vanished.
 //
 // A "group" (one warp, or one CTA) takes configurations from a counter.  It
 // keeps
@@ -184,12 +184,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         item = gs->item;
       }
     }
-    if (kMass) {
-      if (item >= (long long)*a.list_n) break;
-      item = (long long)a.list[item];
-    } else if (item >= a.n_items) {
-      break;
-    }
+    if (item >= a.n_items) break;
     int qi = 0;
     if (a.nq > 1) {  // items come in order: mostly the previous one's query
       if (cur_q >= 0 && item >= a.qs[cur_q].item0 && item < a.qs[cur_q].item0 + a.qs[cur_q].n_cfg) {
@@ -217,6 +212,11 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     const int ring_mask = Q.ring_mask;
     const size_t nu_n = (size_t)(ring_mask < 0 ? L : ring_mask + 1) * P;
     const long long rel = item - Q.item0;
+    if (kMass) {  // percolating configurations only (group-uniform)
+      const bool skip = !Q.want_mass || (a.hard ? !(Q.out.mass[rel] < 0.f) : !Q.out.verdict[rel]);
+      group_sync<kWarp>();  // every thread has read the item
+      if (skip) continue;
+    }
     if (qi != cur_q) {
       cur_q = qi;
       for (int k = tid; k < 8 * (2 * Q.W + 1); k += size) roff[k] = (k & 7) < 4 ? Q.row_off[(k >> 3) * 4 + (k & 7)] : 0;
@@ -712,17 +712,13 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     }
     if (tid == 0) {
       if (kMass) {
-        if (hard) a.hard[atomicAdd(a.hard_n, 1ull)] = (unsigned long long)item;
-        else Q.out.mass[rel] = mass;
+        Q.out.mass[rel] = hard ? -1.f : mass;
       } else {
         Q.out.verdict[rel] = (uint8_t)verdict;
         if (Q.out.first_hit) Q.out.first_hit[rel] = fh;
         if (Q.out.mass) Q.out.mass[rel] = 0.f;
         if (Q.out.m_stop) Q.out.m_stop[rel] = mstop;
-        if (verdict) {
-          if (Q.out.n_perc) atomicAdd(Q.out.n_perc, 1ull);
-          if (Q.want_mass) a.list[atomicAdd(a.list_n, 1ull)] = (unsigned long long)item;
-        }
+        if (verdict && Q.out.n_perc) atomicAdd(Q.out.n_perc, 1ull);
       }
     }
     group_sync<kWarp>();
@@ -792,7 +788,7 @@ struct WaveClass {
   size_t group_smem = 0;
   size_t stride_b = 256, stride_m = 256, stride_h = 256;
   long long grid_b = 0, grid_m = 0, grid_h = 0;
-  size_t scratch = 0, list_b = 0, table_b = 0;
+  size_t scratch = 0, table_b = 0;
 };
 
 // Threads of a group.  With more configurations than groups fit the device,
@@ -853,7 +849,17 @@ int wave_threads(int A, long long n_all) {
   return group_threads(A, n_all, nsm);
 }
 
-pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st) {
+size_t wave_scratch_bytes(const Lattice& lat) {
+  WaveClass c;
+  c.threads = 512;
+  WaveQuery w = {};
+  fill_lattice(w, lat);
+  w.want_mass = 1;
+  place(w, c, 64 * 1024);  // (a smaller window than any device gives it: evicted rows counted)
+  return std::max(c.stride_b, std::max(c.stride_m, c.stride_h));
+}
+
+pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m, size_t limit) {
   int dev = 0, nsm = 0, optin = 0;
   PC_CUDA(cudaGetDevice(&dev));
   PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -866,10 +872,11 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st) {
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return qs[x].lat.N > qs[y].lat.N; });
   long long n_all = 0;
   for (int i : order) n_all += qs[i].n_cfg;
+  if (m) n_all = std::min(n_all, m->max_groups);
   std::vector<WaveClass> cls;
   for (int i : order) {
     const StreamQuery& s = qs[i];
-    const int threads = group_threads(s.lat.A, n_all, nsm);
+    const int threads = std::max(group_threads(s.lat.A, n_all, nsm), m ? 128 : 32);  // (a warp group's scratch comes in fours)
     auto c = std::find_if(cls.begin(), cls.end(), [&](const WaveClass& x) { return x.threads == threads; });
     if (c == cls.end()) {
       cls.emplace_back();
@@ -887,77 +894,90 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st) {
     if (w.want_mass) c->mass_items += s.n_cfg;
     c->q.push_back(w);
   }
-  // grids and device memory: fewer groups where the scratch of all of them
-  // cannot be had
-  char* mem = nullptr;
-  for (size_t total = 24ull << 30;; total /= 8) {
+  // grids and scratch of at most `total` bytes (one group per launch at least)
+  auto plan = [&](size_t total, size_t* bytes) -> pc_status {
     const size_t budget = total / cls.size();
-    size_t bytes = 256 * cls.size();
+    *bytes = 256 * cls.size();
     for (WaveClass& c : cls) {
       const size_t per_cta = c.threads == 32 ? 4 : 1;
       const int block = c.threads * (int)per_cta;
-      const size_t smem = c.group_smem * per_cta;
-      auto grid_of = [&](bool mass, long long items, size_t stride, size_t most, long long* g) -> pc_status {
+      auto grid_of = [&](bool mass, size_t stride, size_t most, long long* g) -> pc_status {
         const void* f = wave_fn(c.threads == 32, c.part, mass);
         // the same limit on every call: calls from several threads never lower it
         PC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
         int per_sm = 0;
-        PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, block, smem));
+        PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, block, c.group_smem * per_cta));
         if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
-        long long n = std::min<long long>((long long)per_sm * nsm, (items + (long long)per_cta - 1) / (long long)per_cta);
+        long long n = std::min<long long>((long long)per_sm * nsm, (c.items + (long long)per_cta - 1) / (long long)per_cta);
         n = std::min<long long>(n, (long long)(most / (stride * per_cta)));
+        if (m) n = std::min(n, m->max_groups);
         *g = std::max<long long>(n, 1);
         return PC_OK;
       };
-      pc_status rc = grid_of(false, c.items, c.stride_b, budget, &c.grid_b);
+      pc_status rc = grid_of(false, c.stride_b, budget, &c.grid_b);
       if (rc) return rc;
       c.scratch = c.stride_b * (size_t)c.grid_b * per_cta;
       if (c.mass_items) {
-        if ((rc = grid_of(true, c.mass_items, c.stride_m, budget, &c.grid_m))) return rc;
+        if ((rc = grid_of(true, c.stride_m, budget, &c.grid_m))) return rc;
         c.scratch = std::max(c.scratch, c.stride_m * (size_t)c.grid_m * per_cta);
-        c.list_b = up(8 * (size_t)c.mass_items, 256);
         if (c.ring) {
-          if ((rc = grid_of(true, c.mass_items, c.stride_h, c.scratch, &c.grid_h))) return rc;
+          if ((rc = grid_of(true, c.stride_h, std::min(budget, c.scratch), &c.grid_h))) return rc;
           c.scratch = std::max(c.scratch, c.stride_h * (size_t)c.grid_h * per_cta);
         }
       }
       c.table_b = c.q.size() > 1 ? up(sizeof(WaveQuery) * c.q.size(), 256) : 0;
-      bytes += c.table_b * (c.ring ? 2 : 1) + c.list_b * (c.ring ? 2 : 1) + c.scratch;
+      *bytes += c.table_b * (c.ring ? 2 : 1) + c.scratch;
     }
-    cudaError_t e = cudaMallocAsync((void**)&mem, bytes, st);
-    if (e == cudaSuccess) break;
-    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "wavefront solver: scratch");
-    cudaGetLastError();
-    if (total < (1ull << 20)) {
-      set_error("wavefront solver: no memory for one configuration's state");
-      return PC_ERR_OOM;
+    return PC_OK;
+  };
+  pc_status rc = PC_OK;
+  cudaError_t e = cudaSuccess;
+  char* mem = nullptr;
+  size_t bytes = 0;
+  if (m) {
+    if ((rc = plan(m->bytes, &bytes))) return rc;
+    if (cls.size() != 1 || cls[0].table_b || cls[0].scratch > m->bytes) {
+      set_error("wavefront solver: the caller's memory does not hold the query");
+      return PC_ERR_INTERNAL;
     }
+  } else {
+    for (size_t total = limit;; total /= 8) {  // fewer groups where the memory for more cannot be had
+      if ((rc = plan(total, &bytes))) return rc;
+      e = cudaMallocAsync((void**)&mem, bytes, st);
+      if (e == cudaSuccess) break;
+      if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "wavefront solver: scratch");
+      cudaGetLastError();
+      if (total < (1ull << 20)) {
+        set_error("wavefront solver: no memory for one configuration's state");
+        return PC_ERR_OOM;
+      }
+    }
+    e = cudaMemsetAsync(mem, 0, 256 * cls.size(), st);
   }
-  cudaError_t e = cudaMemsetAsync(mem, 0, 256 * cls.size(), st);
-  char* at = mem + 256 * cls.size();
+  char* at = m ? m->scratch : mem + 256 * cls.size();
   for (size_t k = 0; k < cls.size(); ++k) {
     WaveClass& c = cls[k];
     const int per_cta = c.threads == 32 ? 4 : 1;  // groups to a CTA
-    unsigned long long* ctr = (unsigned long long*)(mem + 256 * k);
+    unsigned long long* ctr = m ? m->ctr : (unsigned long long*)(mem + 256 * k);
     WaveArgs a = {};
-    a.q0 = c.q[0];
     a.nq = (int)c.q.size();
     a.n_items = c.items;
     a.group_smem = (int)c.group_smem;
-    auto upload = [&](char* to) {
+    auto tables = [&]() {
+      a.q0 = c.q[0];
+      if (!c.table_b) return;
+      a.qs = (const WaveQuery*)at;
       for (size_t b = 0; b < c.q.size() && e == cudaSuccess; b += kUpload) {
         UploadChunk u = {};
         u.n = (int)std::min<size_t>(kUpload, c.q.size() - b);
         for (int i = 0; i < u.n; ++i) u.q[i] = c.q[b + i];
-        wave_upload_kernel<<<1, kUpload, 0, st>>>((WaveQuery*)to + b, u);
+        wave_upload_kernel<<<1, kUpload, 0, st>>>((WaveQuery*)at + b, u);
         e = cudaGetLastError();
       }
+      at += c.table_b;
     };
-    if (c.table_b) { a.qs = (const WaveQuery*)at; upload(at); at += c.table_b; }
-    a.list = (unsigned long long*)at; at += c.list_b;
-    a.list_n = ctr + 1;
-    a.hard_n = ctr + 2;
-    if (c.ring) { a.hard = (unsigned long long*)at; at += c.list_b; }
+    tables();
+    a.scratch = at; at += c.scratch;
     auto launch = [&](bool mass, long long grid, unsigned long long* work, size_t stride) {
       a.work = work;
       a.scratch_stride = (long long)stride;
@@ -966,23 +986,19 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st) {
         e = cudaLaunchKernel(wave_fn(c.threads == 32, c.part, mass), dim3((unsigned)grid), dim3(c.threads * per_cta),
                              args, c.group_smem * per_cta, st);
     };
-    char* table_h = at;
-    if (c.ring) at += c.table_b;
-    a.scratch = at; at += c.scratch;
     launch(false, c.grid_b, ctr, c.stride_b);
     if (c.mass_items) {
-      launch(true, c.grid_m, ctr + 3, c.stride_m);
+      launch(true, c.grid_m, ctr + 1, c.stride_m);
       if (c.ring) {  // frontiers that outgrew the mass rings: a plane for every layer
         for (WaveQuery& w : c.q) w.ring_mask = -1;
-        a.q0 = c.q[0];
-        if (c.table_b) { a.qs = (const WaveQuery*)table_h; upload(table_h); }
-        a.list = a.hard; a.list_n = a.hard_n;
-        launch(true, c.grid_h, ctr + 4, c.stride_h);
+        tables();
+        a.hard = 1;
+        launch(true, c.grid_h, ctr + 2, c.stride_h);
       }
     }
   }
-  pc_status rc = e == cudaSuccess ? PC_OK : cuda_fail(e, "wavefront solver");
-  cudaFreeAsync(mem, st);
+  if (e != cudaSuccess) rc = cuda_fail(e, "wavefront solver");
+  if (mem) cudaFreeAsync(mem, st);
   return rc;
 }
 

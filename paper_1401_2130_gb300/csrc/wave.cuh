@@ -36,18 +36,28 @@ struct WaveArgs {
   const WaveQuery* qs;       // [nq] by increasing item0
   int nq;
   long long n_items;
-  unsigned long long* work;     // next work item (or entry of list)
-  unsigned long long* list;     // percolating items whose mass is wanted
-  unsigned long long* list_n;
-  unsigned long long* hard;     // items whose frontier outgrew the mass rings
-  unsigned long long* hard_n;
+  unsigned long long* work;  // next work item
+  int hard;                  // mass launches: only the items marked by the first one
   int group_smem;
   char* scratch;
   long long scratch_stride;
 };
 
-// Inspects the queries (stream-ordered, no host synchronisation).
-pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st);
+// Device memory that a caller holds for one query's run.
+struct WaveMemory {
+  unsigned long long* ctr;   // 4 zeroed counters
+  char* scratch;
+  size_t bytes;              // at least wave_scratch_bytes of the lattice
+  long long max_groups;      // configurations in work at once
+};
+// Scratch of one configuration in work on a WaveMemory.
+size_t wave_scratch_bytes(const Lattice& lat);
+
+// Inspects the queries (stream-ordered, no host synchronisation).  Without m
+// the scratch is allocated on st, at most `limit` bytes where that is enough
+// for one configuration; with m (one query) nothing is allocated.
+pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m = nullptr,
+                   size_t limit = 24ull << 30);
 // Threads that work on one configuration of an A-column lattice when n_all
 // configurations are inspected together on the current device.
 int wave_threads(int A, long long n_all);
