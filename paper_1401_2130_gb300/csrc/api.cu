@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
 #include "wave.cuh"
 
 namespace pc {
@@ -109,7 +110,7 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
   size_t bytes = 64;  // work counter, percolating counter, streamed-solver error flag
   if (!dev_out) bytes += (size_t)n * (1 + 4 + 4 + 4) + 64;
   Scratch s;
-  PC_CUDA(cudaMallocAsync((void**)&s.base, bytes, st));
+  PC_CUDA(scratch_alloc((void**)&s.base, bytes, st));
   s.work = (unsigned long long*)s.base;
   s.n_perc = s.work + 1;
   if (dev_out) {
@@ -174,16 +175,33 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
     }
     if (rc) break;
     if (!dev_out) {
-      cudaError_t e = cudaMemcpyAsync(verdicts, s.verdict, (size_t)n, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess && first_hit) e = cudaMemcpyAsync(first_hit, s.first_hit, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess && mass) e = cudaMemcpyAsync(mass, s.mass, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess && m_stop) e = cudaMemcpyAsync(m_stop, s.m_stop, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
+      // counters, first hits, masses, step counts and verdicts lie in a row
       unsigned long long cnt = 0;
       int err = 0;
-      if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, s.n_perc, 8, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(&err, s.work + 2, sizeof(int), cudaMemcpyDeviceToHost, st);
+      const size_t all = 64 + (size_t)n * 13;
+      HostStage stage(all);
+      cudaError_t e = cudaSuccess;
+      if (stage.data()) {
+        e = cudaMemcpyAsync(stage.data(), s.base, all, cudaMemcpyDeviceToHost, st);
+      } else {
+        e = cudaMemcpyAsync(verdicts, s.verdict, (size_t)n, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess && first_hit) e = cudaMemcpyAsync(first_hit, s.first_hit, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess && mass) e = cudaMemcpyAsync(mass, s.mass, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess && m_stop) e = cudaMemcpyAsync(m_stop, s.m_stop, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, s.n_perc, 8, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&err, s.work + 2, sizeof(int), cudaMemcpyDeviceToHost, st);
+      }
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
       if (e != cudaSuccess) { rc = cuda_fail(e, "copy outputs"); break; }
+      if (const char* h = stage.data()) {
+        std::memcpy(&cnt, h + 8, 8);
+        std::memcpy(&err, h + 16, sizeof(int));
+        h += 64;
+        if (first_hit) std::memcpy(first_hit, h, (size_t)n * 4);
+        if (mass) std::memcpy(mass, h + (size_t)n * 4, (size_t)n * 4);
+        if (m_stop) std::memcpy(m_stop, h + (size_t)n * 8, (size_t)n * 4);
+        std::memcpy(verdicts, h + (size_t)n * 12, (size_t)n);
+      }
       if (err & 2) { set_error("streamed solver: a bulk-copy wait timed out"); rc = PC_ERR_TIMEOUT; break; }
       if (err) { set_error("streamed solver: tick bound or device check failed"); rc = PC_ERR_INTERNAL; break; }
       if (n_percolating) *n_percolating = (int64_t)cnt;
@@ -286,6 +304,7 @@ pc_status pc_inspect_occupancy(int32_t W, int32_t L, const uint32_t* occ_bits, i
 }
 
 pc_status pc_shutdown(void) {
+  release_pools();
   release_lattices();
   release_static();
   return PC_OK;

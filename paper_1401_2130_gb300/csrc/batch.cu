@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
 #include "tune_file.h"
 #include "wave.cuh"
 
@@ -172,7 +173,7 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
   if (!dev_out)
     for (int64_t i = 0; i < nq; ++i) bytes += ((size_t)q[i].n_configs * 13 + 255) & ~(size_t)255;
   char* mem = nullptr;
-  PC_CUDA(cudaMallocAsync((void**)&mem, bytes, st));
+  PC_CUDA(scratch_alloc((void**)&mem, bytes, st));
   unsigned long long* counts = (unsigned long long*)mem;
   pc_status rc = PC_OK;
   long long n_all = 0;
@@ -218,12 +219,15 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch counts"); break; }
     if (async) break;
     // one copy of the counts and, for host queries, of every output
-    std::vector<char> host(dev_out ? (size_t)nq * 8 : bytes);
-    e = cudaMemcpyAsync(host.data(), mem, host.size(), cudaMemcpyDeviceToHost, st);
+    const size_t all = dev_out ? (size_t)nq * 8 : bytes;
+    HostStage pinned(all);
+    std::vector<char> plain(pinned.data() ? 0 : all);
+    const char* host = pinned.data() ? pinned.data() : plain.data();
+    e = cudaMemcpyAsync((void*)host, mem, all, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch outputs"); break; }
-    const unsigned long long* cnt = (const unsigned long long*)host.data();
-    const char* at = host.data() + ctr_b;
+    const unsigned long long* cnt = (const unsigned long long*)host;
+    const char* at = host + ctr_b;
     for (int64_t i = 0; i < nq; ++i) {
       const size_t n = (size_t)q[i].n_configs;
       if (!dev_out) {

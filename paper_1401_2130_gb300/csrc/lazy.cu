@@ -9,6 +9,7 @@
 // outputs come from the plain inspection's: verdicts, first_hit and m_stop
 // unchanged, mass scaled here on the device.
 #include "common.cuh"
+#include "pool.cuh"
 
 namespace pc {
 namespace {
@@ -53,7 +54,7 @@ extern "C" pc_status pc_lazy_mass(const int32_t* first_hit, const float* mass, i
   // host buffers: stage through one stream-ordered device allocation
   const size_t b4 = (size_t)n_configs * 4;
   char* d = nullptr;
-  PC_CUDA(cudaMallocAsync((void**)&d, 3 * b4, st));
+  PC_CUDA(scratch_alloc((void**)&d, 3 * b4, st));
   int32_t* dfh = (int32_t*)d;
   float* dm = (float*)(d + b4);
   float* dout = (float*)(d + 2 * b4);

@@ -6,6 +6,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
 
 namespace pc {
 
@@ -198,7 +199,7 @@ pc_status launch_occupancy_fixed(const Lattice& lat, const OccStream& os, uint32
   char* mem = nullptr;
   const size_t st_bytes = ((size_t)n_cfg * sizeof(FcState) + 255) & ~(size_t)255;
   const size_t bytes = st_bytes + (size_t)n_cfg * 256 * sizeof(unsigned int) + 256;
-  PC_CUDA(cudaMallocAsync((void**)&mem, bytes, st));
+  PC_CUDA(scratch_alloc((void**)&mem, bytes, st));
   FcState* s = (FcState*)mem;
   unsigned int* hist = (unsigned int*)(mem + st_bytes);
   int* error = (int*)(mem + bytes - 256);

@@ -1,0 +1,101 @@
+// pool.cu -- device scratch and pinned staging kept between calls.
+//
+// Device scratch comes from one memory pool per device, apart from the
+// process's default pool (whose settings are the application's).  A pool with
+// the default release threshold gives its memory back to the system at every
+// synchronisation, and mapping it again cost a call of host outputs 0.2 to 1.5
+// ms (W = 4, L = 16, 1,000 configurations: 327 us alone, against 64 us among
+// others that are not waited for).  This pool keeps at most kKeep bytes.
+// Allocation and free stay stream-ordered, so threads and streams share it
+// safely.
+//
+// Outputs for the host come back in one copy to a pinned buffer: each of the
+// six pageable copies it replaces waits for the stream on its own.  At most
+// kBuffers buffers of kStageBytes are kept; more concurrent calls allocate and
+// free their own.  pc_shutdown gives everything back.
+#include <map>
+#include <mutex>
+#include <vector>
+
+#include "pool.cuh"
+
+namespace pc {
+
+namespace {
+
+constexpr uint64_t kKeep = 1ull << 30;
+constexpr size_t kStageBytes = 4u << 20;
+constexpr size_t kBuffers = 8;
+
+std::mutex g_mu;
+std::map<int, cudaMemPool_t> g_pools;
+std::vector<char*> g_stage;
+
+}  // namespace
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    auto it = g_pools.find(dev);
+    if (it == g_pools.end()) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
+      uint64_t keep = kKeep;
+      e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+      // memory freed on another stream is reused only once that stream has
+      // passed the free: no stream is made to wait for another
+      int no = 0;
+      if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no);
+      if (e != cudaSuccess) { cudaMemPoolDestroy(pool); return e; }
+      it = g_pools.emplace(dev, pool).first;
+    }
+    pool = it->second;
+  }
+  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+
+HostStage::HostStage(size_t bytes) {
+  if (bytes > kStageBytes) return;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (!g_stage.empty()) {
+      p_ = g_stage.back();
+      g_stage.pop_back();
+      return;
+    }
+  }
+  if (cudaMallocHost((void**)&p_, kStageBytes) != cudaSuccess) {
+    cudaGetLastError();
+    p_ = nullptr;
+  }
+}
+
+HostStage::~HostStage() {
+  if (!p_) return;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (g_stage.size() < kBuffers) {
+      g_stage.push_back(p_);
+      return;
+    }
+  }
+  cudaFreeHost(p_);
+}
+
+void release_pools() {
+  std::lock_guard<std::mutex> lk(g_mu);
+  for (auto& kv : g_pools) cudaMemPoolDestroy(kv.second);
+  g_pools.clear();
+  for (char* p : g_stage) cudaFreeHost(p);
+  g_stage.clear();
+  cudaGetLastError();  // after cudaDeviceReset the handles are gone already
+}
+
+}  // namespace pc

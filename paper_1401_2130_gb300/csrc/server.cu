@@ -207,7 +207,11 @@ void worker_main(pc_server* s) {
           const size_t sb = stream_slot_bytes(q.W, q.L);
           if (!s->arena.alloc(ob, &off)) break;
           const size_t room = s->arena.largest();
-          long long k = std::min<long long>(q.n_configs, s->free_slots);
+          // not more than half of the free slots while other queries run or
+          // wait: the next one in a burst would be left with a handful for
+          // its whole run (burst of 8: 5.1 - 6.1 ms without this)
+          const bool alone = running.empty() && to_start.empty() && s->pending.size() == 1;
+          long long k = std::min<long long>(q.n_configs, alone ? s->free_slots : (s->free_slots + 1) / 2);
           k = std::min<long long>(k, std::max(1, s->opts.max_slots_per_query));
           k = std::min<long long>(k, (long long)(room / (sb + 256)));
           size_t soff = 0;

@@ -49,6 +49,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
 #include "wave.cuh"
 
 namespace pc {
@@ -943,7 +944,7 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   } else {
     for (size_t total = limit;; total /= 8) {  // fewer groups where the memory for more cannot be had
       if ((rc = plan(total, &bytes))) return rc;
-      e = cudaMallocAsync((void**)&mem, bytes, st);
+      e = scratch_alloc((void**)&mem, bytes, st);
       if (e == cudaSuccess) break;
       if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "wavefront solver: scratch");
       cudaGetLastError();
