@@ -58,6 +58,7 @@ namespace {
 
 constexpr int kPosBits = 18;  // plane position of a frontier entry; its hexagon row above
 constexpr uint32_t kPosMask = (1u << kPosBits) - 1u;
+constexpr uint32_t kNone = 0xffffffffu;  // empty hash entry (no site packs to it)
 constexpr int kDrawLayers = 8;  // layers drawn at a time (divides 32)
 
 // Contact directions (order of common.cuh, then the end contacts): offset
@@ -119,21 +120,19 @@ __device__ __forceinline__ uint32_t atoms_add(uint32_t a, uint32_t v) {
   asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(r) : "r"(a), "r"(v) : "memory");
   return r;
 }
-// the same under a condition, as predicated instructions (no branches)
-__device__ __forceinline__ uint32_t lds_if(bool c, uint32_t a) {
-  uint32_t v = 0u;
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.shared.u32 %0, [%2];\n\t}" : "+r"(v) : "r"((uint32_t)c), "r"(a));
-  return v;
+template <int OFF>
+__device__ __forceinline__ uint32_t atoms_and_at(uint32_t a, uint32_t m) {
+  uint32_t r;
+  asm volatile("atom.shared.and.b32 %0, [%1+%3], %2;" : "=r"(r) : "r"(a), "r"(m), "n"(OFF) : "memory");
+  return r;
 }
-__device__ __forceinline__ uint32_t atoms_and_if(uint32_t c, uint32_t a, uint32_t m) {
-  uint32_t v = 0u;
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p atom.shared.and.b32 %0, [%2], %3;\n\t}"
-               : "+r"(v) : "r"(c), "r"(a), "r"(m) : "memory");
-  return v;
-}
+// the same under a condition: a predicated instruction, no branch
 __device__ __forceinline__ void sts_u2_if(bool c, uint32_t a, uint32_t x, uint32_t y) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.v2.u32 [%1], {%2, %3};\n\t}"
                :: "r"((uint32_t)c), "r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void sts_u2(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" :: "r"(a), "r"(x), "r"(y) : "memory");
 }
 __device__ __forceinline__ void reds_min(uint32_t a, int v) {
   asm volatile("red.shared.min.s32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
@@ -153,8 +152,13 @@ __device__ __forceinline__ uint32_t smem_at(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-template <bool kWarp, bool kPart, bool kMass>
+// kMode: levels only, or levels with nu -- in shared memory (a hash table of
+// the level's sites) or in planes in device scratch
+enum : int { M_LEVELS = 0, M_HASH = 1, M_PLANES = 2 };
+
+template <bool kWarp, bool kPart, int kMode>
 __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, char* scratch) {
+  constexpr bool kMass = kMode != M_LEVELS;
   const int tid = kWarp ? (threadIdx.x & 31) : threadIdx.x;
   const int size = kWarp ? 32 : blockDim.x;
   const int lane = threadIdx.x & 31;
@@ -208,8 +212,12 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     uint32_t* back = reinterpret_cast<uint32_t*>(scratch + Q.a_back);
     uint32_t* over = reinterpret_cast<uint32_t*>(scratch + Q.a_over);  // two maps of TW rows
     const size_t over_n = (size_t)Q.TW * P;
-    uint32_t* occ = reinterpret_cast<uint32_t*>(scratch + Q.a_occ);
+    uint32_t* occ = Q.o_occ >= 0 ? reinterpret_cast<uint32_t*>(sm + Q.o_occ) : reinterpret_cast<uint32_t*>(scratch + Q.a_occ);
     float* nu = reinterpret_cast<float*>(scratch + Q.a_nu);            // two rings of planes
+    // hash tables (key, entry) of two levels, then nu of the entries of two levels
+    const uint32_t tab_s = smem_at(sm + Q.o_tab), nuq_s = tab_s + 16u * (1u << Q.tab_bits);
+    const int tab_bits = Q.tab_bits;
+    const uint32_t tab_mask = (1u << tab_bits) - 1u;
     const int ring_mask = Q.ring_mask;
     const size_t nu_n = (size_t)(ring_mask < 0 ? L : ring_mask + 1) * P;
     const long long rel = item - Q.item0;
@@ -228,6 +236,8 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         gs->cf[k][0] = 0u; gs->cf[k][1] = 0u; gs->olo[k] = 0x7fffffff; gs->ohi[k] = -1;
       }
     }
+    if (kMode == M_HASH)
+      for (uint32_t k = tid; k < 2u * (tab_mask + 1u); k += size) sts_u2(tab_s + 8u * k, kNone, 0u);
     group_sync<kWarp>();
 
     int G = 0;   // layers drawn
@@ -237,6 +247,15 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       return resident(w) ? win + (w & nr_mask) * P + pos : back + (size_t)w * P + pos;
     };
     auto plane = [&](int t) -> size_t { return (size_t)(t & ring_mask) * P; };
+    // A frontier entry: the site it was claimed from (position, hexagon row;
+    // tube << 4) and the direction, 15 for that site itself.  Its own position,
+    // row and tube:
+    auto decode = [&](uint2 e, uint32_t& ent, int& t) {
+      const uint2 y = lds_u2(dir_s + 8u * (e.y & 15u));
+      const int pos = (int)(e.x & kPosMask), sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
+      ent = e.x + y.x + lds_u<0>(roff_s + ((e.x >> (kPosBits - 5)) & ~31u) + (y.y & 255u));
+      t = (int)(e.y >> 4) + (int)((y.y >> (8 + 2 * sg)) & 3u) - 1;
+    };
     auto row_of = [&](int pos) -> int { return strip_row[(int)__umulhi((unsigned)pos, 0x55555556u) - sb]; };
     // Slide the window by one row: the row that leaves is written back if it
     // was drawn, the row that enters (the same slot) read if it was.
@@ -265,8 +284,10 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       if ((G & 31) == 0) {  // first layers of the row
         for (int k = tid; k < P; k += size) {
           row[k] = 0u;
-          over[(size_t)w * P + k] = 0u;
-          over[over_n + (size_t)w * P + k] = 0u;
+          if (kMode != M_HASH) {
+            over[(size_t)w * P + k] = 0u;
+            over[over_n + (size_t)w * P + k] = 0u;
+          }
         }
         group_sync<kWarp>();
       }
@@ -330,6 +351,32 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       G = Gn;
     };
 
+    // Hash table of a level: the site's key -> its queue entry.  Levels hold
+    // tubes less than 2^14 apart (longer fibres keep nu in planes).
+    auto key_of = [&](uint32_t pos, int t) -> uint32_t { return pos | (uint32_t)t << kPosBits; };
+    auto hash_add = [&](int level, uint32_t key, uint32_t entry) {
+      uint32_t h = (key * 0x9E3779B1u) >> (32 - tab_bits);
+      const uint32_t base = tab_s + 8u * (uint32_t)((level & 1) << tab_bits);
+      for (;;) {
+        uint32_t old;
+        asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(old) : "r"(base + 8u * h), "r"(kNone), "r"(key) : "memory");
+        if (old == kNone) break;
+        h = (h + 1u) & tab_mask;
+      }
+      asm volatile("st.shared.u32 [%0], %1;" :: "r"(base + 8u * h + 4u), "r"(entry) : "memory");
+    };
+    // nu of a site if it belongs to the level, else 0
+    auto hash_nu = [&](int level, uint32_t key) -> float {
+      uint32_t h = (key * 0x9E3779B1u) >> (32 - tab_bits);
+      const uint32_t base = tab_s + 8u * (uint32_t)((level & 1) << tab_bits);
+      for (;;) {
+        const uint2 e = lds_u2(base + 8u * h);
+        if (e.x == key) return __uint_as_float(lds_u<0>(nuq_s + 4u * (uint32_t)((level & 1) * cap) + 4u * e.y));
+        if (e.x == kNone) return 0.f;
+        h = (h + 1u) & tab_mask;
+      }
+    };
+
     draw();
     // level 0: the metallic sites of t = 0
     unsigned total = 0;
@@ -355,8 +402,13 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
           }
           base += __popc(bal & lt);
           if (c) {
-            if (base < (unsigned)cap) queue[base] = make_uint2((uint32_t)pos | (uint32_t)row_of(pos) << kPosBits, 0u);
-            else { atomicOr(over + pos, 1u); gs->olo[0] = 0; gs->ohi[0] = 0; }
+            if (base < (unsigned)cap) {
+              queue[base] = make_uint2((uint32_t)pos | (uint32_t)row_of(pos) << kPosBits, 15u);
+            } else if (kMode != M_HASH) {
+              atomicOr(over + pos, 1u);
+              gs->olo[0] = 0;
+              gs->ohi[0] = 0;
+            }
           }
         }
       }
@@ -403,6 +455,57 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       else r = (((pcs + pd) + pa) + (pbs + e)) + (h + g);
       return inv * r;
     };
+    // M_HASH: nu of the sites of level m, sixteen lanes to a site, one contact
+    // each; true if any is not 0.  The contact values of the previous level
+    // come from its table (others are not in it: 0), the additions are those of
+    // site_value, between lanes.
+    auto level_hash = [&](int m, unsigned n) -> bool {
+      if (tid == 0) gs->nz[m & 1] = 0u;
+      group_sync<kWarp>();
+      const uint32_t q_s = queue_s + 8u * (uint32_t)((m & 1) * cap);
+      const int half = lane & 16;
+      // the lane whose value the first addition takes: the pairs (0,7) (1,8)
+      // (2,5) (3,10) (4,11) (6,9) (12,13), four bits a lane
+      const int mate = half | (int)((0xFECD4361092BA587ull >> (4 * (lane & 15))) & 15u);
+      bool nz = false;
+      for (unsigned i0 = (unsigned)(tid >> 5) * 2u; i0 < n; i0 += (unsigned)(size >> 5) * 2u) {
+        const unsigned i = i0 + (unsigned)(lane >> 4);
+        const bool act = i < n && has16;
+        uint32_t ent;
+        int t;
+        decode(lds_u2(q_s + 8u * (i < n ? i : i0)), ent, t);
+        const int pos = (int)(ent & kPosMask), sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
+        if (i < n && (lane & 15) == 0) hash_add(m, key_of((uint32_t)pos, t), i);
+        const uint32_t np = (ent + e16 + lds_u<0>(roff_s + ((ent >> (kPosBits - 5)) & ~31u) + (y16 & 255u))) & kPosMask;
+        const int tt = t + (int)((y16 >> (8 + 2 * sg)) & 3u) - 1;
+        const bool on = act && (unsigned)tt < (unsigned)L && ((occ[(size_t)(tt >> 5) * P + np] >> (tt & 31)) & 1u);
+        const float v = on && m ? hash_nu(m - 1, key_of(np, tt)) : 0.f;
+        const unsigned bal = __ballot_sync(0xffffffffu, on);
+        const int deg = __popc(bal & (0x3fffu << half)) + (t == L - 1);  // with the detector edge
+        const float x = v + __shfl_sync(0xffffffffu, v, mate);
+        const float pa = __shfl_sync(0xffffffffu, x, half), pbs = __shfl_sync(0xffffffffu, x, half | 1),
+                    g = __shfl_sync(0xffffffffu, x, half | 2), pd = __shfl_sync(0xffffffffu, x, half | 3),
+                    pcs = __shfl_sync(0xffffffffu, x, half | 4), ee = __shfl_sync(0xffffffffu, x, half | 6),
+                    h = __shfl_sync(0xffffffffu, x, half | 12);
+        float r;
+        if (sg == 0) r = (((pa + pbs) + pcs) + (pd + ee)) + (h + g);
+        else if (sg == 1) r = ((pcs + pd) + (pa + pbs)) + ((ee + h) + g);
+        else r = (((pcs + pd) + pa) + (pbs + ee)) + (h + g);
+        const float inv = deg ? __frcp_rn((float)deg) : 0.f;
+        const float val = m ? inv * r : inv * __frcp_rn((float)n0);
+        if (i < n && (lane & 15) == 0) {
+          asm volatile("st.shared.f32 [%0], %1;" :: "r"(nuq_s + 4u * (uint32_t)((m & 1) * cap) + 4u * i), "f"(val) : "memory");
+          nz |= val != 0.f;
+        }
+      }
+      if (nz) gs->nz[m & 1] = 1u;
+      group_sync<kWarp>();
+      const bool live = gs->nz[m & 1] != 0u;
+      // the other table is the next level's
+      for (uint32_t k = tid; k <= tab_mask; k += size) sts_u2(tab_s + 8u * ((uint32_t)(((m + 1) & 1) << tab_bits) + k), kNone, 0u);
+      group_sync<kWarp>();
+      return live;
+    };
     // nu of the sites of level m (queue qn, overflow rows [lo, hi]); true if any is not 0
     auto level_values = [&](int m, unsigned n, const uint2* qn, int lo, int hi) -> bool {
       const float* src = m ? nu + (size_t)((m - 1) & 1) * nu_n : nullptr;
@@ -412,23 +515,25 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       bool nz = false;
       const unsigned stored = min(n, (unsigned)cap);
       for (unsigned i = tid; i < stored; i += size) {
-        const uint2 e = qn[i];
-        const int t = (int)e.y, pos = (int)(e.x & kPosMask);
-        const float x = site_value(t, pos, (int)(e.x >> kPosBits), src);
+        uint32_t ent;
+        int t;
+        decode(qn[i], ent, t);
+        const int pos = (int)(ent & kPosMask);
+        const float x = site_value(t, pos, (int)(ent >> kPosBits), src);
         dst[plane(t) + pos] = x;
         nz |= x != 0.f;
       }
-        for (int w = lo; w <= hi; ++w)
-          for (int pos = tid; pos < P; pos += size) {
-            uint32_t word = over[(size_t)(m & 1) * over_n + (size_t)w * P + pos];
-            while (word) {
-              const int t = 32 * w + __ffs(word) - 1;
-              word &= word - 1;
-              const float x = site_value(t, pos, row_of(pos), src);
-              dst[plane(t) + pos] = x;
-              nz |= x != 0.f;
-            }
+      for (int w = lo; w <= hi; ++w)
+        for (int pos = tid; pos < P; pos += size) {
+          uint32_t word = over[(size_t)(m & 1) * over_n + (size_t)w * P + pos];
+          while (word) {
+            const int t = 32 * w + __ffs(word) - 1;
+            word &= word - 1;
+            const float x = site_value(t, pos, row_of(pos), src);
+            dst[plane(t) + pos] = x;
+            nz |= x != 0.f;
           }
+        }
       if (nz) gs->nz[m & 1] = 1u;
       group_sync<kWarp>();
       return gs->nz[m & 1] != 0u;
@@ -442,7 +547,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         for (int c = tid; c < A; c += 32) {
           const int pos = __ldg(ppos + c), w = (L - 1) >> 5;
           const uint32_t bit = (occ[(size_t)w * P + pos] & ~*word_ptr(w, pos)) >> ((L - 1) & 31);
-          if (bit & 1u) part_sum += dst[plane(L - 1) + pos];
+          if (bit & 1u) part_sum += kMode == M_HASH ? hash_nu(m, key_of((uint32_t)pos, L - 1)) : dst[plane(L - 1) + pos];
         }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) part_sum += __shfl_xor_sync(0xffffffffu, part_sum, o);
@@ -451,15 +556,15 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
 
     int verdict = 0, fh = -1, mstop = 0;
     float mass = 0.f;
-    bool hard = false;
+    bool hard = kMode == M_HASH && total > (unsigned)cap;  // left to the launch with planes
+    if (kMass && n0 > 0 && !hard) {
+      if (kMode == M_HASH) level_hash(0, total);
+      else level_values(0, total, queue, 0, gs->ohi[0]);
+    }
     if (n0 > 0 && L == 1) {
       verdict = 1; fh = 1; mstop = 1;
-      if (kMass) {
-        level_values(0, total, queue, 0, gs->ohi[0]);
-        mass = detector_mass(0);
-      }
-    } else if (n0 > 0) {
-      if (kMass) level_values(0, total, queue, 0, gs->ohi[0]);
+      if (kMass && !hard) mass = detector_mass(0);
+    } else if (n0 > 0 && !hard) {
       int cu_ = 0;  // rotating index of the current level
       for (int m = 1;; ++m) {
         const int nx = cu_ == 2 ? 0 : cu_ + 1, nn = nx == 2 ? 0 : nx + 1;
@@ -473,96 +578,30 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         const int t_lo = kPart ? 32 * wb : 0;
         const unsigned t_span = (unsigned)(min(min(t_need, L - 1), kPart ? 32 * (wb + NR) : 0x7fffffff) - t_lo);
         unsigned count = 0, f = 0;
-        // the site (ent, tt) enters level m as entry idx
-        auto put = [&](bool won, unsigned idx, uint32_t ent, int tt) {
-          sts_u2_if(won && idx < (unsigned)cap, qn_s + 8u * idx, ent, (uint32_t)tt);
-          if (won && (idx >= (unsigned)cap || (unsigned)(tt - t_lo) >= t_span)) {
-            if (idx >= (unsigned)cap) {
-              const int w = tt >> 5;
-              atomicOr(on + (size_t)w * P + (ent & kPosMask), 1u << (tt & 31));
-              reds_min(gs_s + (uint32_t)offsetof(GroupShared, olo) + 4u * (uint32_t)nx, w);
-              reds_max(gs_s + (uint32_t)offsetof(GroupShared, ohi) + 4u * (uint32_t)nx, w);
-            }
-            f |= (tt >= t_need ? F_NEED : 0u) | (tt == L - 1 ? F_HIT : 0u) | (resident(tt >> 5) ? 0u : F_OUT);
-          }
-          if (kMass && won) zero[plane(tt) + (ent & kPosMask)] = 0.f;  // level m holds nothing at step m - 1
-        };
+        // sites at tubes [e_lo, e_lo + e_n) claim nothing outside those
+        const int e_lo = kPart ? t_lo + 1 : 0;
+        const unsigned e_n = (unsigned)max(0, t_lo + (int)t_span - 1 - e_lo);
         // n entries of the next level for this warp
         auto reserve = [&](unsigned n) -> unsigned {
           unsigned base = 0;
-          if (kWarp) {
-            base = count;
-            count += n;
-          } else {
-            if (lane == 0) base = atoms_add(cf_s, n);
-            base = __shfl_sync(0xffffffffu, base, 0);
-          }
-          return base;
+          if (lane == 0) base = atoms_add(cf_s, n);
+          return __shfl_sync(0xffffffffu, base, 0);
         };
         // where the word of (entry, tube) lies in the window
         auto at_of = [&](uint32_t ent, int tt) -> uint32_t {
           return win_s + 4u * (uint32_t)(((tt >> 5) & nr_mask) * P + (int)(ent & kPosMask));
         };
-        auto back_of = [&](uint32_t ent, int tt) -> uint32_t* { return back + (size_t)(tt >> 5) * P + (ent & kPosMask); };
-        // Few sites: sixteen lanes to a site, one contact each, U pairs of
-        // sites at a time, so that the chain of a level is short.
-        auto expand16 = [&](unsigned first, unsigned step, unsigned stored) {
-          constexpr int U = kWarp ? 4 : 2;
-          uint32_t en[U], at[U], got[U];
-          int tt[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const unsigned i = first + (unsigned)u * step + (unsigned)(lane >> 4);
-            const bool act = i < stored && has16;
-            const uint2 e = lds_u2(qc_s + 8u * (act ? i : 0u));
-            const int pos = (int)(e.x & kPosMask), sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
-            en[u] = e.x + e16 + lds_u<0>(roff_s + ((e.x >> (kPosBits - 5)) & ~31u) + (y16 & 255u));
-            tt[u] = (int)e.y + (int)((y16 >> (8 + 2 * sg)) & 3u) - 1;
-            at[u] = at_of(en[u], tt[u]);
-            bool ok = act && tt[u] >= 0;
-            got[u] = 0u;
-            if (kPart && ok && !resident(tt[u] >> 5)) {
-              got[u] = *back_of(en[u], tt[u]);
-              ok = false;
-            }
-            const uint32_t wd = lds_if(ok, at[u]);
-            if (!kPart || ok) got[u] = wd;
-            got[u] &= 1u << (tt[u] & 31);
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const uint32_t bit = got[u];
-            if (kPart && !resident(tt[u] >> 5)) {
-              if (bit) got[u] = atomicAnd(back_of(en[u], tt[u]), ~bit) & bit;
-            } else {
-              got[u] = atoms_and_if(bit, at[u], ~bit) & bit;
-            }
-          }
-          unsigned bal[U], n = 0;
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            bal[u] = __ballot_sync(0xffffffffu, got[u] != 0u);
-            n += (unsigned)__popc(bal[u]);
-          }
-          if (n == 0) return;
-          unsigned base = reserve(n);
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            put(got[u] != 0u, base + (unsigned)__popc(bal[u] & lt), en[u], tt[u]);
-            base += (unsigned)__popc(bal[u]);
-          }
-        };
-        // Many sites: a lane per site.
-        auto expand1 = [&](bool act, uint32_t ent, int t) {
+        // Claims the contacts of a site per lane and appends them
+        // (warp-collective).  The claim is one atomicAnd per contact, issued
+        // without a look at the word first: fourteen in flight, and the old
+        // word says both whether the site was free and that this lane has it.
+        auto expand = [&](bool act, uint32_t ent, int t) {
           const int pos = (int)(ent & kPosMask);
           const int sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
           const uint32_t ro_s = roff_s + 32u * (ent >> kPosBits);
           const int w = t >> 5, b = t & 31;
           const bool s2 = sg == 2, sz = sg == 0;
-          // c: bit d = contact d is metallic and not reached yet.  Each word
-          // is shifted so that the contact's bit comes first and a funnel
-          // shift takes it in.
-          uint32_t c = 0u;
+          uint32_t c = 0u;  // bit d: contact d was free and is this site's
           bool in = act;
           if (kPart) in = act && resident(w) && (b != 31 || resident(w + 1)) && (b != 0 || t == 0 || resident(w - 1));
           if (in) {
@@ -572,15 +611,22 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
             const uint32_t nb = b == 31 ? at_of(ent, t + 1) : base, pbs = b == 0 && t ? at_of(ent, t - 1) : base;
             const uint32_t ub = s2 ? nb : base, db = sz ? pbs : base;
             const uint32_t o2 = 4u * o.x, o1 = 4u * o.y, p1 = 4u * o.z, p2 = 4u * o.w;
-            const uint32_t w13 = lds_u<0>(nb), w12 = lds_u<0>(pbs), w11 = lds_u<0>(db + p1), w10 = lds_u<4>(db + o1),
-                           w9 = lds_u<-4>(db), w8 = lds_u<0>(ub + o1), w7 = lds_u<-4>(ub + p1), w6 = lds_u<4>(ub),
-                           w5 = lds_u<-4>(base + p2), w4 = lds_u<-8>(base + p1), w3 = lds_u<-4>(base + o1),
-                           w2 = lds_u<4>(base + o2), w1 = lds_u<8>(base + o1), w0 = lds_u<4>(base + p1);
-            const int xs = 31 - b, xn = 31 - ((b + 1) & 31), xp = 31 - ((b - 1) & 31);
+            const int bn = (b + 1) & 31, bp = (b - 1) & 31;
+            const uint32_t k0 = ~(1u << b), kn = ~(1u << bn), kp = t ? ~(1u << bp) : 0xffffffffu;
+            const uint32_t ku = s2 ? kn : k0, kd = sz ? kp : k0;
+            const uint32_t w13 = atoms_and_at<0>(nb, kn), w12 = atoms_and_at<0>(pbs, kp), w11 = atoms_and_at<0>(db + p1, kd),
+                           w10 = atoms_and_at<4>(db + o1, kd), w9 = atoms_and_at<-4>(db, kd), w8 = atoms_and_at<0>(ub + o1, ku),
+                           w7 = atoms_and_at<-4>(ub + p1, ku), w6 = atoms_and_at<4>(ub, ku), w5 = atoms_and_at<-4>(base + p2, k0),
+                           w4 = atoms_and_at<-8>(base + p1, k0), w3 = atoms_and_at<-4>(base + o1, k0),
+                           w2 = atoms_and_at<4>(base + o2, k0), w1 = atoms_and_at<8>(base + o1, k0), w0 = atoms_and_at<4>(base + p1, k0);
+            // each word is shifted so that the contact's bit comes first and a
+            // funnel shift takes it in
+            const int xs = 31 - b, xn = 31 - bn, xp = 31 - bp;
             const int xu = s2 ? xn : xs, xd = sz ? xp : xs;
             auto take = [&](uint32_t v, int sh) { c = __funnelshift_l(v << sh, c, 1); };
             take(w13, xn); take(w12, xp); take(w11, xd); take(w10, xd); take(w9, xd); take(w8, xu); take(w7, xu);
             take(w6, xu); take(w5, xs); take(w4, xs); take(w3, xs); take(w2, xs); take(w1, xs); take(w0, xs);
+            if (t == 0) c &= sz ? ~((1u << 12) | (7u << 9)) : ~(1u << 12);
           } else if (act) {  // a row outside the window
             const int4 o = *reinterpret_cast<const int4*>(roff + 8 * (ent >> kPosBits));
             const int ro[5] = {o.x, o.y, o.z, o.w, 0};
@@ -591,54 +637,77 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
               v[d] = tt < 0 ? 0u : *word_ptr(tt >> 5, pos + c_dq(d) + ro[c_row(d)]) >> (tt & 31);
             }
 #pragma unroll
-            for (int d = 0; d < 14; ++d) c |= (v[d] & 1u) << d;
-          }
-          if (t == 0) c &= sz ? ~((1u << 12) | (7u << 9)) : ~(1u << 12);
-          while (__any_sync(0xffffffffu, c != 0u)) {
-            constexpr int K = 3;  // candidates of a lane at a time: their atomics overlap
-            uint32_t en[K], got[K];
-            int tt[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-              const uint2 y = lds_u2(dir_s + 8u * (uint32_t)((__ffs(c) - 1) & 15));
-              en[k] = ent + y.x + lds_u<0>(ro_s + (y.y & 255u));
-              tt[k] = t + (int)((y.y >> (8 + 2 * sg)) & 3u) - 1;
-              const uint32_t bit = c ? 1u << (tt[k] & 31) : 0u;
-              c &= c - 1u;
-              if (kPart && !resident(tt[k] >> 5)) {
-                got[k] = bit ? atomicAnd(back_of(en[k], tt[k]), ~bit) & bit : 0u;
-              } else {
-                got[k] = atoms_and_if(bit, at_of(en[k], tt[k]), ~bit) & bit;
+            for (int d = 0; d < 14; ++d)
+              if (v[d] & 1u) {
+                const int tt = t + c_end(d) + (c_up(d) & s2) - (c_dn(d) & sz);
+                const uint32_t bit = 1u << (tt & 31);
+                if (atomicAnd(word_ptr(tt >> 5, pos + c_dq(d) + ro[c_row(d)]), ~bit) & bit) c |= 1u << d;
               }
+          }
+          // lane after lane's first, then second, .. claim: independent votes
+          // and predicated stores for four (a site rarely claims more), no
+          // branches
+          const unsigned n_c = (unsigned)__popc(c);
+          const unsigned b0 = __ballot_sync(0xffffffffu, n_c > 0u), b1 = __ballot_sync(0xffffffffu, n_c > 1u),
+                         b2 = __ballot_sync(0xffffffffu, n_c > 2u), b3 = __ballot_sync(0xffffffffu, n_c > 3u);
+          if (!b0) return;
+          const uint32_t t4 = (uint32_t)t << 4, claimed = c;
+          const unsigned p0 = (unsigned)__popc(b0), p1 = p0 + (unsigned)__popc(b1), p2 = p1 + (unsigned)__popc(b2);
+          unsigned n_all = p2 + (unsigned)__popc(b3);
+          const bool more = __any_sync(0xffffffffu, n_c > 4u);
+          if (more) n_all = __reduce_add_sync(0xffffffffu, n_c);
+          const unsigned first = kWarp ? count : reserve(n_all);
+          auto append = [&](bool has, unsigned idx) {
+            sts_u2_if(has && idx < (unsigned)cap, qn_s + 8u * idx, ent, t4 | (uint32_t)((__ffs(c) - 1) & 15));
+            c &= c - 1u;
+          };
+          append(n_c > 0u, first + (unsigned)__popc(b0 & lt));
+          append(n_c > 1u, first + p0 + (unsigned)__popc(b1 & lt));
+          append(n_c > 2u, first + p1 + (unsigned)__popc(b2 & lt));
+          append(n_c > 3u, first + p2 + (unsigned)__popc(b3 & lt));
+          unsigned base = first + p2 + (unsigned)__popc(b3);
+          unsigned bal;
+          if (more)
+            while ((bal = __ballot_sync(0xffffffffu, c != 0u)) != 0u) {
+              append(c != 0u, base + (unsigned)__popc(bal & lt));
+              base += (unsigned)__popc(bal);
             }
-            unsigned bal[K], n = 0;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-              bal[k] = __ballot_sync(0xffffffffu, got[k] != 0u);
-              n += (unsigned)__popc(bal[k]);
-            }
-            if (n == 0) continue;
-            unsigned base = reserve(n);
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-              put(got[k] != 0u, base + (unsigned)__popc(bal[k] & lt), en[k], tt[k]);
-              base += (unsigned)__popc(bal[k]);
+          if (kWarp) count = base;
+          // the same once more where a claim needs a look: near layers not
+          // drawn, the end layer or the window's edges, beyond the queue, or
+          // with nu in planes
+          const bool look = claimed && (kMode == M_PLANES || (unsigned)(t - e_lo) >= e_n);
+          if (__any_sync(0xffffffffu, look) || base > (unsigned)cap) {
+            base = first;
+            c = claimed;
+            while ((bal = __ballot_sync(0xffffffffu, c != 0u)) != 0u) {
+              const unsigned idx = base + (unsigned)__popc(bal & lt);
+              if (c) {
+                uint32_t en;
+                int tt;
+                decode(make_uint2(ent, t4 | (uint32_t)(__ffs(c) - 1)), en, tt);
+                if (kMode != M_HASH && idx >= (unsigned)cap) {
+                  atomicOr(on + (size_t)(tt >> 5) * P + (en & kPosMask), 1u << (tt & 31));
+                  reds_min(gs_s + (uint32_t)offsetof(GroupShared, olo) + 4u * (uint32_t)nx, tt >> 5);
+                  reds_max(gs_s + (uint32_t)offsetof(GroupShared, ohi) + 4u * (uint32_t)nx, tt >> 5);
+                }
+                f |= (tt >= t_need ? F_NEED : 0u) | (tt == L - 1 ? F_HIT : 0u) | (resident(tt >> 5) ? 0u : F_OUT);
+                if (kMode == M_PLANES) zero[plane(tt) + (en & kPosMask)] = 0.f;  // level m holds nothing at step m - 1
+                c &= c - 1u;
+              }
+              base += (unsigned)__popc(bal);
             }
           }
         };
         const unsigned stored = min(total, (unsigned)cap);
-        if (stored <= (kWarp ? 16u : (unsigned)size >> 2)) {
-          const unsigned nw2 = (unsigned)(size >> 5) * 2u;  // sites of all warps in one round
-          constexpr unsigned U = kWarp ? 4u : 2u;
-          for (unsigned i = (unsigned)(tid >> 5) * 2u; i < stored; i += U * nw2) expand16(i, nw2, stored);
-        } else {
-          for (unsigned i0 = (unsigned)(tid & ~31); i0 < stored; i0 += (unsigned)size) {
-            const unsigned i = i0 + (unsigned)lane;
-            const uint2 e = lds_u2(qc_s + 8u * (i < stored ? i : i0));
-            expand1(i < stored, e.x, (int)e.y);
-          }
+        for (unsigned i0 = (unsigned)(tid & ~31); i0 < stored; i0 += (unsigned)size) {
+          const unsigned i = i0 + (unsigned)lane;
+          uint32_t ent;
+          int t;
+          decode(lds_u2(qc_s + 8u * (i < stored ? i : i0)), ent, t);
+          expand(i < stored, ent, t);
         }
-        if (total > (unsigned)cap) {  // sites of this level beyond the queue
+        if (kMode != M_HASH && total > (unsigned)cap) {  // sites of this level beyond the queue
           uint32_t* oc = over + (size_t)((m - 1) & 1) * over_n;
           const int lo = gs->olo[cu_], hi = gs->ohi[cu_];
           for (int w = lo; w <= hi; ++w)
@@ -652,7 +721,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
                 const bool act = word != 0u;
                 const int b = act ? __ffs(word) - 1 : 0;
                 word &= word - 1u;
-                expand1(act, ent, 32 * w + b);
+                expand(act, ent, 32 * w + b);
               }
             }
         }
@@ -660,26 +729,35 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         if (kWarp) {
           total = count;
           f = __any_sync(0xffffffffu, f != 0u) ? __reduce_or_sync(0xffffffffu, f) : 0u;
-          if (lane == 0) { gs->olo[nn] = 0x7fffffff; gs->ohi[nn] = -1; }
+          if (total > (unsigned)cap && lane == 0) { gs->olo[nn] = 0x7fffffff; gs->ohi[nn] = -1; }
           __syncwarp();
         } else {
           if (f) reds_or(cf_s + 4u, f);
           if (tid == 0) { gs->cf[nn][0] = 0u; gs->cf[nn][1] = 0u; gs->olo[nn] = 0x7fffffff; gs->ohi[nn] = -1; }
           __syncthreads();
-          total = gs->cf[nx][0];
-          f = gs->cf[nx][1];
+          const uint2 cf = lds_u2(cf_s);
+          total = cf.x;
+          f = cf.y;
         }
         cu_ = nx;
         if (total == 0) { mstop = m; break; }
+        if (kMode == M_HASH && total > (unsigned)cap) { hard = true; break; }
         if (f & F_NEED) draw();  // the new sites have contacts in the next layers
-        if (kMass || (kPart && NR > 0 && (f & F_OUT))) {
+        if (kMode == M_HASH) {
+          const bool live = level_hash(m, total);
+          if (f & F_HIT) { mass = detector_mass(m); break; }
+          if (!live) break;  // nu has underflowed everywhere: the mass is 0
+        }
+        if (kMode == M_PLANES || (kPart && NR > 0 && (f & F_OUT))) {
           int lo = 0, hi = 0;  // tubes of the new level
-          if (!kMass || ring_mask >= 0) {
+          if (kMode != M_PLANES || ring_mask >= 0) {
             if (tid == 0) { gs->span[0] = gs->olo[nx] < 0x7fffffff ? 32 * gs->olo[nx] : 0x7fffffff; gs->span[1] = 32 * gs->ohi[nx] + 31; }
             group_sync<kWarp>();
             lo = 0x7fffffff; hi = -1;
             for (unsigned i = tid; i < min(total, (unsigned)cap); i += size) {
-              const int t = (int)lds_u2(qn_s + 8u * i).y;
+              uint32_t ent;
+              int t;
+              decode(lds_u2(qn_s + 8u * i), ent, t);
               lo = min(lo, t);
               hi = max(hi, t);
             }
@@ -691,7 +769,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
             hi = gs->span[1];
             group_sync<kWarp>();
           }
-          if (kMass) {
+          if (kMode == M_PLANES) {
             // the rings hold the levels m - 1 and m only while their tubes
             // (a level lies within one tube of the previous one's) and the
             // tubes around them are fewer than the rings' planes
@@ -726,26 +804,35 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
   }
 }
 
-// A warp group's registers are bounded so that 24 warps fit an SM.
-template <bool kWarp, bool kPart, bool kMass>
-__global__ void __launch_bounds__(kWarp ? 128 : 512, kWarp ? 6 : 1) wave_kernel(const __grid_constant__ WaveArgs a) {
+// kThreads: threads of a group; 32 = a warp, four to a CTA.  Registers are
+// bounded so that 24 warps (groups of a warp, or of 128 or 256 threads) or one
+// CTA of 512 threads fit an SM.
+template <int kThreads, bool kPart, int kMode>
+__global__ void __launch_bounds__(kThreads == 32 ? 128 : kThreads, kThreads <= 128 ? 6 : kThreads == 256 ? 3 : 1)
+    wave_kernel(const __grid_constant__ WaveArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (kWarp) {
+  if (kThreads == 32) {
     const int w = threadIdx.x >> 5;
-    wave_body<true, kPart, kMass>(a, smem_raw + (size_t)w * a.group_smem,
+    wave_body<true, kPart, kMode>(a, smem_raw + (size_t)w * a.group_smem,
                                   a.scratch + ((long long)blockIdx.x * (blockDim.x >> 5) + w) * a.scratch_stride);
   } else {
-    wave_body<false, kPart, kMass>(a, smem_raw, a.scratch + (long long)blockIdx.x * a.scratch_stride);
+    wave_body<false, kPart, kMode>(a, smem_raw, a.scratch + (long long)blockIdx.x * a.scratch_stride);
   }
 }
 
-const void* wave_fn(bool warp, bool part, bool mass) {
-  static const void* const f[8] = {
-      (const void*)wave_kernel<false, false, false>, (const void*)wave_kernel<false, false, true>,
-      (const void*)wave_kernel<false, true, false>,  (const void*)wave_kernel<false, true, true>,
-      (const void*)wave_kernel<true, false, false>,  (const void*)wave_kernel<true, false, true>,
-      (const void*)wave_kernel<true, true, false>,   (const void*)wave_kernel<true, true, true>};
-  return f[(warp ? 4 : 0) + (part ? 2 : 0) + (mass ? 1 : 0)];
+template <int kThreads>
+const void* wave_fn_of(bool part, int mode) {
+  if (mode == M_LEVELS) return part ? (const void*)wave_kernel<kThreads, true, M_LEVELS> : (const void*)wave_kernel<kThreads, false, M_LEVELS>;
+  constexpr int T = kThreads == 32 ? 128 : kThreads;  // masses: CTAs
+  if (mode == M_HASH) return part ? (const void*)wave_kernel<T, true, M_HASH> : (const void*)wave_kernel<T, false, M_HASH>;
+  return part ? (const void*)wave_kernel<T, true, M_PLANES> : (const void*)wave_kernel<T, false, M_PLANES>;
+}
+
+const void* wave_fn(int threads, bool part, int mode) {
+  return threads == 32    ? wave_fn_of<32>(part, mode)
+         : threads == 128 ? wave_fn_of<128>(part, mode)
+         : threads == 256 ? wave_fn_of<256>(part, mode)
+                          : wave_fn_of<512>(part, mode);
 }
 
 int ceil_log2(long long x) {
@@ -770,7 +857,7 @@ namespace {
 
 // The query table goes through kernel parameters: asynchronous, and no
 // pageable host copy.
-constexpr int kUpload = 16;
+constexpr int kUpload = 14;
 struct UploadChunk {
   int n;
   WaveQuery q[kUpload];
@@ -780,16 +867,16 @@ __global__ void wave_upload_kernel(WaveQuery* dst, const __grid_constant__ Uploa
   if ((int)threadIdx.x < c.n) dst[threadIdx.x] = c.q[threadIdx.x];
 }
 
-// One launch: the queries that run with the same group size.
-struct WaveClass {
-  int threads = 0;           // 32: a group is a warp (four to a CTA), else the CTA
+// One launch over the queries that run with the same group size.
+struct WaveLaunch {
+  int mode = M_LEVELS, threads = 0;
+  bool part = false, hard = false;
   std::vector<WaveQuery> q;
-  long long items = 0, mass_items = 0;
-  bool part = false, ring = false;
-  size_t group_smem = 0;
-  size_t stride_b = 256, stride_m = 256, stride_h = 256;
-  long long grid_b = 0, grid_m = 0, grid_h = 0;
-  size_t scratch = 0, table_b = 0;
+  long long items = 0;
+  size_t group_smem = 0, stride = 256;
+  long long grid = 0;
+  size_t per_cta() const { return threads == 32 ? 4 : 1; }
+  size_t table_b() const { return q.size() > 1 ? up(sizeof(WaveQuery) * q.size(), 256) : 0; }
 };
 
 // Threads of a group.  With more configurations than groups fit the device,
@@ -803,15 +890,27 @@ int group_threads(int A, long long n, int nsm) {
   return 512;
 }
 
-// Shared memory and scratch of query w in a class.
-void place(WaveQuery& w, WaveClass& c, size_t most) {
+// Shared memory (at most `most` bytes) and scratch of query w in a launch.
+// False: no room for the hash tables.
+bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings) {
   const size_t row_b = sizeof(uint32_t) * (size_t)w.P;
+  const bool hash = l.mode == M_HASH;
+  size_t target = l.threads == 32 ? 12 * 1024 : l.threads == 128 ? 36 * 1024 : l.threads == 256 ? 72 * 1024 : most;
+  if (hash) target = std::min(most, 2 * target);
+  w.cap = (int)std::min<long long>(w.A, l.threads == 32 ? 512 : 1200);
+  w.tab_bits = 0;
+  size_t tab = 0;
+  if (hash) {  // the start layer is the largest level to expect
+    const double p = w.occ_bits ? 0.2 : (double)w.occ.T / 4294967296.0;
+    w.cap = (int)std::min<long long>(w.A, (long long)(1.2 * p * w.A) + 96);
+    w.tab_bits = ceil_log2(3 * w.cap / 2 + 1);
+    tab = (16ull << w.tab_bits) + 8 * (size_t)w.cap;
+    if (w.L > 16384) return false;
+  }
   const size_t head = kSharedHead + 32 * (size_t)(2 * w.W + 1);
+  const size_t fixed = head + 2 * sizeof(uint2) * (size_t)w.cap + tab + 64;
   // every word row in shared memory if they fit the target, else a power of
   // two of them
-  const size_t target = c.threads == 32 ? 12 * 1024 : c.threads <= 256 ? 72 * 1024 : most;
-  w.cap = (int)std::min<long long>(w.A, c.threads == 32 ? 512 : 1200);
-  const size_t fixed = head + 2 * sizeof(uint2) * (size_t)w.cap + 32;
   auto fits = [&](int rows, size_t lim) { return fixed + (size_t)rows * row_b <= lim; };
   if (fits(w.TW, target)) {
     w.NR = w.TW; w.nr_mask = -1;
@@ -819,26 +918,64 @@ void place(WaveQuery& w, WaveClass& c, size_t most) {
     w.NR = 0;
     for (int r = 1; r < w.TW && (fits(r, target) || (r <= 2 && fits(r, most))); r *= 2) w.NR = r;
     w.nr_mask = w.NR - 1;
+    if (hash && w.NR < 2) return false;
   }
-  w.o_win = (int)head;
-  w.o_queue = (int)up(w.o_win + w.NR * row_b, 16);
-  c.group_smem = std::max(c.group_smem, up(w.o_queue + 2 * sizeof(uint2) * (size_t)w.cap, 16));
-  c.part = c.part || w.NR < w.TW;
+  size_t o = head;
+  w.o_win = (int)o; o += w.NR * row_b;
+  w.o_occ = -1;
+  if (hash && w.NR == w.TW && fits(2 * w.TW, target)) { w.o_occ = (int)o; o += w.TW * row_b; }
+  o = up(o, 16);
+  w.o_queue = (int)o; o += 2 * sizeof(uint2) * (size_t)w.cap;
+  o = up(o, 16);
+  w.o_tab = (int)o; o += tab;
+  l.group_smem = std::max(l.group_smem, up(o, 16));
+  l.part = l.part || w.NR < w.TW;
   const size_t map_b = up(row_b * w.TW, 256);
-  size_t off = up(2 * row_b * w.TW, 256);
+  size_t off = 0;
   w.a_over = 0;
+  if (!hash) off = up(2 * row_b * w.TW, 256);
   w.a_back = (long long)off;
   if (w.NR < w.TW) off += map_b;
-  c.stride_b = std::max(c.stride_b, off);
-  w.ring_mask = w.L <= 128 ? -1 : 127;
-  if (w.want_mass) {
-    w.a_occ = (long long)off; off += map_b;
+  w.a_occ = w.a_nu = (long long)off;
+  w.ring_mask = -1;
+  if (l.mode != M_LEVELS && w.o_occ < 0) off += map_b;
+  if (l.mode == M_PLANES) {
     w.a_nu = (long long)off;
-    const size_t ring = w.ring_mask < 0 ? (size_t)w.L : 128;
-    c.stride_m = std::max(c.stride_m, off + up(2 * row_b * ring, 256));
-    c.stride_h = std::max(c.stride_h, off + up(2 * row_b * (size_t)w.L, 256));
-    c.ring = c.ring || w.ring_mask >= 0;
+    if (!full_rings && w.L > 128) w.ring_mask = 127;
+    off += up(2 * row_b * (size_t)(w.ring_mask < 0 ? w.L : 128), 256);
   }
+  l.stride = std::max(l.stride, off);
+  return true;
+}
+
+// The launches of a class of queries (item0 set): levels; masses in hash
+// tables, or in rings of planes where a level does not fit the tables; masses
+// that the second left (marked -1), with a plane for every layer.
+std::vector<WaveLaunch> launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, size_t most) {
+  std::vector<WaveLaunch> out;
+  auto add = [&](int mode, int t, bool full) -> bool {
+    WaveLaunch l;
+    l.mode = mode; l.threads = t; l.items = items; l.hard = mode == M_PLANES && full;
+    for (WaveQuery w : qs) {
+      if (!place(w, l, most, full)) return false;
+      l.q.push_back(w);
+    }
+    out.push_back(l);
+    return true;
+  };
+  add(M_LEVELS, threads, false);
+  bool mass = false, rings = false;
+  for (const WaveQuery& w : qs) mass = mass || w.want_mass;
+  if (!mass) return out;
+  const int mt = std::max(threads, 128);
+  if (add(M_HASH, mt, false)) {
+    rings = true;
+  } else {
+    add(M_PLANES, mt, false);
+    for (const WaveQuery& w : out.back().q) rings = rings || w.ring_mask >= 0;
+  }
+  if (rings) add(M_PLANES, mt, true);
+  return out;
 }
 
 }  // namespace
@@ -851,13 +988,18 @@ int wave_threads(int A, long long n_all) {
 }
 
 size_t wave_scratch_bytes(const Lattice& lat) {
-  WaveClass c;
-  c.threads = 512;
   WaveQuery w = {};
   fill_lattice(w, lat);
   w.want_mass = 1;
-  place(w, c, 64 * 1024);  // (a smaller window than any device gives it: evicted rows counted)
-  return std::max(c.stride_b, std::max(c.stride_m, c.stride_h));
+  size_t b = 0;
+  for (int mode : {M_LEVELS, M_HASH, M_PLANES}) {
+    WaveLaunch l;
+    l.mode = mode; l.threads = 128;
+    WaveQuery x = w;
+    // (the smallest window any launch has: evicted rows counted)
+    if (place(x, l, 48 * 1024, true)) b = std::max(b, l.stride);
+  }
+  return b;
 }
 
 pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m, size_t limit) {
@@ -865,7 +1007,8 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   PC_CUDA(cudaGetDevice(&dev));
   PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   PC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  // classes; within one, larger lattices first (their configurations run longest)
+  // classes by group size; within one, larger lattices first (their
+  // configurations run longest)
   std::vector<int> order;
   for (int i = 0; i < nq; ++i)
     if (qs[i].n_cfg > 0) order.push_back(i);
@@ -874,77 +1017,69 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   long long n_all = 0;
   for (int i : order) n_all += qs[i].n_cfg;
   if (m) n_all = std::min(n_all, m->max_groups);
-  std::vector<WaveClass> cls;
-  for (int i : order) {
-    const StreamQuery& s = qs[i];
-    const int threads = std::max(group_threads(s.lat.A, n_all, nsm), m ? 128 : 32);  // (a warp group's scratch comes in fours)
-    auto c = std::find_if(cls.begin(), cls.end(), [&](const WaveClass& x) { return x.threads == threads; });
-    if (c == cls.end()) {
-      cls.emplace_back();
-      c = cls.end() - 1;
-      c->threads = threads;
+  std::vector<WaveLaunch> ls;
+  int classes = 0;
+  for (int threads : {512, 256, 128, 32}) {
+    std::vector<WaveQuery> cq;
+    long long items = 0;
+    for (int i : order) {
+      const StreamQuery& s = qs[i];
+      // (on a caller's memory a configuration is one CTA's)
+      if (std::max(group_threads(s.lat.A, n_all, nsm), m ? 128 : 32) != threads) continue;
+      WaveQuery w = {};
+      fill_lattice(w, s.lat);
+      w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
+      w.out = s.out;
+      w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
+      w.item0 = items; w.n_cfg = s.n_cfg;
+      items += s.n_cfg;
+      cq.push_back(w);
     }
-    WaveQuery w = {};
-    fill_lattice(w, s.lat);
-    w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
-    w.out = s.out;
-    w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
-    w.item0 = c->items; w.n_cfg = s.n_cfg;
-    place(w, *c, (size_t)optin - 64);
-    c->items += s.n_cfg;
-    if (w.want_mass) c->mass_items += s.n_cfg;
-    c->q.push_back(w);
+    if (cq.empty()) continue;
+    ++classes;
+    for (WaveLaunch& l : launches_of(cq, items, threads, (size_t)optin - 64)) ls.push_back(l);
   }
-  // grids and scratch of at most `total` bytes (one group per launch at least)
-  auto plan = [&](size_t total, size_t* bytes) -> pc_status {
-    const size_t budget = total / cls.size();
-    *bytes = 256 * cls.size();
-    for (WaveClass& c : cls) {
-      const size_t per_cta = c.threads == 32 ? 4 : 1;
-      const int block = c.threads * (int)per_cta;
-      auto grid_of = [&](bool mass, size_t stride, size_t most, long long* g) -> pc_status {
-        const void* f = wave_fn(c.threads == 32, c.part, mass);
+  // Grids, and one scratch for all launches (they run one after the other) of
+  // at most `total` bytes, one group at least.  The launch for what the rings
+  // and tables left gets what the others need.
+  auto plan = [&](size_t total, size_t* scratch) -> pc_status {
+    *scratch = 0;
+    for (int pass = 0; pass < 2; ++pass)
+      for (WaveLaunch& l : ls) {
+        if (l.hard != (pass == 1)) continue;
+        const void* f = wave_fn(l.threads, l.part, l.mode);
         // the same limit on every call: calls from several threads never lower it
         PC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
         int per_sm = 0;
-        PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, block, c.group_smem * per_cta));
+        PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, l.threads * (int)l.per_cta(), l.group_smem * l.per_cta()));
         if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
-        long long n = std::min<long long>((long long)per_sm * nsm, (c.items + (long long)per_cta - 1) / (long long)per_cta);
-        n = std::min<long long>(n, (long long)(most / (stride * per_cta)));
+        const size_t cta_b = l.stride * l.per_cta();
+        const size_t most = l.hard ? std::min(total, std::max<size_t>(*scratch, 64u << 20)) : total;
+        long long n = std::min<long long>((long long)per_sm * nsm, (l.items + (long long)l.per_cta() - 1) / (long long)l.per_cta());
+        n = std::min<long long>(n, (long long)(most / cta_b));
         if (m) n = std::min(n, m->max_groups);
-        *g = std::max<long long>(n, 1);
-        return PC_OK;
-      };
-      pc_status rc = grid_of(false, c.stride_b, budget, &c.grid_b);
-      if (rc) return rc;
-      c.scratch = c.stride_b * (size_t)c.grid_b * per_cta;
-      if (c.mass_items) {
-        if ((rc = grid_of(true, c.stride_m, budget, &c.grid_m))) return rc;
-        c.scratch = std::max(c.scratch, c.stride_m * (size_t)c.grid_m * per_cta);
-        if (c.ring) {
-          if ((rc = grid_of(true, c.stride_h, std::min(budget, c.scratch), &c.grid_h))) return rc;
-          c.scratch = std::max(c.scratch, c.stride_h * (size_t)c.grid_h * per_cta);
-        }
+        l.grid = std::max<long long>(n, 1);
+        *scratch = std::max(*scratch, cta_b * (size_t)l.grid);
       }
-      c.table_b = c.q.size() > 1 ? up(sizeof(WaveQuery) * c.q.size(), 256) : 0;
-      *bytes += c.table_b * (c.ring ? 2 : 1) + c.scratch;
-    }
     return PC_OK;
   };
+  size_t tables = 0;
+  for (const WaveLaunch& l : ls) tables += l.table_b();
+  const size_t head = 256 * ls.size();
   pc_status rc = PC_OK;
   cudaError_t e = cudaSuccess;
   char* mem = nullptr;
-  size_t bytes = 0;
+  size_t scratch = 0;
   if (m) {
-    if ((rc = plan(m->bytes, &bytes))) return rc;
-    if (cls.size() != 1 || cls[0].table_b || cls[0].scratch > m->bytes) {
+    if ((rc = plan(m->bytes, &scratch))) return rc;
+    if (classes != 1 || tables || scratch > m->bytes || ls.size() > 3) {
       set_error("wavefront solver: the caller's memory does not hold the query");
       return PC_ERR_INTERNAL;
     }
   } else {
     for (size_t total = limit;; total /= 8) {  // fewer groups where the memory for more cannot be had
-      if ((rc = plan(total, &bytes))) return rc;
-      e = scratch_alloc((void**)&mem, bytes, st);
+      if ((rc = plan(total, &scratch))) return rc;
+      e = scratch_alloc((void**)&mem, head + tables + scratch, st);
       if (e == cudaSuccess) break;
       if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "wavefront solver: scratch");
       cudaGetLastError();
@@ -953,50 +1088,36 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
         return PC_ERR_OOM;
       }
     }
-    e = cudaMemsetAsync(mem, 0, 256 * cls.size(), st);
+    e = cudaMemsetAsync(mem, 0, head, st);
   }
-  char* at = m ? m->scratch : mem + 256 * cls.size();
-  for (size_t k = 0; k < cls.size(); ++k) {
-    WaveClass& c = cls[k];
-    const int per_cta = c.threads == 32 ? 4 : 1;  // groups to a CTA
-    unsigned long long* ctr = m ? m->ctr : (unsigned long long*)(mem + 256 * k);
+  char* at = m ? nullptr : mem + head;  // query tables
+  char* const base = m ? m->scratch : mem + head + tables;
+  for (size_t k = 0; k < ls.size() && e == cudaSuccess; ++k) {
+    WaveLaunch& l = ls[k];
     WaveArgs a = {};
-    a.nq = (int)c.q.size();
-    a.n_items = c.items;
-    a.group_smem = (int)c.group_smem;
-    auto tables = [&]() {
-      a.q0 = c.q[0];
-      if (!c.table_b) return;
+    a.q0 = l.q[0];
+    a.nq = (int)l.q.size();
+    a.n_items = l.items;
+    a.group_smem = (int)l.group_smem;
+    a.hard = l.hard ? 1 : 0;
+    a.work = m ? m->ctr + k : (unsigned long long*)(mem + 256 * k);
+    a.scratch = base;
+    a.scratch_stride = (long long)l.stride;
+    if (l.table_b()) {
       a.qs = (const WaveQuery*)at;
-      for (size_t b = 0; b < c.q.size() && e == cudaSuccess; b += kUpload) {
+      for (size_t b = 0; b < l.q.size() && e == cudaSuccess; b += kUpload) {
         UploadChunk u = {};
-        u.n = (int)std::min<size_t>(kUpload, c.q.size() - b);
-        for (int i = 0; i < u.n; ++i) u.q[i] = c.q[b + i];
+        u.n = (int)std::min<size_t>(kUpload, l.q.size() - b);
+        for (int i = 0; i < u.n; ++i) u.q[i] = l.q[b + i];
         wave_upload_kernel<<<1, kUpload, 0, st>>>((WaveQuery*)at + b, u);
         e = cudaGetLastError();
       }
-      at += c.table_b;
-    };
-    tables();
-    a.scratch = at; at += c.scratch;
-    auto launch = [&](bool mass, long long grid, unsigned long long* work, size_t stride) {
-      a.work = work;
-      a.scratch_stride = (long long)stride;
-      void* args[] = {&a};
-      if (e == cudaSuccess)
-        e = cudaLaunchKernel(wave_fn(c.threads == 32, c.part, mass), dim3((unsigned)grid), dim3(c.threads * per_cta),
-                             args, c.group_smem * per_cta, st);
-    };
-    launch(false, c.grid_b, ctr, c.stride_b);
-    if (c.mass_items) {
-      launch(true, c.grid_m, ctr + 1, c.stride_m);
-      if (c.ring) {  // frontiers that outgrew the mass rings: a plane for every layer
-        for (WaveQuery& w : c.q) w.ring_mask = -1;
-        tables();
-        a.hard = 1;
-        launch(true, c.grid_h, ctr + 2, c.stride_h);
-      }
+      at += l.table_b();
     }
+    void* args[] = {&a};
+    if (e == cudaSuccess)
+      e = cudaLaunchKernel(wave_fn(l.threads, l.part, l.mode), dim3((unsigned)l.grid),
+                           dim3(l.threads * (unsigned)l.per_cta()), args, l.group_smem * l.per_cta(), st);
   }
   if (e != cudaSuccess) rc = cuda_fail(e, "wavefront solver");
   if (mem) cudaFreeAsync(mem, st);

@@ -27,6 +27,7 @@ struct WaveQuery {
   int cap;                   // frontier entries held in shared memory (two levels)
   int ring_mask;             // layers of the mass rings - 1, or -1: every layer has its own plane
   int o_win, o_queue;        // shared memory: window, queues (row offsets at a fixed place)
+  int o_occ, o_tab, tab_bits;  // occupancy (-1: in scratch), hash tables and their size
   long long a_back, a_over, a_occ, a_nu;  // scratch: evicted rows, overflow maps, occupancy, mass rings
 };
 
