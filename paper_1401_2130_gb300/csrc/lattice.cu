@@ -154,7 +154,7 @@ pc_status upload_layout(const PlaneLayout& lay, DevLayout* d) {
   d->P = lay.P; d->s_begin = lay.s_begin; d->n_strips = lay.n_strips;
   PC_CUDA(cudaMalloc(&d->strip_row, sizeof(int16_t) * lay.strip_row.size()));
   PC_CUDA(cudaMalloc(&d->row_off, sizeof(int32_t) * lay.row_off.size()));
-  PC_CUDA(cudaMalloc(&d->ppos, sizeof(int32_t) * lay.ppos.size()));
+  PC_CUDA(cudaMalloc(&d->ppos, sizeof(int32_t) * (lay.ppos.size() + 4)));  // read in fours
   PC_CUDA(cudaMalloc(&d->pcol, sizeof(int32_t) * lay.pcol.size()));
   PC_CUDA(cudaMemcpy(d->strip_row, lay.strip_row.data(), sizeof(int16_t) * lay.strip_row.size(), cudaMemcpyHostToDevice));
   PC_CUDA(cudaMemcpy(d->row_off, lay.row_off.data(), sizeof(int32_t) * lay.row_off.size(), cudaMemcpyHostToDevice));

@@ -143,6 +143,11 @@ __device__ __forceinline__ void reds_max(uint32_t a, int v) {
 __device__ __forceinline__ void reds_or(uint32_t a, uint32_t v) {
   asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
+// or bit into the word at a if u <= last (predicated, no branch)
+__device__ __forceinline__ void reds_or_le(uint32_t u, uint32_t last, uint32_t a, uint32_t bit) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.le.u32 p, %0, %1;\n\t@p red.shared.or.b32 [%2], %3;\n\t}"
+               :: "r"(u), "r"(last), "r"(a), "r"(bit) : "memory");
+}
 __device__ __forceinline__ uint2 lds_u2(uint32_t a) {
   uint2 v;
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
@@ -152,13 +157,74 @@ __device__ __forceinline__ uint32_t smem_at(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Occupancy of layers [G, Gn) of configuration rel, by `size` threads: sets bit
+// t & t_mask of the word of each metallic site's position, in shared memory at
+// row_s (shared) or through set_site(t, position).
+template <class F>
+__device__ __forceinline__ void draw_layers(const WaveQuery& Q, long long rel, int G, int Gn, int tid, int size,
+                                            bool shared, uint32_t row_s, int t_mask, F&& set_site) {
+  const int A = Q.A;
+  const int32_t* ppos = Q.ppos;
+  const uint32_t i0 = (uint32_t)G * (uint32_t)A, i1 = (uint32_t)Gn * (uint32_t)A;
+  const uint32_t divM = Q.divM;
+  const int divS = 31 + Q.divS;
+  if (Q.occ_bits) {
+    const uint32_t* cb = Q.occ_bits + (size_t)rel * Q.words_per_cfg;
+    for (uint32_t wi = (i0 >> 5) + tid; wi <= (i1 - 1) >> 5; wi += size) {
+      uint32_t bits = cb[wi];
+      while (bits) {
+        const uint32_t i = (wi << 5) + __ffs(bits) - 1;
+        bits &= bits - 1;
+        if (i < i0 || i >= i1) continue;
+        const int t = (int)(((uint64_t)i * divM) >> divS), c = (int)(i - (uint32_t)t * A);
+        set_site(t, __ldg(ppos + c));
+      }
+    }
+    return;
+  }
+  // a word u is metallic iff u < T, i.e. u <= T - 1
+  const uint64_t T = Q.occ.T;
+  if (T == 0) return;
+  const uint32_t last = (uint32_t)(T - 1ull), k0 = Q.occ.k0, k1 = Q.occ.k1, wl = Q.occ.wl, cfg = Q.cfg0 + (uint32_t)rel;
+  const uint32_t b_first = i0 >> 2, b_end = (i1 - 1) >> 2;
+  uint32_t bi = b_first + tid;
+  int t = (int)(((uint64_t)(bi << 2) * divM) >> divS), c = (int)((bi << 2) - (uint32_t)t * A);
+  const int dt = (int)(((uint64_t)(4 * size) * divM) >> divS), dc = 4 * size - dt * A;  // one round further
+  for (; bi <= b_end; bi += size) {
+    // a block's four columns (the table is padded by four entries)
+    const int q0 = __ldg(ppos + c), q1 = __ldg(ppos + c + 1), q2 = __ldg(ppos + c + 2), q3 = __ldg(ppos + c + 3);
+    const u32x4 r = philox4x32_10(u32x4{bi, cfg, wl, 0u}, k0, k1);
+    if (shared && c + 3 < A && bi != b_first && bi != b_end) {  // four sites of one layer to draw
+      const uint32_t bit = 1u << (t & t_mask);
+      reds_or_le(r.x, last, row_s + 4u * (uint32_t)q0, bit);
+      reds_or_le(r.y, last, row_s + 4u * (uint32_t)q1, bit);
+      reds_or_le(r.z, last, row_s + 4u * (uint32_t)q2, bit);
+      reds_or_le(r.w, last, row_s + 4u * (uint32_t)q3, bit);
+    } else {  // the chunk's ends, two layers in a block, or no window
+      const uint32_t u[4] = {r.x, r.y, r.z, r.w};
+      int t1 = t, c1 = c;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (u[j] <= last && t1 >= G && t1 < Gn) set_site(t1, __ldg(ppos + c1));
+        if (++c1 == A) { c1 = 0; ++t1; }
+      }
+    }
+    t += dt;
+    c += dc;
+    if (c >= A) { c -= A; ++t; }
+  }
+}
+
 // kMode: levels only, or levels with nu -- in shared memory (a hash table of
 // the level's sites) or in planes in device scratch
-enum : int { M_LEVELS = 0, M_HASH = 1, M_PLANES = 2 };
+// M_PRE: levels, of configurations whose word rows were drawn by a launch
+// before (see run_wave)
+enum : int { M_LEVELS = 0, M_HASH = 1, M_PLANES = 2, M_PRE = 3 };
 
 template <bool kWarp, bool kPart, int kMode>
 __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, char* scratch) {
-  constexpr bool kMass = kMode != M_LEVELS;
+  constexpr bool kMass = kMode == M_HASH || kMode == M_PLANES;
+  constexpr bool kPre = kMode == M_PRE;
   const int tid = kWarp ? (threadIdx.x & 31) : threadIdx.x;
   const int size = kWarp ? 32 : blockDim.x;
   const int lane = threadIdx.x & 31;
@@ -176,9 +242,12 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
   const bool has16 = (lane & 15) < 14;
   const uint32_t e16 = has16 ? c_ent(lane & 15) : 0u, y16 = has16 ? c_cls(lane & 15) : 16u | 0x1500u;
 
-  for (;;) {
+  for (bool once = false;; once = true) {
     long long item;
-    {
+    if (kPre) {  // a CTA per configuration, with its own scratch
+      if (once) break;
+      item = blockIdx.x;
+    } else {
       unsigned long long v = 0;
       if (tid == 0) v = atomicAdd(a.work, 1ull);
       if (kWarp) {
@@ -273,6 +342,18 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     };
     // Draw the next layers (within one word row).  Group-uniform.
     auto draw = [&]() {
+      if (kPre) {  // the next row was drawn into the scratch
+        const int w = G >> 5;
+        if (kPart && NR > 0) {
+          while (w >= wb + NR) slide(1);
+          while (w < wb) slide(-1);
+        }
+        if (!kPart || NR > 0)
+          for (int k = tid; k < P; k += size) win[(w & nr_mask) * P + k] = back[(size_t)w * P + k];
+        G = min(32 * (w + 1), L);
+        group_sync<kWarp>();
+        return;
+      }
       const int Gn = min(G + kDrawLayers, L), w = G >> 5;
       if (kPart && NR > 0) {
         while (w >= wb + NR) slide(1);
@@ -291,53 +372,10 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         }
         group_sync<kWarp>();
       }
-      const uint32_t i0 = (uint32_t)G * (uint32_t)A, i1 = (uint32_t)Gn * (uint32_t)A;
-      const uint32_t divM = Q.divM;
-      const int divS = 31 + Q.divS;
-      auto set_site = [&](int t, int pos) {
+      draw_layers(Q, rel, G, Gn, tid, size, !kPart || NR > 0, row_s, 31, [&](int t, int pos) {
         if (!kPart || NR > 0) reds_or(row_s + 4u * (uint32_t)pos, 1u << (t & 31));
         else atomicOr(row_g + pos, 1u << (t & 31));
-      };
-      if (Q.occ_bits) {
-        const uint32_t* cb = Q.occ_bits + (size_t)rel * Q.words_per_cfg;
-        for (uint32_t wi = (i0 >> 5) + tid; wi <= (i1 - 1) >> 5; wi += size) {
-          uint32_t bits = cb[wi];
-          while (bits) {
-            const uint32_t i = (wi << 5) + __ffs(bits) - 1;
-            bits &= bits - 1;
-            if (i < i0 || i >= i1) continue;
-            const int t = (int)(((uint64_t)i * divM) >> divS), c = (int)(i - (uint32_t)t * A);
-            set_site(t, __ldg(ppos + c));
-          }
-        }
-      } else {
-        OccStream os = Q.occ;
-        os.cfg = Q.cfg0 + (uint32_t)rel;
-        const uint32_t b_end = (i1 - 1) >> 2;
-        uint32_t bi = (i0 >> 2) + tid;
-        int t = (int)(((uint64_t)(bi << 2) * divM) >> divS), c = (int)((bi << 2) - (uint32_t)t * A);
-        const int dt = (int)(((uint64_t)(4 * size) * divM) >> divS), dc = 4 * size - dt * A;  // one round further
-        for (; bi <= b_end; bi += size) {
-          // the four positions are fetched while the block is drawn
-          int tj[4], pj[4];
-          {
-            int t1 = t, c1 = c;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              tj[j] = t1;
-              pj[j] = __ldg(ppos + c1);
-              if (++c1 == A) { c1 = 0; ++t1; }
-            }
-          }
-          const uint32_t bits = os.block_bits(bi);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (((bits >> j) & 1u) && tj[j] >= G && tj[j] < Gn) set_site(tj[j], pj[j]);
-          t += dt;
-          c += dc;
-          if (c >= A) { c -= A; ++t; }
-        }
-      }
+      });
       group_sync<kWarp>();
       if (kMass) {  // the degrees need the occupancy itself
         const int nl = Gn - G;
@@ -377,9 +415,23 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       }
     };
 
+    WaveState* const state = kPre ? a.state + item : nullptr;
+    const int phase = kPre ? state->phase : 0;
+    unsigned total = 0, n_start = 0;
+    int m0 = 0;  // the level the queue holds
+    if (kPre && phase == 2) continue;  // done
+    if (kPre && phase == 1) {          // resume
+      m0 = state->m; total = state->total; wb = state->wb; G = state->G; n_start = state->n0;
+      if (tid == 0) { gs->olo[0] = state->olo; gs->ohi[0] = state->ohi; }
+      const uint2* saved = reinterpret_cast<const uint2*>(scratch + Q.a_nu);
+      for (unsigned k = tid; k < min(total, (unsigned)cap); k += size) queue[(m0 & 1) * cap + k] = saved[k];
+      for (int w = wb; w < wb + NR && 32 * w < G; ++w)
+        for (int k = tid; k < P; k += size) win[(w & nr_mask) * P + k] = back[(size_t)w * P + k];
+      group_sync<kWarp>();
+      draw();  // the rows it waited for
+    } else {
     draw();
     // level 0: the metallic sites of t = 0
-    unsigned total = 0;
     {
       uint32_t* row = !kPart || NR > 0 ? win : back;
       for (int k0 = tid & ~31; k0 < P; k0 += size) {
@@ -415,7 +467,9 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       group_sync<kWarp>();
       if (!kWarp) total = gs->cf[0][0];
     }
-    const unsigned n0 = total;
+    n_start = total;
+    }
+    const unsigned n0 = n_start;
 
     // nu of a new site: (1/degree) x the sum over the contacts of the previous
     // level, whose values lie in src (at level 0: (1/degree) x 1/n0)
@@ -557,6 +611,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     int verdict = 0, fh = -1, mstop = 0;
     float mass = 0.f;
     bool hard = kMode == M_HASH && total > (unsigned)cap;  // left to the launch with planes
+    bool wait = false;
     if (kMass && n0 > 0 && !hard) {
       if (kMode == M_HASH) level_hash(0, total);
       else level_values(0, total, queue, 0, gs->ohi[0]);
@@ -566,7 +621,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       if (kMass && !hard) mass = detector_mass(0);
     } else if (n0 > 0 && !hard) {
       int cu_ = 0;  // rotating index of the current level
-      for (int m = 1;; ++m) {
+      for (int m = m0 + 1;; ++m) {
         const int nx = cu_ == 2 ? 0 : cu_ + 1, nn = nx == 2 ? 0 : nx + 1;
         const uint32_t qc_s = queue_s + 8u * (uint32_t)(((m - 1) & 1) * cap), qn_s = queue_s + 8u * (uint32_t)((m & 1) * cap);
         uint32_t* on = over + (size_t)(m & 1) * over_n;
@@ -742,7 +797,21 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         cu_ = nx;
         if (total == 0) { mstop = m; break; }
         if (kMode == M_HASH && total > (unsigned)cap) { hard = true; break; }
-        if (f & F_NEED) draw();  // the new sites have contacts in the next layers
+        if (f & F_NEED) {  // the new sites have contacts in the next layers
+          if (kPre && !(f & F_HIT) && (G >> 5) >= a.rows_ready) {  // to be drawn by the next launch: leave
+            wait = true;
+            uint2* saved = reinterpret_cast<uint2*>(scratch + Q.a_nu);
+            for (unsigned k = tid; k < min(total, (unsigned)cap); k += size) saved[k] = queue[(m & 1) * cap + k];
+            for (int w = wb; w < wb + NR && 32 * w < G; ++w)
+              for (int k = tid; k < P; k += size) back[(size_t)w * P + k] = win[(w & nr_mask) * P + k];
+            if (tid == 0) {
+              state->phase = 1; state->m = m; state->total = total; state->wb = wb; state->G = G; state->n0 = n0;
+              state->olo = gs->olo[nx]; state->ohi = gs->ohi[nx];
+            }
+            break;
+          }
+          if (kMass || !(f & F_HIT)) draw();
+        }
         if (kMode == M_HASH) {
           const bool live = level_hash(m, total);
           if (f & F_HIT) { mass = detector_mass(m); break; }
@@ -789,7 +858,8 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         }
       }
     }
-    if (tid == 0) {
+    if (tid == 0 && !wait) {
+      if (kPre) state->phase = 2;
       if (kMass) {
         Q.out.mass[rel] = hard ? -1.f : mass;
       } else {
@@ -805,10 +875,12 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
 }
 
 // kThreads: threads of a group; 32 = a warp, four to a CTA.  Registers are
-// bounded so that 24 warps (groups of a warp, or of 128 or 256 threads) or one
-// CTA of 512 threads fit an SM.
+// bounded so that 24 to 28 warps (groups of a warp, or of 128 or 256 threads)
+// or one CTA of 512 threads fit an SM.  (Seven CTAs of 128 threads instead of
+// six, 72 registers: W = 6, L = 96, p = 0.3, 1,024 configurations 734 -> 524
+// us; eight, 64 registers, spill: W = 20, L = 301 1,540 -> 1,690 us.)
 template <int kThreads, bool kPart, int kMode>
-__global__ void __launch_bounds__(kThreads == 32 ? 128 : kThreads, kThreads <= 128 ? 6 : kThreads == 256 ? 3 : 1)
+__global__ void __launch_bounds__(kThreads == 32 ? 128 : kThreads, kThreads == 32 ? 6 : kThreads == 128 ? 7 : kThreads == 256 ? 3 : 1)
     wave_kernel(const __grid_constant__ WaveArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (kThreads == 32) {
@@ -823,7 +895,8 @@ __global__ void __launch_bounds__(kThreads == 32 ? 128 : kThreads, kThreads <= 1
 template <int kThreads>
 const void* wave_fn_of(bool part, int mode) {
   if (mode == M_LEVELS) return part ? (const void*)wave_kernel<kThreads, true, M_LEVELS> : (const void*)wave_kernel<kThreads, false, M_LEVELS>;
-  constexpr int T = kThreads == 32 ? 128 : kThreads;  // masses: CTAs
+  constexpr int T = kThreads == 32 ? 128 : kThreads;  // these: CTAs
+  if (mode == M_PRE) return part ? (const void*)wave_kernel<T, true, M_PRE> : (const void*)wave_kernel<T, false, M_PRE>;
   if (mode == M_HASH) return part ? (const void*)wave_kernel<T, true, M_HASH> : (const void*)wave_kernel<T, false, M_HASH>;
   return part ? (const void*)wave_kernel<T, true, M_PLANES> : (const void*)wave_kernel<T, false, M_PLANES>;
 }
@@ -833,6 +906,46 @@ const void* wave_fn(int threads, bool part, int mode) {
          : threads == 128 ? wave_fn_of<128>(part, mode)
          : threads == 256 ? wave_fn_of<256>(part, mode)
                           : wave_fn_of<512>(part, mode);
+}
+
+// Layers drawn ahead of M_PRE launches: a CTA per configuration and chunk of
+// eight layers of the word rows [row0, row1), into the byte of the words of the
+// row in the configuration's scratch.  The first chunk of a row clears the
+// row of the overflow maps.
+__global__ void __launch_bounds__(512) wave_draw_kernel(const __grid_constant__ WaveArgs a, int row0, int row1) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* tile = reinterpret_cast<uint32_t*>(smem_raw);
+  const int chunks = 4 * (row1 - row0);
+  const long long item = blockIdx.x / chunks;
+  if (a.state[item].phase == 2) return;
+  int qi = 0;
+  if (a.nq > 1) {
+    int hi = a.nq - 1;
+    while (qi < hi) {
+      const int mid = (qi + hi + 1) >> 1;
+      if (a.qs[mid].item0 <= item) qi = mid; else hi = mid - 1;
+    }
+  }
+  const WaveQuery& Q = a.nq > 1 ? a.qs[qi] : a.q0;
+  const int P = Q.P, G = 32 * row0 + 8 * (int)(blockIdx.x % chunks), w = G >> 5, tid = threadIdx.x, size = blockDim.x;
+  char* scratch = a.scratch + item * a.scratch_stride;
+  uint8_t* to = reinterpret_cast<uint8_t*>(scratch + Q.a_back) + 4 * (size_t)w * P + ((G >> 3) & 3);
+  if (w >= Q.TW) return;
+  if ((G & 31) == 0) {
+    uint32_t* over = reinterpret_cast<uint32_t*>(scratch + Q.a_over);
+    for (int k = tid; k < P; k += size) {
+      over[(size_t)w * P + k] = 0u;
+      over[(size_t)(Q.TW + w) * P + k] = 0u;
+    }
+  }
+  for (int k = tid; k < P; k += size) tile[k] = 0u;
+  __syncthreads();
+  const uint32_t tile_s = smem_at(tile);
+  if (G < Q.L)
+    draw_layers(Q, item - Q.item0, G, min(G + 8, Q.L), tid, size, true, tile_s, 7,
+                [&](int t, int pos) { reds_or(tile_s + 4u * (uint32_t)pos, 1u << (t & 7)); });
+  __syncthreads();
+  for (int k = tid; k < P; k += size) to[4 * (size_t)k] = (uint8_t)tile[k];
 }
 
 int ceil_log2(long long x) {
@@ -936,9 +1049,11 @@ bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings) {
   if (!hash) off = up(2 * row_b * w.TW, 256);
   w.a_back = (long long)off;
   if (w.NR < w.TW) off += map_b;
+  if (l.mode == M_PRE && w.NR == w.TW) off += map_b;
   w.a_occ = w.a_nu = (long long)off;
   w.ring_mask = -1;
-  if (l.mode != M_LEVELS && w.o_occ < 0) off += map_b;
+  if (l.mode == M_PRE) off += up(sizeof(uint2) * (size_t)w.cap, 256);  // a queue between launches
+  if ((l.mode == M_HASH || l.mode == M_PLANES) && w.o_occ < 0) off += map_b;
   if (l.mode == M_PLANES) {
     w.a_nu = (long long)off;
     if (!full_rings && w.L > 128) w.ring_mask = 127;
@@ -951,7 +1066,8 @@ bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings) {
 // The launches of a class of queries (item0 set): levels; masses in hash
 // tables, or in rings of planes where a level does not fit the tables; masses
 // that the second left (marked -1), with a plane for every layer.
-std::vector<WaveLaunch> launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, size_t most) {
+std::vector<WaveLaunch> launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, size_t most,
+                                    bool ahead) {
   std::vector<WaveLaunch> out;
   auto add = [&](int mode, int t, bool full) -> bool {
     WaveLaunch l;
@@ -963,7 +1079,7 @@ std::vector<WaveLaunch> launches_of(const std::vector<WaveQuery>& qs, long long 
     out.push_back(l);
     return true;
   };
-  add(M_LEVELS, threads, false);
+  add(ahead ? M_PRE : M_LEVELS, threads, false);
   bool mass = false, rings = false;
   for (const WaveQuery& w : qs) mass = mass || w.want_mass;
   if (!mass) return out;
@@ -1037,7 +1153,17 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
     }
     if (cq.empty()) continue;
     ++classes;
-    for (WaveLaunch& l : launches_of(cq, items, threads, (size_t)optin - 64)) ls.push_back(l);
+    // Few configurations of large lattices: their rows are drawn by the whole
+    // device ahead of the levels, instead of by the one SM that works on them
+    // (a third of its time at W = 64).
+    bool ahead = !m && items <= nsm && threads >= 256;
+    size_t maps = 0;
+    for (const WaveQuery& w : cq) {
+      ahead = ahead && (long long)w.A * w.L >= (1 << 18) && 4 * (size_t)w.P <= (size_t)optin - 64;
+      maps = std::max(maps, 12 * (size_t)w.P * w.TW);
+    }
+    ahead = ahead && maps * (size_t)items <= (2ull << 30);
+    for (WaveLaunch& l : launches_of(cq, items, threads, (size_t)optin - 64, ahead)) ls.push_back(l);
   }
   // Grids, and one scratch for all launches (they run one after the other) of
   // at most `total` bytes, one group at least.  The launch for what the rings
@@ -1054,6 +1180,12 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
         PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, l.threads * (int)l.per_cta(), l.group_smem * l.per_cta()));
         if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
         const size_t cta_b = l.stride * l.per_cta();
+        if (l.mode == M_PRE) {
+          if (per_sm * nsm < l.items) { set_error("wavefront solver: the configurations do not fit the device at once"); return PC_ERR_INTERNAL; }
+          l.grid = l.items;
+          *scratch = std::max(*scratch, cta_b * (size_t)l.grid);
+          continue;
+        }
         const size_t most = l.hard ? std::min(total, std::max<size_t>(*scratch, 64u << 20)) : total;
         long long n = std::min<long long>((long long)per_sm * nsm, (l.items + (long long)l.per_cta() - 1) / (long long)l.per_cta());
         n = std::min<long long>(n, (long long)(most / cta_b));
@@ -1064,8 +1196,12 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
     return PC_OK;
   };
   size_t tables = 0;
-  for (const WaveLaunch& l : ls) tables += l.table_b();
-  const size_t head = 256 * ls.size();
+  size_t states = 0;
+  for (const WaveLaunch& l : ls) {
+    tables += l.table_b();
+    if (l.mode == M_PRE) states += up(sizeof(WaveState) * (size_t)l.items, 256);
+  }
+  const size_t head = 256 * ls.size() + states;
   pc_status rc = PC_OK;
   cudaError_t e = cudaSuccess;
   char* mem = nullptr;
@@ -1092,6 +1228,7 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   }
   char* at = m ? nullptr : mem + head;  // query tables
   char* const base = m ? m->scratch : mem + head + tables;
+  char* state = m ? nullptr : mem + 256 * ls.size();
   for (size_t k = 0; k < ls.size() && e == cudaSuccess; ++k) {
     WaveLaunch& l = ls[k];
     WaveArgs a = {};
@@ -1115,9 +1252,28 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
       at += l.table_b();
     }
     void* args[] = {&a};
-    if (e == cudaSuccess)
-      e = cudaLaunchKernel(wave_fn(l.threads, l.part, l.mode), dim3((unsigned)l.grid),
-                           dim3(l.threads * (unsigned)l.per_cta()), args, l.group_smem * l.per_cta(), st);
+    auto launch = [&]() {
+      if (e == cudaSuccess)
+        e = cudaLaunchKernel(wave_fn(l.threads, l.part, l.mode), dim3((unsigned)l.grid),
+                             dim3(l.threads * (unsigned)l.per_cta()), args, l.group_smem * l.per_cta(), st);
+    };
+    if (l.mode != M_PRE) {
+      launch();
+      continue;
+    }
+    // rows drawn ahead in growing steps, so that configurations which end early
+    // cost little; those that reach the last drawn row wait for the next step
+    a.state = (WaveState*)state;
+    state += up(sizeof(WaveState) * (size_t)l.items, 256);
+    int rows = 0, most_p = 0;
+    for (const WaveQuery& w : l.q) { rows = std::max(rows, w.TW); most_p = std::max(most_p, w.P); }
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(wave_draw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    for (int r0 = 0, r1 = std::min(4, rows); r0 < rows && e == cudaSuccess; r0 = r1, r1 = std::min(4 * r1, rows)) {
+      wave_draw_kernel<<<(unsigned)(l.items * 4 * (r1 - r0)), 512, 4 * (size_t)most_p, st>>>(a, r0, r1);
+      e = cudaGetLastError();
+      a.rows_ready = r1;
+      launch();
+    }
   }
   if (e != cudaSuccess) rc = cuda_fail(e, "wavefront solver");
   if (mem) cudaFreeAsync(mem, st);

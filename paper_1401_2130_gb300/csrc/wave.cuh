@@ -31,6 +31,13 @@ struct WaveQuery {
   long long a_back, a_over, a_occ, a_nu;  // scratch: evicted rows, overflow maps, occupancy, mass rings
 };
 
+// A configuration between two launches over drawn rows.
+struct WaveState {
+  int phase;  // 0: not begun, 1: waits for rows, 2: done
+  int m, wb, G, olo, ohi;
+  unsigned total, n0;
+};
+
 // Queries of one launch and where its groups find their work.
 struct WaveArgs {
   WaveQuery q0;              // the query, if nq == 1
@@ -40,6 +47,8 @@ struct WaveArgs {
   unsigned long long* work;  // next work item
   int hard;                  // mass launches: only the items marked by the first one
   int group_smem;
+  WaveState* state;          // [n_items]: configurations over drawn rows
+  int rows_ready;            // word rows drawn
   char* scratch;
   long long scratch_stride;
 };

@@ -86,6 +86,36 @@ def test_masses_of_the_forced_solvers(W, L, p, n):
         assert np.all(np.abs(a - b) <= 2 * ((P + 31) // 32 + 10) * (2.0 ** -24 * b + 2.0 ** -149)), mode
 
 
+@pytest.mark.parametrize("W,L,p,n", [
+    (24, 300, 0.18, 20),     # every word row in shared memory
+    (24, 145, 0.4, 5),       # rows drawn ahead: the last step ragged
+    (40, 128, 0.19, 30),     # exactly four word rows: one step
+    (40, 129, 0.19, 30),     # one tube more
+    (40, 700, 0.175, 12),    # three steps, a window of rows
+    (64, 600, 0.17, 3),
+    (46, 200, 0.9, 4),       # levels beyond the queue kept over a step
+    (130, 20, 0.3, 2),       # few rows in shared memory
+])
+def test_rows_drawn_ahead(W, L, p, n):
+    """Few configurations of large lattices: their rows are drawn ahead in
+    steps, and a configuration that reaches the last drawn row goes on in the
+    next launch.  Also from caller bits, and beside smaller queries."""
+    import torch
+    ref = oracle.inspect(W, L, p=p, seed=8, cfg0=2, n=n, mode="bfs", threads=THREADS)
+    ref = {k: ref[k] for k in ("verdict", "first_hit", "m_stop")}
+    g = pc.pc_inspect(W, L, p, 8, 2, n)
+    _check(g, ref, W, (W, L, p))
+    many = pc.pc_inspect(W, L, p, 8, 0, 200)  # drawn by the block that works on them
+    for k in ("verdict", "first_hit", "m_stop", "mass"):
+        assert np.array_equal(many[k][2:2 + n], g[k]), k
+    bits = pc.pc_occupancy(W, L, p, 8, 2, n)
+    _check(pc.pc_inspect_occupancy(W, L, bits), ref, W, "caller bits")
+    outs, _ = pc.pc_batch_run([(W, L, p, 8, 2, n), (W, L // 2 + 1, p, 8, 0, 3), (4, 16, 0.2, 8, 0, 100)])
+    for k in ("verdict", "first_hit", "m_stop", "mass"):
+        assert np.array_equal(outs[0][k], g[k]), k
+    torch.cuda.synchronize()
+
+
 def _columns(W):
     return [(q, r) for r in range(-W, W + 1) for q in range(max(-W, -W - r), min(W, W - r) + 1)]
 
