@@ -284,16 +284,16 @@ pc_status pc_server_destroy(pc_server* s);
 
 /*
  * pc_inspect_static -- pc_inspect for callers that must not allocate device
- * memory.  The paper has no counterpart: this is a deployment variant of the
- * resident (shared-memory) solver.
+ * memory.  The paper has no counterpart: this is a deployment variant.
  *
  * Who needs it: processes whose framework has reserved the whole device for
  * its own pool allocator, where a cudaMalloc fails or fragments that pool,
  * and latency-critical loops that cannot afford cudaMalloc / cudaFree, which
  * may synchronise the whole device.  This call performs no device allocation
- * of any kind: its scratch (counters, lattice tables, device staging of the
- * outputs) is one static device array of about 3.9 MB that every GPU loading
- * the library holds until the process exits.
+ * of any kind: its scratch (counters, lattice tables, the solver's maps,
+ * device staging of the outputs) is one static device array of about 7.7 MB
+ * that every GPU loading the library holds until the process exits.  (Pinned
+ * host memory for the copy back is set up by the first call.)
  *
  * Arguments and outputs as pc_inspect with host outputs (all output pointers
  * are HOST pointers; verdicts required, the others optional); the call

@@ -1,5 +1,5 @@
-// noalloc.cu -- pc_inspect_static: the resident inspection without any
-// device-memory allocation.
+// noalloc.cu -- pc_inspect_static: the inspection without any device-memory
+// allocation.
 //
 // Some callers cannot allocate device memory at the point where they need an
 // inspection: a process whose framework has reserved the whole device for
@@ -7,9 +7,9 @@
 // and latency-critical loops for which cudaMalloc / cudaFree are off limits
 // because they can synchronise the whole device.  This entry point serves
 // them: every piece of device scratch it needs -- the work and percolation
-// counters, the lattice tables of the requested W, and the device staging of
-// the per-configuration outputs -- lives in one file-scope static device
-// array, g_static_scratch, of kStaticBytes bytes.  Every GPU that loads the
+// counters, the lattice tables of the requested W, the wavefront solver's
+// scratch and the device staging of the per-configuration outputs -- lives in
+// one file-scope static device array, g_static_scratch, of kStaticBytes bytes.  Every GPU that loads the
 // library holds that array until the process exits.
 //
 // Limits: the lattice must fit the resident (shared-memory) solver and have
@@ -33,10 +33,13 @@
 // one CTA's shared memory (227 KB on GB300), which bounds the lattice long
 // before the tables do: W <= 26 (at L = 1), W = 20 up to L = 8, W = 8 up to
 // L = 74.
+#include <cstring>
 #include <mutex>
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
+#include "wave.cuh"
 
 namespace pc {
 
@@ -48,20 +51,16 @@ constexpr int kStaticMaxP = 9216;             // plane entries of the widest all
 constexpr int kStaticMaxStrips = kStaticMaxP / 3 + 2;
 constexpr int kStaticMaxRows = 2 * kStaticMaxW + 1;
 constexpr int64_t kStaticMaxConfigs = 1 << 18;
+constexpr size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+constexpr size_t kPposBytes = up256(sizeof(int32_t) * (kStaticMaxColumns + 4));  // read in fours
+constexpr size_t kRoffBytes = up256(sizeof(int32_t) * 4 * kStaticMaxRows);
+constexpr size_t kSrowBytes = up256(sizeof(int16_t) * kStaticMaxStrips);
+// scratch of the configurations in work (the solver takes as many as it holds;
+// a resident-size lattice needs at most 232 KB for one)
+constexpr size_t kWaveBytes = 4u << 20;
 constexpr size_t kCtrBytes = 256;
-constexpr size_t kNbrBytes = sizeof(int32_t) * kStaticMaxColumns * kLateral;
-constexpr size_t kSigBytes = kStaticMaxColumns;
-constexpr size_t kLayBytes = sizeof(int32_t) * (kStaticMaxColumns + kStaticMaxP + 4 * kStaticMaxRows) +
-                             sizeof(int16_t) * kStaticMaxStrips;
-constexpr size_t kOutBytes = (size_t)kStaticMaxConfigs * (1 + 4 + 4 + 4);
-constexpr size_t kStaticBytes = kCtrBytes + kNbrBytes + kSigBytes + ((kLayBytes + 255) & ~(size_t)255) + kOutBytes;
-
-// host staging of the layout tables (filled without allocation, then copied)
-std::mutex g_host_mu;
-int32_t h_ppos[kStaticMaxColumns];
-int32_t h_pcol[kStaticMaxP];
-int32_t h_roff[4 * kStaticMaxRows];
-int16_t h_srow[kStaticMaxStrips];
+constexpr size_t kOutBytes = up256((size_t)kStaticMaxConfigs * (1 + 4 + 4 + 4));
+constexpr size_t kStaticBytes = kPposBytes + kRoffBytes + kSrowBytes + kWaveBytes + kCtrBytes + kOutBytes;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
@@ -88,33 +87,42 @@ pc_status static_scratch(unsigned char** out) {
   return PC_OK;
 }
 
-// Lattice tables of radius W (same content as the host-built cache): for each
-// column in row-major order its 12 side-contact neighbour columns (A when
-// outside the hexagon) and its sublattice.
-__global__ void static_tables_kernel(int W, int A, int32_t* nbr, int8_t* sigma) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= A) return;
-  int r = -W, start = 0;
-  for (; r <= W; ++r) {
-    const int len = 2 * W + 1 - (r < 0 ? -r : r);
-    if (a < start + len) break;
-    start += len;
-  }
-  const int qlo = r < 0 ? -W - r : -W;
-  const int q = qlo + (a - start);
-  sigma[a] = (int8_t)(((q - r) % 3 + 3) % 3);
-  for (int d = 0; d < kLateral; ++d) {
-    const int qq = q + dir_dq(d), rr = r + dir_dr(d);
-    int j = A;
-    if (rr >= -W && rr <= W) {
-      const int lo = rr < 0 ? -W - rr : -W, hi = rr < 0 ? W : W - rr;
-      if (qq >= lo && qq <= hi) {
-        int s = 0;
-        for (int x = -W; x < rr; ++x) s += 2 * W + 1 - (x < 0 ? -x : x);
-        j = s + (qq - lo);
-      }
+// The rows of a layout, through kernel parameters (no host copy): first plane
+// position, row offsets.
+struct LayoutRows {
+  int W, s_begin, n_strips;
+  int16_t start[kStaticMaxRows];
+  int16_t off[4 * kStaticMaxRows];
+};
+
+// Tables of the compact layout (the same content as the host-built cache):
+// position of each column, row of each strip, row offsets; zeroed counters.
+__global__ void static_tables_kernel(const __grid_constant__ LayoutRows l, int A, int32_t* ppos, int16_t* strip_row,
+                                     int32_t* row_off, unsigned long long* ctr) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, W = l.W, nr = 2 * W + 1;
+  if (k < (int)(kCtrBytes / 8)) ctr[k] = 0ull;
+  if (k < 4 * nr) row_off[k] = l.off[k];
+  // columns before row i: rows W + 1, .., 2W + 1, .., W + 1 columns long
+  auto before = [W](int i) {
+    const int j = i <= W ? i : 2 * W + 1 - i, s = j * (W + 1) + j * (j - 1) / 2;
+    return i <= W ? s : 3 * W * (W + 1) + 1 - s;
+  };
+  if (k < A) {
+    int lo = 0, hi = nr - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (before(mid) <= k) lo = mid; else hi = mid - 1;
     }
-    nbr[a * kLateral + d] = j;
+    ppos[k] = l.start[lo] + (k - before(lo));
+  }
+  if (k < l.n_strips) {  // the row holding one of the strip's positions, else the row before it
+    const int p2 = 3 * (l.s_begin + k) + 2;
+    int lo = 0, hi = nr - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (l.start[mid] <= p2) lo = mid; else hi = mid - 1;
+    }
+    strip_row[k] = (int16_t)lo;
   }
 }
 
@@ -169,56 +177,66 @@ extern "C" pc_status pc_inspect_static(int32_t W, int32_t L, double p, uint64_t 
     if (Pi) *Pi = 0.0;
     return PC_OK;
   }
-  unsigned long long* work = (unsigned long long*)base;
-  unsigned long long* n_perc = work + 1;
-  int32_t* nbr = (int32_t*)(base + kCtrBytes);
-  int8_t* sig = (int8_t*)(base + kCtrBytes + kNbrBytes);
-  unsigned char* lay = base + kCtrBytes + kNbrBytes + kSigBytes;
-  int32_t* d_ppos = (int32_t*)lay;
-  int32_t* d_pcol = d_ppos + kStaticMaxColumns;
-  int32_t* d_roff = d_pcol + kStaticMaxP;
-  int16_t* d_srow = (int16_t*)(d_roff + 4 * kStaticMaxRows);
-  unsigned char* o = lay + ((kLayBytes + 255) & ~(size_t)255);
-  int32_t* d_fh = (int32_t*)o;
-  float* d_mass = (float*)(o + 4 * (size_t)kStaticMaxConfigs);
-  int32_t* d_ms = (int32_t*)(o + 8 * (size_t)kStaticMaxConfigs);
-  uint8_t* d_v = (uint8_t*)(o + 12 * (size_t)kStaticMaxConfigs);
-
-  PC_CUDA(cudaMemsetAsync(base, 0, kCtrBytes, st));
-  static_tables_kernel<<<(A + 127) / 128, 128, 0, st>>>(W, A, nbr, sig);
-  PC_CUDA(cudaGetLastError());
+  const size_t n = (size_t)n_configs;
+  unsigned char* at = base;
+  int32_t* d_ppos = (int32_t*)at; at += kPposBytes;
+  int32_t* d_roff = (int32_t*)at; at += kRoffBytes;
+  int16_t* d_srow = (int16_t*)at; at += kSrowBytes;
+  char* d_wave = (char*)at; at += kWaveBytes;
+  unsigned long long* ctr = (unsigned long long*)at;  // then the outputs, in a row
+  unsigned char* o = at + kCtrBytes;
+  StreamQuery q;
+  q.out.n_perc = ctr;
+  q.out.first_hit = (int32_t*)o; q.out.mass = (float*)(o + 4 * n);
+  q.out.m_stop = (int32_t*)(o + 8 * n); q.out.verdict = o + 12 * n;
+  LayoutRows rows;
+  rows.W = W; rows.s_begin = s_begin; rows.n_strips = n_strips;
   {
-    // pageable copies from static host tables: they synchronise, but allocate nothing
-    std::lock_guard<std::mutex> lk(g_host_mu);
-    layout_fill(W, nullptr, nullptr, nullptr, h_srow, h_roff, h_ppos, h_pcol);
-    PC_CUDA(cudaMemcpyAsync(d_ppos, h_ppos, sizeof(int32_t) * A, cudaMemcpyHostToDevice, st));
-    PC_CUDA(cudaMemcpyAsync(d_pcol, h_pcol, sizeof(int32_t) * P, cudaMemcpyHostToDevice, st));
-    PC_CUDA(cudaMemcpyAsync(d_roff, h_roff, sizeof(int32_t) * 4 * (2 * W + 1), cudaMemcpyHostToDevice, st));
-    PC_CUDA(cudaMemcpyAsync(d_srow, h_srow, sizeof(int16_t) * n_strips, cudaMemcpyHostToDevice, st));
+    int32_t off[4 * kStaticMaxRows], pp[kStaticMaxColumns];
+    layout_fill(W, nullptr, nullptr, nullptr, nullptr, off, pp, nullptr);
+    for (int i = 0; i < 4 * (2 * W + 1); ++i) rows.off[i] = (int16_t)off[i];
+    for (int i = 0, c = 0; i <= 2 * W; ++i) {
+      rows.start[i] = (int16_t)pp[c];
+      c += 2 * W + 1 - (i < W ? W - i : i - W);
+    }
+  }
+  static_tables_kernel<<<(A + 127) / 128 + 4, 128, 0, st>>>(rows, A, d_ppos, d_srow, d_roff, ctr);
+  PC_CUDA(cudaGetLastError());
+
+  q.lat = Lattice{};
+  q.lat.W = W; q.lat.L = L; q.lat.A = A; q.lat.N = (int64_t)A * L; q.lat.S = A + 1;
+  q.lat.TW = (L + 31) / 32; q.lat.TWP = q.lat.TW + 2;
+  q.lat.P = P; q.lat.s_begin = s_begin; q.lat.n_strips = n_strips;
+  q.lat.strip_row = d_srow; q.lat.row_off = d_roff; q.lat.ppos = d_ppos;
+  q.occ.k0 = (uint32_t)(seed & 0xffffffffu); q.occ.k1 = (uint32_t)(seed >> 32);
+  q.occ.cfg = 0; q.occ.wl = (uint32_t)W | ((uint32_t)L << 8); q.occ.T = threshold_of(p);
+  q.occ_bits = nullptr; q.words_per_cfg = (q.lat.N + 31) / 32;
+  q.n_cfg = n_configs; q.cfg0 = (uint32_t)config_begin;
+  WaveMemory m;
+  m.ctr = ctr + 8; m.scratch = d_wave; m.bytes = kWaveBytes; m.max_groups = n_configs;
+  if ((rc = run_wave(&q, 1, st, &m))) return rc;
+
+  const size_t all = kCtrBytes + 13 * n;
+  HostStage stage(all);  // pinned host memory, kept after the first call
+  unsigned long long cnt = 0;
+  if (stage.data()) {
+    PC_CUDA(cudaMemcpyAsync(stage.data(), ctr, all, cudaMemcpyDeviceToHost, st));
+    PC_CUDA(cudaStreamSynchronize(st));
+    const char* h = stage.data();
+    std::memcpy(&cnt, h, 8);
+    h += kCtrBytes;
+    if (first_hit) std::memcpy(first_hit, h, 4 * n);
+    if (mass) std::memcpy(mass, h + 4 * n, 4 * n);
+    if (m_stop) std::memcpy(m_stop, h + 8 * n, 4 * n);
+    std::memcpy(verdicts, h + 12 * n, n);
+  } else {
+    PC_CUDA(cudaMemcpyAsync(verdicts, q.out.verdict, n, cudaMemcpyDeviceToHost, st));
+    if (first_hit) PC_CUDA(cudaMemcpyAsync(first_hit, q.out.first_hit, n * 4, cudaMemcpyDeviceToHost, st));
+    if (mass) PC_CUDA(cudaMemcpyAsync(mass, q.out.mass, n * 4, cudaMemcpyDeviceToHost, st));
+    if (m_stop) PC_CUDA(cudaMemcpyAsync(m_stop, q.out.m_stop, n * 4, cudaMemcpyDeviceToHost, st));
+    PC_CUDA(cudaMemcpyAsync(&cnt, ctr, 8, cudaMemcpyDeviceToHost, st));
     PC_CUDA(cudaStreamSynchronize(st));
   }
-
-  ResidentArgs a;
-  a.lat.W = W; a.lat.L = L; a.lat.A = A; a.lat.N = (int64_t)A * L; a.lat.S = A + 1;
-  a.lat.TW = (L + 31) / 32; a.lat.TWP = a.lat.TW + 2; a.lat.nbr = nbr; a.lat.sigma = sig;
-  a.lat.P = P; a.lat.s_begin = s_begin; a.lat.n_strips = n_strips;
-  a.lat.strip_row = d_srow; a.lat.row_off = d_roff; a.lat.ppos = d_ppos; a.lat.pcol = d_pcol;
-  a.occ.k0 = (uint32_t)(seed & 0xffffffffu); a.occ.k1 = (uint32_t)(seed >> 32);
-  a.occ.cfg = 0; a.occ.wl = (uint32_t)W | ((uint32_t)L << 8); a.occ.T = threshold_of(p);
-  a.occ_bits = nullptr; a.words_per_cfg = (a.lat.N + 31) / 32;
-  a.n_cfg = n_configs; a.cfg0 = (uint32_t)config_begin;
-  a.verdict = d_v; a.first_hit = d_fh; a.mass = d_mass; a.m_stop = d_ms;
-  a.n_perc = n_perc; a.work = work; a.prep_chunk = 8;
-  if ((rc = launch_resident(a, resident_threads(A, L), st))) return rc;
-
-  const size_t n = (size_t)n_configs;
-  PC_CUDA(cudaMemcpyAsync(verdicts, d_v, n, cudaMemcpyDeviceToHost, st));
-  if (first_hit) PC_CUDA(cudaMemcpyAsync(first_hit, d_fh, n * 4, cudaMemcpyDeviceToHost, st));
-  if (mass) PC_CUDA(cudaMemcpyAsync(mass, d_mass, n * 4, cudaMemcpyDeviceToHost, st));
-  if (m_stop) PC_CUDA(cudaMemcpyAsync(m_stop, d_ms, n * 4, cudaMemcpyDeviceToHost, st));
-  unsigned long long cnt = 0;
-  PC_CUDA(cudaMemcpyAsync(&cnt, n_perc, 8, cudaMemcpyDeviceToHost, st));
-  PC_CUDA(cudaStreamSynchronize(st));
   if (n_percolating) *n_percolating = (int64_t)cnt;
   if (Pi) *Pi = (double)cnt / (double)n_configs;
   return PC_OK;

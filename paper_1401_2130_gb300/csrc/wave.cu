@@ -45,6 +45,9 @@
 // L = 4096, p = 0.17, one configuration 1,248,000 -> 41,700.
 #include <algorithm>
 #include <cstddef>
+#include <map>
+#include <mutex>
+#include <tuple>
 #include <vector>
 
 #include "common.cuh"
@@ -242,6 +245,10 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
   const bool has16 = (lane & 15) < 14;
   const uint32_t e16 = has16 ? c_ent(lane & 15) : 0u, y16 = has16 ? c_cls(lane & 15) : 16u | 0x1500u;
 
+  if (kMass && !(a.full && !a.hard)) {  // nothing to do here?
+    const unsigned long long n = a.count[a.hard ? 1 : 0];
+    if (n < a.min_count || n > a.max_count) return;
+  }
   for (bool once = false;; once = true) {
     long long item;
     if (kPre) {  // a CTA per configuration, with its own scratch
@@ -290,7 +297,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     const int ring_mask = Q.ring_mask;
     const size_t nu_n = (size_t)(ring_mask < 0 ? L : ring_mask + 1) * P;
     const long long rel = item - Q.item0;
-    if (kMass) {  // percolating configurations only (group-uniform)
+    if (kMass && (a.hard || !a.full)) {  // percolating, or marked, configurations only (group-uniform)
       const bool skip = !Q.want_mass || (a.hard ? !(Q.out.mass[rel] < 0.f) : !Q.out.verdict[rel]);
       group_sync<kWarp>();  // every thread has read the item
       if (skip) continue;
@@ -300,6 +307,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       for (int k = tid; k < 8 * (2 * Q.W + 1); k += size) roff[k] = (k & 7) < 4 ? Q.row_off[(k >> 3) * 4 + (k & 7)] : 0;
     }
     if (tid == 0) {
+      gs->nz[0] = 0u;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         gs->cf[k][0] = 0u; gs->cf[k][1] = 0u; gs->olo[k] = 0x7fffffff; gs->ohi[k] = -1;
@@ -472,8 +480,9 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     const unsigned n0 = n_start;
 
     // nu of a new site: (1/degree) x the sum over the contacts of the previous
-    // level, whose values lie in src (at level 0: (1/degree) x 1/n0)
-    auto site_value = [&](int t, int pos, int hrow, const float* src) -> float {
+    // level, whose values value_of gives (0 for other contacts); at level 0:
+    // (1/degree) x 1/n0
+    auto site_value = [&](int t, int pos, int hrow, bool later, auto&& value_of) -> float {
       const int sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
       const int4 o4 = reinterpret_cast<const int4*>(roff)[2 * hrow];
       const int ro[5] = {o4.x, o4.y, o4.z, o4.w, 0};
@@ -491,15 +500,11 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         v[d] = 0.f;
         if (ow[d] & 1u) {
           ++deg;
-          if (src) {
-            const int tt = t + c_end(d) + (c_up(d) & (sg == 2)) - (c_dn(d) & (sg == 0));
-            const int np = pos + c_dq(d) + ro[c_row(d)];
-            if (!((*word_ptr(tt >> 5, np) >> (tt & 31)) & 1u)) v[d] = src[plane(tt) + np];
-          }
+          if (later) v[d] = value_of(t + c_end(d) + (c_up(d) & (sg == 2)) - (c_dn(d) & (sg == 0)), pos + c_dq(d) + ro[c_row(d)]);
         }
       }
       const float inv = deg ? __frcp_rn((float)deg) : 0.f;
-      if (!src) return inv * __frcp_rn((float)n0);
+      if (!later) return inv * __frcp_rn((float)n0);
       // the addition trees of the full recursion (strip_sums in tiling.cuh)
       const float e = v[6] + v[9], h = v[12] + v[13], g = v[5] + v[2];
       const float pa = v[7] + v[0], pbs = v[8] + v[1], pcs = v[4] + v[11], pd = v[3] + v[10];
@@ -514,15 +519,29 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     // come from its table (others are not in it: 0), the additions are those of
     // site_value, between lanes.
     auto level_hash = [&](int m, unsigned n) -> bool {
-      if (tid == 0) gs->nz[m & 1] = 0u;
-      group_sync<kWarp>();
       const uint32_t q_s = queue_s + 8u * (uint32_t)((m & 1) * cap);
       const int half = lane & 16;
       // the lane whose value the first addition takes: the pairs (0,7) (1,8)
       // (2,5) (3,10) (4,11) (6,9) (12,13), four bits a lane
       const int mate = half | (int)((0xFECD4361092BA587ull >> (4 * (lane & 15))) & 15u);
       bool nz = false;
-      for (unsigned i0 = (unsigned)(tid >> 5) * 2u; i0 < n; i0 += (unsigned)(size >> 5) * 2u) {
+      // many sites: a lane per site (about 13 instructions a site in full warps
+      // against 45 with sixteen lanes, but a chain three times as long)
+      const bool lanes = kWarp && n > 6u;  // (in the CTA kernels its registers cost more than it saves)
+      for (unsigned i0 = (unsigned)(tid & ~31); lanes && i0 < n; i0 += (unsigned)size) {
+        const unsigned i = i0 + (unsigned)lane;
+        uint32_t ent;
+        int t;
+        decode(lds_u2(q_s + 8u * (i < n ? i : i0)), ent, t);
+        if (i < n) {
+          hash_add(m, key_of(ent & kPosMask, t), i);
+          const float val = site_value(t, (int)(ent & kPosMask), (int)(ent >> kPosBits), m != 0,
+                                       [&](int tt, int np) { return hash_nu(m - 1, key_of((uint32_t)np, tt)); });
+          asm volatile("st.shared.f32 [%0], %1;" :: "r"(nuq_s + 4u * (uint32_t)((m & 1) * cap) + 4u * i), "f"(val) : "memory");
+          nz |= val != 0.f;
+        }
+      }
+      for (unsigned i0 = (unsigned)(tid >> 5) * 2u; !lanes && i0 < n; i0 += (unsigned)(size >> 5) * 2u) {
         const unsigned i = i0 + (unsigned)(lane >> 4);
         const bool act = i < n && has16;
         uint32_t ent;
@@ -554,16 +573,19 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
       }
       if (nz) gs->nz[m & 1] = 1u;
       group_sync<kWarp>();
-      const bool live = gs->nz[m & 1] != 0u;
-      // the other table is the next level's
+      // the other table and flag are the next level's, which fills them after
+      // the barrier of its claims
+      if (tid == 0) gs->nz[(m + 1) & 1] = 0u;
       for (uint32_t k = tid; k <= tab_mask; k += size) sts_u2(tab_s + 8u * ((uint32_t)(((m + 1) & 1) << tab_bits) + k), kNone, 0u);
-      group_sync<kWarp>();
-      return live;
+      return gs->nz[m & 1] != 0u;
     };
     // nu of the sites of level m (queue qn, overflow rows [lo, hi]); true if any is not 0
     auto level_values = [&](int m, unsigned n, const uint2* qn, int lo, int hi) -> bool {
       const float* src = m ? nu + (size_t)((m - 1) & 1) * nu_n : nullptr;
       float* dst = nu + (size_t)(m & 1) * nu_n;
+      auto value_of = [&](int tt, int np) {  // reached sites: of the previous level, or zeroed when claimed
+        return (*word_ptr(tt >> 5, np) >> (tt & 31)) & 1u ? 0.f : src[plane(tt) + np];
+      };
       if (tid == 0) gs->nz[m & 1] = 0u;
       group_sync<kWarp>();
       bool nz = false;
@@ -573,7 +595,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         int t;
         decode(qn[i], ent, t);
         const int pos = (int)(ent & kPosMask);
-        const float x = site_value(t, pos, (int)(ent >> kPosBits), src);
+        const float x = site_value(t, pos, (int)(ent >> kPosBits), m != 0, value_of);
         dst[plane(t) + pos] = x;
         nz |= x != 0.f;
       }
@@ -583,7 +605,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
           while (word) {
             const int t = 32 * w + __ffs(word) - 1;
             word &= word - 1;
-            const float x = site_value(t, pos, row_of(pos), src);
+            const float x = site_value(t, pos, row_of(pos), m != 0, value_of);
             dst[plane(t) + pos] = x;
             nz |= x != 0.f;
           }
@@ -612,6 +634,7 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     float mass = 0.f;
     bool hard = kMode == M_HASH && total > (unsigned)cap;  // left to the launch with planes
     bool wait = false;
+    bool live = true;  // some nu of the level is not 0
     if (kMass && n0 > 0 && !hard) {
       if (kMode == M_HASH) level_hash(0, total);
       else level_values(0, total, queue, 0, gs->ohi[0]);
@@ -812,10 +835,10 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
           }
           if (kMass || !(f & F_HIT)) draw();
         }
-        if (kMode == M_HASH) {
-          const bool live = level_hash(m, total);
-          if (f & F_HIT) { mass = detector_mass(m); break; }
-          if (!live) break;  // nu has underflowed everywhere: the mass is 0
+        if (kMode == M_HASH && live) {
+          live = level_hash(m, total);
+          if (live && (f & F_HIT)) mass = detector_mass(m);
+          if (!live && !a.full) break;  // nu has underflowed everywhere: the mass is 0
         }
         if (kMode == M_PLANES || (kPart && NR > 0 && (f & F_OUT))) {
           int lo = 0, hi = 0;  // tubes of the new level
@@ -843,16 +866,16 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
             // (a level lies within one tube of the previous one's) and the
             // tubes around them are fewer than the rings' planes
             if (ring_mask >= 0 && hi - lo + 5 > ring_mask + 1) { hard = true; break; }
-            const bool live = level_values(m, total, queue + (m & 1) * cap, gs->olo[nx], gs->ohi[nx]);
-            if (f & F_HIT) { mass = detector_mass(m); break; }
-            if (!live) break;  // nu has underflowed everywhere: the mass is 0
+            if (live) live = level_values(m, total, queue + (m & 1) * cap, gs->olo[nx], gs->ohi[nx]);
+            if (live && (f & F_HIT)) mass = detector_mass(m);
+            if (!live && !a.full) break;  // nu has underflowed everywhere: the mass is 0
           }
           if (kPart && NR > 0 && (f & F_OUT)) {  // keep the window on the frontier
             if ((lo >> 5) < wb && (hi >> 5) < wb + NR - 1) slide(-1);
             else if ((hi >> 5) >= wb + NR && (lo >> 5) > wb) slide(1);
           }
         }
-        if (!kMass && (f & F_HIT)) {
+        if (f & F_HIT) {
           verdict = 1; fh = m + 1; mstop = m + 1;
           break;
         }
@@ -860,14 +883,15 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
     }
     if (tid == 0 && !wait) {
       if (kPre) state->phase = 2;
-      if (kMass) {
-        Q.out.mass[rel] = hard ? -1.f : mass;
-      } else {
+      if (hard) atomicAdd(a.count + 1, 1ull);
+      if (kMass) Q.out.mass[rel] = hard ? -1.f : mass;
+      else if (Q.out.mass) Q.out.mass[rel] = 0.f;
+      if ((!kMass || a.full) && !hard) {
         Q.out.verdict[rel] = (uint8_t)verdict;
         if (Q.out.first_hit) Q.out.first_hit[rel] = fh;
-        if (Q.out.mass) Q.out.mass[rel] = 0.f;
         if (Q.out.m_stop) Q.out.m_stop[rel] = mstop;
         if (verdict && Q.out.n_perc) atomicAdd(Q.out.n_perc, 1ull);
+        if (!kMass && verdict && Q.want_mass) atomicAdd(a.count, 1ull);
       }
     }
     group_sync<kWarp>();
@@ -895,9 +919,9 @@ __global__ void __launch_bounds__(kThreads == 32 ? 128 : kThreads, kThreads == 3
 template <int kThreads>
 const void* wave_fn_of(bool part, int mode) {
   if (mode == M_LEVELS) return part ? (const void*)wave_kernel<kThreads, true, M_LEVELS> : (const void*)wave_kernel<kThreads, false, M_LEVELS>;
+  if (mode == M_HASH) return part ? (const void*)wave_kernel<kThreads, true, M_HASH> : (const void*)wave_kernel<kThreads, false, M_HASH>;
   constexpr int T = kThreads == 32 ? 128 : kThreads;  // these: CTAs
   if (mode == M_PRE) return part ? (const void*)wave_kernel<T, true, M_PRE> : (const void*)wave_kernel<T, false, M_PRE>;
-  if (mode == M_HASH) return part ? (const void*)wave_kernel<T, true, M_HASH> : (const void*)wave_kernel<T, false, M_HASH>;
   return part ? (const void*)wave_kernel<T, true, M_PLANES> : (const void*)wave_kernel<T, false, M_PLANES>;
 }
 
@@ -983,7 +1007,9 @@ __global__ void wave_upload_kernel(WaveQuery* dst, const __grid_constant__ Uploa
 // One launch over the queries that run with the same group size.
 struct WaveLaunch {
   int mode = M_LEVELS, threads = 0;
-  bool part = false, hard = false;
+  bool part = false, hard = false, full = false;
+  int cls = 0;               // launches of one class share the counts
+  unsigned long long min_count = 1, max_count = ~0ull;
   std::vector<WaveQuery> q;
   long long items = 0;
   size_t group_smem = 0, stride = 256;
@@ -1063,38 +1089,105 @@ bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings) {
   return true;
 }
 
-// The launches of a class of queries (item0 set): levels; masses in hash
-// tables, or in rings of planes where a level does not fit the tables; masses
-// that the second left (marked -1), with a plane for every layer.
-std::vector<WaveLaunch> launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, size_t most,
-                                    bool ahead) {
-  std::vector<WaveLaunch> out;
-  auto add = [&](int mode, int t, bool full) -> bool {
-    WaveLaunch l;
-    l.mode = mode; l.threads = t; l.items = items; l.hard = mode == M_PLANES && full;
+// Groups of a launch that fit the device at once.  What the driver says is kept
+// per device, kernel and shared memory (at most kFits entries): asking took
+// several microseconds a launch.
+constexpr size_t kFits = 256;
+std::mutex g_fit_mu;
+std::map<std::tuple<int, const void*, size_t>, int> g_fit;
+
+pc_status resident_groups(const WaveLaunch& l, int nsm, int optin, long long* n) {
+  const void* f = wave_fn(l.threads, l.part, l.mode);
+  int dev = 0;
+  PC_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(g_fit_mu);
+  const auto key = std::make_tuple(dev, f, l.group_smem);
+  const auto known = g_fit.find(key);
+  if (known != g_fit.end()) {
+    *n = (long long)known->second * nsm * (long long)l.per_cta();
+    return PC_OK;
+  }
+  // the same limit on every call: calls from several threads never lower it
+  PC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+  int per_sm = 0;
+  PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, l.threads * (int)l.per_cta(), l.group_smem * l.per_cta()));
+  if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
+  if (g_fit.size() >= kFits) g_fit.clear();
+  g_fit[key] = per_sm;
+  *n = (long long)per_sm * nsm * (long long)l.per_cta();
+  return PC_OK;
+}
+
+// The launches of a class of queries (item0 set).
+//  - Verdicts only: the levels.
+//  - Masses too, and every configuration resident at once: levels and masses in
+//    one pass (the longest configuration's chain of levels is the time, and it
+//    usually percolates).
+//  - Else the levels, then the masses of the percolating ones: in hash tables,
+//    by CTAs while these are few, by warps where more percolate than CTAs fit
+//    (a level then costs fewer instructions); or in rings of planes where a
+//    start layer does not fit the tables.
+//  - Last, masses that did not fit (marked -1), with a plane for every layer.
+pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, int nsm, int optin, bool ahead,
+                      long long at_once, std::vector<WaveLaunch>& out) {
+  auto make = [&](int mode, int t, bool full_rings, WaveLaunch& l) -> bool {
+    l = WaveLaunch();
+    l.mode = mode; l.threads = t; l.items = items; l.hard = mode == M_PLANES && full_rings;
     for (WaveQuery w : qs) {
-      if (!place(w, l, most, full)) return false;
+      if (!place(w, l, (size_t)optin - 64, full_rings)) return false;
       l.q.push_back(w);
     }
-    out.push_back(l);
     return true;
   };
-  add(ahead ? M_PRE : M_LEVELS, threads, false);
-  bool mass = false, rings = false;
-  for (const WaveQuery& w : qs) mass = mass || w.want_mass;
-  if (!mass) return out;
+  bool some = false, all = true;
+  for (const WaveQuery& w : qs) { some = some || w.want_mass; all = all && w.want_mass; }
   const int mt = std::max(threads, 128);
-  if (add(M_HASH, mt, false)) {
-    rings = true;
-  } else {
-    add(M_PLANES, mt, false);
-    for (const WaveQuery& w : out.back().q) rings = rings || w.ring_mask >= 0;
+  WaveLaunch levels, hash, warps, planes;
+  make(ahead ? M_PRE : M_LEVELS, threads, false, levels);
+  if (!some) { out.push_back(levels); return PC_OK; }
+  const bool has_hash = make(M_HASH, mt, false, hash);
+  bool left = true;  // something may be left to the last launch
+  long long fit = 0;
+  if (has_hash) {
+    const pc_status rc = resident_groups(hash, nsm, optin, &fit);
+    if (rc) return rc;
   }
-  if (rings) add(M_PLANES, mt, true);
-  return out;
+  bool full = false;
+  const bool has_warps = threads == 32 && make(M_HASH, 32, false, warps);
+  if (all && !ahead && has_hash && items <= std::min(fit, at_once)) {
+    full = true;
+    hash.full = true;
+    out.push_back(hash);
+  } else {
+    out.push_back(levels);
+    if (has_hash) {
+      if (has_warps) {
+        hash.max_count = (unsigned long long)fit;
+        warps.min_count = (unsigned long long)fit + 1ull;
+        out.push_back(warps);
+      }
+      out.push_back(hash);
+    } else {
+      make(M_PLANES, mt, false, planes);
+      left = false;
+      for (const WaveQuery& w : planes.q) left = left || w.ring_mask >= 0;
+      out.push_back(planes);
+    }
+  }
+  if (left) {
+    make(M_PLANES, mt, true, planes);
+    planes.full = full;
+    out.push_back(planes);
+  }
+  return PC_OK;
 }
 
 }  // namespace
+
+void release_wave() {
+  std::lock_guard<std::mutex> lk(g_fit_mu);
+  g_fit.clear();
+}
 
 int wave_threads(int A, long long n_all) {
   int dev = 0, nsm = 1;
@@ -1163,7 +1256,10 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
       maps = std::max(maps, 12 * (size_t)w.P * w.TW);
     }
     ahead = ahead && maps * (size_t)items <= (2ull << 30);
-    for (WaveLaunch& l : launches_of(cq, items, threads, (size_t)optin - 64, ahead)) ls.push_back(l);
+    const size_t first = ls.size();
+    const pc_status rc = launches_of(cq, items, threads, nsm, optin, ahead, m ? m->max_groups : items, ls);
+    if (rc) return rc;
+    for (size_t k = first; k < ls.size(); ++k) ls[k].cls = classes - 1;
   }
   // Grids, and one scratch for all launches (they run one after the other) of
   // at most `total` bytes, one group at least.  The launch for what the rings
@@ -1173,23 +1269,20 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
     for (int pass = 0; pass < 2; ++pass)
       for (WaveLaunch& l : ls) {
         if (l.hard != (pass == 1)) continue;
-        const void* f = wave_fn(l.threads, l.part, l.mode);
-        // the same limit on every call: calls from several threads never lower it
-        PC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-        int per_sm = 0;
-        PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, l.threads * (int)l.per_cta(), l.group_smem * l.per_cta()));
-        if (per_sm < 1) { set_error("wavefront solver: no block fits an SM"); return PC_ERR_INTERNAL; }
+        long long fit = 0;
+        const pc_status rc = resident_groups(l, nsm, optin, &fit);
+        if (rc) return rc;
+        const long long per_cta = (long long)l.per_cta();
         const size_t cta_b = l.stride * l.per_cta();
         if (l.mode == M_PRE) {
-          if (per_sm * nsm < l.items) { set_error("wavefront solver: the configurations do not fit the device at once"); return PC_ERR_INTERNAL; }
           l.grid = l.items;
           *scratch = std::max(*scratch, cta_b * (size_t)l.grid);
           continue;
         }
         const size_t most = l.hard ? std::min(total, std::max<size_t>(*scratch, 64u << 20)) : total;
-        long long n = std::min<long long>((long long)per_sm * nsm, (l.items + (long long)l.per_cta() - 1) / (long long)l.per_cta());
+        long long n = std::min<long long>(fit / per_cta, (l.items + per_cta - 1) / per_cta);
         n = std::min<long long>(n, (long long)(most / cta_b));
-        if (m) n = std::min(n, m->max_groups);
+        if (m) n = std::min(n, (m->max_groups + per_cta - 1) / per_cta);
         l.grid = std::max<long long>(n, 1);
         *scratch = std::max(*scratch, cta_b * (size_t)l.grid);
       }
@@ -1208,7 +1301,7 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   size_t scratch = 0;
   if (m) {
     if ((rc = plan(m->bytes, &scratch))) return rc;
-    if (classes != 1 || tables || scratch > m->bytes || ls.size() > 3) {
+    if (classes != 1 || tables || scratch > m->bytes || ls.size() > 4) {
       set_error("wavefront solver: the caller's memory does not hold the query");
       return PC_ERR_INTERNAL;
     }
@@ -1237,7 +1330,11 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
     a.n_items = l.items;
     a.group_smem = (int)l.group_smem;
     a.hard = l.hard ? 1 : 0;
+    a.full = l.full ? 1 : 0;
+    a.min_count = l.min_count;
+    a.max_count = l.max_count;
     a.work = m ? m->ctr + k : (unsigned long long*)(mem + 256 * k);
+    a.count = m ? m->ctr + 4 : (unsigned long long*)(mem + 256 * l.cls + 64);
     a.scratch = base;
     a.scratch_stride = (long long)l.stride;
     if (l.table_b()) {

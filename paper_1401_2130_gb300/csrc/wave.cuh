@@ -45,7 +45,10 @@ struct WaveArgs {
   int nq;
   long long n_items;
   unsigned long long* work;  // next work item
+  unsigned long long* count; // percolating items whose mass is wanted; items left to planes
   int hard;                  // mass launches: only the items marked by the first one
+  int full;                  // verdicts and masses in one launch
+  unsigned long long min_count, max_count;  // mass launches: run for so many percolating items
   int group_smem;
   WaveState* state;          // [n_items]: configurations over drawn rows
   int rows_ready;            // word rows drawn
@@ -55,7 +58,7 @@ struct WaveArgs {
 
 // Device memory that a caller holds for one query's run.
 struct WaveMemory {
-  unsigned long long* ctr;   // 4 zeroed counters
+  unsigned long long* ctr;   // 8 zeroed counters
   char* scratch;
   size_t bytes;              // at least wave_scratch_bytes of the lattice
   long long max_groups;      // configurations in work at once
@@ -71,5 +74,6 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
 // Threads that work on one configuration of an A-column lattice when n_all
 // configurations are inspected together on the current device.
 int wave_threads(int A, long long n_all);
+void release_wave();  // pc_shutdown
 
 }  // namespace pc
