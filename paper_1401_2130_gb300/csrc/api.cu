@@ -146,7 +146,7 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
     if ((flags & PC_MODE_RESIDENT) && !resident) {
       set_error("PC_MODE_RESIDENT: lattice state exceeds shared memory"); rc = PC_ERR_OOM; break;
     }
-    if (!(flags & (PC_MODE_RESIDENT | PC_MODE_STREAM))) {
+    if (!(flags & (PC_MODE_RESIDENT | PC_MODE_STREAM)) && !wave_is_slower(lat, os, occ_bits, n)) {
       StreamQuery j;
       j.lat = lat; j.occ = os; j.occ_bits = occ_bits; j.words_per_cfg = wpc;
       j.n_cfg = n; j.cfg0 = (uint32_t)cfg0;

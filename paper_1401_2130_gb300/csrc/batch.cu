@@ -77,7 +77,7 @@ int tuned_threads(const Lattice& lat, double p, uint64_t seed, cudaStream_t st) 
   const int fallback = resident_threads(lat.A, lat.L);
   const int64_t n = 2048;
   char* mem = nullptr;
-  if (cudaMallocAsync((void**)&mem, 64 + n * 13, st) != cudaSuccess) return fallback;
+  if (scratch_alloc((void**)&mem, 64 + n * 13, st) != cudaSuccess) return fallback;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -167,8 +167,9 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
   }
   if (nq == 0) return PC_OK;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // device scratch: a counter per query, and the outputs of host queries
-  const size_t ctr_b = ((size_t)nq * 8 + 255) & ~(size_t)255;
+  // device scratch: a counter per query, the streamed solver's error flags, and
+  // the outputs of host queries
+  const size_t ctr_b = ((size_t)nq * 16 + 255) & ~(size_t)255;
   size_t bytes = ctr_b;
   if (!dev_out)
     for (int64_t i = 0; i < nq; ++i) bytes += ((size_t)q[i].n_configs * 13 + 255) & ~(size_t)255;
@@ -178,6 +179,7 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
   pc_status rc = PC_OK;
   long long n_all = 0;
   std::vector<StreamQuery> sq;
+  std::vector<StreamJob> streamed;  // see wave_is_slower
   std::vector<Lattice> lats((size_t)nq);
   do {
     cudaError_t e = cudaMemsetAsync(mem, 0, ctr_b, st);
@@ -203,10 +205,18 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
         s.out.m_stop = (int32_t*)(stage + 8 * n); s.out.verdict = (uint8_t*)(stage + 12 * n);
         stage += (n * 13 + 255) & ~(size_t)255;
       }
-      sq.push_back(s);
       n_all += s.n_cfg;
+      if (wave_is_slower(s.lat, s.occ, nullptr, s.n_cfg)) {
+        StreamJob j;
+        static_cast<StreamQuery&>(j) = s;
+        j.error_out = (int*)(counts + nq + i);
+        streamed.push_back(j);
+      } else {
+        sq.push_back(s);
+      }
     }
     if (rc == PC_OK) rc = run_wave(sq.data(), (int)sq.size(), st);
+    for (size_t i = 0; i < streamed.size() && rc == PC_OK; ++i) rc = run_stream(streamed[i], st);
     if (rc) break;
     if (dev_out)
       for (int64_t b = 0; b < nq && e == cudaSuccess; b += kCounts) {
@@ -219,7 +229,7 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch counts"); break; }
     if (async) break;
     // one copy of the counts and, for host queries, of every output
-    const size_t all = dev_out ? (size_t)nq * 8 : bytes;
+    const size_t all = dev_out ? (size_t)nq * 16 : bytes;
     HostStage pinned(all);
     std::vector<char> plain(pinned.data() ? 0 : all);
     const char* host = pinned.data() ? pinned.data() : plain.data();
@@ -227,6 +237,10 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch outputs"); break; }
     const unsigned long long* cnt = (const unsigned long long*)host;
+    int err = 0;
+    for (int64_t i = 0; i < nq; ++i) err |= *(const int*)(cnt + nq + i);
+    if (err & 2) { set_error("streamed solver: a bulk-copy wait timed out"); rc = PC_ERR_TIMEOUT; break; }
+    if (err) { set_error("streamed solver: tick bound or segment check failed"); rc = PC_ERR_INTERNAL; break; }
     const char* at = host + ctr_b;
     for (int64_t i = 0; i < nq; ++i) {
       const size_t n = (size_t)q[i].n_configs;

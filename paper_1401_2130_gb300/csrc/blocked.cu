@@ -52,6 +52,7 @@
 #include "blocked_plan.h"
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
 
 namespace pc {
 
@@ -575,7 +576,7 @@ pc_status run_blocked(const StreamJob& job, cudaStream_t st, bool* handled) {
   const size_t head = 256 + a256_host(sizeof(BSlot) * (size_t)K) + a256_host(4 * (size_t)(K + 1));
   static_assert(sizeof(unsigned long long) * 3 + 4 * 3 <= 256, "counters fit the head");
   char* mem = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&mem, head + slot_words * 4 * (size_t)K, st);
+  cudaError_t e = scratch_alloc((void**)&mem, head + slot_words * 4 * (size_t)K, st);
   if (e != cudaSuccess) return cuda_fail(e, "verdict-only solver state");
   BCtx x;
   x.lat = lat; x.occ = job.occ; x.occ_bits = job.occ_bits; x.words_per_cfg = job.words_per_cfg;

@@ -59,10 +59,13 @@ struct StreamQuery {
 };
 struct StreamJob : StreamQuery {
   int* error_out = nullptr;  // device int: 1 if the tick bound was hit
+  char* pool = nullptr;      // the caller's memory for the slots (else allocated)
+  size_t pool_bytes = 0;
 };
 struct StreamPlan;
 // Device resources for a set of queries (stream-ordered allocation on st).
-pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, StreamPlan** out);
+pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, StreamPlan** out,
+                             char* pool = nullptr, size_t pool_bytes = 0);
 // Adds [init -> WHILE(sweep, control)] to g after deps; *last = the WHILE node.
 pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps,
                           cudaGraphNode_t* last);

@@ -121,7 +121,14 @@ pc_status start_query(pc_server* s, Ticket& t) {
   sq.n_cfg = n; sq.cfg0 = (uint32_t)q.config_begin;
   sq.out.verdict = t.v; sq.out.first_hit = t.fh; sq.out.mass = t.mass; sq.out.m_stop = t.ms;
   sq.out.n_perc = t.n_perc;
-  if (t.kind == 0) {
+  if (t.kind == 1 && wave_is_slower(lat, sq.occ, nullptr, n)) {
+    StreamJob j;
+    static_cast<StreamQuery&>(j) = sq;
+    j.error_out = (int*)(t.n_perc + 16);
+    j.pool = s->arena.base + t.off_slots;
+    j.pool_bytes = t.bytes_slots;
+    rc = run_stream(j, st);
+  } else if (t.kind == 0) {
     rc = run_wave(&sq, 1, st, nullptr, kSmallScratch);
   } else {
     WaveMemory m;
@@ -146,7 +153,9 @@ void finish_query(pc_server* s, Ticket& t, cudaStream_t st) {
   cudaError_t e = cudaMemcpyAsync(host.data(), t.n_perc, host.size(), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   unsigned long long cnt = 0;
-  if (e == cudaSuccess) {
+  int err = 0;  // of the streamed solver
+  if (e == cudaSuccess) std::memcpy(&err, host.data() + 128, sizeof(int));
+  if (e == cudaSuccess && !err) {
     const char* h = host.data();
     std::memcpy(&cnt, h, 8);
     h += 256;
@@ -159,6 +168,10 @@ void finish_query(pc_server* s, Ticket& t, cudaStream_t st) {
   if (e != cudaSuccess) {
     t.state = T_FAILED;
     t.status = cuda_fail(e, "server: copy outputs");
+  } else if (err) {
+    set_error("server: streamed solver: device bound reached");
+    t.state = T_FAILED;
+    t.status = (err & 2) ? PC_ERR_TIMEOUT : PC_ERR_INTERNAL;
   } else {
     t.state = T_DONE;
     t.result.n_percolating = (int64_t)cnt;

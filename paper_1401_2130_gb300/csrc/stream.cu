@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
 #include "plan.h"
 #include "tiling.cuh"
 #include "tma.cuh"
@@ -710,29 +711,34 @@ int sweep_grid(const Ctx& x) {
   return nsm * per_sm;
 }
 
-__device__ inline float block_sum_f(float v, float* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Sum of an end layer's values (plane: by position) in the wavefront solver's
+// order -- lane l of one warp adds columns l, l + 32, .., then the lanes by
+// halves -- so that a configuration's mass does not depend on which of the two
+// a call takes.  vals: 8 kCols floats, filled by the whole CTA.  Valid in the
+// first warp.
+__device__ inline float end_mass(const float* plane, const int* ppos, int A, float* vals) {
+  const int tid = threadIdx.x;
+  float sum = 0.f;
+  for (int c0 = 0; c0 < A; c0 += 8 * kCols) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float s = 0.f;
-  if (warp == 0) {
-    s = lane < nw ? red[lane] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[0] = s;
+    for (int i = 0; i < 8; ++i) {
+      const int c = c0 + i * kCols + tid;
+      vals[i * kCols + tid] = c < A ? plane[__ldg(ppos + c)] : 0.f;
+    }
+    __syncthreads();
+    if (tid < 32)
+#pragma unroll 8
+      for (int k = tid; k < 8 * kCols; k += 32) sum += vals[k];
+    __syncthreads();
   }
-  __syncthreads();
-  s = red[0];
-  __syncthreads();
-  return s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return sum;
 }
 
 // One CTA per slot; the last CTA to finish plans the next tick.
 __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
-  __shared__ float red[32];
+  __shared__ float vals[8 * kCols];
   __shared__ int s_n0;
   __shared__ bool s_last;
   const int slot = blockIdx.x, tid = threadIdx.x;
@@ -763,7 +769,6 @@ __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
         finish = true;
       } else {
         const float inv = __frcp_rn((float)n0);
-        float part = 0.f;
         for (int a = tid; a < A; a += blockDim.x) {
           const uint32_t b = v.occw[S + a] & 1u;
           v.R0[S + a] = b;
@@ -772,10 +777,10 @@ __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
           const int d = v.dg[pos];
           const float val = b ? (d ? __frcp_rn((float)d) : 0.f) * inv : 0.f;
           v.nu0[(size_t)2 * lat.P + pos] = val;
-          part += val;
         }
         if (L == 1) {
-          mass = Q.bits_only ? 0.f : block_sum_f(part, red);
+          __syncthreads();
+          mass = Q.bits_only ? 0.f : end_mass(v.nu0 + (size_t)2 * lat.P, lat.ppos, A, vals);
           finish = true; verdict = 1; fh = 1; mstop = 1;
         } else {
           c.phase = PH_STEP; c.m = 1; c.flags = 0u;
@@ -787,10 +792,7 @@ __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
       c.flags = 0u;
       if (f & kEnd) {
         const float* dst = (c.m & 1) ? v.nu1 : v.nu0;
-        float part = 0.f;
-        for (int k = Q.bits_only ? lat.P : tid; k < lat.P; k += blockDim.x)
-          part += dst[(size_t)(L + 1) * lat.P + k];
-        mass = Q.bits_only ? 0.f : block_sum_f(part, red);
+        mass = Q.bits_only ? 0.f : end_mass(dst + (size_t)(L + 1) * lat.P, lat.ppos, A, vals);
         finish = true; verdict = 1; fh = c.m + 1; mstop = c.m + 1;
       } else if (!(f & kGrow)) {
         finish = true; mstop = c.m;
@@ -851,7 +853,8 @@ struct StreamPlan {
   int* error_dev = nullptr;
 };
 
-pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, StreamPlan** out) {
+pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, StreamPlan** out, char* pool,
+                             size_t pool_bytes) {
   *out = nullptr;
   long long n_items = 0;
   size_t slot = 0;
@@ -867,22 +870,23 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   }
   size_t free_b = 0, total_b = 0;
   PC_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  const size_t budget = free_b / 2;
+  const size_t budget = pool ? pool_bytes : free_b / 2;
   long long K = std::min<long long>(n_items, kMaxSlots);
   // PC_STREAM_MAX_SLOTS caps the pool (tests use it to force slot reuse)
   if (const char* cap = std::getenv("PC_STREAM_MAX_SLOTS")) {
     const long long c = std::atoll(cap);
     if (c > 0) K = std::min<long long>(K, c);
   }
-  K = std::min<long long>(K, (long long)(budget / (slot + 1)));
+  K = std::min<long long>(K, (long long)(budget / (pool ? slot : slot + 1)));
   if (n_items > 0 && K < 1) {
-    set_error("streamed solver: one configuration's state exceeds half the free device memory");
+    set_error(pool ? "streamed solver: one configuration's state exceeds the memory given"
+                   : "streamed solver: one configuration's state exceeds half the free device memory");
     return PC_ERR_OOM;
   }
   if (K < 1) K = 1;
   const size_t hdr = a256(sizeof(QDev) * nq) + a256(sizeof(Ctl) * K) + a256(sizeof(int) * (K + 1)) + 256;
   StreamPlan* P = new StreamPlan();
-  cudaError_t e = cudaMallocAsync((void**)&P->mem, hdr + (size_t)K * slot + 256, st);
+  cudaError_t e = scratch_alloc((void**)&P->mem, hdr + (pool ? 0 : (size_t)K * slot) + 256, st);
   if (e != cudaSuccess) { delete P; return cuda_fail(e, "stream plan alloc"); }
   char* q = P->mem;
   Ctx& x = P->x;
@@ -897,7 +901,7 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   x.error = (int*)(x.ticks + 2);
   x.next_unit = x.ticks + 3;
   q += 256;
-  x.pool = q;
+  x.pool = pool ? pool : q;
   x.slot_bytes = slot;
   x.use_cond = 0;
   x.fp = 0;
@@ -996,7 +1000,7 @@ pc_status run_stream_verdict_first(const StreamJob& job, cudaStream_t st) {
   // 2. the FP32 recursion on the percolating configurations only: the same
   // steps as the single pass, so every output equals it to the bit
   char* mem = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&mem, 256 + sizeof(int64_t) * (size_t)job.n_cfg, st);
+  cudaError_t e = scratch_alloc((void**)&mem, 256 + sizeof(int64_t) * (size_t)job.n_cfg, st);
   if (e != cudaSuccess) return cuda_fail(e, "verdict-first selection");
   unsigned long long* cnt = (unsigned long long*)mem;
   int64_t* sel = (int64_t*)(mem + 256);
@@ -1037,7 +1041,7 @@ pc_status run_stream(const StreamJob& job, cudaStream_t st) {
   q.lat = job.lat; q.occ = job.occ; q.occ_bits = job.occ_bits; q.words_per_cfg = job.words_per_cfg;
   q.n_cfg = job.n_cfg; q.cfg0 = job.cfg0; q.out = job.out; q.bits_only = job.bits_only; q.sel = job.sel;
   StreamPlan* P = nullptr;
-  pc_status rc = stream_plan_create(&q, 1, st, &P);
+  pc_status rc = stream_plan_create(&q, 1, st, &P, job.pool, job.pool_bytes);
   if (rc) return rc;
   if (std::getenv("PC_STREAM_HOST_LOOP")) {
     // profiling aid: the same ticks launched from a host loop (profilers do

@@ -1018,44 +1018,73 @@ struct WaveLaunch {
   size_t table_b() const { return q.size() > 1 ? up(sizeof(WaveQuery) * q.size(), 256) : 0; }
 };
 
+// Density of metallic sites (caller bits: a guess near the threshold).
+double density(const WaveQuery& w) { return w.occ_bits ? 0.2 : (double)w.occ.T / 4294967296.0; }
+// Sites of a level, on average over a percolating configuration: the start
+// layer, p A sites, is also about the largest (measured at W = 24: 85 at p =
+// 0.18, 141 at 0.2, 347 at 0.3, 1,576 at 0.9).
+double level_sites(const WaveQuery& w) {
+  const double p = std::max(density(w), 1e-9), f = 1.0 - 0.0256 / (p * p);
+  return p * w.A * std::max(f, 0.1);
+}
+
 // Threads of a group.  With more configurations than groups fit the device,
 // few (more configurations in flight; a level's fixed cost is paid by every
 // warp); else more (a level is a chain of instructions: more warps, fewer
-// sites each).
+// sites each), and more still where levels are large for their lattice.
 int group_threads(int A, long long n, int nsm) {
   if (A <= 640) return n <= 8ll * nsm ? 128 : 32;
   if (A <= 2000) return n <= 2ll * nsm ? 256 : 128;
   if (A <= 5000) return n <= nsm ? 512 : 256;
   return 512;
 }
+int group_threads(const WaveQuery& w, long long n, int nsm) {
+  const int t = group_threads(w.A, n, nsm);
+  const double s = 20.0 * level_sites(w);
+  if (n <= nsm) return std::max(t, s > 2000.0 ? 512 : s > 640.0 ? 256 : 32);
+  return n <= 2ll * nsm && s > 640.0 ? std::max(t, 256) : t;
+}
 
-// Shared memory (at most `most` bytes) and scratch of query w in a launch.
+// Shared memory (at most `most` bytes; `share`: of an SM's, per configuration,
+// if all of them are resident) and scratch of query w in a launch.
 // False: no room for the hash tables.
-bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings) {
+bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings, size_t share) {
   const size_t row_b = sizeof(uint32_t) * (size_t)w.P;
   const bool hash = l.mode == M_HASH;
   size_t target = l.threads == 32 ? 12 * 1024 : l.threads == 128 ? 36 * 1024 : l.threads == 256 ? 72 * 1024 : most;
   if (hash) target = std::min(most, 2 * target);
-  w.cap = (int)std::min<long long>(w.A, l.threads == 32 ? 512 : 1200);
+  target = std::max(target, std::min(most, share));
+  w.cap = (int)std::min<long long>(w.A, (long long)(1.1 * density(w) * w.A) + 64);
+  const size_t head = kSharedHead + 32 * (size_t)(2 * w.W + 1);
   w.tab_bits = 0;
   size_t tab = 0;
-  if (hash) {  // the start layer is the largest level to expect
-    const double p = w.occ_bits ? 0.2 : (double)w.occ.T / 4294967296.0;
-    w.cap = (int)std::min<long long>(w.A, (long long)(1.2 * p * w.A) + 96);
-    w.tab_bits = ceil_log2(3 * w.cap / 2 + 1);
+  bool window = true;
+  if (!hash) {
+    // near the threshold levels are small after the first few and span up to 90
+    // tubes: a window of four rows before room for those few; else room for
+    // large levels, of a tube or two, and two rows
+    const int least = (int)std::min<long long>(w.A, l.threads == 32 ? 512 : 1200);
+    const bool small = 1.5 * level_sites(w) <= least;
+    auto with = [&](int n) { return head + 128 + 2 * sizeof(uint2) * (size_t)least + std::min(w.TW, n) * row_b; };
+    window = with(1) <= most;  // W <= 128
+    const size_t rows = head + 128 + std::min(w.TW, with(2) <= most ? 2 : window ? 1 : 0) * row_b;
+    const int room = most > rows ? (int)((most - rows) / (2 * sizeof(uint2))) : 0;
+    w.cap = std::min(w.cap, small && window ? least : std::max(least, room));
+  } else {
+    w.cap = std::min(w.A, w.cap + w.cap / 8 + 32);
+    w.tab_bits = ceil_log2(std::max(3 * w.cap / 2, (int)(4.0 * level_sites(w))) + 1);
     tab = (16ull << w.tab_bits) + 8 * (size_t)w.cap;
     if (w.L > 16384) return false;
   }
-  const size_t head = kSharedHead + 32 * (size_t)(2 * w.W + 1);
   const size_t fixed = head + 2 * sizeof(uint2) * (size_t)w.cap + tab + 64;
   // every word row in shared memory if they fit the target, else a power of
   // two of them
   auto fits = [&](int rows, size_t lim) { return fixed + (size_t)rows * row_b <= lim; };
-  if (fits(w.TW, target)) {
+  if (fits(w.TW, target) || (w.TW <= 2 && fits(w.TW, most))) {
     w.NR = w.TW; w.nr_mask = -1;
   } else {
     w.NR = 0;
-    for (int r = 1; r < w.TW && (fits(r, target) || (r <= 2 && fits(r, most))); r *= 2) w.NR = r;
+    for (int r = 1; window && r < w.TW && (fits(r, target) || (r <= 2 && fits(r, most))); r *= 2) w.NR = r;
     w.nr_mask = w.NR - 1;
     if (hash && w.NR < 2) return false;
   }
@@ -1079,7 +1108,7 @@ bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings) {
   w.a_occ = w.a_nu = (long long)off;
   w.ring_mask = -1;
   if (l.mode == M_PRE) off += up(sizeof(uint2) * (size_t)w.cap, 256);  // a queue between launches
-  if ((l.mode == M_HASH || l.mode == M_PLANES) && w.o_occ < 0) off += map_b;
+  if ((hash || l.mode == M_PLANES) && w.o_occ < 0) off += map_b;
   if (l.mode == M_PLANES) {
     w.a_nu = (long long)off;
     if (!full_rings && w.L > 128) w.ring_mask = 127;
@@ -1126,26 +1155,36 @@ pc_status resident_groups(const WaveLaunch& l, int nsm, int optin, long long* n)
 //  - Else the levels, then the masses of the percolating ones: in hash tables,
 //    by CTAs while these are few, by warps where more percolate than CTAs fit
 //    (a level then costs fewer instructions); or in rings of planes where a
-//    start layer does not fit the tables.
+//    start layer does not fit the tables, or levels are large: sixteen lanes a
+//    site cost most there (W = 24, L = 16, p = 0.95, 1,500 configurations:
+//    12,260 -> 2,410 us; L = 64, 4 configurations, 40 sites a level: 410 us in
+//    tables, 660 in planes).
 //  - Last, masses that did not fit (marked -1), with a plane for every layer.
 pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, int nsm, int optin, bool ahead,
                       long long at_once, std::vector<WaveLaunch>& out) {
+  const long long per_sm = (std::min(items, at_once) + nsm - 1) / nsm;
+  const size_t share = per_sm > 32 ? 0 : (size_t)optin / (size_t)per_sm - (per_sm > 1 ? 1024 : 64);
   auto make = [&](int mode, int t, bool full_rings, WaveLaunch& l) -> bool {
     l = WaveLaunch();
     l.mode = mode; l.threads = t; l.items = items; l.hard = mode == M_PLANES && full_rings;
     for (WaveQuery w : qs) {
-      if (!place(w, l, (size_t)optin - 64, full_rings)) return false;
+      if (!place(w, l, (size_t)optin / l.per_cta() - 64, full_rings, share)) return false;
       l.q.push_back(w);
     }
     return true;
   };
   bool some = false, all = true;
-  for (const WaveQuery& w : qs) { some = some || w.want_mass; all = all && w.want_mass; }
+  double sites = 0.0;
+  for (const WaveQuery& w : qs) {
+    some = some || w.want_mass;
+    all = all && w.want_mass;
+    sites = std::max(sites, level_sites(w));
+  }
   const int mt = std::max(threads, 128);
   WaveLaunch levels, hash, warps, planes;
   make(ahead ? M_PRE : M_LEVELS, threads, false, levels);
   if (!some) { out.push_back(levels); return PC_OK; }
-  const bool has_hash = make(M_HASH, mt, false, hash);
+  const bool has_hash = sites <= 3.0 * mt / 8 && make(M_HASH, mt, false, hash);
   bool left = true;  // something may be left to the last launch
   long long fit = 0;
   if (has_hash) {
@@ -1184,6 +1223,25 @@ pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int thr
 
 }  // namespace
 
+bool wave_is_slower(const Lattice& lat, const OccStream& occ, const uint32_t* occ_bits, long long n) {
+  // (the resident solver's masses depend on its CTA size in their last bits)
+  if (lat.A < 3000 || resident_fits(lat.W, lat.L)) return false;
+  int dev = 0, nsm = 1, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  WaveQuery w = {};
+  fill_lattice(w, lat);
+  w.occ = occ;
+  w.occ_bits = occ_bits;
+  WaveLaunch l;
+  l.threads = 512;
+  if (!place(w, l, (size_t)optin - 64, false, 0) || w.NR == 0) return true;
+  const double sites = level_sites(w), k = 152.0 * (double)n / nsm;
+  if (w.NR < std::min(w.TW, 2) || sites > 0.8 * w.cap || density(w) * w.A > 4.5 * w.cap) return sites > 760.0 + 20.0 * k;
+  return sites > 2600.0 + 60.0 * k;
+}
+
 void release_wave() {
   std::lock_guard<std::mutex> lk(g_fit_mu);
   g_fit.clear();
@@ -1206,7 +1264,7 @@ size_t wave_scratch_bytes(const Lattice& lat) {
     l.mode = mode; l.threads = 128;
     WaveQuery x = w;
     // (the smallest window any launch has: evicted rows counted)
-    if (place(x, l, 48 * 1024, true)) b = std::max(b, l.stride);
+    if (place(x, l, 48 * 1024, true, 0)) b = std::max(b, l.stride);
   }
   return b;
 }
@@ -1234,11 +1292,11 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
     for (int i : order) {
       const StreamQuery& s = qs[i];
       // (on a caller's memory a configuration is one CTA's)
-      if (std::max(group_threads(s.lat.A, n_all, nsm), m ? 128 : 32) != threads) continue;
       WaveQuery w = {};
       fill_lattice(w, s.lat);
       w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
       w.out = s.out;
+      if (std::max(group_threads(w, n_all, nsm), m ? 128 : 32) != threads) continue;
       w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
       w.item0 = items; w.n_cfg = s.n_cfg;
       items += s.n_cfg;

@@ -74,6 +74,19 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
 // Threads that work on one configuration of an A-column lattice when n_all
 // configurations are inspected together on the current device.
 int wave_threads(int A, long long n_all);
+// Whether the streamed and blocked solvers, which work on a configuration with
+// the whole device, are the faster ones for n configurations: each of this
+// solver's is one SM's, so that few of them with large levels leave the device
+// idle; and a cross-section beyond one SM's shared memory (W >= 129), or levels
+// beyond its queue, are walked in device memory.  Where the line lies, in sites
+// of a level (us of this solver / of the others): W = 64, L = 32, one
+// configuration, p = 0.3 (2,700 sites a level) 1,370 / 1,530, p = 0.4 (4,200)
+// 1,750 / 1,400, p = 0.95 4,690 / 1,240; 16 of them, p = 0.4 1,860 / 1,900, p =
+// 0.55 (6,300) 2,480 / 1,780; 64 of them, p = 0.75 as fast.  Beyond the queue:
+// W = 90, L = 128, verdicts, one configuration, p = 0.18 (930 sites) 1,900 /
+// 7,800, p = 0.21 (2,200) 12,000 / 5,140; W = 128, L = 512, p = 0.165 (820)
+// 127,000 / 57,100, 16 of them, L = 128, 19,900 / 18,300.
+bool wave_is_slower(const Lattice& lat, const OccStream& occ, const uint32_t* occ_bits, long long n);
 void release_wave();  // pc_shutdown
 
 }  // namespace pc

@@ -240,3 +240,34 @@ def test_calls_on_several_streams_and_threads():
         for g in got[i]:
             for key in ("verdict", "first_hit", "m_stop", "mass"):
                 assert np.array_equal(g[key], w[key]), (specs[i], key)
+
+
+@pytest.mark.parametrize("W,L,p,n", [
+    (52, 33, 0.9, 5), (64, 33, 0.5, 5),   # levels too large for few SMs
+    (64, 32, 0.24, 9), (64, 65, 0.18, 3),  # levels for which these are the faster ones
+    (90, 40, 0.25, 3),                    # a window of one row of two
+    (125, 9, 0.4, 3),                     # no window row in shared memory
+])
+def test_the_solver_does_not_show(W, L, p, n):
+    """A configuration's outputs are the same bits whatever solver a call takes:
+    alone, among many, forced, in a batch beside small queries, in a server."""
+    ref = pc.pc_inspect(W, L, p, 6, 0, n, mode=pc.PC_MODE_STREAM)
+    many = pc.pc_inspect(W, L, p, 6, 0, 160)
+    g = pc.pc_inspect(W, L, p, 6, 0, n)
+    one = pc.pc_inspect(W, L, p, 6, 1, 1)
+    v = pc.pc_inspect(W, L, p, 6, 0, n, verdict_first=True)
+    outs, res = pc.pc_batch_run([(3, 9, 0.4, 6, 0, 50), (W, L, p, 6, 0, n)])
+    assert res[1]["n_percolating"] == int(ref["verdict"].sum())
+    srv = pc.Server(hbm_budget_bytes=1 << 30, max_slots=16, max_slots_per_query=4)
+    try:
+        t = srv.submit((W, L, p, 6, 0, n))
+        served = srv.poll(t, 60.0)
+        for k in ("verdict", "first_hit", "m_stop", "mass"):
+            for what, o in (("many", many), ("default", g), ("verdict first", v), ("batch", outs[1]), ("server", served)):
+                assert np.array_equal(np.asarray(o[k])[:n], ref[k]), (what, k)
+            assert one[k][0] == ref[k][1], k
+    finally:
+        srv.close()
+    b = pc.pc_inspect(W, L, p, 6, 0, n, bits_only=True)
+    for k in ("verdict", "first_hit", "m_stop"):
+        assert np.array_equal(b[k], ref[k]), k
