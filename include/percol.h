@@ -225,7 +225,8 @@ pc_status pc_batch_run(const pc_query* queries, int64_t n_queries, pc_result* ou
  * device at pc_server_create).  Queries are admitted in arrival order as soon
  * as their HBM footprint -- output buffers, plus the state of max(1, min(slots
  * free, max_slots_per_query)) configurations when the lattice exceeds shared
- * memory (half of the free slots while other queries run or wait) -- fits the server's device arena of hbm_budget_bytes.  Each admitted
+ * memory (half of the free slots while other queries run or wait) -- fits the
+ * server's device arena of hbm_budget_bytes.  Each admitted
  * query is one run of the wavefront solver on a side stream, in its own
  * memory: as many configurations in work at once as it has slots, the next
  * ones taken on the device; queries run beside each other, and new ones are

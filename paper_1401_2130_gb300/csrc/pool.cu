@@ -15,7 +15,7 @@
 // free their own.  pc_shutdown gives everything back.
 #include <map>
 #include <mutex>
-#include <vector>
+#include <new>
 
 #include "pool.cuh"
 
@@ -29,7 +29,8 @@ constexpr size_t kBuffers = 8;
 
 std::mutex g_mu;
 std::map<int, cudaMemPool_t> g_pools;
-std::vector<char*> g_stage;
+char* g_stage[kBuffers];
+size_t g_stages = 0;
 
 }  // namespace
 
@@ -54,7 +55,12 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
       int no = 0;
       if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no);
       if (e != cudaSuccess) { cudaMemPoolDestroy(pool); return e; }
-      it = g_pools.emplace(dev, pool).first;
+      try {
+        it = g_pools.emplace(dev, pool).first;
+      } catch (const std::bad_alloc&) {
+        cudaMemPoolDestroy(pool);
+        return cudaErrorMemoryAllocation;
+      }
     }
     pool = it->second;
   }
@@ -65,9 +71,8 @@ HostStage::HostStage(size_t bytes) {
   if (bytes > kStageBytes) return;
   {
     std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_stage.empty()) {
-      p_ = g_stage.back();
-      g_stage.pop_back();
+    if (g_stages > 0) {
+      p_ = g_stage[--g_stages];
       return;
     }
   }
@@ -81,8 +86,8 @@ HostStage::~HostStage() {
   if (!p_) return;
   {
     std::lock_guard<std::mutex> lk(g_mu);
-    if (g_stage.size() < kBuffers) {
-      g_stage.push_back(p_);
+    if (g_stages < kBuffers) {
+      g_stage[g_stages++] = p_;
       return;
     }
   }
@@ -93,8 +98,7 @@ void release_pools() {
   std::lock_guard<std::mutex> lk(g_mu);
   for (auto& kv : g_pools) cudaMemPoolDestroy(kv.second);
   g_pools.clear();
-  for (char* p : g_stage) cudaFreeHost(p);
-  g_stage.clear();
+  while (g_stages > 0) cudaFreeHost(g_stage[--g_stages]);
   cudaGetLastError();  // after cudaDeviceReset the handles are gone already
 }
 

@@ -164,6 +164,8 @@ void finish_query(pc_server* s, Ticket& t, cudaStream_t st) {
     if (t.q.m_stop) std::memcpy(t.q.m_stop, h + 8 * n, 4 * (size_t)n);
     if (t.q.verdicts) std::memcpy(t.q.verdicts, h + 12 * n, (size_t)n);
   }
+  // (no CUDA call under s->mu, which the host callbacks take)
+  if (t.ev) { cudaEventDestroy(t.ev); t.ev = nullptr; }
   std::lock_guard<std::mutex> lk(s->mu);
   if (e != cudaSuccess) {
     t.state = T_FAILED;
@@ -189,7 +191,6 @@ void finish_query(pc_server* s, Ticket& t, cudaStream_t st) {
   s->arena.release(t.off_out, t.bytes_out);
   if (t.bytes_slots) s->arena.release(t.off_slots, t.bytes_slots);
   s->free_slots += t.nslots;
-  if (t.ev) { cudaEventDestroy(t.ev); t.ev = nullptr; }
   s->cv_done.notify_all();
 }
 
@@ -246,12 +247,12 @@ void worker_main(pc_server* s) {
       const pc_status rc = start_query(s, t);
       if (rc) {
         cudaStreamSynchronize(s->streams[t.stream_idx]);  // nothing of it runs on in memory given back
+        if (t.ev) { cudaEventDestroy(t.ev); t.ev = nullptr; }
         std::lock_guard<std::mutex> lk(s->mu);
         t.state = T_FAILED; t.status = rc;
         s->arena.release(t.off_out, t.bytes_out);
         if (t.bytes_slots) s->arena.release(t.off_slots, t.bytes_slots);
         s->free_slots += t.nslots;
-        if (t.ev) { cudaEventDestroy(t.ev); t.ev = nullptr; }
         s->cv_done.notify_all();
       } else {
         running.push_back(started[i]);

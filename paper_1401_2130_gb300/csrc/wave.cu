@@ -47,6 +47,7 @@
 #include <cstddef>
 #include <map>
 #include <mutex>
+#include <new>
 #include <tuple>
 #include <vector>
 
@@ -1269,7 +1270,7 @@ size_t wave_scratch_bytes(const Lattice& lat) {
   return b;
 }
 
-pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m, size_t limit) {
+pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m, size_t limit) try {
   int dev = 0, nsm = 0, optin = 0;
   PC_CUDA(cudaGetDevice(&dev));
   PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -1433,6 +1434,9 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   if (e != cudaSuccess) rc = cuda_fail(e, "wavefront solver");
   if (mem) cudaFreeAsync(mem, st);
   return rc;
+} catch (const std::bad_alloc&) {  // of the plan, before any device memory is taken
+  set_error("wavefront solver: no host memory for the plan");
+  return PC_ERR_OOM;
 }
 
 }  // namespace pc
