@@ -10,7 +10,11 @@ block of 8 configurations at each of the three p (three inspection calls);
 the steps cycle through the 8 blocks of the 64 configurations.  Metric:
 site-updates per second (every step m of the forward recursion sweeps the
 causal window of min(m+1, L) layers of A sites), roofline against the
-measured HBM copy bandwidth at 8.375 B per site-update.
+measured HBM copy bandwidth at 8.375 B per site-update.  The solver of these
+lines is forced (PC_MODE_STREAM, and PC_MODE_RESIDENT in the p-sweep): the
+default one updates each reached site once, so that a rate of site-updates
+would count work that it does not do; its configurations/s stand beside the
+value ("default_path").
 
 Other workloads: ``--workload psweep`` (W = 8, L = 64, p = 0.100 .. 0.200, 10^4
 configurations per p, seed 2, the shared-memory resident solver), ``batch``,
@@ -320,7 +324,7 @@ def solve_ticks(verdict, first_hit, m_stop) -> int:
 
 def run_large(args, pc, torch, rank, world, local, dist):
     """W = 64, L = 4096 (51.1 M sites), p in {0.14, 0.1533, 0.17}, 64
-    configurations each, seed 4: the streamed solver, HBM bound.  One step =
+    configurations each, seed 4: the streamed solver (forced), HBM bound.  One step =
     one block of configurations at each p; steps cycle through the blocks."""
     ps = list(LPS) if args.large_p is None else [float(v) for v in args.large_p.split(",")]
     n = args.large_configs
@@ -340,17 +344,17 @@ def run_large(args, pc, torch, rank, world, local, dist):
         return {"verdict": o["verdict"][sl], "first_hit": o["first_hit"][sl], "mass": o["mass"][sl],
                 "m_stop": o["m_stop"][sl], "n_percolating": nperc[b, i:i + 1]}
 
-    def step(b):
+    def step(b, mode=pc.PC_MODE_STREAM):
         for i, p in enumerate(ps):
             pc.pc_inspect(LW, LL, p, LSEED, base + b * block, block, device=True, out=block_out(i, p, b),
-                          stream=stream, bits_only=args.bits_only)
+                          stream=stream, bits_only=args.bits_only, mode=mode)
 
     # warm-up: one configuration per p, outside the timed configuration range
     wo = pc._alloc_outputs(1, True, pc.ALL_OUTPUTS)
     for w in range(args.warmup):
         for p in ps:
             pc.pc_inspect(LW, LL, p, LSEED, base + nb * block + w, 1, device=True, out=wo, stream=stream,
-                          bits_only=args.bits_only)
+                          bits_only=args.bits_only, mode=pc.PC_MODE_STREAM)
     torch.cuda.synchronize()
     times, blocks = [], []
     with Clocks(local) as clk:
@@ -411,7 +415,8 @@ def run_large(args, pc, torch, rank, world, local, dist):
     for k in range(e2e_steps):
         b = k % nb
         for p in ps:
-            r = pc.pc_inspect(LW, LL, p, LSEED, base + b * block, block, bits_only=args.bits_only)
+            r = pc.pc_inspect(LW, LL, p, LSEED, base + b * block, block, bits_only=args.bits_only,
+                              mode=pc.PC_MODE_STREAM)
             su_e2e += site_updates(LA, LL, r["verdict"], r["first_hit"], r["m_stop"])
     e2e_t = time.perf_counter() - t0
     if dist is not None:
@@ -421,6 +426,22 @@ def run_large(args, pc, torch, rank, world, local, dist):
         st_ = torch.tensor([float(su_e2e)], dtype=torch.float64, device="cuda")
         dist.all_reduce(st_, op=dist.ReduceOp.SUM)
         su_e2e = int(st_.item())
+
+    # the same step by the default path, which performs one update per reached
+    # site instead of one per site of the window and step: configurations/s
+    # only, after the outputs of the timed region were read
+    step(0, 0)
+    torch.cuda.synchronize()
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    e0.record(stream)
+    step(0, 0)
+    e1.record(stream)
+    torch.cuda.synchronize()
+    t_default = e0.elapsed_time(e1) / 1e3
+    first = slice(0, block)
+    same_default = 0 not in blocks or all(
+        np.array_equal(outs[p][k][first].cpu().numpy(), host[p][k][first])
+        for p in ps for k in ("verdict", "first_hit", "m_stop"))
 
     peaks = measured_peaks()
     hbm = peaks.get("hbm_gbs") or 6800.0
@@ -448,6 +469,10 @@ def run_large(args, pc, torch, rank, world, local, dist):
                    "parallelism": f"configs sharded over {world} GPU(s)",
                    "l2": "inputs larger than L2 (each configuration's state is ~0.5 GB), no flush"},
         "configs_per_s": block * len(ps) * world * len(times) / t_max,
+        "default_path": {"configs_per_s_per_gpu": block * len(ps) / t_default, "ms_per_step": t_default * 1e3,
+                         "results_identical": bool(same_default),
+                         "note": "the step without a forced solver (wavefront solver); no site-updates are claimed "
+                                 "for it"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                      "frac": achieved / hbm, "traffic": traffic,
                      "traffic_note": ("ncu DRAM bytes (read + write) per site-update of "
@@ -526,7 +551,7 @@ def large_cpu_leg(args, host, ps, block, seen):
 
 def run_batch(args, pc, torch):
     """28 (W, L) queries of the finite-size-scaling set, 10^4 configurations
-    each at p = 0.1533, seed 3: one batched submission (cached CUDA graph)
+    each at p = 0.1533, seed 3: one batched submission
     against 28 plain one-lattice-per-launch calls."""
     specs = batching_specs(args.batch_configs)
     stream = torch.cuda.current_stream()
@@ -568,7 +593,7 @@ def run_batch(args, pc, torch):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1)
         h = {k: v.cpu().numpy() for k, v in o.items()}
-        su_q = site_updates(3 * W_ * (W_ + 1) + 1, L_, h["verdict"], h["first_hit"], h["m_stop"])
+        su_q = site_updates(3 * W_ * (W_ + 1) + 1, L_, h["verdict"], h["first_hit"], h["m_stop"])  # the recursion's
         per_query_ms[f"{W_},{L_}"] = round(ms, 3)
         per_query_su_s[f"{W_},{L_}"] = float(f"{su_q / (ms / 1e3):.4g}")
     # a naive GPU path for contrast: one configuration per launch, on a
@@ -602,10 +627,10 @@ def run_batch(args, pc, torch):
                    "queries": len(specs), "configs_per_query": args.batch_configs,
                    "l2": "no flush (per-launch working sets differ; see plain)"},
         "plain_configs_per_s": n_tot / tp, "batched_over_plain": tp / tb,
-        "plain_ms_per_query": per_query_ms, "plain_site_updates_per_s": per_query_su_s,
+        "plain_ms_per_query": per_query_ms, "plain_recursion_site_updates_per_s": per_query_su_s,
         "one_config_per_launch": {"configs_per_s": n_tot / t_one, "batched_over": t_one / tb,
                                   "sample": f"first {n_one} configurations of each size, extrapolated"},
-        "site_updates_per_s_batched": su / tb, "results_identical": bool(same),
+        "recursion_site_updates_per_s_batched": su / tb, "results_identical": bool(same),
         "clocks": clk.summary(),
     }
 
@@ -749,7 +774,7 @@ def run_psweep(args, pc, torch, rank, world, local, dist):
             if evs is not None:
                 evs[i][0].record(stream)
             pc.pc_inspect(W, L, p, SEED, cfg0, n_cfg, device=True, out=outs[i], stream=stream,
-                          verdict_first=args.verdict_first)
+                          verdict_first=args.verdict_first, mode=pc.PC_MODE_RESIDENT)
             if evs is not None:
                 evs[i][1].record(stream)
 
@@ -804,7 +829,8 @@ def run_psweep(args, pc, torch, rank, world, local, dist):
     t0 = time.perf_counter()
     for _ in range(e2e_steps):
         for p in PS:
-            pc.pc_inspect(W, L, p, SEED, cfg0, n_cfg, device=False, verdict_first=args.verdict_first)
+            pc.pc_inspect(W, L, p, SEED, cfg0, n_cfg, device=False, verdict_first=args.verdict_first,
+                          mode=pc.PC_MODE_RESIDENT)
     e2e_t = (time.perf_counter() - t0) / e2e_steps
     if dist is not None:
         tt = torch.tensor([e2e_t], device="cuda")
