@@ -674,6 +674,10 @@ __device__ __forceinline__ void wave_body(const WaveArgs& a, unsigned char* sm, 
         // (warp-collective).  The claim is one atomicAnd per contact, issued
         // without a look at the word first: fourteen in flight, and the old
         // word says both whether the site was free and that this lane has it.
+        // (Fourteen loads first and claims of the set bits alone: fewer atomics,
+        // one more round of latency.  us per call without and with them: W =
+        // 64, L = 4096 17,489 and 22,956; W = 8, L = 64, 10^4 configurations 492
+        // and 519 in CTAs, 594 in warps as well.)
         auto expand = [&](bool act, uint32_t ent, int t) {
           const int pos = (int)(ent & kPosMask);
           const int sg = pos - 3 * (int)__umulhi((unsigned)pos, 0x55555556u);
