@@ -108,14 +108,9 @@ __global__ void __launch_bounds__(256) fc_hist_kernel(OccStream os, uint32_t cfg
   }
 }
 
-// One warp per configuration: descend into the bin holding the wanted rank.
-__global__ void fc_select_kernel(FcState* st, unsigned int* hist, int64_t n_cfg) {
-  const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (c >= n_cfg) return;
-  FcState s = st[c];
-  unsigned int* h = hist + c * 256;
-  if (s.resolved) return;  // warp-uniform
+// A warp descends into the bin holding the wanted rank and clears the
+// histogram h for the next digit.
+__device__ __forceinline__ void fc_descend(FcState& s, unsigned int* h, int lane) {
   unsigned int v[8], sum = 0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) { v[k] = h[lane * 8 + k]; sum += v[k]; }
@@ -142,17 +137,85 @@ __global__ void fc_select_kernel(FcState* st, unsigned int* hist, int64_t n_cfg)
   below = __shfl_sync(0xffffffffu, below, src);
   cnt = __shfl_sync(0xffffffffu, cnt, src);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) h[lane * 8 + k] = 0u;  // ready for the next pass
-  if (lane == 0) {
-    if (found < 0) {  // cannot happen: the ranks of the histogram cover rank
-      s.resolved = 2;
-    } else {
-      s.prefix = (s.shift < 64 ? (s.prefix << 8) : 0ull) | (uint64_t)found;
-      s.shift -= 8;
-      s.rank -= below;
-      if (cnt == 1 || s.shift == 0) s.resolved = 1;
+  for (int k = 0; k < 8; ++k) h[lane * 8 + k] = 0u;
+  if (found < 0) {  // cannot happen: the ranks of the histogram cover rank
+    s.resolved = 2;
+  } else {
+    s.prefix = (s.shift < 64 ? (s.prefix << 8) : 0ull) | (uint64_t)found;
+    s.shift -= 8;
+    s.rank -= below;
+    if (cnt == 1 || s.shift == 0) s.resolved = 1;
+  }
+}
+
+// One warp per configuration.
+__global__ void fc_select_kernel(FcState* st, unsigned int* hist, int64_t n_cfg) {
+  const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (c >= n_cfg) return;
+  FcState s = st[c];
+  if (s.resolved) return;  // warp-uniform
+  fc_descend(s, hist + c * 256, lane);
+  if (lane == 0) st[c] = s;
+}
+
+// The whole selection of a configuration whose words fit shared memory: a CTA
+// draws them once, counts the first digit on the way, descends digit by digit
+// over the stored words (two or three of the eight digits settle it: N keys
+// spread over 256 bins a digit) and writes the occupancy, a ballot per word.
+// What bounds it: the draw's integer instructions and one shared atomic a site;
+// HBM carries the N / 8 bytes written.  The kernels above, which draw the words
+// in every pass, remain for lattices beyond shared memory.
+// us per call, multi-launch kernels and this one (one fifth of the sites): W =
+// 8, L = 24, 4,000 configurations 220 and 104; W = 3, L = 7, 50,000 560 and 127;
+// W = 16, L = 64, 1,000 373 and 202; the largest that fit, W = 16, L = 70, one
+// configuration 109 and 66; one site, 100 configurations 119 and 42.
+__global__ void __launch_bounds__(1024) fc_shared_kernel(OccStream os, uint32_t cfg0, int64_t n_cfg, int N, int64_t wpc,
+                                                         int64_t n_metallic, uint32_t* __restrict__ out,
+                                                         int* __restrict__ error) {
+  extern __shared__ __align__(16) uint4 fc_words[];  // the configuration's words, four a block
+  __shared__ unsigned int h[256];
+  __shared__ FcState sh;
+  const int tid = threadIdx.x, size = blockDim.x, lane = tid & 31, nblk = (N + 3) / 4;
+  const uint32_t* u = reinterpret_cast<const uint32_t*>(fc_words);
+  for (int k = tid; k < 256; k += size) h[k] = 0u;
+  __syncthreads();
+  for (int64_t c = blockIdx.x; c < n_cfg; c += gridDim.x) {
+    const uint32_t cfg = cfg0 + (uint32_t)c;
+    for (int b = tid; b < nblk; b += size) {
+      const u32x4 r = philox4x32_10(u32x4{(uint32_t)b, cfg, os.wl, 0u}, os.k0, os.k1);
+      fc_words[b] = make_uint4(r.x, r.y, r.z, r.w);
+      atomicAdd(&h[r.x >> 24], 1u);
+      if (4 * b + 1 < N) atomicAdd(&h[r.y >> 24], 1u);
+      if (4 * b + 2 < N) atomicAdd(&h[r.z >> 24], 1u);
+      if (4 * b + 3 < N) atomicAdd(&h[r.w >> 24], 1u);
     }
-    st[c] = s;
+    FcState s;
+    s.prefix = 0; s.shift = 64; s.rank = n_metallic - 1; s.resolved = 0;
+    for (;;) {  // at most eight digits
+      __syncthreads();
+      if (tid < 32) {
+        fc_descend(s, h, lane);
+        if (lane == 0) sh = s;
+      }
+      __syncthreads();
+      s = sh;
+      if (s.resolved) break;  // block-uniform
+      const int dshift = s.shift - 8;
+      for (int i = tid; i < N; i += size) {
+        const uint64_t key = fc_key(u[i], i);
+        if ((key >> s.shift) == s.prefix) atomicAdd(&h[(key >> dshift) & 255u], 1u);
+      }
+    }
+    if (s.resolved != 1 && tid == 0) atomicOr(error, 1);  // the selection did not converge (never expected)
+    const int warps = size >> 5;
+    for (int w = tid >> 5; w < (int)wpc; w += warps) {
+      const int i = 32 * w + lane;
+      const bool metallic = s.resolved == 1 && i < N && (fc_key(u[min(i, N - 1)], i) >> s.shift) <= s.prefix;
+      const unsigned int word = __ballot_sync(0xffffffffu, metallic);
+      if (lane == 0) out[c * wpc + w] = word;
+    }
+    __syncthreads();  // the words, the histogram and sh are the next configuration's
   }
 }
 
@@ -196,6 +259,31 @@ pc_status launch_occupancy_fixed(const Lattice& lat, const OccStream& os, uint32
   int dev = 0, nsm = 0;
   PC_CUDA(cudaGetDevice(&dev));
   PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  int optin = 0;
+  PC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const int64_t words_b = 16 * ((lat.N + 3) / 4);
+  if (n_metallic > 0 && words_b <= optin - 2048) {
+    // threads: a few rounds of the draw for small lattices (eight CTAs or more
+    // an SM), an SM's all where one CTA fills its shared memory
+    const int threads = lat.N <= 1024 ? 64 : lat.N <= 8192 ? 256 : lat.N <= 24576 ? 512 : 1024;
+    int* error = nullptr;
+    PC_CUDA(scratch_alloc((void**)&error, 256, st));
+    cudaError_t e = cudaMemsetAsync(error, 0, 256, st);
+    // the same limit on every call: calls from several threads never lower it
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fc_shared_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 2048);
+    if (e == cudaSuccess) {
+      fc_shared_kernel<<<(unsigned)std::min<int64_t>(n_cfg, 1 << 20), threads, (size_t)words_b, st>>>(
+          os, cfg0, n_cfg, (int)lat.N, wpc, n_metallic, occ_bits, error);
+      e = cudaGetLastError();
+    }
+    int err = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, error, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFreeAsync(error, st);
+    if (e != cudaSuccess) return cuda_fail(e, "fixed-count kernel");
+    if (err) { set_error("fixed-count selection did not converge"); return PC_ERR_INTERNAL; }
+    return PC_OK;
+  }
   char* mem = nullptr;
   const size_t st_bytes = ((size_t)n_cfg * sizeof(FcState) + 255) & ~(size_t)255;
   const size_t bytes = st_bytes + (size_t)n_cfg * 256 * sizeof(unsigned int) + 256;
