@@ -55,7 +55,6 @@ struct Smem {
   int* roff;
   float* inv;       // [16]
   uint32_t* flags;  // [3]
-  float* redf;      // [32]
   long long* redi;  // [32]
   long long* scal;  // [4]
 };
@@ -94,31 +93,25 @@ __device__ inline Smem carve(unsigned char* base, int W, int A, int L, int P, in
   s.roff = (int*)take(sizeof(int) * 4 * (size_t)(2 * W + 1));
   s.inv = (float*)take(sizeof(float) * 16);
   s.flags = (uint32_t*)take(sizeof(uint32_t) * 4);
-  s.redf = (float*)take(sizeof(float) * 32);
+  take(sizeof(float) * 32);  // spare: which lattices fit does not change with it
   s.redi = (long long*)take(sizeof(long long) * 32);
   s.scal = (long long*)take(sizeof(long long) * 4);
   return s;
 }
 
-// Deterministic block reductions (fixed tree for a fixed block size).
-__device__ inline float block_sum_f(float v, float* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Sum of an end layer's values (plane: by position) in the order of the other
+// solvers -- lane l of one warp adds columns l, l + 32, .., then the lanes by
+// halves -- so that a configuration's mass depends neither on the CTA size nor
+// on the solver a call takes.  Valid in the first warp.
+__device__ inline float end_mass(const float* plane, const int32_t* ppos, int A) {
+  float sum = 0.f;
+  if (threadIdx.x < 32) {
+#pragma unroll 4
+    for (int c = threadIdx.x; c < A; c += 32) sum += plane[__ldg(ppos + c)];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float s = 0.f;
-  if (warp == 0) {
-    s = lane < nw ? red[lane] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[0] = s;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   }
-  __syncthreads();
-  s = red[0];
-  __syncthreads();
-  return s;
+  return sum;
 }
 
 __device__ inline long long block_sum_i(long long v, long long* red) {
@@ -360,9 +353,7 @@ __device__ __forceinline__ void solve_config(const ResidentArgs& Pa, const Query
       if (!no_fp) start_nu();
       else __syncthreads();
       if (L == 1) {
-        float part = 0.f;
-        for (int k = tid; k < P; k += T) part += sm.nu[0][2 * P + k];
-        mass = bits_only ? 0.f : block_sum_f(part, sm.redf);
+        mass = bits_only ? 0.f : end_mass(sm.nu[0] + 2 * P, lat.ppos, A);
         verdict = 1; fh = 1; mstop = 1;
       } else {
         for (int m = 1;; ++m) {
@@ -413,9 +404,7 @@ __device__ __forceinline__ void solve_config(const ResidentArgs& Pa, const Query
           const uint32_t f = sm.flags[m % 3];
           if (tid == 0) sm.flags[(m + 2) % 3] = 0u;
           if (f & kEnd) {
-            float part = 0.f;
-            for (int k = no_fp ? P : tid; k < P; k += T) part += dst[(size_t)(L + 1) * P + k];
-            mass = no_fp ? 0.f : block_sum_f(part, sm.redf);
+            mass = no_fp ? 0.f : end_mass(dst + (size_t)(L + 1) * P, lat.ppos, A);
             verdict = 1; fh = m + 1; mstop = m + 1;
             break;
           }
@@ -435,9 +424,7 @@ __device__ __forceinline__ void solve_config(const ResidentArgs& Pa, const Query
             __syncthreads();
           }
           const float* last = ((fh - 1) & 1) ? sm.nu[1] : sm.nu[0];
-          float part = 0.f;
-          for (int k = tid; k < P; k += T) part += last[(size_t)(L + 1) * P + k];
-          mass = block_sum_f(part, sm.redf);
+          mass = end_mass(last + (size_t)(L + 1) * P, lat.ppos, A);
         }
       }
     }
