@@ -1,8 +1,7 @@
 // api.cu -- the extern "C" entry points of libpercol (include/percol.h).
 //
-// Validates arguments, chooses the solver (shared-memory resident when the
-// configuration's state fits one CTA, streamed otherwise), allocates the
-// call's stream-ordered scratch and marshals host or device outputs.
+// Validates arguments, chooses the solver (route_of), allocates the call's
+// stream-ordered scratch and marshals host or device outputs.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -11,6 +10,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "pool.cuh"
+#include "route.h"
 #include "wave.cuh"
 
 namespace pc {
@@ -60,13 +60,32 @@ bool resident_fits(int W, int L) {
   return resident_smem(lat) <= (size_t)max_smem;
 }
 
-int resident_threads(int A, int L) {
-  // about one (strip, 16-layer chunk) item per thread; strips ~ A / 3
-  const long long items = ((long long)A / 3 + 1) * ((L + 15) / 16);
-  long long t = (items + 31) / 32 * 32;
-  if (t < 128) t = 128;
-  if (t > 640) t = 640;
-  return (int)t;
+int resident_threads(const Lattice& lat, long long n) {
+  int dev = 0, nsm = 1, sm_smem = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  return resident_cta(lat.A, lat.L, n, nsm, resident_smem(lat), (size_t)sm_smem);
+}
+
+pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStream_t st) {
+  ResidentArgs a;
+  a.lat = q.lat; a.occ = q.occ; a.occ_bits = q.occ_bits; a.words_per_cfg = q.words_per_cfg;
+  a.n_cfg = q.n_cfg; a.cfg0 = q.cfg0;
+  a.verdict = q.out.verdict; a.first_hit = q.out.first_hit; a.mass = q.out.mass; a.m_stop = q.out.m_stop;
+  a.n_perc = q.out.n_perc; a.work = work; a.prep_chunk = 8;
+  a.bits_only = q.bits_only;
+  a.verdict_first = q.verdict_first;
+  return launch_resident(a, resident_threads(q.lat, q.n_cfg), st);
+}
+
+Route route_of(const Lattice& lat, const OccStream& occ, long long n, bool bits_only) {
+  if (!resident_fits(lat.W, lat.L)) return wave_is_slower(lat, occ, nullptr, n) ? Route::kDevice : Route::kWave;
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const double p = (double)occ.T / 4294967296.0;
+  return !bits_only && p >= resident_from(lat.W, lat.A, lat.L, n, nsm) ? Route::kResident : Route::kWave;
 }
 
 namespace {
@@ -141,37 +160,34 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
     os.T = occ_bits ? 0 : threshold_of(p);
     const int64_t wpc = (lat.N + 31) / 32;
 
-    bool resident = resident_fits(W, L);
-    if (flags & PC_MODE_STREAM) resident = false;
-    if ((flags & PC_MODE_RESIDENT) && !resident) {
-      set_error("PC_MODE_RESIDENT: lattice state exceeds shared memory"); rc = PC_ERR_OOM; break;
-    }
-    if (!(flags & (PC_MODE_RESIDENT | PC_MODE_STREAM)) && !wave_is_slower(lat, os, occ_bits, n)) {
-      StreamQuery j;
-      j.lat = lat; j.occ = os; j.occ_bits = occ_bits; j.words_per_cfg = wpc;
-      j.n_cfg = n; j.cfg0 = (uint32_t)cfg0;
-      j.out.verdict = s.verdict; j.out.first_hit = s.first_hit; j.out.mass = s.mass;
-      j.out.m_stop = s.m_stop; j.out.n_perc = s.n_perc;
-      j.bits_only = (flags & PC_BITS_ONLY) ? 1 : 0;
-      rc = run_wave(&j, 1, st);
-    } else if (resident) {
+    const bool first = (flags & PC_VERDICT_FIRST) != 0;
+    StreamJob j;
+    j.lat = lat; j.occ = os; j.occ_bits = occ_bits; j.words_per_cfg = wpc;
+    j.n_cfg = n; j.cfg0 = (uint32_t)cfg0;
+    j.out.verdict = s.verdict; j.out.first_hit = s.first_hit; j.out.mass = s.mass;
+    j.out.m_stop = s.m_stop; j.out.n_perc = s.n_perc;
+    j.bits_only = (flags & PC_BITS_ONLY) ? 1 : 0;
+    j.verdict_first = first ? 1 : 0;
+    j.error_out = (int*)(s.work + 2);
+    if (flags & PC_MODE_RESIDENT) {
+      if (!resident_fits(W, L)) {
+        set_error("PC_MODE_RESIDENT: lattice state exceeds shared memory"); rc = PC_ERR_OOM; break;
+      }
       ResidentArgs a;
       a.lat = lat; a.occ = os; a.occ_bits = occ_bits; a.words_per_cfg = wpc;
       a.n_cfg = n; a.cfg0 = (uint32_t)cfg0;
       a.verdict = s.verdict; a.first_hit = s.first_hit; a.mass = s.mass; a.m_stop = s.m_stop;
       a.n_perc = s.n_perc; a.work = s.work; a.prep_chunk = 8;
-      a.bits_only = (flags & PC_BITS_ONLY) ? 1 : 0;
-      a.verdict_first = (flags & PC_VERDICT_FIRST) ? 1 : 0;
+      a.bits_only = j.bits_only;
+      a.verdict_first = first ? 1 : 0;
       rc = launch_resident(a, tuned_threads(lat, occ_bits ? 0.2 : p, seed, st), st);
     } else {
-      StreamJob j;
-      j.lat = lat; j.occ = os; j.occ_bits = occ_bits; j.words_per_cfg = wpc;
-      j.n_cfg = n; j.cfg0 = (uint32_t)cfg0;
-      j.out.verdict = s.verdict; j.out.first_hit = s.first_hit; j.out.mass = s.mass;
-      j.out.m_stop = s.m_stop; j.out.n_perc = s.n_perc;
-      j.bits_only = (flags & PC_BITS_ONLY) ? 1 : 0;
-      j.error_out = (int*)(s.work + 2);
-      rc = (!j.bits_only && (flags & PC_VERDICT_FIRST)) ? run_stream_verdict_first(j, st) : run_stream(j, st);
+      const Route route = (flags & PC_MODE_STREAM) ? Route::kDevice
+                          : occ_bits               ? (wave_is_slower(lat, os, occ_bits, n) ? Route::kDevice : Route::kWave)
+                                                   : route_of(lat, os, n, j.bits_only != 0);
+      if (route == Route::kWave) rc = run_wave(&j, 1, st);
+      else if (route == Route::kResident) rc = run_resident(j, s.work, st);
+      else rc = (!j.bits_only && first) ? run_stream_verdict_first(j, st) : run_stream(j, st);
     }
     if (rc) break;
     if (!dev_out) {

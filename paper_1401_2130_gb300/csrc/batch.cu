@@ -74,7 +74,7 @@ int tuned_threads(const Lattice& lat, double p, uint64_t seed, cudaStream_t st) 
   const std::tuple<int, int, int> key{lat.W, lat.L, p_bin(p)};
   auto it = g_tune.find(key);
   if (it != g_tune.end()) return it->second;
-  const int fallback = resident_threads(lat.A, lat.L);
+  const int fallback = resident_threads(lat, 2048);
   const int64_t n = 2048;
   char* mem = nullptr;
   if (scratch_alloc((void**)&mem, 64 + n * 13, st) != cudaSuccess) return fallback;

@@ -35,8 +35,8 @@ struct ResidentArgs {
 constexpr int kResidentMaxThreads = 640;  // resident CTA size limit: 20 warps at <= 96 registers
 size_t resident_smem(const Lattice& lat);
 pc_status launch_resident(const ResidentArgs& args, int threads, cudaStream_t st);
-// default CTA size of the resident solver (about 16 tube layers per thread)
-int resident_threads(int A, int L);
+// CTA size of the resident solver for n configurations (route.h)
+int resident_threads(const Lattice& lat, long long n);
 // CTA size picked by the autotuner for (W, L, p bin) (batch.cu); times
 // candidates on a miss, outside any stream capture
 int tuned_threads(const Lattice& lat, double p, uint64_t seed, cudaStream_t st);
@@ -53,10 +53,17 @@ struct StreamQuery {
   uint32_t cfg0;
   Outputs out;
   int bits_only = 0;  // reached set only: no FP units, mass written 0
+  int verdict_first = 0;  // the caller asks for verdicts first (a hint: the outputs are the same)
   // device list of n_cfg configurations (indices from 0 within the query) to
   // solve, outputs written at those indices; null = configurations 0..n_cfg-1
   const int64_t* sel = nullptr;
 };
+// q on the resident solver, in CTAs of resident_threads; work: a zeroed counter.
+pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStream_t st);
+// The solver that a call without a PC_MODE flag takes for n configurations of
+// occupancy stream occ.
+enum class Route { kWave, kResident, kDevice };  // one SM a configuration, .., the whole device (stream.cu, blocked.cu)
+Route route_of(const Lattice& lat, const OccStream& occ, long long n, bool bits_only);
 struct StreamJob : StreamQuery {
   int* error_out = nullptr;  // device int: 1 if the tick bound was hit
   char* pool = nullptr;      // the caller's memory for the slots (else allocated)

@@ -466,9 +466,13 @@ static pc_status resident_config(const ResidentArgs& args, int threads, void** f
     return PC_ERR_ARG;
   }
   *smem = resident_smem(args.lat);
-  PC_CUDA(cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem));
-  int dev = 0, nsm = 0, per_sm = 0;
+  int dev = 0, nsm = 0, per_sm = 0, optin = 0;
   PC_CUDA(cudaGetDevice(&dev));
+  PC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  // the same limit on every call: calls from several threads never lower it
+  cudaFuncAttributes fa;
+  PC_CUDA(cudaFuncGetAttributes(&fa, resident_kernel));
+  PC_CUDA(cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes));
   PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_kernel, threads, *smem));
   if (per_sm < 1) {

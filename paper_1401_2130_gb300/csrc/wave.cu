@@ -1183,7 +1183,8 @@ pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int thr
   for (const WaveQuery& w : qs) {
     some = some || w.want_mass;
     all = all && w.want_mass;
-    sites = std::max(sites, level_sites(w));
+    // in a short fibre the start layer is one of few levels
+    sites = std::max({sites, level_sites(w), density(w) * w.A / w.L});
   }
   const int mt = std::max(threads, 128);
   WaveLaunch levels, hash, warps, planes;

@@ -39,3 +39,25 @@ def test_masses_of_the_solvers_are_the_same_bits(W, L, p, n):
     for first in (False, True):
         _equal(pc.pc_inspect(W, L, p, 31, 7, n, mode=pc.PC_MODE_RESIDENT, verdict_first=first), ref, ("resident", first))
         _equal(pc.pc_inspect(W, L, p, 31, 7, n, verdict_first=first), ref, ("default", first))
+
+
+@pytest.mark.parametrize("W,L,ps,n", [
+    (8, 8, (0.45, 0.7), 4000), (14, 14, (0.2, 0.4, 0.95), 1), (3, 18, (0.15, 0.3), 20), (6, 2, (0.1, 0.3), 900),
+    (20, 6, (0.6, 1.0), 500), (2, 5, (0.0, 1.0), 30), (25, 1, (0.15, 0.3), 700),
+])
+def test_default_calls_on_both_sides_of_the_line(W, L, ps, n):
+    """pc_inspect without a mode: the densities lie on both sides of the one
+    from which the resident solver takes the call."""
+    import torch
+    for p in ps:
+        ref = pc.pc_inspect(W, L, p, 12, 3, n, mode=pc.PC_MODE_STREAM)
+        g = pc.pc_inspect(W, L, p, 12, 3, n)
+        _equal(g, ref, p)
+        assert g["n_percolating"] == ref["n_percolating"]
+        d = pc.pc_inspect(W, L, p, 12, 3, n, device=True, verdict_first=True)
+        torch.cuda.synchronize()
+        assert int(d.pop("n_percolating")[0]) == ref["n_percolating"]
+        _equal({k: v.cpu().numpy() for k, v in d.items()}, ref, (p, "device"))
+        b = pc.pc_inspect(W, L, p, 12, 3, n, bits_only=True)
+        _equal(dict(b, mass=ref["mass"]), ref, (p, "verdicts"))
+        assert not b["mass"].any()
