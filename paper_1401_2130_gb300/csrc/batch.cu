@@ -196,6 +196,7 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
       s.occ_bits = nullptr; s.words_per_cfg = (s.lat.N + 31) / 32;
       s.n_cfg = q[i].n_configs; s.cfg0 = (uint32_t)q[i].config_begin;
       s.bits_only = (flags & PC_BITS_ONLY) ? 1 : 0;
+      s.verdict_first = (flags & PC_VERDICT_FIRST) ? 1 : 0;
       s.out.n_perc = counts + i;
       if (dev_out) {
         s.out.verdict = q[i].verdicts; s.out.first_hit = q[i].first_hit;

@@ -54,6 +54,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "pool.cuh"
+#include "route.h"
 #include "wave.cuh"
 
 namespace pc {
@@ -1156,7 +1157,8 @@ pc_status resident_groups(const WaveLaunch& l, int nsm, int optin, long long* n)
 //  - Verdicts only: the levels.
 //  - Masses too, and every configuration resident at once: levels and masses in
 //    one pass (the longest configuration's chain of levels is the time, and it
-//    usually percolates).
+//    usually percolates).  Not where the caller asks for verdicts first and
+//    hardly one is expected to percolate (`few`).
 //  - Else the levels, then the masses of the percolating ones: in hash tables,
 //    by CTAs while these are few, by warps where more percolate than CTAs fit
 //    (a level then costs fewer instructions); or in rings of planes where a
@@ -1166,7 +1168,7 @@ pc_status resident_groups(const WaveLaunch& l, int nsm, int optin, long long* n)
 //    tables, 660 in planes).
 //  - Last, masses that did not fit (marked -1), with a plane for every layer.
 pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, int nsm, int optin, bool ahead,
-                      long long at_once, std::vector<WaveLaunch>& out) {
+                      bool few, long long at_once, std::vector<WaveLaunch>& out) {
   const long long per_sm = (std::min(items, at_once) + nsm - 1) / nsm;
   const size_t share = per_sm > 32 ? 0 : (size_t)optin / (size_t)per_sm - (per_sm > 1 ? 1024 : 64);
   auto make = [&](int mode, int t, bool full_rings, WaveLaunch& l) -> bool {
@@ -1199,7 +1201,7 @@ pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int thr
   }
   bool full = false;
   const bool has_warps = threads == 32 && make(M_HASH, 32, false, warps);
-  if (all && !ahead && has_hash && items <= std::min(fit, at_once)) {
+  if (all && !ahead && !few && has_hash && items <= std::min(fit, at_once)) {
     full = true;
     hash.full = true;
     out.push_back(hash);
@@ -1295,6 +1297,7 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   for (int threads : {512, 256, 128, 32}) {
     std::vector<WaveQuery> cq;
     long long items = 0;
+    bool few = true;  // most configurations are not expected to percolate, and the caller says so
     for (int i : order) {
       const StreamQuery& s = qs[i];
       // (on a caller's memory a configuration is one CTA's)
@@ -1304,6 +1307,7 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
       w.out = s.out;
       if (std::max(group_threads(w, n_all, nsm), m ? 128 : 32) != threads) continue;
       w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
+      few = few && s.verdict_first && !s.occ_bits && few_percolate(w.W, w.L, density(w), s.n_cfg);
       w.item0 = items; w.n_cfg = s.n_cfg;
       items += s.n_cfg;
       cq.push_back(w);
@@ -1321,7 +1325,7 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
     }
     ahead = ahead && maps * (size_t)items <= (2ull << 30);
     const size_t first = ls.size();
-    const pc_status rc = launches_of(cq, items, threads, nsm, optin, ahead, m ? m->max_groups : items, ls);
+    const pc_status rc = launches_of(cq, items, threads, nsm, optin, ahead, few, m ? m->max_groups : items, ls);
     if (rc) return rc;
     for (size_t k = first; k < ls.size(); ++k) ls[k].cls = classes - 1;
   }

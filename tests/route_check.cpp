@@ -43,6 +43,16 @@ int main() {
         }
       }
     }
+  // near the threshold law's own points: wider fibres percolate earlier
+  if (!(fibre_threshold(8, 48) > 0.19 && fibre_threshold(16, 48) < fibre_threshold(4, 48) && fibre_threshold(20, 20) < 0.19)) {
+    std::printf("threshold\n");
+    return 1;
+  }
+  if (!few_percolate(8, 48, 0.18, 100) || few_percolate(8, 48, 0.2, 100) || few_percolate(20, 301, 0.172, 500) ||
+      few_percolate(4, 12, 0.16, 300) || !few_percolate(6, 36, 0.19, 200)) {
+    std::printf("few\n");
+    return 1;
+  }
   std::printf("ok\n");
   return 0;
 }

@@ -61,3 +61,14 @@ def test_default_calls_on_both_sides_of_the_line(W, L, ps, n):
         b = pc.pc_inspect(W, L, p, 12, 3, n, bits_only=True)
         _equal(dict(b, mass=ref["mass"]), ref, (p, "verdicts"))
         assert not b["mass"].any()
+
+
+@pytest.mark.parametrize("W,L,p,n", [(8, 48, 0.18, 100), (6, 36, 0.19, 200), (4, 48, 0.24, 700), (10, 40, 0.185, 16),
+                                     (12, 24, 0.15, 100)])
+def test_verdicts_first_below_the_threshold(W, L, p, n):
+    """Levels of all configurations and then the masses of the few that
+    percolate, where both would go in one pass without the flag."""
+    g = pc.pc_inspect(W, L, p, 3, 0, n)
+    _equal(pc.pc_inspect(W, L, p, 3, 0, n, verdict_first=True), g, "call")
+    outs, _ = pc.pc_batch_run([(W, L, p, 3, 0, n), (W, L, p, 4, 0, n)], verdict_first=True)
+    _equal(outs[0], g, "batch")
