@@ -9,8 +9,14 @@
 // them: every piece of device scratch it needs -- the work and percolation
 // counters, the lattice tables of the requested W, the wavefront solver's
 // scratch and the device staging of the per-configuration outputs -- lives in
-// one file-scope static device array, g_static_scratch, of kStaticBytes bytes.  Every GPU that loads the
-// library holds that array until the process exits.
+// one file-scope static device array, g_static_scratch, of kStaticBytes bytes.
+// Every GPU that loads the library holds that array until the process exits.
+//
+// Solvers: the resident one, which needs no scratch, unless the wavefront
+// solver is the faster one (route_of) and has room in the array for as many
+// configurations at once as the device takes.  (Masses in device planes with a
+// few dozen configurations in work: W = 16, L = 16, p = 0.95, 10,000
+// configurations 93,700 us, on the resident solver 6,800.)
 //
 // Limits: the lattice must fit the resident (shared-memory) solver and have
 // at most kStaticMaxColumns columns; at most kStaticMaxConfigs configurations
@@ -33,6 +39,7 @@
 // one CTA's shared memory (227 KB on GB300), which bounds the lattice long
 // before the tables do: W <= 26 (at L = 1), W = 20 up to L = 8, W = 8 up to
 // L = 74.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -55,12 +62,16 @@ constexpr size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t kPposBytes = up256(sizeof(int32_t) * (kStaticMaxColumns + 4));  // read in fours
 constexpr size_t kRoffBytes = up256(sizeof(int32_t) * 4 * kStaticMaxRows);
 constexpr size_t kSrowBytes = up256(sizeof(int16_t) * kStaticMaxStrips);
+constexpr size_t kPcolBytes = up256(sizeof(int32_t) * kStaticMaxP);
+constexpr size_t kNbrBytes = up256(sizeof(int32_t) * kStaticMaxColumns * kLateral);
+constexpr size_t kSigBytes = up256(kStaticMaxColumns);
 // scratch of the configurations in work (the solver takes as many as it holds;
 // a resident-size lattice needs at most 232 KB for one)
 constexpr size_t kWaveBytes = 4u << 20;
 constexpr size_t kCtrBytes = 256;
 constexpr size_t kOutBytes = up256((size_t)kStaticMaxConfigs * (1 + 4 + 4 + 4));
-constexpr size_t kStaticBytes = kPposBytes + kRoffBytes + kSrowBytes + kWaveBytes + kCtrBytes + kOutBytes;
+constexpr size_t kStaticBytes = kPposBytes + kRoffBytes + kSrowBytes + kPcolBytes + kNbrBytes + kSigBytes + kWaveBytes +
+                                kCtrBytes + kOutBytes;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
@@ -96,9 +107,12 @@ struct LayoutRows {
 };
 
 // Tables of the compact layout (the same content as the host-built cache):
-// position of each column, row of each strip, row offsets; zeroed counters.
-__global__ void static_tables_kernel(const __grid_constant__ LayoutRows l, int A, int32_t* ppos, int16_t* strip_row,
-                                     int32_t* row_off, unsigned long long* ctr) {
+// position of each column, row of each strip, row offsets; for the resident
+// solver (pcol not null) also the column at each position and each column's
+// sublattice and neighbours.  Zeroed counters.
+__global__ void static_tables_kernel(const __grid_constant__ LayoutRows l, int A, int P, int32_t* ppos, int16_t* strip_row,
+                                     int32_t* row_off, int32_t* pcol, int8_t* sigma, int32_t* nbr,
+                                     unsigned long long* ctr) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x, W = l.W, nr = 2 * W + 1;
   if (k < (int)(kCtrBytes / 8)) ctr[k] = 0ull;
   if (k < 4 * nr) row_off[k] = l.off[k];
@@ -114,6 +128,23 @@ __global__ void static_tables_kernel(const __grid_constant__ LayoutRows l, int A
       if (before(mid) <= k) lo = mid; else hi = mid - 1;
     }
     ppos[k] = l.start[lo] + (k - before(lo));
+    if (pcol) {
+      const int r = lo - W, q = (r < 0 ? -W - r : -W) + (k - before(lo));
+      sigma[k] = (int8_t)(((q - r) % 3 + 3) % 3);
+      for (int d = 0; d < kLateral; ++d) {
+        const int qq = q + dir_dq(d), rr = r + dir_dr(d), qlo = rr < 0 ? -W - rr : -W, qhi = rr < 0 ? W : W - rr;
+        nbr[k * kLateral + d] = rr >= -W && rr <= W && qq >= qlo && qq <= qhi ? before(rr + W) + (qq - qlo) : A;
+      }
+    }
+  }
+  if (pcol && k < P) {
+    int lo = 0, hi = nr - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (l.start[mid] <= k) lo = mid; else hi = mid - 1;
+    }
+    const int j = k - l.start[lo];
+    pcol[k] = j >= 0 && j < before(lo + 1) - before(lo) ? before(lo) + j : -1;
   }
   if (k < l.n_strips) {  // the row holding one of the strip's positions, else the row before it
     const int p2 = 3 * (l.s_begin + k) + 2;
@@ -182,6 +213,9 @@ extern "C" pc_status pc_inspect_static(int32_t W, int32_t L, double p, uint64_t 
   int32_t* d_ppos = (int32_t*)at; at += kPposBytes;
   int32_t* d_roff = (int32_t*)at; at += kRoffBytes;
   int16_t* d_srow = (int16_t*)at; at += kSrowBytes;
+  int32_t* d_pcol = (int32_t*)at; at += kPcolBytes;
+  int32_t* d_nbr = (int32_t*)at; at += kNbrBytes;
+  int8_t* d_sig = (int8_t*)at; at += kSigBytes;
   char* d_wave = (char*)at; at += kWaveBytes;
   unsigned long long* ctr = (unsigned long long*)at;  // then the outputs, in a row
   unsigned char* o = at + kCtrBytes;
@@ -200,21 +234,24 @@ extern "C" pc_status pc_inspect_static(int32_t W, int32_t L, double p, uint64_t 
       c += 2 * W + 1 - (i < W ? W - i : i - W);
     }
   }
-  static_tables_kernel<<<(A + 127) / 128 + 4, 128, 0, st>>>(rows, A, d_ppos, d_srow, d_roff, ctr);
-  PC_CUDA(cudaGetLastError());
-
   q.lat = Lattice{};
   q.lat.W = W; q.lat.L = L; q.lat.A = A; q.lat.N = (int64_t)A * L; q.lat.S = A + 1;
   q.lat.TW = (L + 31) / 32; q.lat.TWP = q.lat.TW + 2;
   q.lat.P = P; q.lat.s_begin = s_begin; q.lat.n_strips = n_strips;
-  q.lat.strip_row = d_srow; q.lat.row_off = d_roff; q.lat.ppos = d_ppos;
+  q.lat.strip_row = d_srow; q.lat.row_off = d_roff; q.lat.ppos = d_ppos; q.lat.pcol = d_pcol;
+  q.lat.nbr = d_nbr; q.lat.sigma = d_sig;
   q.occ.k0 = (uint32_t)(seed & 0xffffffffu); q.occ.k1 = (uint32_t)(seed >> 32);
   q.occ.cfg = 0; q.occ.wl = (uint32_t)W | ((uint32_t)L << 8); q.occ.T = threshold_of(p);
   q.occ_bits = nullptr; q.words_per_cfg = (q.lat.N + 31) / 32;
   q.n_cfg = n_configs; q.cfg0 = (uint32_t)config_begin;
   WaveMemory m;
   m.ctr = ctr + 8; m.scratch = d_wave; m.bytes = kWaveBytes; m.max_groups = n_configs;
-  if ((rc = run_wave(&q, 1, st, &m))) return rc;
+  const bool wave = route_of(q.lat, q.occ, n_configs, false) == Route::kWave && wave_memory_suffices(q, m);
+  static_tables_kernel<<<(std::max(A, P) + 127) / 128 + 4, 128, 0, st>>>(rows, A, P, d_ppos, d_srow, d_roff,
+                                                                         wave ? nullptr : d_pcol, d_sig, d_nbr, ctr);
+  PC_CUDA(cudaGetLastError());
+  rc = wave ? run_wave(&q, 1, st, &m) : run_resident(q, ctr + 8, st);
+  if (rc) return rc;
 
   const size_t all = kCtrBytes + 13 * n;
   HostStage stage(all);  // pinned host memory, kept after the first call

@@ -1250,6 +1250,30 @@ bool wave_is_slower(const Lattice& lat, const OccStream& occ, const uint32_t* oc
   return sites > 2600.0 + 60.0 * k;
 }
 
+bool wave_memory_suffices(const StreamQuery& s, const WaveMemory& m) try {
+  int dev = 0, nsm = 1, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  WaveQuery w = {};
+  fill_lattice(w, s.lat);
+  w.occ = s.occ; w.occ_bits = s.occ_bits;
+  w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
+  w.n_cfg = s.n_cfg;
+  const int threads = std::max(group_threads(w, std::min<long long>(s.n_cfg, m.max_groups), nsm), 128);
+  std::vector<WaveLaunch> ls;
+  if (launches_of({w}, s.n_cfg, threads, nsm, optin, false, false, m.max_groups, ls)) return false;
+  for (const WaveLaunch& l : ls) {
+    long long fit = 0;
+    if (l.hard) continue;
+    if (resident_groups(l, nsm, optin, &fit)) return false;
+    if (3 * (m.bytes / l.stride) < (size_t)std::min(fit, l.items)) return false;
+  }
+  return true;
+} catch (const std::bad_alloc&) {
+  return false;
+}
+
 void release_wave() {
   std::lock_guard<std::mutex> lk(g_fit_mu);
   g_fit.clear();

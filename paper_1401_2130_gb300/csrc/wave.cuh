@@ -65,6 +65,9 @@ struct WaveMemory {
 };
 // Scratch of one configuration in work on a WaveMemory.
 size_t wave_scratch_bytes(const Lattice& lat);
+// Whether m holds at least a third of the groups that the device would take at
+// once (fewer leave SMs idle).
+bool wave_memory_suffices(const StreamQuery& q, const WaveMemory& m);
 
 // Inspects the queries (stream-ordered, no host synchronisation).  Without m
 // the scratch is allocated on st, at most `limit` bytes where that is enough
