@@ -27,7 +27,7 @@ namespace pc {
 inline double resident_from(int W, int A, int L, long long n, int nsm) {
   if (L > 16 * W + 12 && (W == 0 || n > nsm)) return 1e9;  // at no density
   const double q = std::min(std::max((double)n / nsm, 1.0), 60.0);
-  return 0.018 * std::pow((double)L, 0.58) * std::pow((double)A, 0.19) * std::pow(q, 0.29);
+  return 0.0055 * std::pow((double)L, 0.7) * std::pow((double)A, 0.32) * std::pow(q, 0.4);
 }
 
 // CTA size of the resident solver for n configurations of a lattice whose
