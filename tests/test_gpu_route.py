@@ -72,3 +72,16 @@ def test_verdicts_first_below_the_threshold(W, L, p, n):
     _equal(pc.pc_inspect(W, L, p, 3, 0, n, verdict_first=True), g, "call")
     outs, _ = pc.pc_batch_run([(W, L, p, 3, 0, n), (W, L, p, 4, 0, n)], verdict_first=True)
     _equal(outs[0], g, "batch")
+
+
+@pytest.mark.parametrize("W,L,p,n", [(16, 40, 0.4, 300), (20, 33, 0.95, 60), (24, 150, 0.6, 20), (30, 9, 0.8, 200)])
+def test_dense_calls_in_one_pass(W, L, p, n):
+    """Lattices beyond shared memory with large levels that nearly all
+    percolate: levels and masses together, in planes of all layers (L <= 128)
+    or in rings of them."""
+    ref = pc.pc_inspect(W, L, p, 8, 1, n, mode=pc.PC_MODE_STREAM)
+    assert ref["verdict"].all()
+    _equal(pc.pc_inspect(W, L, p, 8, 1, n), ref, "call")
+    outs, _ = pc.pc_batch_run([(W, L, p, 8, 1, n), (W, L, 0.0, 8, 1, 3), (W, L + 1, p, 8, 1, 2)])
+    _equal(outs[0], ref, "batch")
+    assert not outs[1]["verdict"].any() and not outs[1]["mass"].any()
