@@ -2,6 +2,7 @@
 //
 // Validates arguments, chooses the solver (route_of), allocates the call's
 // stream-ordered scratch and marshals host or device outputs.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -76,11 +77,12 @@ pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStrea
   a.n_perc = q.out.n_perc; a.work = work; a.prep_chunk = 8;
   a.bits_only = q.bits_only;
   a.verdict_first = q.verdict_first;
+  a.gate = q.gate;
   return launch_resident(a, resident_threads(q.lat, q.n_cfg), st);
 }
 
 Route route_of(const Lattice& lat, const OccStream& occ, long long n, bool bits_only) {
-  if (!resident_fits(lat.W, lat.L)) return wave_is_slower(lat, occ, nullptr, n) ? Route::kDevice : Route::kWave;
+  if (!resident_fits(lat.W, lat.L)) return wave_is_slower(lat, (double)occ.T / 4294967296.0, n, bits_only) ? Route::kDevice : Route::kWave;
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -89,6 +91,61 @@ Route route_of(const Lattice& lat, const OccStream& occ, long long n, bool bits_
 }
 
 namespace {
+
+// Caller occupancies.  The host does not know how dense they are, and waiting
+// for the answer would make an asynchronous call wait for its stream: a sample
+// on the device opens the launches that are for its density and closes the
+// others (each an empty launch, about 2 us).  Sparse: the wavefront solver,
+// queues and tables sized for up to a quarter of the sites.  Denser: sized for
+// all of them (near 0.2 that costs occupancy).  Denser still: the solver that
+// route_of gives such a stream.  Verdicts first: masses in a pass of their own.  ctr: counters of the call, zeroed; ctr[0] is
+// the resident solver's, ctr[3] takes the sample.
+// us per call, all launches sized for a density of 0.2 and now: W = 8, L = 48,
+// p = 0.7, 16 configurations 1,664 and 221; W = 64, L = 128, p = 0.95, verdicts
+// of one 6,218 and 598.
+pc_status inspect_bits(StreamJob j, unsigned long long* ctr, cudaStream_t st) {
+  constexpr double kSparse = 0.25;
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const Lattice& lat = j.lat;
+  const bool res = resident_fits(lat.W, lat.L);
+  double top = 2.0;  // density from which the resident, or the device-wide, solver takes over
+  if (res) {
+    if (!j.bits_only) top = resident_from(lat.W, lat.A, lat.L, j.n_cfg, nsm);
+    if (top <= 0.15) return run_resident(j, ctr, st);
+  } else {
+    if (wave_is_slower(lat, 0.2, j.n_cfg, j.bits_only != 0)) return run_stream(j, st);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    // (a small lattice is done before the device-wide solvers' graph is built)
+    if (lat.N >= 100000 && capture == cudaStreamCaptureStatusNone)
+      for (int d = 5; d <= 20 && top > 1.0; ++d)
+        if (wave_is_slower(lat, 0.05 * d, j.n_cfg, j.bits_only != 0)) top = 0.05 * d;
+  }
+  j.gate.at = (const unsigned*)(ctr + 3);
+  pc_status rc = launch_bits_density(lat, j.occ_bits, j.words_per_cfg, j.n_cfg, (unsigned*)(ctr + 3), st);
+  if (rc) return rc;
+  auto between = [&](double lo, double hi, double density, double most) {
+    j.gate.lo = (unsigned)(lo * 65536.0); j.gate.hi = hi > 1.0 ? ~0u : (unsigned)(hi * 65536.0);
+    j.density = density; j.density_most = most;
+  };
+  // (what is sized for a quarter of few columns holds all of them)
+  const double split = top <= 0.5 && 1.1 * kSparse * lat.A + 64 >= lat.A ? top : std::min(kSparse, top);
+  between(0.0, split, 0.2, kSparse);
+  if ((rc = run_wave(&j, 1, st))) return rc;
+  if (top <= 1.0) {
+    between(top, 2.0, 0.6, 1.0);
+    rc = res ? run_resident(j, ctr, st) : run_stream(j, st);
+    if (rc == PC_ERR_OOM && !res) { top = 2.0; rc = PC_OK; }  // no memory for it: the wavefront solver needs less
+    if (rc) return rc;
+  }
+  if (top > split) {
+    between(split, top, 0.6, 1.0);
+    rc = run_wave(&j, 1, st);
+  }
+  return rc;
+}
 
 struct Scratch {
   unsigned long long* work = nullptr;
@@ -182,10 +239,9 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
       a.verdict_first = first ? 1 : 0;
       rc = launch_resident(a, tuned_threads(lat, occ_bits ? 0.2 : p, seed, st), st);
     } else {
-      const Route route = (flags & PC_MODE_STREAM) ? Route::kDevice
-                          : occ_bits               ? (wave_is_slower(lat, os, occ_bits, n) ? Route::kDevice : Route::kWave)
-                                                   : route_of(lat, os, n, j.bits_only != 0);
-      if (route == Route::kWave) rc = run_wave(&j, 1, st);
+      const Route route = (flags & PC_MODE_STREAM) ? Route::kDevice : route_of(lat, os, n, j.bits_only != 0);
+      if (occ_bits && !(flags & PC_MODE_STREAM)) rc = inspect_bits(j, s.work, st);
+      else if (route == Route::kWave) rc = run_wave(&j, 1, st);
       else if (route == Route::kResident) rc = run_resident(j, s.work, st);
       else rc = (!j.bits_only && first) ? run_stream_verdict_first(j, st) : run_stream(j, st);
     }

@@ -207,7 +207,7 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
         stage += (n * 13 + 255) & ~(size_t)255;
       }
       n_all += s.n_cfg;
-      if (wave_is_slower(s.lat, s.occ, nullptr, s.n_cfg)) {
+      if (wave_is_slower(s.lat, q[i].p, s.n_cfg, s.bits_only != 0)) {
         StreamJob j;
         static_cast<StreamQuery&>(j) = s;
         j.error_out = (int*)(counts + nq + i);

@@ -103,7 +103,11 @@ struct BCtx {
   unsigned long long max_ticks;
   cudaGraphConditionalHandle cond;
   int cs;                      // CTAs per cluster the kernel was planned for
+  Gate gate;
 };
+
+// Configurations of the run (none behind a closed gate).
+__device__ inline long long items_of(const BCtx& x) { return x.gate.closed() ? 0 : x.n_cfg; }
 
 // --- cluster primitives (PTX ISA: mapa, ld.shared::cluster, barrier.cluster)
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -162,7 +166,7 @@ __device__ inline void plan_slot(const BCtx& x, BSlot& c) {
 
 __device__ inline void take(const BCtx& x, BSlot& c, unsigned long long item) {
   c.item = (long long)item; c.m0 = 0; c.G = 0; c.par = 0; c.gmask = 0u; c.hmask = 0u;
-  c.phase = (long long)item < x.n_cfg ? BP_DRAW0 : BP_EMPTY;
+  c.phase = (long long)item < items_of(x) ? BP_DRAW0 : BP_EMPTY;
   plan_slot(x, c);
 }
 
@@ -217,6 +221,7 @@ __global__ void blocked_init_kernel(BCtx x) {
   if (threadIdx.x == 0) {
     *x.work = (unsigned long long)x.K;
     *x.n_done = 0ull; *x.next_item = 0u; *x.arrive = 0u; *x.ticks = 0ull; *x.error = 0;
+    if (x.use_cond && items_of(x) == 0) cudaGraphSetConditional(x.cond, 0u);
   }
 }
 
@@ -499,7 +504,7 @@ __global__ void __launch_bounds__(kCtlThreads) blocked_control_kernel(BCtx x) {
     const unsigned long long t = *x.ticks + 1ull;
     *x.ticks = t;
     if (x.use_cond) {  // the loop ends when every configuration is done
-      const bool more = __ldcg(x.n_done) < (unsigned long long)x.n_cfg;
+      const bool more = __ldcg(x.n_done) < (unsigned long long)items_of(x);
       if (more && t >= x.max_ticks) *x.error = 1;
       cudaGraphSetConditional(x.cond, (more && t < x.max_ticks) ? 1u : 0u);
     }
@@ -577,8 +582,14 @@ pc_status run_blocked(const StreamJob& job, cudaStream_t st, bool* handled) {
   static_assert(sizeof(unsigned long long) * 3 + 4 * 3 <= 256, "counters fit the head");
   char* mem = nullptr;
   cudaError_t e = scratch_alloc((void**)&mem, head + slot_words * 4 * (size_t)K, st);
-  if (e != cudaSuccess) return cuda_fail(e, "verdict-only solver state");
+  if (e != cudaSuccess) {
+    const pc_status rc = cuda_fail(e, "verdict-only solver state");
+    if (!job.gate.at || e != cudaErrorMemoryAllocation) return rc;
+    cudaGetLastError();  // the caller has another solver for the call
+    return PC_ERR_OOM;
+  }
   BCtx x;
+  x.gate = job.gate;
   x.lat = lat; x.occ = job.occ; x.occ_bits = job.occ_bits; x.words_per_cfg = job.words_per_cfg;
   x.n_cfg = job.n_cfg; x.cfg0 = job.cfg0; x.out = job.out; x.K = (int)K;
   unsigned long long* ctr = (unsigned long long*)mem;
@@ -614,6 +625,12 @@ pc_status run_blocked(const StreamJob& job, cudaStream_t st, bool* handled) {
     blocked_init_kernel<<<1, 256, 0, st>>>(x);
     e = cudaGetLastError();
     unsigned long long ticks = 0;
+    if (e == cudaSuccess && x.gate.at) {
+      unsigned g = 0;
+      e = cudaMemcpyAsync(&g, x.gate.at, sizeof(g), cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e == cudaSuccess && (g < x.gate.lo || g >= x.gate.hi)) *done_h = (unsigned long long)job.n_cfg;
+    }
     while (e == cudaSuccess && *done_h < (unsigned long long)job.n_cfg) {
       for (int i = 0; i < kChunk && e == cudaSuccess; ++i) {
         e = cudaLaunchKernelEx(&cfg, blocked_pass_kernel, x);

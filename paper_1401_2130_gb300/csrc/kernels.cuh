@@ -14,6 +14,14 @@ struct Outputs {
   unsigned long long* n_perc;  // atomically incremented per percolating config
 };
 
+// Work that runs only where a density sampled on the device (65,536ths of the
+// sites) lies in [lo, hi).  Open if at is null.
+struct Gate {
+  const unsigned* at = nullptr;
+  unsigned lo = 0, hi = ~0u;
+  __device__ bool closed() const { return at && (*at < lo || *at >= hi); }
+};
+
 // Resident (shared-memory) solver, resident.cu.
 struct ResidentArgs {
   Lattice lat;
@@ -31,6 +39,7 @@ struct ResidentArgs {
   int prep_chunk;            // layers prepared per lazy chunk (>= 3)
   int bits_only = 0;         // reached set only: no FP32 sweep, mass written 0
   int verdict_first = 0;     // reached set first, FP32 recursion only where it percolates
+  Gate gate;
 };
 constexpr int kResidentMaxThreads = 640;  // resident CTA size limit: 20 warps at <= 96 registers
 size_t resident_smem(const Lattice& lat);
@@ -57,6 +66,10 @@ struct StreamQuery {
   // device list of n_cfg configurations (indices from 0 within the query) to
   // solve, outputs written at those indices; null = configurations 0..n_cfg-1
   const int64_t* sel = nullptr;
+  // caller occupancies: what the launches are sized for (levels, start layer),
+  // and the sampled densities that they are for
+  double density = 0.2, density_most = 0.25;
+  Gate gate;
 };
 // q on the resident solver, in CTAs of resident_threads; work: a zeroed counter.
 pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStream_t st);
@@ -91,6 +104,10 @@ pc_status run_blocked(const StreamJob& job, cudaStream_t st, bool* handled);
 // Whether run_blocked takes PC_BITS_ONLY jobs of this lattice on this device.
 bool blocked_takes(const Lattice& lat);
 
+// Largest density of a sample of caller occupancies (runs of at least 4,096
+// sites) to the zeroed word at, in 65,536ths (occupancy.cu).
+pc_status launch_bits_density(const Lattice& lat, const uint32_t* occ_bits, int64_t words_per_cfg, int64_t n_cfg,
+                              unsigned* at, cudaStream_t st);
 // Standalone occupancy draw, occupancy.cu.
 pc_status launch_occupancy(const Lattice& lat, const OccStream& os, uint32_t cfg0,
                            int64_t n_cfg, uint32_t* occ_bits, cudaStream_t st);

@@ -443,6 +443,7 @@ __device__ __forceinline__ void solve_config(const ResidentArgs& Pa, const Query
 __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(ResidentArgs Pa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long s_item;
+  if (Pa.gate.closed()) return;
   QueryState qs;
   setup_query(Pa, smem_raw, qs);
   for (;;) {

@@ -27,7 +27,7 @@ namespace pc {
 inline double resident_from(int W, int A, int L, long long n, int nsm) {
   if (L > 16 * W + 12 && (W == 0 || n > nsm)) return 1e9;  // at no density
   const double q = std::min(std::max((double)n / nsm, 1.0), 60.0);
-  return 0.0055 * std::pow((double)L, 0.7) * std::pow((double)A, 0.32) * std::pow(q, 0.4);
+  return 0.0053 * std::pow((double)L, 0.7) * std::pow((double)A, 0.32) * std::pow(q, 0.4);
 }
 
 // CTA size of the resident solver for n configurations of a lattice whose
@@ -58,15 +58,15 @@ inline double fibre_threshold(int W, int L) {
   return 0.156 + 0.58 * std::pow(w / l, -1.22) * s - 0.39 * s;
 }
 
-// Whether hardly one of n configurations of density p is expected to
+// Density below which hardly one of n configurations is expected to
 // percolate: with verdicts asked for first, their masses are then better left
 // to a pass of their own than computed for all.  Long fibres only, and the
 // farther below the threshold the more configurations there are and the
 // softer the transition is (1,854 calls measured both ways; us in one pass and
 // in two: W = 8, L = 48, 100 configurations, p = 0.18 206 / 94, p = 0.2 245 /
 // 358; W = 4, L = 48, p = 0.21, 800 of them 161 / 94).
-inline bool few_percolate(int W, int L, double p, long long n) {
-  return L >= 20 && fibre_threshold(W, L) - p > 0.1 * std::pow((double)n, 0.3) / std::sqrt((double)L * std::max(W, 1));
+inline double few_percolate_below(int W, int L, long long n) {
+  return L >= 20 ? fibre_threshold(W, L) - 0.1 * std::pow((double)n, 0.3) / std::sqrt((double)L * std::max(W, 1)) : 0.0;
 }
 
 }  // namespace pc

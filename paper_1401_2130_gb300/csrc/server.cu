@@ -121,7 +121,7 @@ pc_status start_query(pc_server* s, Ticket& t) {
   sq.n_cfg = n; sq.cfg0 = (uint32_t)q.config_begin;
   sq.out.verdict = t.v; sq.out.first_hit = t.fh; sq.out.mass = t.mass; sq.out.m_stop = t.ms;
   sq.out.n_perc = t.n_perc;
-  if (t.kind == 1 && wave_is_slower(lat, sq.occ, nullptr, n)) {
+  if (t.kind == 1 && wave_is_slower(lat, q.p, n, false)) {
     StreamJob j;
     static_cast<StreamQuery&>(j) = sq;
     j.error_out = (int*)(t.n_perc + 16);

@@ -117,7 +117,12 @@ struct Ctx {
   int nring;                    // ring slots (3 .. kMaxRing)
   int fp;                       // some query runs the FP32 recursion (else: the bits-only kernel)
   int use_cond;                 // set the WHILE condition at the end of a tick
+  Gate gate;
 };
+
+// Work items of the run (none behind a closed gate).
+__device__ inline long long items_of(const Ctx& x) { return x.gate.closed() ? 0 : x.n_items; }
+
 
 
 // items along the plane / column axis of one unit row, per kind: strip pairs
@@ -184,7 +189,7 @@ __device__ inline void fill_plan(Ctl& c, const QDev& Q) {
 __device__ inline void assign(const Ctx& x, Ctl& c, unsigned long long item) {
   c.item = (long long)item; c.m = 0; c.G = 0; c.F = 0; c.flags = 0u;
   for (int k = 0; k < U_KINDS; ++k) c.units[k] = 0;
-  if ((long long)item < x.n_items) {
+  if ((long long)item < items_of(x)) {
     c.q = query_of(x, (long long)item);
     c.phase = PH_DRAW0;
     fill_plan(c, x.qs[c.q]);
@@ -260,6 +265,7 @@ __global__ void __launch_bounds__(1024) stream_init_kernel(Ctx x) {
     *x.arrive = 0u;
     *x.next_unit = 0u;
     *x.error = 0;
+    if (x.use_cond && items_of(x) == 0) cudaGraphSetConditional(x.cond, 0u);
   }
   __threadfence();
   __syncthreads();
@@ -830,7 +836,7 @@ __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
     const unsigned t = *x.ticks + 1u;
     *x.ticks = t;
     // an error bit (expired wait, failed check) ends the loop at once
-    const bool more = *x.n_done < (unsigned long long)x.n_items && *x.error == 0;
+    const bool more = *x.n_done < (unsigned long long)items_of(x) && *x.error == 0;
     if (x.use_cond) {
       if (more && t >= x.max_ticks) *x.error = 1;
       cudaGraphSetConditional(x.cond, (more && t < x.max_ticks) ? 1u : 0u);
@@ -839,6 +845,12 @@ __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
 }
 
 }  // namespace
+
+__global__ void __launch_bounds__(256) zero_pool_kernel(Ctx x, size_t n) {
+  if (x.gate.closed()) return;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    reinterpret_cast<uint4*>(x.pool)[i] = make_uint4(0u, 0u, 0u, 0u);
+}
 
 size_t stream_slot_bytes(int W, int L) {
   int P = 0;
@@ -870,7 +882,8 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   }
   size_t free_b = 0, total_b = 0;
   PC_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  const size_t budget = pool ? pool_bytes : free_b / 2;
+  // (behind a gate, which is mostly closed, no more than the scratch pool keeps)
+  const size_t budget = pool ? pool_bytes : qs[0].gate.at ? std::min(free_b / 2, std::max(slot + 1, (size_t)1 << 30)) : free_b / 2;
   long long K = std::min<long long>(n_items, kMaxSlots);
   // PC_STREAM_MAX_SLOTS caps the pool (tests use it to force slot reuse)
   if (const char* cap = std::getenv("PC_STREAM_MAX_SLOTS")) {
@@ -887,7 +900,13 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   const size_t hdr = a256(sizeof(QDev) * nq) + a256(sizeof(Ctl) * K) + a256(sizeof(int) * (K + 1)) + 256;
   StreamPlan* P = new StreamPlan();
   cudaError_t e = scratch_alloc((void**)&P->mem, hdr + (pool ? 0 : (size_t)K * slot) + 256, st);
-  if (e != cudaSuccess) { delete P; return cuda_fail(e, "stream plan alloc"); }
+  if (e != cudaSuccess) {
+    delete P;
+    const pc_status rc = cuda_fail(e, "stream plan alloc");
+    if (!qs[0].gate.at || e != cudaErrorMemoryAllocation) return rc;
+    cudaGetLastError();  // the caller has another solver for the call
+    return PC_ERR_OOM;
+  }
   char* q = P->mem;
   Ctx& x = P->x;
   x.qs = (const QDev*)q; q += a256(sizeof(QDev) * nq);
@@ -904,6 +923,7 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   x.pool = pool ? pool : q;
   x.slot_bytes = slot;
   x.use_cond = 0;
+  x.gate = nq == 1 ? qs[0].gate : Gate();
   x.fp = 0;
   for (int i = 0; i < nq; ++i) x.fp |= qs[i].bits_only ? 0 : 1;
   {
@@ -929,7 +949,12 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
     e = cudaGetLastError();
   }
   // pool must start zeroed: padding rows / sentinel columns are never written
-  if (e == cudaSuccess) e = cudaMemsetAsync(x.pool, 0, (size_t)K * slot, st);
+  if (e == cudaSuccess && x.gate.at) {
+    zero_pool_kernel<<<1024, 256, 0, st>>>(x, (size_t)K * slot / sizeof(uint4));
+    e = cudaGetLastError();
+  } else if (e == cudaSuccess) {
+    e = cudaMemsetAsync(x.pool, 0, (size_t)K * slot, st);
+  }
   if (e != cudaSuccess) { cudaFreeAsync(P->mem, st); delete P; return cuda_fail(e, "stream plan init"); }
   P->grid = sweep_grid(x);
   *out = P;
@@ -1040,6 +1065,7 @@ pc_status run_stream(const StreamJob& job, cudaStream_t st) {
   StreamQuery q;
   q.lat = job.lat; q.occ = job.occ; q.occ_bits = job.occ_bits; q.words_per_cfg = job.words_per_cfg;
   q.n_cfg = job.n_cfg; q.cfg0 = job.cfg0; q.out = job.out; q.bits_only = job.bits_only; q.sel = job.sel;
+  q.gate = job.gate;
   StreamPlan* P = nullptr;
   pc_status rc = stream_plan_create(&q, 1, st, &P, job.pool, job.pool_bytes);
   if (rc) return rc;
@@ -1048,8 +1074,15 @@ pc_status run_stream(const StreamJob& job, cudaStream_t st) {
     // not look inside graphs with conditional nodes)
     Ctx& x = P->x;
     stream_init_kernel<<<1, 1024, 0, st>>>(x);
+    unsigned g = ~0u;
+    if (x.gate.at) {
+      cudaError_t e = cudaMemcpyAsync(&g, x.gate.at, sizeof(g), cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e != cudaSuccess) rc = cuda_fail(e, "host loop");
+    }
+    const bool closed = x.gate.at && (g < x.gate.lo || g >= x.gate.hi);
     unsigned long long done = 0;
-    for (int chunk = 0; rc == PC_OK && done < (unsigned long long)x.n_items; ++chunk) {
+    for (int chunk = 0; rc == PC_OK && !closed && done < (unsigned long long)x.n_items; ++chunk) {
       for (int i = 0; i < 32; ++i) {
         if (x.fp) sweep_kernel<true><<<P->grid, kCols, sweep_smem_bytes(x.seg_cap, x.nring, x.K), st>>>(x);
         else sweep_kernel<false><<<P->grid, kCols, sweep_smem_bytes(x.seg_cap, x.nring, x.K), st>>>(x);

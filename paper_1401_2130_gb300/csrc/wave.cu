@@ -913,6 +913,7 @@ template <int kThreads, bool kPart, int kMode>
 __global__ void __launch_bounds__(kThreads == 32 ? 128 : kThreads, kThreads == 32 ? 6 : kThreads == 128 ? 7 : kThreads == 256 ? 3 : 1)
     wave_kernel(const __grid_constant__ WaveArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (a.gate.closed()) return;
   if (kThreads == 32) {
     const int w = threadIdx.x >> 5;
     wave_body<true, kPart, kMode>(a, smem_raw + (size_t)w * a.group_smem,
@@ -947,6 +948,7 @@ __global__ void __launch_bounds__(512) wave_draw_kernel(const __grid_constant__ 
   uint32_t* tile = reinterpret_cast<uint32_t*>(smem_raw);
   const int chunks = 4 * (row1 - row0);
   const long long item = blockIdx.x / chunks;
+  if (a.gate.closed()) return;
   if (a.state[item].phase == 2) return;
   int qi = 0;
   if (a.nq > 1) {
@@ -1024,8 +1026,12 @@ struct WaveLaunch {
   size_t table_b() const { return q.size() > 1 ? up(sizeof(WaveQuery) * q.size(), 256) : 0; }
 };
 
-// Density of metallic sites (caller bits: a guess near the threshold).
-double density(const WaveQuery& w) { return w.occ_bits ? 0.2 : (double)w.occ.T / 4294967296.0; }
+double density(const WaveQuery& w) { return w.density; }
+void fill_density(WaveQuery& w, const StreamQuery& s) {
+  const double p = (double)s.occ.T / 4294967296.0;
+  w.density = (float)(s.occ_bits ? s.density : p);
+  w.density_most = (float)(s.occ_bits ? s.density_most : p);
+}
 // Sites of a level, on average over a percolating configuration: the start
 // layer, p A sites, is also about the largest (measured at W = 24: 85 at p =
 // 0.18, 141 at 0.2, 347 at 0.3, 1,576 at 0.9).
@@ -1060,7 +1066,7 @@ bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings, size_t sha
   size_t target = l.threads == 32 ? 12 * 1024 : l.threads == 128 ? 36 * 1024 : l.threads == 256 ? 72 * 1024 : most;
   if (hash) target = std::min(most, 2 * target);
   target = std::max(target, std::min(most, share));
-  w.cap = (int)std::min<long long>(w.A, (long long)(1.1 * density(w) * w.A) + 64);
+  w.cap = (int)std::min<long long>(w.A, (long long)(1.1 * w.density_most * w.A) + 64);
   const size_t head = kSharedHead + 32 * (size_t)(2 * w.W + 1);
   w.tab_bits = 0;
   size_t tab = 0;
@@ -1241,23 +1247,21 @@ pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int thr
 
 }  // namespace
 
-bool wave_is_slower(const Lattice& lat, const OccStream& occ, const uint32_t* occ_bits, long long n) {
-  // (the resident solver's masses depend on its CTA size in their last bits)
-  if (lat.A < 3000 || resident_fits(lat.W, lat.L)) return false;
+bool wave_is_slower(const Lattice& lat, double p, long long n, bool bits_only) {
+  if (lat.A < (bits_only ? 2700 : 3000) || resident_fits(lat.W, lat.L)) return false;
   int dev = 0, nsm = 1, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   WaveQuery w = {};
   fill_lattice(w, lat);
-  w.occ = occ;
-  w.occ_bits = occ_bits;
+  w.density = w.density_most = (float)p;
   WaveLaunch l;
   l.threads = 512;
   if (!place(w, l, (size_t)optin - 64, false, 0) || w.NR == 0) return true;
   const double sites = level_sites(w), k = 152.0 * (double)n / nsm;
   if (w.NR < std::min(w.TW, 2) || sites > 0.8 * w.cap || density(w) * w.A > 4.5 * w.cap) return sites > 760.0 + 20.0 * k;
-  return sites > 2600.0 + 60.0 * k;
+  return sites > (bits_only ? 2040.0 : 2600.0) + 60.0 * k;
 }
 
 bool wave_memory_suffices(const StreamQuery& s, const WaveMemory& m) try {
@@ -1268,6 +1272,7 @@ bool wave_memory_suffices(const StreamQuery& s, const WaveMemory& m) try {
   WaveQuery w = {};
   fill_lattice(w, s.lat);
   w.occ = s.occ; w.occ_bits = s.occ_bits;
+  fill_density(w, s);
   w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
   w.n_cfg = s.n_cfg;
   const int threads = std::max(group_threads(w, std::min<long long>(s.n_cfg, m.max_groups), nsm), 128);
@@ -1339,9 +1344,10 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
       fill_lattice(w, s.lat);
       w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
       w.out = s.out;
+      fill_density(w, s);
       if (std::max(group_threads(w, n_all, nsm), m ? 128 : 32) != threads) continue;
       w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
-      few = few && s.verdict_first && !s.occ_bits && few_percolate(w.W, w.L, density(w), s.n_cfg);
+      few = few && s.verdict_first && (s.occ_bits || density(w) < few_percolate_below(w.W, w.L, s.n_cfg));
       w.item0 = items; w.n_cfg = s.n_cfg;
       items += s.n_cfg;
       cq.push_back(w);
@@ -1435,6 +1441,7 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
     a.full = l.full ? 1 : 0;
     a.min_count = l.min_count;
     a.max_count = l.max_count;
+    if (nq == 1) a.gate = qs[0].gate;
     a.work = m ? m->ctr + k : (unsigned long long*)(mem + 256 * k);
     a.count = m ? m->ctr + 4 : (unsigned long long*)(mem + 256 * l.cls + 64);
     a.scratch = base;

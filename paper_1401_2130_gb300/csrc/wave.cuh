@@ -21,6 +21,7 @@ struct WaveQuery {
   uint32_t cfg0;
   Outputs out;
   int want_mass;
+  float density, density_most;  // of metallic sites: as levels, and as the start layer, are sized for
   long long item0, n_cfg;    // the query's work items
   int NR;                    // word rows of the unvisited map held in shared memory
   int nr_mask;               // row w has slot w & nr_mask
@@ -50,6 +51,7 @@ struct WaveArgs {
   int full;                  // verdicts and masses in one launch
   unsigned long long min_count, max_count;  // mass launches: run for so many percolating items
   int group_smem;
+  Gate gate;
   WaveState* state;          // [n_items]: configurations over drawn rows
   int rows_ready;            // word rows drawn
   char* scratch;
@@ -88,8 +90,10 @@ int wave_threads(int A, long long n_all);
 // 0.55 (6,300) 2,480 / 1,780; 64 of them, p = 0.75 as fast.  Beyond the queue:
 // W = 90, L = 128, verdicts, one configuration, p = 0.18 (930 sites) 1,900 /
 // 7,800, p = 0.21 (2,200) 12,000 / 5,140; W = 128, L = 512, p = 0.165 (820)
-// 127,000 / 57,100, 16 of them, L = 128, 19,900 / 18,300.
-bool wave_is_slower(const Lattice& lat, const OccStream& occ, const uint32_t* occ_bits, long long n);
+// 127,000 / 57,100, 16 of them, L = 128, 19,900 / 18,300.  Verdicts of one: W =
+// 30, L = 180, p = 0.95 (2,580) 881 / 764, p = 0.7 (1,850) 700 / 775; W = 52, L =
+// 312, p = 0.35 (2,290) 1,841 / 1,675, p = 0.25 (1,220) 1,498 / 1,857.
+bool wave_is_slower(const Lattice& lat, double density, long long n, bool bits_only);
 void release_wave();  // pc_shutdown
 
 }  // namespace pc

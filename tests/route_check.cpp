@@ -48,8 +48,8 @@ int main() {
     std::printf("threshold\n");
     return 1;
   }
-  if (!few_percolate(8, 48, 0.18, 100) || few_percolate(8, 48, 0.2, 100) || few_percolate(20, 301, 0.172, 500) ||
-      few_percolate(4, 12, 0.16, 300) || !few_percolate(6, 36, 0.19, 200)) {
+  auto few = [](int W, int L, double p, long long n) { return p < few_percolate_below(W, L, n); };
+  if (!few(8, 48, 0.18, 100) || few(8, 48, 0.2, 100) || few(20, 301, 0.172, 500) || few(4, 12, 0.16, 300) || !few(6, 36, 0.19, 200)) {
     std::printf("few\n");
     return 1;
   }
