@@ -115,7 +115,8 @@ pc_status inspect_bits(StreamJob j, unsigned long long* ctr, cudaStream_t st) {
     if (!j.bits_only) top = resident_from(lat.W, lat.A, lat.L, j.n_cfg, nsm);
     if (top <= 0.15) return run_resident(j, ctr, st);
   } else {
-    if (wave_is_slower(lat, 0.2, j.n_cfg, j.bits_only != 0)) return run_stream(j, st);
+    if (wave_is_slower(lat, 0.2, j.n_cfg, j.bits_only != 0))
+      return !j.bits_only && j.verdict_first ? run_stream_verdict_first(j, false, st) : run_stream(j, st);
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
     // (a small lattice is done before the device-wide solvers' graph is built)
@@ -243,13 +244,17 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
       if (occ_bits && !(flags & PC_MODE_STREAM)) rc = inspect_bits(j, s.work, st);
       else if (route == Route::kWave) rc = run_wave(&j, 1, st);
       else if (route == Route::kResident) rc = run_resident(j, s.work, st);
-      else rc = (!j.bits_only && first) ? run_stream_verdict_first(j, st) : run_stream(j, st);
+      else if (j.bits_only || !first) rc = run_stream(j, st);
+      // (without PC_MODE_STREAM no call waits for its stream; where most
+      // percolate, one pass is the faster way)
+      else if (!(flags & PC_MODE_STREAM) && p >= fibre_threshold(W, L)) rc = run_stream(j, st);
+      else rc = run_stream_verdict_first(j, (flags & PC_MODE_STREAM) != 0, st);
     }
     if (rc) break;
     if (!dev_out) {
       // counters, first hits, masses, step counts and verdicts lie in a row
       unsigned long long cnt = 0;
-      int err = 0;
+      int errs[2] = {0, 0};  // of the streamed solver, two passes with verdicts first
       const size_t all = 64 + (size_t)n * 13;
       HostStage stage(all);
       cudaError_t e = cudaSuccess;
@@ -261,19 +266,20 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
         if (e == cudaSuccess && mass) e = cudaMemcpyAsync(mass, s.mass, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess && m_stop) e = cudaMemcpyAsync(m_stop, s.m_stop, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, s.n_perc, 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&err, s.work + 2, sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(errs, s.work + 2, sizeof(errs), cudaMemcpyDeviceToHost, st);
       }
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
       if (e != cudaSuccess) { rc = cuda_fail(e, "copy outputs"); break; }
       if (const char* h = stage.data()) {
         std::memcpy(&cnt, h + 8, 8);
-        std::memcpy(&err, h + 16, sizeof(int));
+        std::memcpy(errs, h + 16, sizeof(errs));
         h += 64;
         if (first_hit) std::memcpy(first_hit, h, (size_t)n * 4);
         if (mass) std::memcpy(mass, h + (size_t)n * 4, (size_t)n * 4);
         if (m_stop) std::memcpy(m_stop, h + (size_t)n * 8, (size_t)n * 4);
         std::memcpy(verdicts, h + (size_t)n * 12, (size_t)n);
       }
+      const int err = errs[0] | errs[1];
       if (err & 2) { set_error("streamed solver: a bulk-copy wait timed out"); rc = PC_ERR_TIMEOUT; break; }
       if (err) { set_error("streamed solver: tick bound or device check failed"); rc = PC_ERR_INTERNAL; break; }
       if (n_percolating) *n_percolating = (int64_t)cnt;

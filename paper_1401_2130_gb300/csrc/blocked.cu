@@ -697,7 +697,7 @@ pc_status run_blocked(const StreamJob& job, cudaStream_t st, bool* handled) {
     if (job.error_out) e = cudaMemcpyAsync(job.error_out, x.error, sizeof(int), cudaMemcpyDeviceToDevice, st);
   } while (0);
   if (e != cudaSuccess) rc = cuda_fail(e, "verdict-only solver graph");
-  if (ex) cudaGraphExecDestroy(ex);  // an in-flight executable is freed on completion
+  if (ex) retire_graph(ex, st);
   if (g) cudaGraphDestroy(g);
   cudaFreeAsync(mem, st);
   *handled = true;

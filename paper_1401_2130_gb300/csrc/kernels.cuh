@@ -78,14 +78,16 @@ pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStrea
 enum class Route { kWave, kResident, kDevice };  // one SM a configuration, .., the whole device (stream.cu, blocked.cu)
 Route route_of(const Lattice& lat, const OccStream& occ, long long n, bool bits_only);
 struct StreamJob : StreamQuery {
-  int* error_out = nullptr;  // device int: 1 if the tick bound was hit
+  int* error_out = nullptr;  // device int: 1 if the tick bound was hit (verdict first without a wait: two ints)
+  const unsigned long long* n_dev = nullptr;  // device count of configurations (at most n_cfg; null: n_cfg)
   char* pool = nullptr;      // the caller's memory for the slots (else allocated)
   size_t pool_bytes = 0;
 };
 struct StreamPlan;
 // Device resources for a set of queries (stream-ordered allocation on st).
 pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, StreamPlan** out,
-                             char* pool = nullptr, size_t pool_bytes = 0);
+                             char* pool = nullptr, size_t pool_bytes = 0,
+                             const unsigned long long* n_dev = nullptr);
 // Adds [init -> WHILE(sweep, control)] to g after deps; *last = the WHILE node.
 pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps,
                           cudaGraphNode_t* last);
@@ -94,9 +96,10 @@ void stream_plan_release(StreamPlan* P, cudaStream_t st);
 size_t stream_slot_bytes(int W, int L);
 pc_status run_stream(const StreamJob& job, cudaStream_t st);
 // PC_VERDICT_FIRST on the streamed path: a verdict-only solve of every
-// configuration, then the full solve of the percolating ones (the host waits
-// for the first to count them).
-pc_status run_stream_verdict_first(const StreamJob& job, cudaStream_t st);
+// configuration, then the full solve of the percolating ones.  wait: the host
+// waits for the first to count them, and takes slots for so many; else they are
+// counted on the device, and the slots are those that the scratch pool keeps.
+pc_status run_stream_verdict_first(const StreamJob& job, bool wait, cudaStream_t st);
 // Verdict-only solver with temporal blocking (blocked.cu): runs a PC_BITS_ONLY
 // job when a thread-block cluster holds the lattice's cross-section
 // (*handled = true), else leaves it to the step-synchronous solver.

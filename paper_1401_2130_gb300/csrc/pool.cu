@@ -12,7 +12,14 @@
 // Outputs for the host come back in one copy to a pinned buffer: each of the
 // six pageable copies it replaces waits for the stream on its own.  At most
 // kBuffers buffers of kStageBytes are kept; more concurrent calls allocate and
-// free their own.  pc_shutdown gives everything back.
+// free their own.
+//
+// Executable graphs are destroyed many at a time: cudaGraphExecDestroy waits
+// until the device is idle, also for a graph that has ended (290 ms behind a
+// kernel of 290 ms), and would make an asynchronous call wait for its stream.
+// At most kRetired are kept; every kRetired-th call waits.
+//
+// pc_shutdown gives everything back.
 #include <map>
 #include <mutex>
 #include <new>
@@ -31,6 +38,11 @@ std::mutex g_mu;
 std::map<int, cudaMemPool_t> g_pools;
 char* g_stage[kBuffers];
 size_t g_stages = 0;
+
+constexpr size_t kRetired = 64;
+struct Retired { cudaGraphExec_t ex; cudaEvent_t ev; };
+Retired g_retired[kRetired];
+size_t g_retireds = 0;
 
 }  // namespace
 
@@ -94,8 +106,42 @@ HostStage::~HostStage() {
   cudaFreeHost(p_);
 }
 
+void retire_graph(cudaGraphExec_t ex, cudaStream_t st) {
+  cudaEvent_t ev = nullptr;
+  if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(ev, st) != cudaSuccess) {
+    cudaGetLastError();
+    if (ev) cudaEventDestroy(ev);
+    cudaGraphExecDestroy(ex);
+    return;
+  }
+  Retired done[kRetired];
+  size_t n = 0;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (g_retireds == kRetired) {
+      size_t left = 0;
+      for (size_t i = 0; i < kRetired; ++i) {
+        if (i == 0 || cudaEventQuery(g_retired[i].ev) == cudaSuccess) done[n++] = g_retired[i];
+        else g_retired[left++] = g_retired[i];
+      }
+      cudaGetLastError();  // "not ready"
+      g_retireds = left;
+    }
+    g_retired[g_retireds++] = Retired{ex, ev};
+  }
+  for (size_t i = 0; i < n; ++i) {
+    cudaGraphExecDestroy(done[i].ex);
+    cudaEventDestroy(done[i].ev);
+  }
+}
+
 void release_pools() {
   std::lock_guard<std::mutex> lk(g_mu);
+  for (size_t i = 0; i < g_retireds; ++i) {
+    cudaGraphExecDestroy(g_retired[i].ex);
+    cudaEventDestroy(g_retired[i].ev);
+  }
+  g_retireds = 0;
   for (auto& kv : g_pools) cudaMemPoolDestroy(kv.second);
   g_pools.clear();
   while (g_stages > 0) cudaFreeHost(g_stage[--g_stages]);

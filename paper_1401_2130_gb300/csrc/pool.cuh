@@ -24,6 +24,9 @@ class HostStage {
   char* p_ = nullptr;
 };
 
+// Takes an executable graph launched on st, to be destroyed later (pool.cu).
+void retire_graph(cudaGraphExec_t ex, cudaStream_t st);
+
 void release_pools();  // pc_shutdown
 
 }  // namespace pc

@@ -118,10 +118,13 @@ struct Ctx {
   int fp;                       // some query runs the FP32 recursion (else: the bits-only kernel)
   int use_cond;                 // set the WHILE condition at the end of a tick
   Gate gate;
+  const unsigned long long* n_dev;  // items counted on the device (null: n_items)
 };
 
 // Work items of the run (none behind a closed gate).
-__device__ inline long long items_of(const Ctx& x) { return x.gate.closed() ? 0 : x.n_items; }
+__device__ inline long long items_of(const Ctx& x) {
+  return x.gate.closed() ? 0 : x.n_dev ? min(x.n_items, (long long)*x.n_dev) : x.n_items;
+}
 
 
 
@@ -846,8 +849,8 @@ __global__ void __launch_bounds__(kCols) control_kernel(Ctx x) {
 
 }  // namespace
 
-__global__ void __launch_bounds__(256) zero_pool_kernel(Ctx x, size_t n) {
-  if (x.gate.closed()) return;
+__global__ void __launch_bounds__(256) zero_pool_kernel(Ctx x) {
+  const size_t n = (size_t)min((long long)x.K, items_of(x)) * x.slot_bytes / sizeof(uint4);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     reinterpret_cast<uint4*>(x.pool)[i] = make_uint4(0u, 0u, 0u, 0u);
 }
@@ -866,7 +869,7 @@ struct StreamPlan {
 };
 
 pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, StreamPlan** out, char* pool,
-                             size_t pool_bytes) {
+                             size_t pool_bytes, const unsigned long long* n_dev) {
   *out = nullptr;
   long long n_items = 0;
   size_t slot = 0;
@@ -882,8 +885,9 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   }
   size_t free_b = 0, total_b = 0;
   PC_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  // (behind a gate, which is mostly closed, no more than the scratch pool keeps)
-  const size_t budget = pool ? pool_bytes : qs[0].gate.at ? std::min(free_b / 2, std::max(slot + 1, (size_t)1 << 30)) : free_b / 2;
+  // (for what is mostly behind a closed gate, or few, no more than the scratch pool keeps)
+  const bool little = qs[0].gate.at || n_dev;
+  const size_t budget = pool ? pool_bytes : little ? std::min(free_b / 2, std::max(slot + 1, (size_t)1 << 30)) : free_b / 2;
   long long K = std::min<long long>(n_items, kMaxSlots);
   // PC_STREAM_MAX_SLOTS caps the pool (tests use it to force slot reuse)
   if (const char* cap = std::getenv("PC_STREAM_MAX_SLOTS")) {
@@ -924,6 +928,7 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   x.slot_bytes = slot;
   x.use_cond = 0;
   x.gate = nq == 1 ? qs[0].gate : Gate();
+  x.n_dev = n_dev;
   x.fp = 0;
   for (int i = 0; i < nq; ++i) x.fp |= qs[i].bits_only ? 0 : 1;
   {
@@ -949,8 +954,8 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
     e = cudaGetLastError();
   }
   // pool must start zeroed: padding rows / sentinel columns are never written
-  if (e == cudaSuccess && x.gate.at) {
-    zero_pool_kernel<<<1024, 256, 0, st>>>(x, (size_t)K * slot / sizeof(uint4));
+  if (e == cudaSuccess && (x.gate.at || x.n_dev)) {
+    zero_pool_kernel<<<1024, 256, 0, st>>>(x);
     e = cudaGetLastError();
   } else if (e == cudaSuccess) {
     e = cudaMemsetAsync(x.pool, 0, (size_t)K * slot, st);
@@ -1015,7 +1020,7 @@ __global__ void select_percolating_kernel(const uint8_t* verdict, int64_t n, int
 }
 }  // namespace
 
-pc_status run_stream_verdict_first(const StreamJob& job, cudaStream_t st) {
+pc_status run_stream_verdict_first(const StreamJob& job, bool wait, cudaStream_t st) {
   if (job.n_cfg <= 0) return PC_OK;
   // 1. the exact reached set decides every configuration (mass written 0)
   StreamJob b = job;
@@ -1036,21 +1041,24 @@ pc_status run_stream_verdict_first(const StreamJob& job, cudaStream_t st) {
     select_percolating_kernel<<<grid, 256, 0, st>>>(job.out.verdict, job.n_cfg, sel, cnt);
     e = cudaGetLastError();
   }
+  StreamJob f = job;
+  f.bits_only = 0;
+  f.sel = sel;
+  f.out.n_perc = nullptr;  // counted by the first pass
   int err1 = 0;  // the verdict pass's error flag: the FP32 pass rewrites error_out
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&n_sel, cnt, sizeof(n_sel), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && job.error_out)
-    e = cudaMemcpyAsync(&err1, job.error_out, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (!wait) {
+    f.n_dev = cnt;
+    if (f.error_out) ++f.error_out;
+  } else {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&n_sel, cnt, sizeof(n_sel), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && job.error_out)
+      e = cudaMemcpyAsync(&err1, job.error_out, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    f.n_cfg = (int64_t)n_sel;
+  }
   if (e != cudaSuccess) rc = cuda_fail(e, "verdict-first selection");
   else if (err1) { set_error("verdict pass: a device bound was reached"); rc = (err1 & 2) ? PC_ERR_TIMEOUT : PC_ERR_INTERNAL; }
-  if (rc == PC_OK && n_sel > 0) {
-    StreamJob f = job;
-    f.bits_only = 0;
-    f.sel = sel;
-    f.n_cfg = (int64_t)n_sel;
-    f.out.n_perc = nullptr;  // counted by the first pass
-    rc = run_stream(f, st);
-  }
+  if (rc == PC_OK && f.n_cfg > 0) rc = run_stream(f, st);
   cudaFreeAsync(mem, st);
   return rc;
 }
@@ -1062,12 +1070,8 @@ pc_status run_stream(const StreamJob& job, cudaStream_t st) {
     const pc_status rb = run_blocked(job, st, &handled);
     if (handled || rb != PC_OK) return rb;
   }
-  StreamQuery q;
-  q.lat = job.lat; q.occ = job.occ; q.occ_bits = job.occ_bits; q.words_per_cfg = job.words_per_cfg;
-  q.n_cfg = job.n_cfg; q.cfg0 = job.cfg0; q.out = job.out; q.bits_only = job.bits_only; q.sel = job.sel;
-  q.gate = job.gate;
   StreamPlan* P = nullptr;
-  pc_status rc = stream_plan_create(&q, 1, st, &P, job.pool, job.pool_bytes);
+  pc_status rc = stream_plan_create(&job, 1, st, &P, job.pool, job.pool_bytes, job.n_dev);
   if (rc) return rc;
   if (std::getenv("PC_STREAM_HOST_LOOP")) {
     // profiling aid: the same ticks launched from a host loop (profilers do
@@ -1075,14 +1079,16 @@ pc_status run_stream(const StreamJob& job, cudaStream_t st) {
     Ctx& x = P->x;
     stream_init_kernel<<<1, 1024, 0, st>>>(x);
     unsigned g = ~0u;
-    if (x.gate.at) {
-      cudaError_t e = cudaMemcpyAsync(&g, x.gate.at, sizeof(g), cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    unsigned long long done = 0, items = (unsigned long long)x.n_items;
+    {
+      cudaError_t e = cudaSuccess;
+      if (x.gate.at) e = cudaMemcpyAsync(&g, x.gate.at, sizeof(g), cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess && x.n_dev) e = cudaMemcpyAsync(&items, x.n_dev, 8, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess && (x.gate.at || x.n_dev)) e = cudaStreamSynchronize(st);
       if (e != cudaSuccess) rc = cuda_fail(e, "host loop");
+      if (x.gate.at && (g < x.gate.lo || g >= x.gate.hi)) items = 0;
     }
-    const bool closed = x.gate.at && (g < x.gate.lo || g >= x.gate.hi);
-    unsigned long long done = 0;
-    for (int chunk = 0; rc == PC_OK && !closed && done < (unsigned long long)x.n_items; ++chunk) {
+    for (int chunk = 0; rc == PC_OK && done < items; ++chunk) {
       for (int i = 0; i < 32; ++i) {
         if (x.fp) sweep_kernel<true><<<P->grid, kCols, sweep_smem_bytes(x.seg_cap, x.nring, x.K), st>>>(x);
         else sweep_kernel<false><<<P->grid, kCols, sweep_smem_bytes(x.seg_cap, x.nring, x.K), st>>>(x);
@@ -1115,7 +1121,7 @@ pc_status run_stream(const StreamJob& job, cudaStream_t st) {
       if (e != cudaSuccess) { rc = cuda_fail(e, "error copy"); break; }
     }
   } while (0);
-  if (ex) cudaGraphExecDestroy(ex);  // an in-flight executable is freed on completion
+  if (ex) retire_graph(ex, st);
   if (g) cudaGraphDestroy(g);
   stream_plan_release(P, st);
   return rc;
