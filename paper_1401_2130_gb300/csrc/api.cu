@@ -69,15 +69,21 @@ int resident_threads(const Lattice& lat, long long n) {
   return resident_cta(lat.A, lat.L, n, nsm, resident_smem(lat), (size_t)sm_smem);
 }
 
-pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStream_t st) {
+ResidentArgs resident_args(const StreamQuery& q) {
   ResidentArgs a;
   a.lat = q.lat; a.occ = q.occ; a.occ_bits = q.occ_bits; a.words_per_cfg = q.words_per_cfg;
   a.n_cfg = q.n_cfg; a.cfg0 = q.cfg0;
   a.verdict = q.out.verdict; a.first_hit = q.out.first_hit; a.mass = q.out.mass; a.m_stop = q.out.m_stop;
-  a.n_perc = q.out.n_perc; a.work = work; a.prep_chunk = 8;
+  a.n_perc = q.out.n_perc; a.work = nullptr; a.prep_chunk = 8;
   a.bits_only = q.bits_only;
   a.verdict_first = q.verdict_first;
   a.gate = q.gate;
+  return a;
+}
+
+pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStream_t st) {
+  ResidentArgs a = resident_args(q);
+  a.work = work;
   return launch_resident(a, resident_threads(q.lat, q.n_cfg), st);
 }
 

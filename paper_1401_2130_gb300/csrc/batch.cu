@@ -1,13 +1,13 @@
 // batch.cu -- pc_batch_run (one GPU submission for many queries of mixed
-// lattice sizes, on the wavefront solver) and the autotuner of the forced
-// resident solver's CTA size.
+// lattice sizes) and the autotuner of the forced resident solver's CTA size.
 //
 // A batch is the launches of run_wave: one for the levels and one for the
 // masses of each group size its lattices take, each over the configurations of
-// all its queries in decreasing lattice size.  Nothing is kept between calls.
-// (It was a CUDA graph of one resident or slot-pool launch per size class,
-// built on a batch's first call: 8 sizes x 400 configurations took 42 - 53 ms,
-// of which the W = 32 slots' ticks were most.)
+// all its queries in decreasing lattice size.  Short, thin or dense lattices of
+// resident size go to the resident solver, together, and wide dense ones to the
+// device-wide solvers.  Nothing is kept between calls.
+// (8 sizes x 400 configurations near the threshold: 1.2 ms; 42 ms as a CUDA
+// graph of the full recursion, of which the W = 32 slots' ticks were most.)
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -22,6 +22,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "pool.cuh"
+#include "route.h"
 #include "tune_file.h"
 #include "wave.cuh"
 
@@ -142,6 +143,51 @@ int size_class(const pc_query& q, const Lattice& lat, int32_t flags) {
   return (flags & PC_BITS_ONLY) && blocked_takes(lat) ? 2 : 1;
 }
 
+// Whether the queries, all of resident size, are the resident solver's: by the
+// line for their configurations together, each query with the weight of its
+// sites (so that they stay together: one launch, or a few, for all of them).
+// W = 6, 10 and 12, L = W, 10 configurations each: p = 0.25 126 us on the
+// resident solver, 158 on the wavefront solver.
+bool residents_are_faster(const std::vector<StreamQuery>& res) {
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  long long n = 0;
+  for (const StreamQuery& s : res) n += s.n_cfg;
+  double score = 0.0;
+  for (const StreamQuery& s : res) {
+    const double p = std::max((double)s.occ.T / 4294967296.0, 1e-3);
+    const double over = std::log(p / resident_from(s.lat.W, s.lat.A, s.lat.L, n, nsm));
+    score += (double)s.lat.N * (double)s.n_cfg * std::min(std::max(over, -1.0), 1.0);
+  }
+  return score > 0.0;
+}
+
+// The queries of the solvers that work on a configuration with the whole
+// device: verdicts alone one after the other where a cluster holds the
+// cross-section, the others in one pool of slots, larger lattices first (their
+// steps overlap: W = 36 and 64, L = W, p = 0.9, 10 configurations each 2,590 us,
+// one query after the other 3,618).
+pc_status run_device(std::vector<StreamQuery>& qs, int* error, cudaStream_t st) {
+  std::vector<StreamQuery> together;
+  together.reserve(qs.size());
+  int flags = 0;  // error flags used (one of each query at most)
+  for (const StreamQuery& s : qs) {
+    if (!s.bits_only || !blocked_takes(s.lat)) { together.push_back(s); continue; }
+    StreamJob j;
+    static_cast<StreamQuery&>(j) = s;
+    j.error_out = error + 2 * flags++;
+    const pc_status rc = run_stream(j, st);
+    if (rc) return rc;
+  }
+  if (together.empty()) return PC_OK;
+  std::stable_sort(together.begin(), together.end(),
+                   [](const StreamQuery& x, const StreamQuery& y) { return x.lat.N > y.lat.N; });
+  StreamJob j;
+  j.error_out = error + 2 * flags;
+  return run_streams(together.data(), (int)together.size(), j, st);
+}
+
 }  // namespace
 
 }  // namespace pc
@@ -167,9 +213,9 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
   }
   if (nq == 0) return PC_OK;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // device scratch: a counter per query, the streamed solver's error flags, and
-  // the outputs of host queries
-  const size_t ctr_b = ((size_t)nq * 16 + 255) & ~(size_t)255;
+  // device scratch: a counter per query, the streamed solver's error flags, the
+  // resident launches' counters, and the outputs of host queries
+  const size_t ctr_b = ((size_t)nq * 16 + 24 + 255) & ~(size_t)255;
   size_t bytes = ctr_b;
   if (!dev_out)
     for (int64_t i = 0; i < nq; ++i) bytes += ((size_t)q[i].n_configs * 13 + 255) & ~(size_t)255;
@@ -177,10 +223,10 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
   PC_CUDA(scratch_alloc((void**)&mem, bytes, st));
   unsigned long long* counts = (unsigned long long*)mem;
   pc_status rc = PC_OK;
-  long long n_all = 0;
-  std::vector<StreamQuery> sq;
-  std::vector<StreamJob> streamed;  // see wave_is_slower
+  std::vector<StreamQuery> sq, res, streamed;  // wavefront, resident (candidates at first), device-wide solvers
+  std::vector<int64_t> sq_i, res_i;            // their places in q
   std::vector<Lattice> lats((size_t)nq);
+  std::vector<int> threads((size_t)nq);
   do {
     cudaError_t e = cudaMemsetAsync(mem, 0, ctr_b, st);
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch counters"); break; }
@@ -206,18 +252,27 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
         s.out.m_stop = (int32_t*)(stage + 8 * n); s.out.verdict = (uint8_t*)(stage + 12 * n);
         stage += (n * 13 + 255) & ~(size_t)255;
       }
-      n_all += s.n_cfg;
-      if (wave_is_slower(s.lat, q[i].p, s.n_cfg, s.bits_only != 0)) {
-        StreamJob j;
-        static_cast<StreamQuery&>(j) = s;
-        j.error_out = (int*)(counts + nq + i);
-        streamed.push_back(j);
-      } else {
-        sq.push_back(s);
-      }
+      if (!s.bits_only && resident_fits(q[i].W, q[i].L)) { res.push_back(s); res_i.push_back(i); }
+      else if (wave_is_slower(s.lat, q[i].p, s.n_cfg, s.bits_only != 0)) streamed.push_back(s);
+      else { sq.push_back(s); sq_i.push_back(i); }
+    }
+    if (rc) break;
+    if (!residents_are_faster(res)) {
+      sq.insert(sq.end(), res.begin(), res.end());
+      sq_i.insert(sq_i.end(), res_i.begin(), res_i.end());
+      res.clear();
+      res_i.clear();
+    }
+    long long n_wave = 0;
+    for (const StreamQuery& s : sq) n_wave += s.n_cfg;
+    for (size_t k = 0; k < sq.size(); ++k) threads[(size_t)sq_i[k]] = wave_threads(sq[k], n_wave);
+    if (!res.empty()) {
+      std::vector<int> t(res.size());
+      rc = run_residents(res.data(), (int)res.size(), counts + 2 * nq, t.data(), st);
+      for (size_t k = 0; k < res.size(); ++k) threads[(size_t)res_i[k]] = t[k];
     }
     if (rc == PC_OK) rc = run_wave(sq.data(), (int)sq.size(), st);
-    for (size_t i = 0; i < streamed.size() && rc == PC_OK; ++i) rc = run_stream(streamed[i], st);
+    if (rc == PC_OK && !streamed.empty()) rc = run_device(streamed, (int*)(counts + nq), st);
     if (rc) break;
     if (dev_out)
       for (int64_t b = 0; b < nq && e == cudaSuccess; b += kCounts) {
@@ -259,7 +314,7 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
         out[i].n_percolating = (int64_t)cnt[i];
         out[i].Pi = n ? (double)cnt[i] / (double)n : 0.0;
         out[i].solver = n ? size_class(q[i], lats[(size_t)i], flags) : 0;
-        out[i].threads = out[i].solver == 0 && n ? wave_threads(lats[(size_t)i].A, n_all) : 0;
+        out[i].threads = out[i].solver == 0 && n ? threads[(size_t)i] : 0;
       }
     }
   } while (0);

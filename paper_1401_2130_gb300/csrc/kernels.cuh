@@ -73,6 +73,10 @@ struct StreamQuery {
 };
 // q on the resident solver, in CTAs of resident_threads; work: a zeroed counter.
 pc_status run_resident(const StreamQuery& q, unsigned long long* work, cudaStream_t st);
+ResidentArgs resident_args(const StreamQuery& q);  // without a work counter
+// The queries in one launch for each class of shared memory; work: three zeroed
+// counters; threads[q]: the CTA size that query q ran with.
+pc_status run_residents(const StreamQuery* qs, int nq, unsigned long long* work, int* threads, cudaStream_t st);
 // The solver that a call without a PC_MODE flag takes for n configurations of
 // occupancy stream occ.
 enum class Route { kWave, kResident, kDevice };  // one SM a configuration, .., the whole device (stream.cu, blocked.cu)
@@ -95,6 +99,9 @@ int* stream_plan_error(StreamPlan* P);
 void stream_plan_release(StreamPlan* P, cudaStream_t st);
 size_t stream_slot_bytes(int W, int L);
 pc_status run_stream(const StreamJob& job, cudaStream_t st);
+// The queries in one pool of slots that refill as configurations finish (job:
+// the run's error flag, pool and count).
+pc_status run_streams(const StreamQuery* qs, int nq, const StreamJob& job, cudaStream_t st);
 // PC_VERDICT_FIRST on the streamed path: a verdict-only solve of every
 // configuration, then the full solve of the percolating ones.  wait: the host
 // waits for the first to count them, and takes slots for so many; else they are

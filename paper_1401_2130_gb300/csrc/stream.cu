@@ -1070,8 +1070,12 @@ pc_status run_stream(const StreamJob& job, cudaStream_t st) {
     const pc_status rb = run_blocked(job, st, &handled);
     if (handled || rb != PC_OK) return rb;
   }
+  return run_streams(&job, 1, job, st);
+}
+
+pc_status run_streams(const StreamQuery* qs, int nq, const StreamJob& job, cudaStream_t st) {
   StreamPlan* P = nullptr;
-  pc_status rc = stream_plan_create(&job, 1, st, &P, job.pool, job.pool_bytes, job.n_dev);
+  pc_status rc = stream_plan_create(qs, nq, st, &P, job.pool, job.pool_bytes, job.n_dev);
   if (rc) return rc;
   if (std::getenv("PC_STREAM_HOST_LOOP")) {
     // profiling aid: the same ticks launched from a host loop (profilers do

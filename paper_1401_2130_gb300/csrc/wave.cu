@@ -1294,11 +1294,14 @@ void release_wave() {
   g_fit.clear();
 }
 
-int wave_threads(int A, long long n_all) {
+int wave_threads(const StreamQuery& q, long long n_all) {
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  return group_threads(A, n_all, nsm);
+  WaveQuery w = {};
+  fill_lattice(w, q.lat);
+  fill_density(w, q);
+  return group_threads(w, n_all, nsm);
 }
 
 size_t wave_scratch_bytes(const Lattice& lat) {
