@@ -15,6 +15,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -188,39 +189,11 @@ pc_status run_device(std::vector<StreamQuery>& qs, int* error, cudaStream_t st) 
   return run_streams(together.data(), (int)together.size(), j, st);
 }
 
-}  // namespace
-
-}  // namespace pc
-
-using namespace pc;
-
-extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags,
-                                  void* cuda_stream) {
-  NvtxRange nvtx_("pc_batch_run");
-  if (nq < 0 || (nq > 0 && !q)) { set_error("pc_batch_run: bad query array"); return PC_ERR_ARG; }
-  if (flags & ~(PC_OUT_DEVICE | PC_ASYNC | PC_BITS_ONLY | PC_VERDICT_FIRST)) { set_error("pc_batch_run: unknown flag bits"); return PC_ERR_ARG; }
+// A batch on its device scratch: counters in the first ctr_b bytes, then the
+// staging of host outputs.
+pc_status batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags, cudaStream_t st, char* mem, size_t ctr_b,
+                    size_t bytes) {
   const bool dev_out = (flags & PC_OUT_DEVICE) != 0, async = (flags & PC_ASYNC) != 0;
-  if (async && (!dev_out || out)) { set_error("PC_ASYNC needs PC_OUT_DEVICE and out == NULL"); return PC_ERR_ARG; }
-  for (int64_t i = 0; i < nq; ++i) {
-    const pc_query& x = q[i];
-    if (x.W < 0 || x.W > 255 || x.L < 1 || x.L >= (1 << 24)) { set_error("pc_batch_run: bad W or L"); return PC_ERR_ARG; }
-    if ((n_columns(x.W) + 1) * ((int64_t)x.L + 2) >= ((int64_t)1 << 31)) { set_error("pc_batch_run: lattice too large"); return PC_ERR_ARG; }
-    if (!(x.p >= 0.0 && x.p <= 1.0)) { set_error("pc_batch_run: p must be in [0, 1]"); return PC_ERR_ARG; }
-    if (x.n_configs < 0 || x.config_begin < 0 || x.config_begin + x.n_configs > ((int64_t)1 << 32)) {
-      set_error("pc_batch_run: bad configuration range"); return PC_ERR_ARG;
-    }
-    if (x.n_configs > 0 && !x.verdicts) { set_error("pc_batch_run: verdicts must not be NULL"); return PC_ERR_ARG; }
-  }
-  if (nq == 0) return PC_OK;
-  cudaStream_t st = (cudaStream_t)cuda_stream;
-  // device scratch: a counter per query, the streamed solver's error flags, the
-  // resident launches' counters, and the outputs of host queries
-  const size_t ctr_b = ((size_t)nq * 16 + 24 + 255) & ~(size_t)255;
-  size_t bytes = ctr_b;
-  if (!dev_out)
-    for (int64_t i = 0; i < nq; ++i) bytes += ((size_t)q[i].n_configs * 13 + 255) & ~(size_t)255;
-  char* mem = nullptr;
-  PC_CUDA(scratch_alloc((void**)&mem, bytes, st));
   unsigned long long* counts = (unsigned long long*)mem;
   pc_status rc = PC_OK;
   std::vector<StreamQuery> sq, res, streamed;  // wavefront, resident (candidates at first), device-wide solvers
@@ -284,12 +257,27 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
       }
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch counts"); break; }
     if (async) break;
-    // one copy of the counts and, for host queries, of every output
-    const size_t all = dev_out ? (size_t)nq * 16 : bytes;
-    HostStage pinned(all);
-    std::vector<char> plain(pinned.data() ? 0 : all);
+    // one copy of the counts and, for host queries, of every output; where that
+    // is more than the pinned buffer holds, of the counts, and each output to the
+    // caller's own array
+    HostStage pinned(dev_out ? (size_t)nq * 16 : bytes);
+    std::vector<char> plain(pinned.data() ? 0 : (size_t)nq * 16);
     const char* host = pinned.data() ? pinned.data() : plain.data();
-    e = cudaMemcpyAsync((void*)host, mem, all, cudaMemcpyDeviceToHost, st);
+    e = cudaMemcpyAsync((void*)host, mem, pinned.data() && !dev_out ? bytes : (size_t)nq * 16, cudaMemcpyDeviceToHost, st);
+    if (!pinned.data() && !dev_out) {
+      const char* from = mem + ctr_b;
+      for (int64_t i = 0; i < nq && e == cudaSuccess; ++i) {
+        const size_t n = (size_t)q[i].n_configs;
+        auto copy = [&](void* to, size_t off, size_t b) {
+          if (to && b && e == cudaSuccess) e = cudaMemcpyAsync(to, from + off, b, cudaMemcpyDeviceToHost, st);
+        };
+        copy(q[i].first_hit, 0, 4 * n);
+        copy(q[i].mass, 4 * n, 4 * n);
+        copy(q[i].m_stop, 8 * n, 4 * n);
+        copy(q[i].verdicts, 12 * n, n);
+        from += (n * 13 + 255) & ~(size_t)255;
+      }
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch outputs"); break; }
     const unsigned long long* cnt = (const unsigned long long*)host;
@@ -301,7 +289,7 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
     for (int64_t i = 0; i < nq; ++i) {
       const size_t n = (size_t)q[i].n_configs;
       if (!dev_out) {
-        if (n > 0) {
+        if (n > 0 && pinned.data()) {
           if (q[i].first_hit) std::memcpy(q[i].first_hit, at, 4 * n);
           if (q[i].mass) std::memcpy(q[i].mass, at + 4 * n, 4 * n);
           if (q[i].m_stop) std::memcpy(q[i].m_stop, at + 8 * n, 4 * n);
@@ -318,6 +306,49 @@ extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out,
       }
     }
   } while (0);
+  return rc;
+}
+
+}  // namespace
+
+}  // namespace pc
+
+using namespace pc;
+
+extern "C" pc_status pc_batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags,
+                                  void* cuda_stream) {
+  NvtxRange nvtx_("pc_batch_run");
+  if (nq < 0 || (nq > 0 && !q)) { set_error("pc_batch_run: bad query array"); return PC_ERR_ARG; }
+  if (flags & ~(PC_OUT_DEVICE | PC_ASYNC | PC_BITS_ONLY | PC_VERDICT_FIRST)) { set_error("pc_batch_run: unknown flag bits"); return PC_ERR_ARG; }
+  const bool dev_out = (flags & PC_OUT_DEVICE) != 0, async = (flags & PC_ASYNC) != 0;
+  if (async && (!dev_out || out)) { set_error("PC_ASYNC needs PC_OUT_DEVICE and out == NULL"); return PC_ERR_ARG; }
+  for (int64_t i = 0; i < nq; ++i) {
+    const pc_query& x = q[i];
+    if (x.W < 0 || x.W > 255 || x.L < 1 || x.L >= (1 << 24)) { set_error("pc_batch_run: bad W or L"); return PC_ERR_ARG; }
+    if ((n_columns(x.W) + 1) * ((int64_t)x.L + 2) >= ((int64_t)1 << 31)) { set_error("pc_batch_run: lattice too large"); return PC_ERR_ARG; }
+    if (!(x.p >= 0.0 && x.p <= 1.0)) { set_error("pc_batch_run: p must be in [0, 1]"); return PC_ERR_ARG; }
+    if (x.n_configs < 0 || x.config_begin < 0 || x.config_begin + x.n_configs > ((int64_t)1 << 32)) {
+      set_error("pc_batch_run: bad configuration range"); return PC_ERR_ARG;
+    }
+    if (x.n_configs > 0 && !x.verdicts) { set_error("pc_batch_run: verdicts must not be NULL"); return PC_ERR_ARG; }
+  }
+  if (nq == 0) return PC_OK;
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  // device scratch: a counter per query, the streamed solver's error flags, the
+  // resident launches' counters, and the outputs of host queries
+  const size_t ctr_b = ((size_t)nq * 16 + 24 + 255) & ~(size_t)255;
+  size_t bytes = ctr_b;
+  if (!dev_out)
+    for (int64_t i = 0; i < nq; ++i) bytes += ((size_t)q[i].n_configs * 13 + 255) & ~(size_t)255;
+  char* mem = nullptr;
+  PC_CUDA(scratch_alloc((void**)&mem, bytes, st));
+  pc_status rc = PC_OK;
+  try {
+    rc = batch_run(q, nq, out, flags, st, mem, ctr_b, bytes);
+  } catch (const std::bad_alloc&) {
+    set_error("pc_batch_run: no host memory");
+    rc = PC_ERR_OOM;
+  }
   const cudaError_t fe = cudaFreeAsync(mem, st);
   if (rc == PC_OK && fe != cudaSuccess) rc = cuda_fail(fe, "batch: free");
   return rc;

@@ -60,3 +60,21 @@ def test_wide_dense_queries_together():
 
 def test_sparse_and_dense_queries():
     _check([(8, 60, 0.2, 1, 0, 400), (4, 4, 0.9, 2, 0, 30), (14, 10, 0.16, 3, 0, 100), (30, 40, 0.5, 4, 0, 6)])
+
+
+def test_outputs_beyond_the_pinned_buffer():
+    """More than 4 MB of host outputs: each array goes straight to the caller's,
+    and arrays that the caller leaves out are not touched."""
+    specs = [(2, 2, 0.3, 1, 0, 300_000), (0, 1, 0.5, 2, 0, 7), (3, 2, 0.2, 3, 5, 200_000), (1, 1, 0.4, 4, 0, 0)]
+    queries, outs = pc.batch_queries(specs, device=False)
+    queries[2].first_hit = None
+    queries[0].mass = None
+    untouched = [outs[2]["first_hit"].copy(), outs[0]["mass"].copy()]
+    _, res = pc.pc_batch_run(specs, outs=outs, queries=queries)
+    assert np.array_equal(outs[2]["first_hit"], untouched[0]) and np.array_equal(outs[0]["mass"], untouched[1])
+    for i, (spec, o, r) in enumerate(zip(specs[:3], outs, res)):
+        ref = pc.pc_inspect(*spec)
+        for k in KEYS:
+            if (i, k) not in ((2, "first_hit"), (0, "mass")):
+                assert np.array_equal(o[k], ref[k]), (spec, k)
+        assert r["n_percolating"] == ref["n_percolating"]
