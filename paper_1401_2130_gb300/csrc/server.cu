@@ -9,7 +9,7 @@
 // scratch in its slots (k configurations in work at once; the device takes the
 // next configuration without the host), so queries run beside each other.  A
 // host callback behind each run wakes the worker, which copies the outputs out
-// (one copy), returns memory and slots, and admits more queries.
+// on a stream of their own, returns memory and slots, and admits more queries.
 // Latency = completion time - submission time.
 // Results equal pc_inspect's: the occupancy stream is counter based and the
 // per-configuration solve does not depend on what runs beside it.
@@ -30,6 +30,7 @@
 #include "arena.h"
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pool.cuh"
 #include "wave.cuh"
 
 namespace pc {
@@ -37,7 +38,13 @@ namespace {
 
 using Clock = std::chrono::steady_clock;
 
-constexpr int kStreams = 8;
+// Run streams.  A query has one of its own while it runs, and admission waits
+// for an idle one.  With the copies' stream they are as many as the device has
+// hardware queues by default: further streams share a queue, and a run's later
+// launches then wait behind another query's (a burst of 100 queries, W <= 32, L
+// <= 12 W, 50 to 500 configurations: 20 ms with 7, 94 with 16, 208 with 32; 8
+// given out in turn whether idle or not 189).
+constexpr int kStreams = 7;
 // scratch of a query whose state fits shared memory: stream-ordered, and at most this
 constexpr size_t kSmallScratch = 64ull << 20;
 
@@ -51,7 +58,7 @@ struct Ticket {
   pc_result result = {};
   // running state
   int kind = 0;                 // 0: fits shared memory, 1: state in arena slots
-  int stream_idx = 0;
+  int stream_idx = -1;          // its run stream
   size_t off_out = 0, bytes_out = 0, off_slots = 0, bytes_slots = 0;
   int nslots = 0;               // slots held until the query finishes
   cudaEvent_t ev = nullptr;
@@ -66,7 +73,8 @@ struct pc_server {
   pc_server_opts opts;
   int device = 0;
   cudaStream_t streams[pc::kStreams] = {};
-  int next_stream = 0;
+  cudaStream_t copy = nullptr;     // outputs of finished queries
+  bool busy[pc::kStreams] = {};    // (worker)
   char* arena_mem = nullptr;
   pc::Arena arena;
   int free_slots = 0;
@@ -113,7 +121,7 @@ pc_status start_query(pc_server* s, Ticket& t) {
   t.v = (uint8_t*)(d + 12 * n);
   cudaStream_t st = s->streams[t.stream_idx];
   PC_CUDA(cudaMemsetAsync(o, 0, 256, st));
-  StreamQuery sq;
+  StreamQuery sq;  // (counters in the first 256 bytes: percolating, the solvers' from 64 and, error flag, 128 on)
   sq.lat = lat;
   sq.occ.k0 = (uint32_t)(q.seed & 0xffffffffu); sq.occ.k1 = (uint32_t)(q.seed >> 32);
   sq.occ.cfg = 0; sq.occ.wl = (uint32_t)q.W | ((uint32_t)q.L << 8); sq.occ.T = threshold_of(q.p);
@@ -129,7 +137,8 @@ pc_status start_query(pc_server* s, Ticket& t) {
     j.pool_bytes = t.bytes_slots;
     rc = run_stream(j, st);
   } else if (t.kind == 0) {
-    rc = run_wave(&sq, 1, st, nullptr, kSmallScratch);
+    rc = route_of(lat, sq.occ, n, false) == Route::kResident ? PC_ERR_OOM : run_wave(&sq, 1, st, nullptr, kSmallScratch);
+    if (rc == PC_ERR_OOM) rc = run_resident(sq, t.n_perc + 8, st);  // needs no scratch
   } else {
     WaveMemory m;
     m.ctr = t.n_perc + 8;
@@ -145,24 +154,36 @@ pc_status start_query(pc_server* s, Ticket& t) {
   return PC_OK;
 }
 
-// Copy a finished query's outputs to the caller, release its resources.
-void finish_query(pc_server* s, Ticket& t, cudaStream_t st) {
+// Copy a finished query's outputs to the caller, release its resources.  On a
+// stream of its own: the run stream may hold the next query's run by then.
+void finish_query(pc_server* s, Ticket& t) {
   const int64_t n = t.q.n_configs;
-  // one copy: the count, then first hits, masses, step counts, verdicts
-  std::vector<char> host(256 + 13 * (size_t)n);
-  cudaError_t e = cudaMemcpyAsync(host.data(), t.n_perc, host.size(), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  // one copy: the count, then first hits, masses, step counts, verdicts; large
+  // outputs each to the caller's array
+  const size_t all = 256 + 13 * (size_t)n;
+  HostStage stage(all);
+  char head[256] = {};
+  const char* h = stage.data() ? stage.data() : head;
+  const char* o = (const char*)t.n_perc;
+  cudaError_t e = cudaMemcpyAsync((void*)h, o, stage.data() ? all : sizeof(head), cudaMemcpyDeviceToHost, s->copy);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->copy);
   unsigned long long cnt = 0;
   int err = 0;  // of the streamed solver
-  if (e == cudaSuccess) std::memcpy(&err, host.data() + 128, sizeof(int));
-  if (e == cudaSuccess && !err) {
-    const char* h = host.data();
+  if (e == cudaSuccess) {
     std::memcpy(&cnt, h, 8);
-    h += 256;
-    if (t.q.first_hit) std::memcpy(t.q.first_hit, h, 4 * (size_t)n);
-    if (t.q.mass) std::memcpy(t.q.mass, h + 4 * n, 4 * (size_t)n);
-    if (t.q.m_stop) std::memcpy(t.q.m_stop, h + 8 * n, 4 * (size_t)n);
-    if (t.q.verdicts) std::memcpy(t.q.verdicts, h + 12 * n, (size_t)n);
+    std::memcpy(&err, h + 128, sizeof(int));
+  }
+  if (e == cudaSuccess && !err) {
+    auto give = [&](void* to, size_t off, size_t b) {
+      if (!to || e != cudaSuccess) return;
+      if (stage.data()) std::memcpy(to, h + 256 + off, b);
+      else e = cudaMemcpyAsync(to, o + 256 + off, b, cudaMemcpyDeviceToHost, s->copy);
+    };
+    give(t.q.first_hit, 0, 4 * (size_t)n);
+    give(t.q.mass, 4 * (size_t)n, 4 * (size_t)n);
+    give(t.q.m_stop, 8 * (size_t)n, 4 * (size_t)n);
+    give(t.q.verdicts, 12 * (size_t)n, (size_t)n);
+    if (e == cudaSuccess && !stage.data()) e = cudaStreamSynchronize(s->copy);
   }
   // (no CUDA call under s->mu, which the host callbacks take)
   if (t.ev) { cudaEventDestroy(t.ev); t.ev = nullptr; }
@@ -209,13 +230,16 @@ void worker_main(pc_server* s) {
         const uint64_t id = s->pending.front();
         auto found = s->tickets.find(id);  // a cancelled ticket may already be polled away
         if (found == s->tickets.end() || found->second.state == T_CANCELLED) { s->pending.pop_front(); continue; }
+        int idle = 0;
+        while (idle < kStreams && s->busy[idle]) ++idle;
+        if (idle == kStreams) break;
         Ticket& t = found->second;
         const pc_query& q = t.q;
         size_t off = 0;
         const size_t ob = out_bytes(q.n_configs);
-        if (resident_fits(q.W, q.L)) {
+        if (t.kind == 0) {
           if (!s->arena.alloc(ob, &off)) break;
-          t.kind = 0; t.off_out = off; t.bytes_out = ob;
+          t.off_out = off; t.bytes_out = ob;
         } else {
           if (s->free_slots == 0) break;
           const size_t sb = stream_slot_bytes(q.W, q.L);
@@ -230,12 +254,12 @@ void worker_main(pc_server* s) {
           k = std::min<long long>(k, (long long)(room / (sb + 256)));
           size_t soff = 0;
           if (k < 1 || !s->arena.alloc((size_t)k * sb, &soff)) { s->arena.release(off, ob); break; }
-          t.kind = 1; t.off_out = off; t.bytes_out = ob;
+          t.off_out = off; t.bytes_out = ob;
           t.off_slots = soff; t.bytes_slots = (size_t)k * sb; t.nslots = (int)k;
           s->free_slots -= t.nslots;
         }
-        t.stream_idx = s->next_stream;
-        s->next_stream = (s->next_stream + 1) % kStreams;
+        t.stream_idx = idle;
+        s->busy[idle] = true;
         t.state = T_RUNNING;
         s->pending.pop_front();
         to_start.push_back(&t);  // a running ticket stays in the map (and in place) until it is polled when done
@@ -248,6 +272,7 @@ void worker_main(pc_server* s) {
       if (rc) {
         cudaStreamSynchronize(s->streams[t.stream_idx]);  // nothing of it runs on in memory given back
         if (t.ev) { cudaEventDestroy(t.ev); t.ev = nullptr; }
+        s->busy[t.stream_idx] = false;
         std::lock_guard<std::mutex> lk(s->mu);
         t.state = T_FAILED; t.status = rc;
         s->arena.release(t.off_out, t.bytes_out);
@@ -267,8 +292,12 @@ void worker_main(pc_server* s) {
         std::lock_guard<std::mutex> lk(s->mu);
         tp = &s->tickets[id];
       }
-      if (cudaEventQuery(tp->ev) != cudaErrorNotReady) finish_query(s, *tp, s->streams[tp->stream_idx]);
-      else still.push_back(id);
+      if (cudaEventQuery(tp->ev) != cudaErrorNotReady) {
+        s->busy[tp->stream_idx] = false;
+        finish_query(s, *tp);
+      } else {
+        still.push_back(id);
+      }
     }
     const bool freed = still.size() < running.size();
     running.swap(still);
@@ -308,11 +337,13 @@ pc_status pc_server_create(const pc_server_opts* opts, pc_server** out) {
   cudaGetDevice(&s->device);
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < kStreams && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&s->streams[i], cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->copy, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->arena_mem, o.hbm_budget_bytes);
   if (e != cudaSuccess) {
     pc_status rc = cuda_fail(e, "pc_server_create");
     if (s->arena_mem) cudaFree(s->arena_mem);
     for (auto r : s->streams) if (r) cudaStreamDestroy(r);
+    if (s->copy) cudaStreamDestroy(s->copy);
     delete s;
     return rc == PC_ERR_CUDA && e == cudaErrorMemoryAllocation ? PC_ERR_OOM : rc;
   }
@@ -334,7 +365,8 @@ pc_status pc_server_submit(pc_server* s, const pc_query* q, uint64_t* ticket) {
     set_error("pc_server_submit: bad p or configuration range"); return PC_ERR_ARG;
   }
   size_t need = out_bytes(q->n_configs);
-  if (!resident_fits(q->W, q->L)) {
+  const bool small = resident_fits(q->W, q->L);
+  if (!small) {
     if (q->W > s->opts.max_W) { set_error("pc_server_submit: lattice wider than the server's max_W"); return PC_ERR_ARG; }
     need += stream_slot_bytes(q->W, q->L) + 256;
   }
@@ -347,6 +379,7 @@ pc_status pc_server_submit(pc_server* s, const pc_query* q, uint64_t* ticket) {
   const uint64_t id = s->next_ticket++;
   Ticket& t = s->tickets[id];
   t.q = *q;
+  t.kind = small ? 0 : 1;
   t.t_submit = Clock::now();
   if (!s->any) { s->any = true; s->t_first = t.t_submit; }
   s->submitted += 1;
@@ -431,6 +464,7 @@ pc_status pc_server_destroy(pc_server* s) {
   for (auto& kv : s->tickets) if (kv.second.ev) cudaEventDestroy(kv.second.ev);
   cudaFree(s->arena_mem);
   for (auto r : s->streams) cudaStreamDestroy(r);
+  cudaStreamDestroy(s->copy);
   delete s;
   return PC_OK;
 }
