@@ -1336,42 +1336,49 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
   if (m) n_all = std::min(n_all, m->max_groups);
   std::vector<WaveLaunch> ls;
   int classes = 0;
-  for (int threads : {512, 256, 128, 32}) {
-    std::vector<WaveQuery> cq;
-    long long items = 0;
-    bool few = true;  // most configurations are not expected to percolate, and the caller says so
-    for (int i : order) {
-      const StreamQuery& s = qs[i];
-      // (on a caller's memory a configuration is one CTA's)
-      WaveQuery w = {};
-      fill_lattice(w, s.lat);
-      w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
-      w.out = s.out;
-      fill_density(w, s);
-      if (std::max(group_threads(w, n_all, nsm), m ? 128 : 32) != threads) continue;
-      w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
-      few = few && s.verdict_first && (s.occ_bits || density(w) < few_percolate_below(w.W, w.L, s.n_cfg));
-      w.item0 = items; w.n_cfg = s.n_cfg;
-      items += s.n_cfg;
-      cq.push_back(w);
+  auto build = [&](size_t most_ahead) -> pc_status {
+    ls.clear();
+    classes = 0;
+    for (int threads : {512, 256, 128, 32}) {
+      std::vector<WaveQuery> cq;
+      long long items = 0;
+      bool few = true;  // most configurations are not expected to percolate, and the caller says so
+      for (int i : order) {
+        const StreamQuery& s = qs[i];
+        // (on a caller's memory a configuration is one CTA's)
+        WaveQuery w = {};
+        fill_lattice(w, s.lat);
+        w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
+        w.out = s.out;
+        fill_density(w, s);
+        if (std::max(group_threads(w, n_all, nsm), m ? 128 : 32) != threads) continue;
+        w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
+        few = few && s.verdict_first && (s.occ_bits || density(w) < few_percolate_below(w.W, w.L, s.n_cfg));
+        w.item0 = items; w.n_cfg = s.n_cfg;
+        items += s.n_cfg;
+        cq.push_back(w);
+      }
+      if (cq.empty()) continue;
+      ++classes;
+      // Few configurations of large lattices: their rows are drawn by the whole
+      // device ahead of the levels, instead of by the one SM that works on them
+      // (a third of its time at W = 64).
+      bool ahead = !m && items <= nsm && threads >= 256;
+      size_t maps = 0;
+      for (const WaveQuery& w : cq) {
+        ahead = ahead && (long long)w.A * w.L >= (1 << 18) && 4 * (size_t)w.P <= (size_t)optin - 64;
+        maps = std::max(maps, 12 * (size_t)w.P * w.TW);
+      }
+      ahead = ahead && maps * (size_t)items <= most_ahead;
+      const size_t first = ls.size();
+      const pc_status rc = launches_of(cq, items, threads, nsm, optin, ahead, few, m ? m->max_groups : items, ls);
+      if (rc) return rc;
+      for (size_t k = first; k < ls.size(); ++k) ls[k].cls = classes - 1;
     }
-    if (cq.empty()) continue;
-    ++classes;
-    // Few configurations of large lattices: their rows are drawn by the whole
-    // device ahead of the levels, instead of by the one SM that works on them
-    // (a third of its time at W = 64).
-    bool ahead = !m && items <= nsm && threads >= 256;
-    size_t maps = 0;
-    for (const WaveQuery& w : cq) {
-      ahead = ahead && (long long)w.A * w.L >= (1 << 18) && 4 * (size_t)w.P <= (size_t)optin - 64;
-      maps = std::max(maps, 12 * (size_t)w.P * w.TW);
-    }
-    ahead = ahead && maps * (size_t)items <= (2ull << 30);
-    const size_t first = ls.size();
-    const pc_status rc = launches_of(cq, items, threads, nsm, optin, ahead, few, m ? m->max_groups : items, ls);
-    if (rc) return rc;
-    for (size_t k = first; k < ls.size(); ++k) ls[k].cls = classes - 1;
-  }
+    return PC_OK;
+  };
+  pc_status rc = build(std::min<size_t>(limit, 2ull << 30));
+  if (rc) return rc;
   // Grids, and one scratch for all launches (they run one after the other) of
   // at most `total` bytes, one group at least.  The launch for what the rings
   // and tables left gets what the others need.
@@ -1399,14 +1406,16 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
       }
     return PC_OK;
   };
-  size_t tables = 0;
-  size_t states = 0;
-  for (const WaveLaunch& l : ls) {
-    tables += l.table_b();
-    if (l.mode == M_PRE) states += up(sizeof(WaveState) * (size_t)l.items, 256);
-  }
-  const size_t head = 256 * ls.size() + states;
-  pc_status rc = PC_OK;
+  size_t tables = 0, states = 0, head = 0;
+  auto sizes = [&]() {
+    tables = states = 0;
+    for (const WaveLaunch& l : ls) {
+      tables += l.table_b();
+      if (l.mode == M_PRE) states += up(sizeof(WaveState) * (size_t)l.items, 256);
+    }
+    head = 256 * ls.size() + states;
+  };
+  sizes();
   cudaError_t e = cudaSuccess;
   char* mem = nullptr;
   size_t scratch = 0;
@@ -1423,6 +1432,10 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
       if (e == cudaSuccess) break;
       if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "wavefront solver: scratch");
       cudaGetLastError();
+      if (states) {  // rows drawn ahead need every configuration's at once: drawn by their groups instead
+        if ((rc = build(0))) return rc;
+        sizes();
+      }
       if (total < (1ull << 20)) {
         set_error("wavefront solver: no memory for one configuration's state");
         return PC_ERR_OOM;
