@@ -92,10 +92,8 @@ struct StreamPlan;
 pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, StreamPlan** out,
                              char* pool = nullptr, size_t pool_bytes = 0,
                              const unsigned long long* n_dev = nullptr);
-// Adds [init -> WHILE(sweep, control)] to g after deps; *last = the WHILE node.
-pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps,
-                          cudaGraphNode_t* last);
-int* stream_plan_error(StreamPlan* P);
+// Adds [init -> WHILE(sweep, control)] to g.
+pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g);
 void stream_plan_release(StreamPlan* P, cudaStream_t st);
 size_t stream_slot_bytes(int W, int L);
 pc_status run_stream(const StreamJob& job, cudaStream_t st);

@@ -966,9 +966,8 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
   return PC_OK;
 }
 
-// Adds [init kernel -> WHILE(sweep, control)] to graph g after deps.
-pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps,
-                          cudaGraphNode_t* last) {
+// Adds [init kernel -> WHILE(sweep, control)] to graph g.
+pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g) {
   Ctx& x = P->x;
   PC_CUDA(cudaGraphConditionalHandleCreate(&x.cond, g, 1, cudaGraphCondAssignDefault));
   x.use_cond = 1;
@@ -977,7 +976,7 @@ pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g, const cudaGraphNode_t* d
   kp.func = (void*)stream_init_kernel;
   kp.gridDim = dim3(1); kp.blockDim = dim3(1024); kp.sharedMemBytes = 0; kp.kernelParams = args;
   cudaGraphNode_t n_init;
-  PC_CUDA(cudaGraphAddKernelNode(&n_init, g, deps, ndeps, &kp));
+  PC_CUDA(cudaGraphAddKernelNode(&n_init, g, nullptr, 0, &kp));
   cudaGraphNodeParams cp = {};
   cp.type = cudaGraphNodeTypeConditional;
   cp.conditional.handle = x.cond;
@@ -996,11 +995,8 @@ pc_status stream_plan_add(StreamPlan* P, cudaGraph_t g, const cudaGraphNode_t* d
   cpk.func = (void*)control_kernel;
   cpk.gridDim = dim3(x.K); cpk.blockDim = dim3(kCols); cpk.kernelParams = args;
   PC_CUDA(cudaGraphAddKernelNode(&n_ctl, body, &n_sweep, 1, &cpk));
-  *last = n_while;
   return PC_OK;
 }
-
-int* stream_plan_error(StreamPlan* P) { return P->error_dev; }
 
 void stream_plan_release(StreamPlan* P, cudaStream_t st) {
   if (!P) return;
@@ -1114,8 +1110,7 @@ pc_status run_streams(const StreamQuery* qs, int nq, const StreamJob& job, cudaS
   do {
     cudaError_t e = cudaGraphCreate(&g, 0);
     if (e != cudaSuccess) { rc = cuda_fail(e, "graph create"); break; }
-    cudaGraphNode_t last;
-    if ((rc = stream_plan_add(P, g, nullptr, 0, &last))) break;
+    if ((rc = stream_plan_add(P, g))) break;
     e = cudaGraphInstantiate(&ex, g, 0);
     if (e != cudaSuccess) { rc = cuda_fail(e, "graph instantiate"); break; }
     e = cudaGraphLaunch(ex, st);

@@ -1304,21 +1304,6 @@ int wave_threads(const StreamQuery& q, long long n_all) {
   return group_threads(w, n_all, nsm);
 }
 
-size_t wave_scratch_bytes(const Lattice& lat) {
-  WaveQuery w = {};
-  fill_lattice(w, lat);
-  w.want_mass = 1;
-  size_t b = 0;
-  for (int mode : {M_LEVELS, M_HASH, M_PLANES}) {
-    WaveLaunch l;
-    l.mode = mode; l.threads = 128;
-    WaveQuery x = w;
-    // (the smallest window any launch has: evicted rows counted)
-    if (place(x, l, 48 * 1024, true, 0)) b = std::max(b, l.stride);
-  }
-  return b;
-}
-
 pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m, size_t limit) try {
   int dev = 0, nsm = 0, optin = 0;
   PC_CUDA(cudaGetDevice(&dev));

@@ -62,11 +62,11 @@ struct WaveArgs {
 struct WaveMemory {
   unsigned long long* ctr;   // 8 zeroed counters
   char* scratch;
-  size_t bytes;              // at least wave_scratch_bytes of the lattice
+  size_t bytes;              // for one configuration at least (a streamed solver's slot is larger:
+                             // its two FP32 planes of L + 4 layers and its bytes of degrees exceed
+                             // this solver's two of L layers and four bit maps)
   long long max_groups;      // configurations in work at once
 };
-// Scratch of one configuration in work on a WaveMemory.
-size_t wave_scratch_bytes(const Lattice& lat);
 // Whether m holds at least a third of the groups that the device would take at
 // once (fewer leave SMs idle).
 bool wave_memory_suffices(const StreamQuery& q, const WaveMemory& m);
