@@ -246,7 +246,14 @@ extern "C" pc_status pc_inspect_static(int32_t W, int32_t L, double p, uint64_t 
   q.n_cfg = n_configs; q.cfg0 = (uint32_t)config_begin;
   WaveMemory m;
   m.ctr = ctr + 8; m.scratch = d_wave; m.bytes = kWaveBytes; m.max_groups = n_configs;
-  const bool wave = route_of(q.lat, q.occ, n_configs, false) == Route::kWave && wave_memory_suffices(q, m);
+  bool wave = route_of(q.lat, q.occ, n_configs, false) == Route::kWave;
+  if (wave) {  // groups of one warp where the array holds enough of them, else of a CTA
+    m.warps = true;
+    if (!wave_memory_suffices(q, m)) {
+      m.warps = false;
+      wave = wave_memory_suffices(q, m);
+    }
+  }
   static_tables_kernel<<<(std::max(A, P) + 127) / 128 + 4, 128, 0, st>>>(rows, A, P, d_ppos, d_srow, d_roff,
                                                                          wave ? nullptr : d_pcol, d_sig, d_nbr, ctr);
   PC_CUDA(cudaGetLastError());

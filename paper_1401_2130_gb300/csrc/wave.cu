@@ -1275,7 +1275,7 @@ bool wave_memory_suffices(const StreamQuery& s, const WaveMemory& m) try {
   fill_density(w, s);
   w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
   w.n_cfg = s.n_cfg;
-  const int threads = std::max(group_threads(w, std::min<long long>(s.n_cfg, m.max_groups), nsm), 128);
+  const int threads = std::max(group_threads(w, std::min<long long>(s.n_cfg, m.max_groups), nsm), m.warps ? 32 : 128);
   std::vector<WaveLaunch> ls;
   if (launches_of({w}, s.n_cfg, threads, nsm, optin, false, false, m.max_groups, ls)) return false;
   for (const WaveLaunch& l : ls) {
@@ -1330,13 +1330,12 @@ pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMem
       bool few = true;  // most configurations are not expected to percolate, and the caller says so
       for (int i : order) {
         const StreamQuery& s = qs[i];
-        // (on a caller's memory a configuration is one CTA's)
         WaveQuery w = {};
         fill_lattice(w, s.lat);
         w.occ = s.occ; w.occ_bits = s.occ_bits; w.words_per_cfg = s.words_per_cfg; w.cfg0 = s.cfg0;
         w.out = s.out;
         fill_density(w, s);
-        if (std::max(group_threads(w, n_all, nsm), m ? 128 : 32) != threads) continue;
+        if (std::max(group_threads(w, n_all, nsm), m && !m->warps ? 128 : 32) != threads) continue;
         w.want_mass = (!s.bits_only && s.out.mass) ? 1 : 0;
         few = few && s.verdict_first && (s.occ_bits || density(w) < few_percolate_below(w.W, w.L, s.n_cfg));
         w.item0 = items; w.n_cfg = s.n_cfg;

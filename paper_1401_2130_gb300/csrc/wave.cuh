@@ -66,6 +66,7 @@ struct WaveMemory {
                              // its two FP32 planes of L + 4 layers and its bytes of degrees exceed
                              // this solver's two of L layers and four bit maps)
   long long max_groups;      // configurations in work at once
+  bool warps = false;        // groups of one warp too (else a configuration is a CTA's)
 };
 // Whether m holds at least a third of the groups that the device would take at
 // once (fewer leave SMs idle).
