@@ -82,15 +82,15 @@ typedef int32_t pc_status;
                                   Sec. II.B), so the reached set decides every
                                   configuration first and the FP32 recursion
                                   then runs, for exactly first_hit - 1 steps,
-                                  on the percolating ones only.  The wavefront
-                                  solver always decides first; the forced
-                                  solvers do with this flag, and with
-                                  PC_MODE_STREAM the call waits for
-                                  the verdicts before it starts the FP32
+                                  on the percolating ones only.  Without a
+                                  PC_MODE flag it is a hint that few of them
+                                  do: a pass that would compute all masses
+                                  beside the verdicts is split where that
+                                  pays.  The forced solvers decide first with
+                                  this flag; with PC_MODE_STREAM the call waits
+                                  for the verdicts before it starts the FP32
                                   solves (it synchronises cuda_stream even with
-                                  PC_OUT_DEVICE).  pc_batch_run's streamed
-                                  queries run their single pass.  Ignored with
-                                  PC_BITS_ONLY */
+                                  PC_OUT_DEVICE).  Ignored with PC_BITS_ONLY */
 
 /*
  * Lattice size (Sec. II.A): n_columns = A = 3W(W+1)+1, n_sites = A*L.
@@ -142,16 +142,22 @@ pc_status pc_occupancy_fixed(int32_t W, int32_t L, int64_t n_metallic, uint64_t 
  * PC_ERR_TIMEOUT if a bounded device wait of the streamed solver expires
  * (host outputs only: with PC_OUT_DEVICE the call returns before the device
  * work ends, except with PC_VERDICT_FIRST and PC_MODE_STREAM).
- * Solvers: without a PC_MODE flag the wavefront solver, which updates each
- * reached site once, at the step at which mass first arrives there (the
+ * (Every 64th call that the streamed solver takes waits until the device is
+ * idle.)
+ * Solvers: without a PC_MODE flag mostly the wavefront solver, which updates
+ * each reached site once, at the step at which mass first arrives there (the
  * probability at the first hit is a sum over shortest walks, so nothing else
  * of the vector enters it; its terms and their additions are the full
- * recursion's, only the last sum over the end layer has a fixed order of its
- * own).  PC_MODE_RESIDENT and PC_MODE_STREAM run the full recursion over the
- * causal window: the resident one keeps a configuration's state in one CTA's
- * shared memory (PC_ERR_OOM where it does not fit), the streamed one in HBM;
- * with PC_BITS_ONLY the streamed path runs 32 steps per visit of a slab where
- * one thread-block cluster holds the cross-section (pc_bits_blocked_shape).
+ * recursion's).  Two other solvers run the full recursion over the causal
+ * window: the resident one keeps a configuration's state in one CTA's shared
+ * memory, the streamed one in HBM; with PC_BITS_ONLY the streamed path runs 32
+ * steps per visit of a slab where one thread-block cluster holds the
+ * cross-section (pc_bits_blocked_shape).  Without a PC_MODE flag the resident
+ * one takes short, thin or dense lattices that fit it, the streamed path dense
+ * cross-sections of about 3,000 columns and more in few configurations, and
+ * those of W >= 129.  PC_MODE_RESIDENT (PC_ERR_OOM where the state does not
+ * fit) and PC_MODE_STREAM force one.  The outputs are the same bits whichever
+ * runs: the last sum, over the end layer, has one order in all of them.
  */
 pc_status pc_inspect(int32_t W, int32_t L, double p, uint64_t seed,
                      int64_t config_begin, int64_t n_configs,
@@ -162,6 +168,9 @@ pc_status pc_inspect(int32_t W, int32_t L, double p, uint64_t seed,
 /*
  * As pc_inspect, for caller-given occupancies: occ_bits is a DEVICE buffer of
  * n_configs * ceil(N/32) uint32 words in the layout pc_occupancy writes.
+ * Without a PC_MODE flag the solver is chosen on the device, from the densest
+ * part of a sample of the bits, without a wait; while cuda_stream is being
+ * captured it is the wavefront or the resident one.
  */
 pc_status pc_inspect_occupancy(int32_t W, int32_t L, const uint32_t* occ_bits,
                                int64_t n_configs, uint8_t* verdicts,
@@ -195,16 +204,20 @@ typedef struct pc_result {
                                CTA's shared memory, 2 = synchronous PC_BITS_ONLY
                                batches: one thread-block cluster holds its
                                cross-section (pc_bits_blocked_shape), 1 = else */
-  int32_t threads;          /* class 0: threads that worked on a configuration */
+  int32_t threads;          /* class 0: threads of the group or CTA that worked
+                               on a configuration's levels */
 } pc_result;
 
 /*
  * Inspect many queries of mixed lattice sizes in one GPU submission (the
- * batching of a finite-size-scaling sweep, Sec. III) on the wavefront solver:
+ * batching of a finite-size-scaling sweep, Sec. III).  On the wavefront solver:
  * one persistent launch for the levels, and one for the masses, of each group
  * size that the batch's lattices take (a warp, or a CTA of 128 to 512
  * threads), each taking the configurations of its queries from one list
- * ordered by decreasing lattice size.
+ * ordered by decreasing lattice size.  Where the queries that fit one CTA's
+ * shared memory are mostly short or dense they share a launch of the resident
+ * solver for each class of shared memory (a quarter, a half, all of an SM's);
+ * wide dense ones share one pool of the streamed solver's slots.
  * out: [n_queries] host summaries, or NULL.  Unless flags has PC_ASYNC the
  * call synchronises cuda_stream and fills out; with PC_ASYNC (requires
  * PC_OUT_DEVICE and out == NULL) it returns after enqueueing.  PC_BITS_ONLY
@@ -213,7 +226,9 @@ typedef struct pc_result {
  * Results equal those of pc_inspect on each query.
  * Threads: calls from several host threads are safe; nothing is shared
  * between calls.  Batches on several streams that name the same output
- * buffers rewrite them without waiting for one another.
+ * buffers rewrite them without waiting for one another; a caller that reads
+ * them between two such batches makes the second stream wait for its read
+ * (cudaStreamWaitEvent), or gives each batch buffers of its own.
  * Errors: PC_ERR_ARG, PC_ERR_OOM, PC_ERR_CUDA, PC_ERR_INTERNAL.
  */
 #define PC_ASYNC 0x2
@@ -226,13 +241,14 @@ pc_status pc_batch_run(const pc_query* queries, int64_t n_queries, pc_result* ou
  * as their HBM footprint -- output buffers, plus the state of max(1, min(slots
  * free, max_slots_per_query)) configurations when the lattice exceeds shared
  * memory (half of the free slots while other queries run or wait) -- fits the
- * server's device arena of hbm_budget_bytes.  Each admitted
- * query is one run of the wavefront solver on a side stream, in its own
- * memory: as many configurations in work at once as it has slots, the next
- * ones taken on the device; queries run beside each other, and new ones are
- * admitted when one ends.  (A query without slots uses at most 64 MB of
- * stream-ordered scratch besides.)  Each query's results equal pc_inspect's on
- * the same query.
+ * server's device arena of hbm_budget_bytes, and one of seven run streams is
+ * idle.  Each admitted query is one run of the solver that pc_inspect would
+ * take (but with as many configurations in work at once as it has slots), on a
+ * stream and in memory of its own; queries run beside each other, outputs are
+ * copied beside them, and new queries are admitted when one ends.  (A query
+ * without slots uses at most 64 MB of stream-ordered scratch besides, or none
+ * where it cannot be had.)  Each query's results equal pc_inspect's on the same
+ * query.
  */
 typedef struct pc_server pc_server;
 
@@ -292,7 +308,7 @@ pc_status pc_server_destroy(pc_server* s);
  * and latency-critical loops that cannot afford cudaMalloc / cudaFree, which
  * may synchronise the whole device.  This call performs no device allocation
  * of any kind: its scratch (counters, lattice tables, the solver's maps,
- * device staging of the outputs) is one static device array of about 7.7 MB
+ * device staging of the outputs) is one static device array of about 8.1 MB
  * that every GPU loading the library holds until the process exits.  (Pinned
  * host memory for the copy back is set up by the first call.)
  *
@@ -383,8 +399,9 @@ pc_status pc_bits_blocked_shape(int32_t W, int32_t* cluster_size, int32_t* colum
 pc_status pc_lazy_mass(const int32_t* first_hit, const float* mass, int64_t n_configs,
                        double hold, float* mass_lazy, int32_t flags, void* cuda_stream);
 
-/* Release cached lattice tables of every device,
- * and forget the static array's cached device addresses (pc_inspect_static).
+/* Release cached lattice tables of every device, the scratch kept between
+ * calls and executable graphs not destroyed yet (it waits for them), and forget
+ * the static array's cached device addresses (pc_inspect_static).
  * Call it after cudaDeviceReset, before any further call of the library. */
 pc_status pc_shutdown(void);
 

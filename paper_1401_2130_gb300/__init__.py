@@ -224,8 +224,9 @@ def pc_inspect(W: int, L: int, p: float, seed: int, config_begin: int, n_configs
 
     bits_only: propagate the exact reached set alone (verdicts, first_hit,
     m_stop; mass is 0).
-    verdict_first: the same outputs, bit for bit, with the FP32 recursion run
-    only on the configurations that percolate (the default solver always does).
+    verdict_first: the same outputs, bit for bit; a hint that few
+    configurations percolate (masses of these only, in a pass of their own
+    where that pays).
 
     device=False: numpy outputs plus ``n_percolating`` and ``Pi`` (the call
     synchronises).  device=True: torch CUDA tensors written asynchronously on

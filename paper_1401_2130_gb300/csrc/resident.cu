@@ -110,7 +110,7 @@ __device__ inline Smem carve(unsigned char* base, int W, int A, int L, int P, in
 __device__ inline float end_mass(const float* plane, const int32_t* ppos, int A) {
   float sum = 0.f;
   if (threadIdx.x < 32) {
-#pragma unroll 4
+#pragma unroll 16
     for (int c = threadIdx.x; c < A; c += 32) sum += plane[__ldg(ppos + c)];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);

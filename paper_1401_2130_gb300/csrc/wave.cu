@@ -15,10 +15,14 @@
 // to it to the bit.  Once every entry of a level has underflowed to 0 all
 // later ones are 0, as in the full FP32 recursion.
 //
-// wave_kernel<.., false>: levels of every configuration (verdict, first_hit,
-//   m_stop; mass 0).
-// wave_kernel<.., true>: the levels of the percolating ones again, with nu,
-//   until the end layer is reached or nu has vanished.
+// wave_kernel, by its mode:
+//   M_LEVELS, M_PRE  levels of every configuration (verdict, first_hit, m_stop;
+//                    mass 0); M_PRE: over word rows drawn by a launch before.
+//   M_HASH, M_PLANES levels with nu, until the end layer is reached or nu has
+//                    vanished: of the percolating ones after a launch for the
+//                    levels, or of all ("full", verdicts too).  nu of two levels
+//                    lives in a hash table in shared memory or in planes in
+//                    device scratch.
 //
 // A "group" (one warp, or one CTA) takes configurations from a counter.  It
 // keeps
@@ -28,21 +32,24 @@
 //          hexagon are zero).  Word rows [wb, wb + NR) live in shared memory
 //          (a ring), the others in device scratch, where the few sites whose
 //          contacts lie outside the window are handled with global atomics.
-//   queues the sites of the current and of the next level, packed t << pb |
-//          pos.  Sites beyond the queue's capacity are kept as bits of an
-//          overflow map in device scratch, so that no level is too large.
-// A level: each site of the current one tests its 14 contacts in U and claims
-// the set ones (atomicAnd), the winner appends the site to the next level.
-// One barrier per level.  Occupancy is drawn a few layers ahead of the
-// frontier from the same Philox stream as every other path.
+//   queues the sites of the current and of the next level, each as the site it
+//          was claimed from (position and hexagon row; tube) and the direction.
+//          Sites beyond the queue's capacity are kept as bits of an overflow
+//          map in device scratch, so that no level is too large.
+// A level: each site of the current one claims its 14 contacts in U, one
+// atomicAnd each without a look at the word first; whoever finds the bit still
+// set appends the contact to the next level.  One barrier per level.  Occupancy
+// is drawn a few layers ahead of the frontier from the same Philox stream as
+// every other path.
 //
 // What bounds it: a level is a chain of dependent shared-memory accesses and
 // integer instructions of one or a few warps (a warp issues one every 4.8
 // cycles), and there are first_hit - 1 of them; HBM traffic is nil.  Against
 // the full recursion, which updates every site of the window at every step
-// (us per call): W = 8, L = 64, p = 0.185, 10^4 configurations 7,230 -> 698;
-// W = 46, L = 400, p = 0.165, 32 configurations 273,000 -> 3,840; W = 64,
-// L = 4096, p = 0.17, one configuration 1,248,000 -> 41,700.
+// (us per call): W = 8, L = 64, p = 0.185, 10^4 configurations 7,230 -> 498;
+// W = 46, L = 400, p = 0.165, 32 configurations 258,000 -> 2,280; W = 64,
+// L = 4096, p = 0.17, one configuration 1,250,000 -> 17,600.  Where it is not
+// the faster one: route.h, wave_is_slower.
 #include <algorithm>
 #include <cstddef>
 #include <map>
@@ -1043,7 +1050,11 @@ double level_sites(const WaveQuery& w) {
 // Threads of a group.  With more configurations than groups fit the device,
 // few (more configurations in flight; a level's fixed cost is paid by every
 // warp); else more (a level is a chain of instructions: more warps, fewer
-// sites each), and more still where levels are large for their lattice.
+// sites each), and more still where levels are large for their lattice (from 32
+// and 100 sites a level on; without that, times what it takes: W = 24, L = 64, p
+// = 0.3, 20 configurations 1.49, W = 14, L = 100, p = 0.2, 300 of them 1.33, W =
+// 12, L = 200, p = 0.2, 60 of them 1.22; twice or half the sites: no gain in 15
+// calls).
 int group_threads(int A, long long n, int nsm) {
   if (A <= 640) return n <= 8ll * nsm ? 128 : 32;
   if (A <= 2000) return n <= 2ll * nsm ? 256 : 128;
@@ -1060,6 +1071,11 @@ int group_threads(const WaveQuery& w, long long n, int nsm) {
 // Shared memory (at most `most` bytes; `share`: of an SM's, per configuration,
 // if all of them are resident) and scratch of query w in a launch.
 // False: no room for the hash tables.
+// The targets leave an SM as many groups as its registers allow; with masses in
+// tables twice that, as fewer configurations percolate than have levels.  Half
+// of them: W = 20, L = 301, p = 0.172, 500 configurations 1.75 times the time,
+// 14 other calls as before, but W = 10, L = 100, p = 0.22, 3,000 of them 0.93.
+// Tables of twice or half the size: within 2 % over 15 calls.
 bool place(WaveQuery& w, WaveLaunch& l, size_t most, bool full_rings, size_t share) {
   const size_t row_b = sizeof(uint32_t) * (size_t)w.P;
   const bool hash = l.mode == M_HASH;
@@ -1171,7 +1187,9 @@ pc_status resident_groups(const WaveLaunch& l, int nsm, int optin, long long* n)
 //    start layer does not fit the tables, or levels are large: sixteen lanes a
 //    site cost most there (W = 24, L = 16, p = 0.95, 1,500 configurations:
 //    12,260 -> 2,410 us; L = 64, 4 configurations, 40 sites a level: 410 us in
-//    tables, 660 in planes).  With planes and nearly every configuration
+//    tables, 660 in planes).  The line, 48 sites for 128 threads: a third of it
+//    costs 1.2 to 1.3 times the time in four of 15 calls and saves 11 % in one,
+//    five times as much 1.5 to 2 times in four.  With planes and nearly every configuration
 //    percolating, levels and masses go in one pass again, with one draw (W = 14,
 //    L = 14, 1,500 configurations, p = 0.95 770 us in two passes, 588 in one; at p
 //    = 0.35 still 1.2 to 1.4 times as fast over 16 lattices) -- where no ring
@@ -1180,6 +1198,7 @@ pc_status resident_groups(const WaveLaunch& l, int nsm, int optin, long long* n)
 pc_status launches_of(const std::vector<WaveQuery>& qs, long long items, int threads, int nsm, int optin, bool ahead,
                       bool few, long long at_once, std::vector<WaveLaunch>& out) {
   const long long per_sm = (std::min(items, at_once) + nsm - 1) / nsm;
+  // (more than 32 to an SM: less than any target; not taken into account or always, 15 calls take the same)
   const size_t share = per_sm > 32 ? 0 : (size_t)optin / (size_t)per_sm - (per_sm > 1 ? 1024 : 64);
   auto make = [&](int mode, int t, bool full_rings, WaveLaunch& l) -> bool {
     l = WaveLaunch();
