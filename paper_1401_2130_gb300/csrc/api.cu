@@ -137,8 +137,12 @@ pc_status inspect_bits(StreamJob j, unsigned long long* ctr, cudaStream_t st) {
     j.gate.lo = (unsigned)(lo * 65536.0); j.gate.hi = hi > 1.0 ? ~0u : (unsigned)(hi * 65536.0);
     j.density = density; j.density_most = most;
   };
-  // (what is sized for a quarter of few columns holds all of them)
-  const double split = top <= 0.5 && 1.1 * kSparse * lat.A + 64 >= lat.A ? top : std::min(kSparse, top);
+  // (what is sized for a quarter of few columns holds more; and where the
+  // resident solver takes over soon, it takes all that is not sparse: two
+  // launches fewer)
+  const double sparse = lat.A <= 1000 ? 0.3 : kSparse;
+  if (res && top <= 0.5) top = std::min(top, sparse);
+  const double split = std::min(sparse, top);
   between(0.0, split, 0.2, kSparse);
   if ((rc = run_wave(&j, 1, st))) return rc;
   if (top <= 1.0) {
