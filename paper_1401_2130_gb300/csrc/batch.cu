@@ -139,8 +139,8 @@ __global__ void batch_counts_kernel(const unsigned long long* counts, const __gr
 // The size class of a query (pc_result.solver): 0 where its state fits one
 // CTA's shared memory, 2 where a thread-block cluster holds the cross-section
 // of a synchronous verdict-only query, else 1.
-int size_class(const pc_query& q, const Lattice& lat, int32_t flags) {
-  if (resident_fits(q.W, q.L)) return 0;
+int size_class(const Lattice& lat, bool fits, int32_t flags) {
+  if (fits) return 0;
   return (flags & PC_BITS_ONLY) && blocked_takes(lat) ? 2 : 1;
 }
 
@@ -149,10 +149,7 @@ int size_class(const pc_query& q, const Lattice& lat, int32_t flags) {
 // sites (so that they stay together: one launch, or a few, for all of them).
 // W = 6, 10 and 12, L = W, 10 configurations each: p = 0.25 126 us on the
 // resident solver, 158 on the wavefront solver.
-bool residents_are_faster(const std::vector<StreamQuery>& res) {
-  int dev = 0, nsm = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+bool residents_are_faster(const std::vector<StreamQuery>& res, int nsm) {
   long long n = 0;
   for (const StreamQuery& s : res) n += s.n_cfg;
   double score = 0.0;
@@ -200,6 +197,12 @@ pc_status batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags
   std::vector<int64_t> sq_i, res_i;            // their places in q
   std::vector<Lattice> lats((size_t)nq);
   std::vector<int> threads((size_t)nq);
+  std::vector<char> fits((size_t)nq);  // of resident size
+  // (what the device says once: asked for each query it is a microsecond of each)
+  int dev = 0, nsm = 1, optin = 0;
+  PC_CUDA(cudaGetDevice(&dev));
+  PC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  PC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   do {
     cudaError_t e = cudaMemsetAsync(mem, 0, ctr_b, st);
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch counters"); break; }
@@ -225,12 +228,13 @@ pc_status batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags
         s.out.m_stop = (int32_t*)(stage + 8 * n); s.out.verdict = (uint8_t*)(stage + 12 * n);
         stage += (n * 13 + 255) & ~(size_t)255;
       }
-      if (!s.bits_only && resident_fits(q[i].W, q[i].L)) { res.push_back(s); res_i.push_back(i); }
-      else if (wave_is_slower(s.lat, q[i].p, s.n_cfg, s.bits_only != 0)) streamed.push_back(s);
+      fits[(size_t)i] = s.lat.A <= 32767 && resident_smem(s.lat) <= (size_t)optin;
+      if (!s.bits_only && fits[(size_t)i]) { res.push_back(s); res_i.push_back(i); }
+      else if (!fits[(size_t)i] && wave_is_slower(s.lat, q[i].p, s.n_cfg, s.bits_only != 0)) streamed.push_back(s);
       else { sq.push_back(s); sq_i.push_back(i); }
     }
     if (rc) break;
-    if (!residents_are_faster(res)) {
+    if (!residents_are_faster(res, nsm)) {
       sq.insert(sq.end(), res.begin(), res.end());
       sq_i.insert(sq_i.end(), res_i.begin(), res_i.end());
       res.clear();
@@ -238,7 +242,7 @@ pc_status batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags
     }
     long long n_wave = 0;
     for (const StreamQuery& s : sq) n_wave += s.n_cfg;
-    for (size_t k = 0; k < sq.size(); ++k) threads[(size_t)sq_i[k]] = wave_threads(sq[k], n_wave);
+    for (size_t k = 0; k < sq.size(); ++k) threads[(size_t)sq_i[k]] = wave_threads(sq[k], n_wave, nsm);
     if (!res.empty()) {
       std::vector<int> t(res.size());
       rc = run_residents(res.data(), (int)res.size(), counts + 2 * nq, t.data(), st);
@@ -301,7 +305,7 @@ pc_status batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags
       if (out) {
         out[i].n_percolating = (int64_t)cnt[i];
         out[i].Pi = n ? (double)cnt[i] / (double)n : 0.0;
-        out[i].solver = n ? size_class(q[i], lats[(size_t)i], flags) : 0;
+        out[i].solver = n ? size_class(lats[(size_t)i], fits[(size_t)i] != 0, flags) : 0;
         out[i].threads = out[i].solver == 0 && n ? threads[(size_t)i] : 0;
       }
     }

@@ -498,7 +498,10 @@ struct ResidentChunk {
 };
 static_assert(sizeof(ResidentChunk) <= 4000, "kernel parameters");
 __global__ void resident_upload_kernel(ResidentQuery* dst, const __grid_constant__ ResidentChunk c) {
-  if ((int)threadIdx.x < c.n) dst[threadIdx.x] = c.q[threadIdx.x];
+  constexpr int kWords = sizeof(ResidentQuery) / 4;  // a word a thread
+  static_assert(sizeof(ResidentQuery) % 4 == 0, "whole words");
+  for (int i = threadIdx.x; i < c.n * kWords; i += blockDim.x)
+    reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(c.q)[i];
 }
 
 // Grid of a resident kernel in CTAs of `threads` with smem bytes.
@@ -586,7 +589,7 @@ pc_status run_residents(const StreamQuery* qs, int nq, unsigned long long* work,
       ResidentChunk c;
       c.n = (int)std::min<size_t>(kUpload, rq.size() - b);
       for (int i = 0; i < c.n; ++i) c.q[i] = rq[b + i];
-      resident_upload_kernel<<<1, kUpload, 0, st>>>(at + b, c);
+      resident_upload_kernel<<<1, 512, 0, st>>>(at + b, c);
       e = cudaGetLastError();
     }
     long long grid = 0;

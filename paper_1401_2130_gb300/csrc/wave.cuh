@@ -78,8 +78,8 @@ bool wave_memory_suffices(const StreamQuery& q, const WaveMemory& m);
 pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m = nullptr,
                    size_t limit = 24ull << 30);
 // Threads that work on one configuration of q (its levels) when n_all
-// configurations are inspected together on the current device.
-int wave_threads(const StreamQuery& q, long long n_all);
+// configurations are inspected together on nsm SMs.
+int wave_threads(const StreamQuery& q, long long n_all, int nsm);
 // Whether the streamed and blocked solvers, which work on a configuration with
 // the whole device, are the faster ones for n configurations: each of this
 // solver's is one SM's, so that few of them with large levels leave the device
