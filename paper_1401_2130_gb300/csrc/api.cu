@@ -3,6 +3,7 @@
 // Validates arguments, chooses the solver (route_of), allocates the call's
 // stream-ordered scratch and marshals host or device outputs.
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -109,13 +110,23 @@ namespace {
 // us per call, all launches sized for a density of 0.2 and now: W = 8, L = 48,
 // p = 0.7, 16 configurations 1,664 and 221; W = 64, L = 128, p = 0.95, verdicts
 // of one 6,218 and 598.
-pc_status inspect_bits(StreamJob j, unsigned long long* ctr, cudaStream_t st) {
+// Beyond resident size what stands behind a closed gate is not cheap: planes of
+// hundreds of MB to map, or a graph to build, 100 to 200 us of the host and 50 of
+// the device.  There the host looks for the sample for at most as long (in a
+// call that waits for its stream anyway, until it comes) and leaves the rest out,
+// or opens it, if it has come.
+pc_status inspect_bits(StreamJob j, unsigned long long* ctr, bool waits, cudaStream_t st) {
   constexpr double kSparse = 0.25;
+  // scratch of launches that may never run: within what the pool keeps
+  constexpr size_t kUnsure = 768ull << 20;
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const Lattice& lat = j.lat;
   const bool res = resident_fits(lat.W, lat.L);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+  const bool captured = capture != cudaStreamCaptureStatusNone;
   double top = 2.0;  // density from which the resident, or the device-wide, solver takes over
   if (res) {
     if (!j.bits_only) top = resident_from(lat.W, lat.A, lat.L, j.n_cfg, nsm);
@@ -123,37 +134,55 @@ pc_status inspect_bits(StreamJob j, unsigned long long* ctr, cudaStream_t st) {
   } else {
     if (wave_is_slower(lat, 0.2, j.n_cfg, j.bits_only != 0))
       return !j.bits_only && j.verdict_first ? run_stream_verdict_first(j, false, st) : run_stream(j, st);
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
     // (a small lattice is done before the device-wide solvers' graph is built)
-    if (lat.N >= 100000 && capture == cudaStreamCaptureStatusNone)
+    if (lat.N >= 100000 && !captured)
       for (int d = 5; d <= 20 && top > 1.0; ++d)
         if (wave_is_slower(lat, 0.05 * d, j.n_cfg, j.bits_only != 0)) top = 0.05 * d;
   }
-  j.gate.at = (const unsigned*)(ctr + 3);
-  pc_status rc = launch_bits_density(lat, j.occ_bits, j.words_per_cfg, j.n_cfg, (unsigned*)(ctr + 3), st);
-  if (rc) return rc;
-  auto between = [&](double lo, double hi, double density, double most) {
-    j.gate.lo = (unsigned)(lo * 65536.0); j.gate.hi = hi > 1.0 ? ~0u : (unsigned)(hi * 65536.0);
-    j.density = density; j.density_most = most;
-  };
   // (what is sized for a quarter of few columns holds more; and where the
   // resident solver takes over soon, it takes all that is not sparse: two
   // launches fewer)
-  const double sparse = lat.A <= 1000 ? 0.3 : kSparse;
+  const double sparse = lat.A <= 2200 ? 0.3 : kSparse;
   if (res && top <= 0.5) top = std::min(top, sparse);
   const double split = std::min(sparse, top);
+  const Mail mail = !res && !captured ? take_mail() : Mail();
+  pc_status rc = launch_bits_density(lat, j.occ_bits, j.words_per_cfg, j.n_cfg, (unsigned*)(ctr + 3), mail, st);
+  if (rc) return rc;
+  auto of = [](double d) { return d > 1.0 ? ~0u : (unsigned)(d * 65536.0); };
+  auto between = [&](double lo, double hi, double density, double most) {
+    j.gate.at = (const unsigned*)(ctr + 3);
+    j.gate.lo = of(lo); j.gate.hi = of(hi);
+    j.density = density; j.density_most = most;
+  };
   between(0.0, split, 0.2, kSparse);
   if ((rc = run_wave(&j, 1, st))) return rc;
-  if (top <= 1.0) {
+  unsigned g = 0;
+  bool known = false;
+  if (mail.at) {
+    const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(300);
+    while (!(known = mail.answer(&g)) && std::chrono::steady_clock::now() < until) {}
+    if (!known && waits) {
+      PC_CUDA(cudaStreamSynchronize(st));
+      known = mail.answer(&g);
+    }
+  }
+  if (known && g < of(split)) return PC_OK;
+  if (top <= 1.0 && (!known || g >= of(top))) {
     between(top, 2.0, 0.6, 1.0);
+    if (known) j.gate = Gate();
     rc = res ? run_resident(j, ctr, st) : run_stream(j, st);
-    if (rc == PC_ERR_OOM && !res) { top = 2.0; rc = PC_OK; }  // no memory for it: the wavefront solver needs less
-    if (rc) return rc;
+    // no memory for it: the wavefront solver needs less
+    if (rc != PC_ERR_OOM || res) {
+      if (rc || known) return rc;
+    } else {
+      top = 2.0;
+      rc = PC_OK;
+    }
   }
   if (top > split) {
     between(split, top, 0.6, 1.0);
-    rc = run_wave(&j, 1, st);
+    if (known) j.gate = Gate();
+    rc = run_wave(&j, 1, st, nullptr, known ? kWaveLimit : kUnsure);
   }
   return rc;
 }
@@ -251,7 +280,7 @@ pc_status inspect_impl(int32_t W, int32_t L, double p, uint64_t seed, int64_t cf
       rc = launch_resident(a, tuned_threads(lat, occ_bits ? 0.2 : p, seed, st), st);
     } else {
       const Route route = (flags & PC_MODE_STREAM) ? Route::kDevice : route_of(lat, os, n, j.bits_only != 0);
-      if (occ_bits && !(flags & PC_MODE_STREAM)) rc = inspect_bits(j, s.work, st);
+      if (occ_bits && !(flags & PC_MODE_STREAM)) rc = inspect_bits(j, s.work, !dev_out, st);
       else if (route == Route::kWave) rc = run_wave(&j, 1, st);
       else if (route == Route::kResident) rc = run_resident(j, s.work, st);
       else if (j.bits_only || !first) rc = run_stream(j, st);

@@ -112,10 +112,12 @@ pc_status run_blocked(const StreamJob& job, cudaStream_t st, bool* handled);
 // Whether run_blocked takes PC_BITS_ONLY jobs of this lattice on this device.
 bool blocked_takes(const Lattice& lat);
 
-// Largest density of a sample of caller occupancies (runs of at least 4,096
-// sites) to the zeroed word at, in 65,536ths (occupancy.cu).
+// Largest density of a sample of caller occupancies (runs of at least 1,024
+// sites), in 65,536ths: to the first of three zeroed words at, and to mail
+// (occupancy.cu).
+struct Mail;  // pool.cuh
 pc_status launch_bits_density(const Lattice& lat, const uint32_t* occ_bits, int64_t words_per_cfg, int64_t n_cfg,
-                              unsigned* at, cudaStream_t st);
+                              unsigned* at, const Mail& mail, cudaStream_t st);
 // Standalone occupancy draw, occupancy.cu.
 pc_status launch_occupancy(const Lattice& lat, const OccStream& os, uint32_t cfg0,
                            int64_t n_cfg, uint32_t* occ_bits, cudaStream_t st);

@@ -253,32 +253,45 @@ __global__ void fc_write_kernel(OccStream os, uint32_t cfg0, int64_t n_cfg, int6
 }  // namespace
 
 // A warp per run of `chunk` configurations: `words` words of each, evenly
-// spaced.
+// spaced.  The last block (at[2] counts them) answers in mail.
 static __global__ void __launch_bounds__(256) bits_density_kernel(const uint32_t* bits, int64_t wpc, int64_t n_cfg, int64_t N,
-                                                                  int64_t runs, int64_t chunk, int words, unsigned* at) {
+                                                                  int64_t runs, int64_t chunk, int words, unsigned* at,
+                                                                  Mail mail) {
   const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (r >= runs) return;
-  const int64_t c0 = runs > 1 ? r * (n_cfg - chunk) / (runs - 1) : 0;
-  unsigned set = 0, sites = 0;
-  for (int64_t k = lane; k < chunk * words; k += 32) {
-    const int64_t c = k / words, w = (k - c * words) * wpc / words, here = min((int64_t)32, N - 32 * w);
-    const uint32_t word = bits[(c0 + c) * wpc + w] & (here < 32 ? (1u << here) - 1u : 0xffffffffu);
-    set += __popc(word);
-    sites += (unsigned)here;
+  if (r < runs) {
+    const int64_t c0 = runs > 1 ? r * (n_cfg - chunk) / (runs - 1) : 0;
+    unsigned set = 0, sites = 0;
+#pragma unroll 4
+    for (int64_t k = lane; k < chunk * words; k += 32) {
+      const int64_t c = k / words, w = (k - c * words) * wpc / words, here = min((int64_t)32, N - 32 * w);
+      const uint32_t word = bits[(c0 + c) * wpc + w] & (here < 32 ? (1u << here) - 1u : 0xffffffffu);
+      set += __popc(word);
+      sites += (unsigned)here;
+    }
+    set = __reduce_add_sync(0xffffffffu, set);
+    sites = __reduce_add_sync(0xffffffffu, sites);
+    if (lane == 0 && sites) atomicMax(at, (unsigned)(((uint64_t)set << 16) / sites));
   }
-  set = __reduce_add_sync(0xffffffffu, set);
-  sites = __reduce_add_sync(0xffffffffu, sites);
-  if (lane == 0 && sites) atomicMax(at, (unsigned)(((uint64_t)set << 16) / sites));
+  if (!mail.at) return;  // grid-uniform
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(at + 2, 1u) == gridDim.x - 1) {
+      __threadfence();
+      *(volatile unsigned long long*)mail.at = (unsigned long long)mail.tag << 32 | atomicMax(at, 0u);
+      __threadfence_system();
+    }
+  }
 }
 
 pc_status launch_bits_density(const Lattice& lat, const uint32_t* occ_bits, int64_t words_per_cfg, int64_t n_cfg,
-                              unsigned* at, cudaStream_t st) {
-  const int64_t chunk = std::min<int64_t>(n_cfg, (4096 + lat.N - 1) / lat.N);
+                              unsigned* at, const Mail& mail, cudaStream_t st) {
+  const int64_t chunk = std::min<int64_t>(n_cfg, (1024 + lat.N - 1) / lat.N);
   const int words = (int)std::min<int64_t>(words_per_cfg, 128);
   const int64_t runs = std::min<int64_t>(n_cfg / chunk, 4096);
   bits_density_kernel<<<(unsigned)((runs * 32 + 255) / 256), 256, 0, st>>>(occ_bits, words_per_cfg, n_cfg, lat.N, runs, chunk,
-                                                                          words, at);
+                                                                          words, at, mail);
   PC_CUDA(cudaGetLastError());
   return PC_OK;
 }

@@ -19,10 +19,13 @@
 // kernel of 290 ms), and would make an asynchronous call wait for its stream.
 // At most kRetired are kept; every kRetired-th call waits.
 //
+// Mails (take_mail) are kMails words of pinned memory.
+//
 // pc_shutdown gives everything back.
 #include <map>
 #include <mutex>
 #include <new>
+#include <vector>
 
 #include "pool.cuh"
 
@@ -38,6 +41,10 @@ std::mutex g_mu;
 std::map<int, cudaMemPool_t> g_pools;
 char* g_stage[kBuffers];
 size_t g_stages = 0;
+
+constexpr unsigned kMails = 4096;
+unsigned long long* g_mail = nullptr;
+unsigned g_tag = 0;
 
 constexpr size_t kRetired = 64;
 struct Retired { cudaGraphExec_t ex; cudaEvent_t ev; };
@@ -106,6 +113,31 @@ HostStage::~HostStage() {
   cudaFreeHost(p_);
 }
 
+bool Mail::answer(unsigned* v) const {
+  if (!at) return false;
+  const unsigned long long x = *(const volatile unsigned long long*)at;
+  *v = (unsigned)x;
+  return (unsigned)(x >> 32) == tag;
+}
+
+Mail take_mail() {
+  Mail m;
+  std::lock_guard<std::mutex> lk(g_mu);
+  if (!g_mail) {
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, kMails * sizeof(unsigned long long), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      return m;
+    }
+    g_mail = (unsigned long long*)p;
+    for (size_t i = 0; i < kMails; ++i) g_mail[i] = 0ull;
+  }
+  if (++g_tag == 0u) ++g_tag;
+  m.tag = g_tag;
+  m.at = g_mail + g_tag % kMails;
+  return m;
+}
+
 void retire_graph(cudaGraphExec_t ex, cudaStream_t st) {
   cudaEvent_t ev = nullptr;
   if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(ev, st) != cudaSuccess) {
@@ -142,9 +174,22 @@ void release_pools() {
     cudaEventDestroy(g_retired[i].ev);
   }
   g_retireds = 0;
+  std::vector<int> devices;
+  for (const auto& kv : g_pools) devices.push_back(kv.first);
   for (auto& kv : g_pools) cudaMemPoolDestroy(kv.second);
   g_pools.clear();
   while (g_stages > 0) cudaFreeHost(g_stage[--g_stages]);
+  if (g_mail) {  // no kernel may still write into it
+    int now = 0;
+    cudaGetDevice(&now);
+    for (int dev : devices) {
+      cudaSetDevice(dev);
+      cudaDeviceSynchronize();
+    }
+    cudaSetDevice(now);
+    cudaFreeHost(g_mail);
+  }
+  g_mail = nullptr;
   cudaGetLastError();  // after cudaDeviceReset the handles are gone already
 }
 

@@ -27,6 +27,16 @@ class HostStage {
 // Takes an executable graph launched on st, to be destroyed later (pool.cu).
 void retire_graph(cudaGraphExec_t ex, cudaStream_t st);
 
+// A word of pinned memory that a kernel answers a call in: it writes tag << 32 |
+// answer.  Nobody waits for it, and the word is another call's kMails calls
+// later: an answer with another tag is no answer.
+struct Mail {
+  unsigned long long* at = nullptr;  // null: no pinned memory
+  unsigned tag = 0;
+  bool answer(unsigned* v) const;    // (host) true if it has come
+};
+Mail take_mail();
+
 void release_pools();  // pc_shutdown
 
 }  // namespace pc

@@ -75,8 +75,9 @@ bool wave_memory_suffices(const StreamQuery& q, const WaveMemory& m);
 // Inspects the queries (stream-ordered, no host synchronisation).  Without m
 // the scratch is allocated on st, at most `limit` bytes where that is enough
 // for one configuration; with m (one query) nothing is allocated.
+constexpr size_t kWaveLimit = 24ull << 30;
 pc_status run_wave(const StreamQuery* qs, int nq, cudaStream_t st, const WaveMemory* m = nullptr,
-                   size_t limit = 24ull << 30);
+                   size_t limit = kWaveLimit);
 // Threads that work on one configuration of q (its levels) when n_all
 // configurations are inspected together on nsm SMs.
 int wave_threads(const StreamQuery& q, long long n_all, int nsm);

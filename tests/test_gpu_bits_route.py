@@ -36,13 +36,16 @@ def _check(W, L, bits, what):
     n = bits.shape[0]
     ref = pc.pc_inspect_occupancy(W, L, bits, mode=pc.PC_MODE_STREAM)
     for mode in (0, pc.PC_BITS_ONLY, pc.PC_VERDICT_FIRST):
-        for device in (False, True):
+        # the sample comes in time, or behind other work on the stream it does not
+        for device, busy in ((False, False), (True, False), (True, True), (False, True)):
+            if busy:
+                torch.cuda._sleep(1_000_000)
             g = pc.pc_inspect_occupancy(W, L, bits, mode=mode, device=device)
             torch.cuda.synchronize()
             g = {k: v.cpu().numpy() if hasattr(v, "cpu") else v for k, v in g.items()}
             for k in KEYS:
                 want = np.zeros(n, np.float32) if k == "mass" and mode == pc.PC_BITS_ONLY else ref[k]
-                assert np.array_equal(g[k], want), (what, mode, device, k)
+                assert np.array_equal(g[k], want), (what, mode, device, busy, k)
             assert int(np.asarray(g["n_percolating"]).reshape(-1)[0]) == ref["n_percolating"]
 
 
