@@ -168,9 +168,11 @@ pc_status pc_inspect(int32_t W, int32_t L, double p, uint64_t seed,
 /*
  * As pc_inspect, for caller-given occupancies: occ_bits is a DEVICE buffer of
  * n_configs * ceil(N/32) uint32 words in the layout pc_occupancy writes.
- * Without a PC_MODE flag the solver is chosen on the device, from the densest
- * part of a sample of the bits, without a wait; while cuda_stream is being
- * captured it is the wavefront or the resident one.
+ * Without a PC_MODE flag the solver follows from the densest part of a sample of
+ * the bits that the device takes.  No call with PC_OUT_DEVICE waits for its
+ * stream; for lattices beyond shared memory the host looks for the sample for at
+ * most 0.3 ms before it leaves the choice to the device.  While cuda_stream is
+ * being captured the solver is the wavefront or the resident one.
  */
 pc_status pc_inspect_occupancy(int32_t W, int32_t L, const uint32_t* occ_bits,
                                int64_t n_configs, uint8_t* verdicts,
