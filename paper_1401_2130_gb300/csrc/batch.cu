@@ -149,9 +149,18 @@ int size_class(const Lattice& lat, bool fits, int32_t flags) {
 // sites (so that they stay together: one launch, or a few, for all of them).
 // W = 6, 10 and 12, L = W, 10 configurations each: p = 0.25 126 us on the
 // resident solver, 158 on the wavefront solver.
-bool residents_are_faster(const std::vector<StreamQuery>& res, int nsm) {
+// Never beside as many sites on the wavefront solver: its launch takes them along
+// (W = 3, 23 and 32, L = 3 W and 4 W, p = 0.137, 34 configurations each 261 us, with
+// W = 3 on the resident solver 314).
+bool residents_are_faster(const std::vector<StreamQuery>& res, const std::vector<StreamQuery>& wave, int nsm) {
   long long n = 0;
-  for (const StreamQuery& s : res) n += s.n_cfg;
+  double sites = 0.0;
+  for (const StreamQuery& s : res) {
+    n += s.n_cfg;
+    sites += (double)s.lat.N * (double)s.n_cfg;
+  }
+  for (const StreamQuery& s : wave) sites -= (double)s.lat.N * (double)s.n_cfg;
+  if (sites <= 0.0) return false;
   double score = 0.0;
   for (const StreamQuery& s : res) {
     const double p = std::max((double)s.occ.T / 4294967296.0, 1e-3);
@@ -234,7 +243,7 @@ pc_status batch_run(const pc_query* q, int64_t nq, pc_result* out, int32_t flags
       else { sq.push_back(s); sq_i.push_back(i); }
     }
     if (rc) break;
-    if (!residents_are_faster(res, nsm)) {
+    if (!residents_are_faster(res, sq, nsm)) {
       sq.insert(sq.end(), res.begin(), res.end());
       sq_i.insert(sq_i.end(), res_i.begin(), res_i.end());
       res.clear();
