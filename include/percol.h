@@ -243,7 +243,7 @@ pc_status pc_batch_run(const pc_query* queries, int64_t n_queries, pc_result* ou
  * as their HBM footprint -- output buffers, plus the state of max(1, min(slots
  * free, max_slots_per_query)) configurations when the lattice exceeds shared
  * memory (half of the free slots while other queries run or wait) -- fits the
- * server's device arena of hbm_budget_bytes, and one of seven run streams is
+ * server's device arena of hbm_budget_bytes, and one of six run streams is
  * idle.  Each admitted query is one run of the solver that pc_inspect would
  * take (but with as many configurations in work at once as it has slots), on a
  * stream and in memory of its own; queries run beside each other, outputs are

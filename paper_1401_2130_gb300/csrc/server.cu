@@ -39,12 +39,13 @@ namespace {
 using Clock = std::chrono::steady_clock;
 
 // Run streams.  A query has one of its own while it runs, and admission waits
-// for an idle one.  With the copies' stream they are as many as the device has
-// hardware queues by default: further streams share a queue, and a run's later
-// launches then wait behind another query's (a burst of 100 queries, W <= 32, L
-// <= 12 W, 50 to 500 configurations: 20 ms with 7, 94 with 16, 208 with 32; 8
-// given out in turn whether idle or not 189).
-constexpr int kStreams = 7;
+// for an idle one.  With the copies' stream they are fewer than the device's
+// hardware queues by default (eight): further streams share a queue, and a run's
+// later launches then wait behind another query's (a burst of 100 queries, W <=
+// 32, L <= 12 W, 50 to 500 configurations: 20 ms with 6 or 7, 94 with 16, 208 with
+// 32; 8 given out in turn whether idle or not 189).  50 bursts of 3 to 9 queries:
+// 6 are 3 % faster than 7 or 8, and 6 % than 10.
+constexpr int kStreams = 6;
 // scratch of a query whose state fits shared memory: stream-ordered, and at most this
 constexpr size_t kSmallScratch = 64ull << 20;
 
