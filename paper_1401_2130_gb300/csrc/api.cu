@@ -108,8 +108,8 @@ namespace {
 // route_of gives such a stream.  Verdicts first: masses in a pass of their own.  ctr: counters of the call, zeroed; ctr[0] is
 // the resident solver's, ctr[3] takes the sample.
 // us per call, all launches sized for a density of 0.2 and now: W = 8, L = 48,
-// p = 0.7, 16 configurations 1,664 and 221; W = 64, L = 128, p = 0.95, verdicts
-// of one 6,218 and 598.
+// p = 0.7, 16 configurations 1,664 and 212; W = 64, L = 128, p = 0.95, verdicts
+// of one 6,218 and 503.
 // Beyond resident size what stands behind a closed gate is not cheap: planes of
 // hundreds of MB to map, or a graph to build, 100 to 200 us of the host and 50 of
 // the device.  There the host looks for the sample for at most as long (in a
