@@ -105,16 +105,17 @@ namespace {
 // others (each an empty launch, about 2 us).  Sparse: the wavefront solver,
 // queues and tables sized for up to a quarter of the sites.  Denser: sized for
 // all of them (near 0.2 that costs occupancy).  Denser still: the solver that
-// route_of gives such a stream.  Verdicts first: masses in a pass of their own.  ctr: counters of the call, zeroed; ctr[0] is
-// the resident solver's, ctr[3] takes the sample.
+// route_of gives such a stream.  Verdicts first: masses in a pass of their own.
 // us per call, all launches sized for a density of 0.2 and now: W = 8, L = 48,
 // p = 0.7, 16 configurations 1,664 and 212; W = 64, L = 128, p = 0.95, verdicts
 // of one 6,218 and 503.
 // Beyond resident size what stands behind a closed gate is not cheap: planes of
 // hundreds of MB to map, or a graph to build, 100 to 200 us of the host and 50 of
-// the device.  There the host looks for the sample for at most as long (in a
-// call that waits for its stream anyway, until it comes) and leaves the rest out,
-// or opens it, if it has come.
+// the device.  There the host looks for the sample for 0.3 ms at most (in a call
+// that waits for its stream anyway, until it comes) and leaves the rest out, or
+// opens it, if it has come.
+// ctr: counters of the call, zeroed; ctr[0] is the resident solver's, ctr[3] and
+// ctr[4] are the sample's.
 pc_status inspect_bits(StreamJob j, unsigned long long* ctr, bool waits, cudaStream_t st) {
   constexpr double kSparse = 0.25;
   // scratch of launches that may never run: within what the pool keeps
