@@ -535,7 +535,8 @@ bool pick_shape(const Lattice& lat, Shape* out) {
     Shape s;
     s.cs = cs; s.cpr = cpr; s.threads = (cpr + 31) / 32 * 32; s.nrow = 4 * nq;
     s.smem = 48 * (cpr + 1) * nq;
-    if (cudaFuncSetAttribute(blocked_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem) != cudaSuccess) {
+    // the same limit on every call: calls from several threads never lower it
+    if (cudaFuncSetAttribute(blocked_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, budget) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }

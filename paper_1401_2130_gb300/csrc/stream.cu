@@ -936,8 +936,14 @@ pc_status stream_plan_create(const StreamQuery* qs, int nq, cudaStream_t st, Str
     for (int i = 0; i < nq; ++i) cap = std::max(cap, max_pair_segment(qs[i].lat.W, kCols) + 16);
     x.seg_cap = x.fp ? cap : 0;
     x.nring = x.fp ? ring_depth(cap) : 0;
-    const int bytes = sweep_smem_bytes(x.seg_cap, x.nring, x.K);
-    cudaError_t ea = cudaFuncSetAttribute(sweep_fn(x), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    // the same limit on every call: calls from several threads never lower it
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t ea = cudaGetDevice(&dev);
+    if (ea == cudaSuccess) ea = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (ea == cudaSuccess) ea = cudaFuncGetAttributes(&fa, sweep_fn(x));
+    if (ea == cudaSuccess)
+      ea = cudaFuncSetAttribute(sweep_fn(x), cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
     if (ea != cudaSuccess) { cudaFreeAsync(P->mem, st); delete P; return cuda_fail(ea, "sweep smem"); }
   }
   // every configuration needs at most N + 3 ticks; slots run concurrently
